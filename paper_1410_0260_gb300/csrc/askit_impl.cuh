@@ -38,6 +38,34 @@ void askit_set_error(const char *fmt, ...);
         ASK_CUDA(cudaGetLastError());                \
     } while (0)
 
+// Launches kernel k so that it may start while the kernel before it on the
+// stream still runs (programmatic stream serialization).  Every kernel launched
+// this way calls pdl_wait() in every thread before it reads or writes anything
+// that an earlier kernel of the stream touches; what it does before that
+// (barriers, TMEM, operands fixed at setup) overlaps the earlier kernel's tail.
+// The first kernel of a call is launched normally.
+template <class... KArgs, class... Args>
+inline askit_status launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                               const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    ASK_CUDA(cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...));
+    return ASKIT_OK;
+}
+// Lets the next kernel of the stream be launched once every block has got here.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Waits until the earlier kernels of the stream have completed (no-op after a
+// normal launch).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Sticky device status codes (written by kernels with bounded waits).
 enum { ASK_DEV_OK = 0, ASK_DEV_TIMEOUT = 1, ASK_DEV_BAD_ITEM = 2 };
 
@@ -215,8 +243,11 @@ struct askit_tree_s {
     int32_t *skel_ids = nullptr;  // [skel_total]
     int32_t *piv = nullptr;       // [piv_total]
     double *P64 = nullptr;        // [p_total]
-    float *P32 = nullptr;         // [p_total]
-    int64_t *d_skoff = nullptr, *d_pivoff = nullptr, *d_poff = nullptr, *d_spool = nullptr;
+    // FP32 copy for the upward pass: node a's rows start at d_p32off[a] and are
+    // (c_a - s_a) floats padded with zeros to a multiple of 4 apart (16-byte loads)
+    float *P32 = nullptr;
+    std::vector<int> lvl_nr;      // [L + 1] largest c_a - s_a of each level
+    int64_t *d_skoff = nullptr, *d_pivoff = nullptr, *d_p32off = nullptr, *d_spool = nullptr;
     int32_t *d_s = nullptr, *d_ncol = nullptr;
 
     // evaluation operands

@@ -239,9 +239,9 @@ askit_status setup_impl(askit_tree t, const float *X_dev, int64_t ldx, const flo
         t->h_poff.assign(nn + 1, 0); t->h_spool.assign(nn + 1, 0);
         ASK_TRY(t->arena.alloc(&t->skel_ids, 1)); ASK_TRY(t->arena.alloc(&t->piv, 1));
         ASK_TRY(t->arena.alloc(&t->P64, 1)); ASK_TRY(t->arena.alloc(&t->P32, 1));
-        ASK_TRY(t->arena.alloc(&t->d_poff, nn + 1)); ASK_TRY(t->arena.alloc(&t->d_skoff, nn + 1));
+        ASK_TRY(t->arena.alloc(&t->d_p32off, nn + 1)); ASK_TRY(t->arena.alloc(&t->d_skoff, nn + 1));
         ASK_TRY(t->arena.alloc(&t->d_pivoff, nn + 1)); ASK_TRY(t->arena.alloc(&t->d_spool, nn + 1));
-        ASK_CUDA(cudaMemsetAsync(t->d_poff, 0, sizeof(int64_t) * (nn + 1), s));
+        ASK_CUDA(cudaMemsetAsync(t->d_p32off, 0, sizeof(int64_t) * (nn + 1), s));
         ASK_CUDA(cudaMemsetAsync(t->d_skoff, 0, sizeof(int64_t) * (nn + 1), s));
         ASK_CUDA(cudaMemsetAsync(t->d_pivoff, 0, sizeof(int64_t) * (nn + 1), s));
         ASK_CUDA(cudaMemsetAsync(t->d_spool, 0, sizeof(int64_t) * (nn + 1), s));

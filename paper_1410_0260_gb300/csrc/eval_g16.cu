@@ -229,6 +229,7 @@ eval_g16_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_const
                      ::"r"(smem_u32(tmem_slot)), "r"(G_TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();          // the set-up above overlaps the kernels before; everything below reads their results
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -699,11 +700,13 @@ eval_g16_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_const
 template <int RC>
 __global__ void g16_cols_kernel(const int64_t *sb_row0, const int32_t *sb_nr, int64_t n_leaf_sub, const float *Wt,
                                 const float *Ws, int r, float *colw) {
+    pdl_trigger();
     const int64_t b = blockIdx.x;
     const int t = threadIdx.x;
     const bool far = b >= n_leaf_sub;
     const int64_t row = sb_row0[b] + t;
     const bool valid = t < sb_nr[b];
+    pdl_wait();
     const float *w = (far ? Ws : Wt) + row * r;
 #pragma unroll
     for (int z = 0; z < RC; ++z) colw[(b * 128 + t) * RC + z] = (valid && z < r) ? w[z] : 0.f;
@@ -717,10 +720,12 @@ __global__ void g16_cols_kernel(const int64_t *sb_row0, const int32_t *sb_nr, in
 // and vectors past r are zero.
 __global__ void g16_wcols_kernel(const int64_t *sb_row0, const int32_t *sb_nr, int64_t n_leaf_sub, const float *Wt,
                                  const float *Ws, int r, uint8_t *colw) {
+    pdl_trigger();
     __shared__ float wmax[4][16];
     const int64_t b = blockIdx.x;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const bool valid = t < sb_nr[b];
+    pdl_wait();
     const float *w = (b >= n_leaf_sub ? Ws : Wt) + (sb_row0[b] + t) * r;
     float v[16];
 #pragma unroll
@@ -784,10 +789,8 @@ askit_status launch_g16(G16State *st, const G16Args &a, int grid, cudaStream_t s
     static const cudaError_t attr = cudaFuncSetAttribute(eval_g16_kernel<RC, NA, NB>,
                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     ASK_CUDA(attr);
-    eval_g16_kernel<RC, NA, NB><<<(unsigned)grid, S::THREADS, smem, s>>>(st->map[0], st->map[1], st->map[2],
-                                                                         st->map[3], a);
-    ASK_LAUNCH();
-    return ASKIT_OK;
+    return launch_pdl(eval_g16_kernel<RC, NA, NB>, dim3((unsigned)grid), dim3(S::THREADS), smem, s, st->map[0],
+                      st->map[1], st->map[2], st->map[3], a);
 }
 
 template <int RC>
@@ -798,12 +801,11 @@ askit_status run_g16(askit_tree t, const WeightCtx &c, G16State *st, G16Args a, 
     // weights, r > 4 split for the weight MMA
     float *colw = RC == 1 ? reinterpret_cast<float *>(c.colv) : c.colw;
     if constexpr (SG<RC, 3, 1>::WMMA)
-        g16_wcols_kernel<<<(unsigned)t->n_sub, 128, 0, s>>>(t->sb_row0, t->sb_nr, t->n_leaf_sub, c.Wt, c.Ws, c.r,
-                                                            reinterpret_cast<uint8_t *>(colw));
+        ASK_TRY(launch_pdl(g16_wcols_kernel, dim3((unsigned)t->n_sub), dim3(128), 0, s, t->sb_row0, t->sb_nr,
+                           t->n_leaf_sub, c.Wt, c.Ws, c.r, reinterpret_cast<uint8_t *>(colw)));
     else
-        g16_cols_kernel<RC><<<(unsigned)t->n_sub, 128, 0, s>>>(t->sb_row0, t->sb_nr, t->n_leaf_sub, c.Wt, c.Ws, c.r,
-                                                               colw);
-    ASK_LAUNCH();
+        ASK_TRY(launch_pdl(g16_cols_kernel<RC>, dim3((unsigned)t->n_sub), dim3(128), 0, s, t->sb_row0, t->sb_nr,
+                           t->n_leaf_sub, c.Wt, c.Ws, c.r, colw));
     a.colw = colw;
     ASK_TRY(ktimer_mark(t, s, false));
     // three or four target-row stages (one or two items' copies in flight);

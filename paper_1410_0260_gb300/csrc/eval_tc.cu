@@ -153,6 +153,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
                      ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();          // the set-up above overlaps the kernels before; everything below reads their results
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -639,9 +640,8 @@ askit_status launch(askit_tree t, TcState *st, const CUtensorMap &map_q, const T
     }
     const unsigned grid = (unsigned)a_grid;
     ASK_TRY(ktimer_mark(t, s, false));
-    eval_tc_kernel<P, RC><<<grid, TC_THREADS, smem, s>>>(st->map[pi][0], st->map[pi][1], st->map[pi][2],
-                                                         st->map[pi][3], map_q, st->raw_t, st->raw_s, a);
-    ASK_LAUNCH();
+    ASK_TRY(launch_pdl(eval_tc_kernel<P, RC>, dim3(grid), dim3(TC_THREADS), smem, s, st->map[pi][0], st->map[pi][1],
+                       st->map[pi][2], st->map[pi][3], map_q, st->raw_t, st->raw_s, a));
     return ktimer_mark(t, s, true);
 }
 

@@ -178,6 +178,7 @@ eval_tc16_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                      ::"r"(smem_u32(tmem_slot)), "r"(T16_TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();          // the set-up above overlaps the kernels before; everything below reads their results
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -659,11 +660,13 @@ template <int RC, int UNI>
 __global__ void tc16_cols_kernel(const int64_t *sb_row0, const int32_t *sb_nr, int64_t n_leaf_sub, const float *sc_t,
                                  const float *sc_s, const float *nrm_t, const float *nrm_s, const float *Wt,
                                  const float *Ws, int r, float g_unscale, float4 *colv, float *colw) {
+    pdl_trigger();
     const int64_t b = blockIdx.x;
     const int t = threadIdx.x;
     const bool far = b >= n_leaf_sub;
     const int64_t row = sb_row0[b] + t;
     const bool valid = t < sb_nr[b];
+    pdl_wait();
     const float sc = valid ? (far ? sc_s : sc_t)[row] : 0.f;
     const float nrm = valid ? (far ? nrm_s : nrm_t)[row] : 0.f;
     const float *w = (far ? Ws : Wt) + row * r;
@@ -761,10 +764,8 @@ askit_status launch16(T16State *st, int pi, const CUtensorMap &map_q, const CUte
     static const cudaError_t attr = cudaFuncSetAttribute(eval_tc16_kernel<P, RC, NRAW, NB, UNI>,
                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     ASK_CUDA(attr);
-    eval_tc16_kernel<P, RC, NRAW, NB, UNI><<<(unsigned)grid, S::THREADS, smem, s>>>(
-        st->map[pi][0], st->map[pi][1], st->map[pi][2], st->map[pi][3], map_q, map_q8, a);
-    ASK_LAUNCH();
-    return ASKIT_OK;
+    return launch_pdl(eval_tc16_kernel<P, RC, NRAW, NB, UNI>, dim3((unsigned)grid), dim3(S::THREADS), smem, s,
+                      st->map[pi][0], st->map[pi][1], st->map[pi][2], st->map[pi][3], map_q, map_q8, a);
 }
 
 template <int P, int RC>
@@ -779,15 +780,14 @@ askit_status run16(askit_tree t, const WeightCtx &c, T16State *st, int pi, const
         const float sc = (float)(t->prm.kernel_scale * 1.4426950408889634 / (hf * hf));
         a.uni_a = 2.f * g_unscale * sc;
         a.uni_c = -sc;
-        tc16_cols_kernel<RC, 1><<<(unsigned)t->n_sub, 128, 0, s>>>(t->sb_row0, t->sb_nr, t->n_leaf_sub, t->sc_t,
-                                                                   t->sc_s, t->nrmc_t, t->nrmc_s, c.Wt, c.Ws, c.r,
-                                                                   g_unscale, c.colv, c.colw);
+        ASK_TRY(launch_pdl(tc16_cols_kernel<RC, 1>, dim3((unsigned)t->n_sub), dim3(128), 0, s, t->sb_row0, t->sb_nr,
+                           t->n_leaf_sub, t->sc_t, t->sc_s, t->nrmc_t, t->nrmc_s, c.Wt, c.Ws, c.r, g_unscale, c.colv,
+                           c.colw));
     } else {
-        tc16_cols_kernel<RC, 0><<<(unsigned)t->n_sub, 128, 0, s>>>(t->sb_row0, t->sb_nr, t->n_leaf_sub, t->sc_t,
-                                                                   t->sc_s, t->nrmc_t, t->nrmc_s, c.Wt, c.Ws, c.r,
-                                                                   g_unscale, c.colv, c.colw);
+        ASK_TRY(launch_pdl(tc16_cols_kernel<RC, 0>, dim3((unsigned)t->n_sub), dim3(128), 0, s, t->sb_row0, t->sb_nr,
+                           t->n_leaf_sub, t->sc_t, t->sc_s, t->nrmc_t, t->nrmc_s, c.Wt, c.Ws, c.r, g_unscale, c.colv,
+                           c.colw));
     }
-    ASK_LAUNCH();
     a.colv = c.colv;
     a.colw = c.colw;
     auto go = [&]() -> askit_status {

@@ -178,6 +178,7 @@ eval_tcw_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_const
                      ::"r"(smem_u32(tmem_slot)), "r"(W_TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_wait();          // the set-up above overlaps the kernels before; everything below reads their results
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -662,8 +663,8 @@ askit_status launch_w(askit_tree t, TcwState *st, int pi, const TcwArgs &a, int 
     ASK_CUDA(attr);
     ASK_TRY(ktimer_mark(t, s, false));
     const CUtensorMap *m = st->map[pi][NB - 1];
-    eval_tcw_kernel<P, RC, NB><<<(unsigned)grid, W_THREADS, smem, s>>>(m[0], m[1], m[2], m[3], m[4], m[5], a);
-    ASK_LAUNCH();
+    ASK_TRY(launch_pdl(eval_tcw_kernel<P, RC, NB>, dim3((unsigned)grid), dim3(W_THREADS), smem, s, m[0], m[1], m[2],
+                       m[3], m[4], m[5], a));
     return ktimer_mark(t, s, true);
 }
 

@@ -280,17 +280,28 @@ __global__ void __launch_bounds__(QR_THREADS) cpqr_kernel(
 __global__ void skel_out_kernel(const int32_t *batch_nodes, int64_t a0, const int64_t *poff_ws,
                                 const int64_t *poff_lvl, const int32_t *s, const int32_t *ncol,
                                 const int32_t *cols, int cmax, const int32_t *piv_fixed, int s_max,
-                                const double *work, int32_t *skel_fixed, double *P64, float *P32) {
+                                const double *work, int32_t *skel_fixed, double *P64) {
     int g = blockIdx.x;
     int64_t a = batch_nodes[g];
     int sa = s[a], c = ncol[a];
     for (int q = threadIdx.x; q < sa; q += blockDim.x)
         skel_fixed[a * s_max + q] = cols[(a - a0) * cmax + piv_fixed[a * cmax + q]];
     int64_t np = (int64_t)sa * (c - sa);
-    for (int64_t e = threadIdx.x; e < np; e += blockDim.x) {
-        double x = work[poff_ws[g] + e];
-        P64[poff_lvl[g] + e] = x;
-        P32[poff_lvl[g] + e] = (float)x;
+    for (int64_t e = threadIdx.x; e < np; e += blockDim.x) P64[poff_lvl[g] + e] = work[poff_ws[g] + e];
+}
+
+// The FP32 copy of P the upward pass reads: node a = 2 + block, rows padded
+// with zeros to a multiple of 4 columns.
+__global__ void p32_kernel(const double *P64, const int64_t *poff, const int64_t *p32off, const int32_t *s,
+                           const int32_t *ncol, float *P32) {
+    const int64_t a = 2 + blockIdx.x;
+    const int sa = s[a], nr = ncol[a] - sa, ldp = (nr + 3) & ~3;
+    const double *src = P64 + poff[a];
+    float *dst = P32 + p32off[a];
+    for (int64_t e = threadIdx.x; e < (int64_t)sa * ldp; e += blockDim.x) {
+        const int64_t q = e / ldp;
+        const int u = (int)(e % ldp);
+        dst[e] = u < nr ? (float)src[q * nr + u] : 0.f;
     }
 }
 
@@ -419,7 +430,6 @@ askit_status skeletonize(askit_tree t, cudaStream_t s) {
     ASK_CUDA(cudaMemsetAsync(t->d_s, 0, sizeof(int32_t) * nn, s));
 
     std::vector<double *> lvl_P64(L + 1, nullptr);
-    std::vector<float *> lvl_P32(L + 1, nullptr);
     std::vector<int64_t> lvl_ptot(L + 1, 0);
     std::vector<int64_t> node_poff(nn, 0);   // offset within its level pool
     const size_t budget = (size_t)6 << 30;   // FP64 workspace per batch
@@ -437,8 +447,7 @@ askit_status skeletonize(askit_tree t, cudaStream_t s) {
         ASK_LAUNCH();
         // level pool for P (sizes known only after the QR of each batch)
         std::vector<double *> batch_P64;
-        std::vector<float *> batch_P32;
-            std::vector<int64_t> batch_tot;
+        std::vector<int64_t> batch_tot;
         int64_t a = a0;
         int64_t lvl_run = 0;   // offset of the current batch inside the level pool
         while (a < a1) {
@@ -495,17 +504,14 @@ askit_status skeletonize(askit_tree t, cudaStream_t s) {
                 tot += (int64_t)t->h_s[nd] * (t->h_ncol[nd] - t->h_s[nd]);
             }
             double *P64 = nullptr;
-            float *P32 = nullptr;
             ASK_CUDA(cudaMalloc(&P64, sizeof(double) * (tot ? tot : 1)));
-            ASK_CUDA(cudaMalloc(&P32, sizeof(float) * (tot ? tot : 1)));
             ASK_CUDA(cudaMemcpyAsync(d_plvl, plvl.data(), sizeof(int64_t) * nb, cudaMemcpyHostToDevice, s));
             skel_out_kernel<<<nb, 256, 0, s>>>(d_nodes, a0, d_pws, d_plvl, t->d_s, t->d_ncol, cols, cmax,
-                                              piv_fixed, s_max, work, skel_fixed, P64, P32);
+                                              piv_fixed, s_max, work, skel_fixed, P64);
             ASK_LAUNCH();
             ASK_CUDA(cudaStreamSynchronize(s));
             cudaFree(work); cudaFree(d_nodes); cudaFree(d_woff); cudaFree(d_pws); cudaFree(d_plvl);
             batch_P64.push_back(P64);
-            batch_P32.push_back(P32);
             batch_tot.push_back(tot);
             lvl_run += tot;
         }
@@ -514,15 +520,13 @@ askit_status skeletonize(askit_tree t, cudaStream_t s) {
         int64_t ltot = 0;
         for (auto x : batch_tot) ltot += x;
         ASK_CUDA(cudaMalloc(&lvl_P64[depth], sizeof(double) * (ltot ? ltot : 1)));
-        ASK_CUDA(cudaMalloc(&lvl_P32[depth], sizeof(float) * (ltot ? ltot : 1)));
         int64_t off = 0;
         for (size_t b = 0; b < batch_tot.size(); ++b) {
             ASK_CUDA(cudaMemcpyAsync(lvl_P64[depth] + off, batch_P64[b], sizeof(double) * batch_tot[b], cudaMemcpyDeviceToDevice, s));
-            ASK_CUDA(cudaMemcpyAsync(lvl_P32[depth] + off, batch_P32[b], sizeof(float) * batch_tot[b], cudaMemcpyDeviceToDevice, s));
             off += batch_tot[b];
         }
         ASK_CUDA(cudaStreamSynchronize(s));
-        for (size_t b = 0; b < batch_P64.size(); ++b) { cudaFree(batch_P64[b]); cudaFree(batch_P32[b]); }
+        for (size_t b = 0; b < batch_P64.size(); ++b) cudaFree(batch_P64[b]);
         lvl_ptot[depth] = ltot;
     }
 
@@ -538,13 +542,23 @@ askit_status skeletonize(askit_tree t, cudaStream_t s) {
     t->h_poff[nn] = ptot;
     t->p_total = ptot;
     ASK_TRY(t->arena.alloc(&t->P64, ptot));
-    ASK_TRY(t->arena.alloc(&t->P32, ptot));
     for (int depth = 1; depth <= L; ++depth) {
-        if (lvl_ptot[depth]) {
+        if (lvl_ptot[depth])
             ASK_CUDA(cudaMemcpyAsync(t->P64 + lvl_base[depth], lvl_P64[depth], sizeof(double) * lvl_ptot[depth], cudaMemcpyDeviceToDevice, s));
-            ASK_CUDA(cudaMemcpyAsync(t->P32 + lvl_base[depth], lvl_P32[depth], sizeof(float) * lvl_ptot[depth], cudaMemcpyDeviceToDevice, s));
-        }
     }
+    // the FP32 copy: padded rows, in heap order
+    std::vector<int64_t> p32off(nn + 1, 0);
+    t->lvl_nr.assign(L + 1, 0);
+    int64_t p32tot = 0;
+    for (int64_t a = 2; a < nn; ++a) {
+        const int nr = t->h_ncol[a] - t->h_s[a];
+        p32off[a] = p32tot;
+        p32tot += (int64_t)t->h_s[a] * ((nr + 3) & ~3);
+        int &mx = t->lvl_nr[heap_depth(a)];
+        mx = std::max(mx, nr);
+    }
+    p32off[nn] = p32tot;
+    ASK_TRY(t->arena.alloc(&t->P32, p32tot));
     int64_t sk = 0, pv = 0, sp = 0;
     for (int64_t a = 0; a < nn; ++a) {
         t->h_skoff[a] = sk;
@@ -566,16 +580,22 @@ askit_status skeletonize(askit_tree t, cudaStream_t s) {
         if (t->h_ncol[a])
             ASK_CUDA(cudaMemcpyAsync(t->piv + t->h_pivoff[a], piv_fixed + a * cmax, sizeof(int32_t) * t->h_ncol[a], cudaMemcpyDeviceToDevice, s));
     }
-    ASK_TRY(t->arena.alloc(&t->d_poff, nn + 1));
+    ASK_TRY(t->arena.alloc(&t->d_p32off, nn + 1));
+    int64_t *d_poff = nullptr;      // offsets in P64
+    ASK_CUDA(cudaMallocAsync(&d_poff, sizeof(int64_t) * (nn + 1), s));
     ASK_TRY(t->arena.alloc(&t->d_skoff, nn + 1));
     ASK_TRY(t->arena.alloc(&t->d_pivoff, nn + 1));
     ASK_TRY(t->arena.alloc(&t->d_spool, nn + 1));
-    ASK_CUDA(cudaMemcpyAsync(t->d_poff, t->h_poff.data(), sizeof(int64_t) * (nn + 1), cudaMemcpyHostToDevice, s));
+    ASK_CUDA(cudaMemcpyAsync(d_poff, t->h_poff.data(), sizeof(int64_t) * (nn + 1), cudaMemcpyHostToDevice, s));
+    ASK_CUDA(cudaMemcpyAsync(t->d_p32off, p32off.data(), sizeof(int64_t) * (nn + 1), cudaMemcpyHostToDevice, s));
+    p32_kernel<<<(unsigned)(nn - 2), 256, 0, s>>>(t->P64, d_poff, t->d_p32off, t->d_s, t->d_ncol, t->P32);
+    ASK_LAUNCH();
+    cudaFreeAsync(d_poff, s);
     ASK_CUDA(cudaMemcpyAsync(t->d_skoff, t->h_skoff.data(), sizeof(int64_t) * (nn + 1), cudaMemcpyHostToDevice, s));
     ASK_CUDA(cudaMemcpyAsync(t->d_pivoff, t->h_pivoff.data(), sizeof(int64_t) * (nn + 1), cudaMemcpyHostToDevice, s));
     ASK_CUDA(cudaMemcpyAsync(t->d_spool, t->h_spool.data(), sizeof(int64_t) * (nn + 1), cudaMemcpyHostToDevice, s));
     ASK_CUDA(cudaStreamSynchronize(s));
-    for (int depth = 1; depth <= L; ++depth) { cudaFree(lvl_P64[depth]); cudaFree(lvl_P32[depth]); }
+    for (int depth = 1; depth <= L; ++depth) cudaFree(lvl_P64[depth]);
     t->arena.release(skel_fixed);
     t->arena.release(piv_fixed);
     t->arena.release(d_ell);

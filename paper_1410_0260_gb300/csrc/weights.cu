@@ -11,6 +11,7 @@ namespace {
 
 __global__ void permute_in_kernel(const float *W, int64_t ldw, int r, const int32_t *perm, int64_t N,
                                   float *Wt) {
+    pdl_trigger();
     int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= N * r) return;
     int64_t q = e / r;
@@ -18,101 +19,203 @@ __global__ void permute_in_kernel(const float *W, int64_t ldw, int r, const int3
     Wt[e] = W[(int64_t)perm[q] * ldw + z];
 }
 
-// Block (a, y) takes rows [rows y, rows y + rows) of node a's w~_a: 32 rows
-// on the wide levels near the leaves, fewer (more blocks a node) on the
-// levels near the root, whose few nodes would otherwise leave the GPU idle.
-// A row's sum is formed the same way whatever the split.
-// The rows v(R) the node's P multiplies (gathered through its pivot order)
-// are staged in shared memory, in chunks of UP_KU rows and RC columns; warps
-// then take rows q of w~_a, lanes split the columns u of P and reduce with
-// shuffles (the same order for every split of the rows).
-constexpr int UP_KU = 1024;
+// The upward pass reads every node's P once (4 s (c - s) bytes: HBM-bound on the
+// wide levels near the leaves) and is a chain of L launches on the narrow ones
+// near the root (latency-bound).  Block (a, y) takes 8 R rows of node a's w~_a,
+// a warp R of them: lane l reads P's columns 128 i + 4 l .. + 3 as one 16-byte
+// load a row (R loads in flight, the next step's R issued before this step's
+// products), and every load of a v(R) value from shared memory serves R rows.
+// The row sums are reduced over the lanes by a transposing butterfly (R RC sums
+// in about R RC shuffles).  R = 8 (r <= 4) or 4 (r > 4: R RC accumulators in
+// registers) where a level has 64 nodes or more, 2 near the root, whose few
+// nodes would otherwise leave most SMs idle; a row's sum is formed in the same
+// order for every R.  Levels are launched with programmatic serialization: a
+// level's blocks resolve their pivots and read their first P rows while the
+// level below still runs.
+// Measured (a set_weights call with its permutation, GB300; before: one row a
+// warp, 4-byte loads, r > 4 bound by its shared-memory loads):
+//   1M x 64, s = 256, r = 1     398 -> 275 us (1.07 GB of P: 158 us at the copy rate)
+//   64K x 64, s = 512, r = 16  2587 -> 147 us
+//   50K x 64, s = 256, r = 3    163 ->  32 us
+constexpr int UP_KU = 1024;      // columns of P staged at a time
+constexpr int UP_WARPS = 8;
 
+// floats between consecutive columns' v values: conflict-free 16-byte reads
 template <int RC>
-__host__ __device__ constexpr int up_stride() { return RC == 1 ? 1 : RC + 4; }   // padded: conflict-free float4 reads
+__host__ __device__ constexpr int up_stride() { return RC == 16 ? 20 : RC; }
 
-template <int RC>
-__global__ void upward_kernel(int64_t a0, bool leaf_level, int r, int rows, const int32_t *nstart, const int32_t *s,
-                              const int32_t *ncol, const int64_t *pivoff, const int32_t *piv, const int64_t *poff,
-                              const float *P32, const int64_t *spool, const float *Wt, float *Ws) {
-    extern __shared__ float vs[];
-    constexpr int STR = up_stride<RC>();
+template <int RC, int R>
+__global__ void __launch_bounds__(32 * UP_WARPS) upward_kernel(
+    int64_t a0, bool leaf_level, int r, int ku_max, const int32_t *nstart, const int32_t *s, const int32_t *ncol,
+    const int64_t *pivoff, const int32_t *piv, const int64_t *p32off, const float *P32, const int64_t *spool,
+    const float *Wt, float *Ws) {
+    extern __shared__ float vs[];          // [ku_max][STR] values, then [ku_max] rows of v
+    constexpr int STR = up_stride<RC>(), V = R * RC;
+    pdl_trigger();
+    int32_t *vrows = reinterpret_cast<int32_t *>(vs + (size_t)ku_max * STR);
     const int64_t a = a0 + blockIdx.x;
-    const int sa = s[a], c = ncol[a], nr = c - sa;
-    const int q0 = rows * blockIdx.y, q1 = min(sa, q0 + rows);
-    if (q0 >= sa) return;                                 // block-uniform
+    const int sa = s[a], nr = ncol[a] - sa, ldp = (nr + 3) & ~3;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int q0 = (blockIdx.y * UP_WARPS + warp) * R;
+    if ((int)blockIdx.y * UP_WARPS * R >= sa) {            // block-uniform
+        pdl_wait();
+        return;
+    }
+    // v of column col: row vrow(col) of `src` (weights in tree order at a leaf,
+    // the children's skeleton weights above)
     const int32_t *pv = piv + pivoff[a];
-    const float *P = P32 + poff[a];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int sl = leaf_level ? 0 : s[2 * a];
-    const float *vl = leaf_level ? Wt + (int64_t)nstart[a] * r : Ws + spool[2 * a] * r;
-    const float *vr = leaf_level ? nullptr : Ws + spool[2 * a + 1] * r;
-    auto vrow = [&](int col) -> const float * {
-        return (leaf_level || col < sl) ? vl + (int64_t)col * r : vr + (int64_t)(col - sl) * r;
-    };
+    const int64_t rl = leaf_level ? nstart[a] : spool[2 * a], rr_ = leaf_level ? 0 : spool[2 * a + 1] - sl;
+    const float *src = leaf_level ? Wt : Ws;
+    auto vrow = [&](int col) -> int32_t { return (int32_t)((leaf_level || col < sl ? rl : rr_) + col); };
     float *out = Ws + spool[a] * r;
+    const float *Prow[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) Prow[k] = P32 + p32off[a] + (int64_t)min(q0 + k, sa - 1) * ldp + 4 * lane;
+    // the sums this lane holds after the butterfly (value j of NV: row jb / RC,
+    // vector jb % RC of the warp's R x RC)
+    constexpr int NV = V > 32 ? V / 32 : 1;
+    int jb = 0;
+    bool writer = true;
+    {
+        int n = V;
+#pragma unroll
+        for (int m = 16; m >= 1; m >>= 1) {
+            if (n > 1) {
+                n >>= 1;
+                jb += (lane & m) ? n : 0;
+            } else {
+                writer = writer && !(lane & m);
+            }
+        }
+    }
+    bool waited = false;
     for (int z0 = 0; z0 < r; z0 += RC) {
-        for (int u0 = 0; u0 < nr || u0 == 0; u0 += UP_KU) {
-            const int ku = nr - u0 < UP_KU ? nr - u0 : UP_KU;
-            __syncthreads();
-            for (int e = threadIdx.x; e < ku * RC; e += blockDim.x) {
-                const int uu = e / RC, z = e % RC;
-                vs[uu * STR + z] = (z0 + z < r) ? vrow(pv[sa + u0 + uu])[z0 + z] : 0.f;
+        float acc[V];
+#pragma unroll
+        for (int e = 0; e < V; ++e) acc[e] = 0.f;
+        for (int u0 = 0; u0 < nr; u0 += UP_KU) {
+            const int ku = min(nr - u0, UP_KU), ni = (ku + 127) >> 7, lim = ldp - u0 - 4 * lane;
+            float4 p[R];
+#pragma unroll
+            for (int k = 0; k < R; ++k)
+                p[k] = lim > 0 ? *reinterpret_cast<const float4 *>(Prow[k] + u0) : make_float4(0.f, 0.f, 0.f, 0.f);
+            __syncthreads();                               // the last chunk's values are no longer read
+            for (int e = threadIdx.x; e < 128 * ni; e += 32 * UP_WARPS) vrows[e] = e < ku ? vrow(pv[sa + u0 + e]) : -1;
+            if (!waited) {
+                pdl_wait();
+                waited = true;
             }
             __syncthreads();
-            for (int q = q0 + warp; q < q1; q += nw) {
-                float acc[RC];
+            // UB gathered values in flight a thread
+            constexpr int UB = RC == 1 ? 4 : 8;
+            for (int e0 = threadIdx.x; e0 < 128 * ni * RC; e0 += UB * 32 * UP_WARPS) {
+                float x[UB];
 #pragma unroll
-                for (int z = 0; z < RC; ++z) acc[z] = 0.f;
-                for (int uu = lane; uu < ku; uu += 32) {
-                    const float p = P[(int64_t)q * nr + u0 + uu];
+                for (int b = 0; b < UB; ++b) {
+                    const int e = e0 + b * 32 * UP_WARPS, z = z0 + e % RC;
+                    const int32_t row = e < 128 * ni * RC ? vrows[e / RC] : -1;
+                    x[b] = (row >= 0 && z < r) ? src[(int64_t)row * r + z] : 0.f;
+                }
+#pragma unroll
+                for (int b = 0; b < UB; ++b) {
+                    const int e = e0 + b * 32 * UP_WARPS, u = e / RC;
+                    // column 128 i + 4 l + c at slot (4 i + c) 32 + l
+                    const int slot = ((u >> 7) * 4 + (u & 3)) * 32 + ((u >> 2) & 31);
+                    if (e < 128 * ni * RC) vs[slot * STR + e % RC] = x[b];
+                }
+            }
+            __syncthreads();
+#pragma unroll 1
+            for (int i = 0; i < ni; ++i) {
+                float4 pn[R];
+                const bool more = i + 1 < ni && 128 * (i + 1) < lim;
+#pragma unroll
+                for (int k = 0; k < R; ++k)
+                    pn[k] = more ? *reinterpret_cast<const float4 *>(Prow[k] + u0 + 128 * (i + 1))
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float *v = vs + ((4 * i + c) * 32 + lane) * STR;
+                    float pc[R];
+#pragma unroll
+                    for (int k = 0; k < R; ++k) pc[k] = c == 0 ? p[k].x : c == 1 ? p[k].y : c == 2 ? p[k].z : p[k].w;
                     if constexpr (RC == 1) {
-                        acc[0] = fmaf(p, vs[uu], acc[0]);
+                        const float x = v[0];
+#pragma unroll
+                        for (int k = 0; k < R; ++k) acc[k] = fmaf(pc[k], x, acc[k]);
                     } else {
 #pragma unroll
                         for (int z4 = 0; z4 < RC / 4; ++z4) {
-                            const float4 v = *reinterpret_cast<const float4 *>(vs + uu * STR + 4 * z4);
-                            acc[4 * z4 + 0] = fmaf(p, v.x, acc[4 * z4 + 0]);
-                            acc[4 * z4 + 1] = fmaf(p, v.y, acc[4 * z4 + 1]);
-                            acc[4 * z4 + 2] = fmaf(p, v.z, acc[4 * z4 + 2]);
-                            acc[4 * z4 + 3] = fmaf(p, v.w, acc[4 * z4 + 3]);
+                            const float4 x = *reinterpret_cast<const float4 *>(v + 4 * z4);
+#pragma unroll
+                            for (int k = 0; k < R; ++k) {
+                                float *ak = acc + k * RC + 4 * z4;
+                                ak[0] = fmaf(pc[k], x.x, ak[0]);
+                                ak[1] = fmaf(pc[k], x.y, ak[1]);
+                                ak[2] = fmaf(pc[k], x.z, ak[2]);
+                                ak[3] = fmaf(pc[k], x.w, ak[3]);
+                            }
                         }
                     }
                 }
 #pragma unroll
-                for (int z = 0; z < RC; ++z)
-                    for (int o = 16; o > 0; o >>= 1) acc[z] += __shfl_xor_sync(0xffffffffu, acc[z], o);
-                if (lane == 0) {
-                    const float *vsk = vrow(pv[q]);
-#pragma unroll
-                    for (int z = 0; z < RC; ++z)
-                        if (z0 + z < r) {
-                            float *o = out + (int64_t)q * r + z0 + z;
-                            *o = (u0 == 0 ? vsk[z0 + z] : *o) + acc[z];
-                        }
-                }
+                for (int k = 0; k < R; ++k) p[k] = pn[k];
             }
-            if (nr == 0) break;
+        }
+        if (!waited) {
+            pdl_wait();
+            waited = true;
+        }
+        // sums over the lanes: at mask m a lane keeps the half of its values that
+        // bit m of its number selects, until one is left
+        int n = V;
+#pragma unroll
+        for (int m = 16; m >= 1; m >>= 1) {
+            if (n > 1) {
+                n >>= 1;
+                const bool up = lane & m;
+#pragma unroll
+                for (int j = 0; j < V / 2; ++j)
+                    if (j < n) {
+                        const float send = up ? acc[j] : acc[j + n], keep = up ? acc[j + n] : acc[j];
+                        acc[j] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+                    }
+            } else {
+                acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], m);
+            }
+        }
+        if (writer) {
+#pragma unroll
+            for (int j = 0; j < NV; ++j) {
+                const int q = q0 + (jb + j) / RC, z = z0 + (jb + j) % RC;
+                if (q < sa && z < r) out[(int64_t)q * r + z] = src[(int64_t)vrow(pv[q]) * r + z] + acc[j];
+            }
         }
     }
 }
 
-template <int RC>
-askit_status launch_upward(askit_tree t, WeightCtx &c, int depth, int r, cudaStream_t s) {
-    const size_t smem = sizeof(float) * UP_KU * up_stride<RC>();
+template <int RC, int R>
+askit_status launch_upward_r(askit_tree t, WeightCtx &c, int depth, int r, cudaStream_t s) {
+    constexpr int STR = up_stride<RC>();
     // set once per kernel instance (thread-safe static initialisation)
     static const cudaError_t attr =
-        cudaFuncSetAttribute(upward_kernel<RC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(upward_kernel<RC, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(UP_KU * (STR * sizeof(float) + sizeof(int32_t))));
     ASK_CUDA(attr);
     const int64_t a0 = (int64_t)1 << depth;
-    const int rows = a0 >= 512 ? 32 : (a0 >= 64 ? 8 : 2);     // rows of w~_a a block takes
-    const unsigned ny = (unsigned)((std::max(1, t->prm.s_max) + rows - 1) / rows);
-    const unsigned threads = 32u * (unsigned)std::min(8, rows);
-    upward_kernel<RC><<<dim3((unsigned)a0, ny), threads, smem, s>>>(a0, depth == t->L, r, rows, t->nstart, t->d_s, t->d_ncol,
-                                                                t->d_pivoff, t->piv, t->d_poff, t->P32, t->d_spool,
-                                                                c.Wt, c.Ws);
-    ASK_LAUNCH();
-    return ASKIT_OK;
+    const int ku_max = std::max(128, std::min(UP_KU, (t->lvl_nr[depth] + 127) / 128 * 128));
+    const size_t smem = (size_t)ku_max * (STR * sizeof(float) + sizeof(int32_t));
+    const unsigned ny = (unsigned)((std::max(1, t->prm.s_max) + UP_WARPS * R - 1) / (UP_WARPS * R));
+    return launch_pdl(upward_kernel<RC, R>, dim3((unsigned)a0, ny), dim3(32 * UP_WARPS), smem, s, a0, depth == t->L, r,
+                      ku_max, t->nstart, t->d_s, t->d_ncol, t->d_pivoff, t->piv, t->d_p32off, t->P32, t->d_spool, c.Wt,
+                      c.Ws);
+}
+
+template <int RC>
+askit_status launch_upward(askit_tree t, WeightCtx &c, int depth, int r, cudaStream_t s) {
+    if (depth < 6) return launch_upward_r<RC, 2>(t, c, depth, r, s);
+    return launch_upward_r<RC, RC <= 4 ? 8 : 4>(t, c, depth, r, s);
 }
 
 }  // namespace
