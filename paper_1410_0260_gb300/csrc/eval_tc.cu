@@ -79,8 +79,8 @@ struct Smem {
     static constexpr int COLV = ANORM + 2 * 128 * 4;       // float4 [2][128]: per source pair {A, B}, {C, w} (see loader)
     static constexpr int RC_MAX = 16;
     static constexpr int COLW = COLV + 2 * 128 * 16;       // float [2][128][RC_MAX] weights (r > 1)
-    static constexpr int BAR = COLW + 2 * 128 * RC_MAX * 4;   // 14 mbarriers
-    static constexpr int MISC = BAR + 14 * 8;              // tmem address, abort flag
+    static constexpr int BAR = COLW + 2 * 128 * RC_MAX * 4;   // 15 mbarriers
+    static constexpr int MISC = BAR + 16 * 8;              // tmem address, abort flag
     static constexpr int BYTES = MISC + 16;
 };
 
@@ -121,7 +121,13 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
     const uint32_t bar0 = sbase + S::BAR;
     auto BAR_A_FULL = [&](int s) { return bar0 + 8 * s; };
     auto BAR_A_EMPTY = [&](int s) { return bar0 + 8 * (2 + s); };
-    const uint32_t BAR_B_FULL = bar0 + 8 * 4, BAR_B_EMPTY = bar0 + 8 * 5;
+    // the sub-block's tiles: block lb completes phase lb >> 1 of barrier lb & 1.
+    // A loader group may have no item in a block, but has one in any two
+    // consecutive blocks, so it never waits for a phase more than one ahead of
+    // the last one it knows complete (with one barrier for all blocks it did,
+    // and could pass on the parity of a phase two back).
+    auto BAR_B_FULL = [&](int s) { return bar0 + 8 * (s ? 14 : 4); };
+    const uint32_t BAR_B_EMPTY = bar0 + 8 * 5;
     auto BAR_T_FULL = [&](int a) { return bar0 + 8 * (6 + a); };
     auto BAR_T_EMPTY = [&](int a) { return bar0 + 8 * (8 + a); };
     auto BAR_R_FULL = [&](int a) { return bar0 + 8 * (10 + a); };    // gathered target rows landed
@@ -135,7 +141,8 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
         mbar_init(BAR_A_FULL(1), 128);
         mbar_init(BAR_A_EMPTY(0), 1);
         mbar_init(BAR_A_EMPTY(1), 1);
-        mbar_init(BAR_B_FULL, 1);
+        mbar_init(BAR_B_FULL(0), 1);
+        mbar_init(BAR_B_FULL(1), 1);
         mbar_init(BAR_B_EMPTY, 1);
         mbar_init(BAR_T_FULL(0), 1);
         mbar_init(BAR_T_FULL(1), 1);
@@ -216,7 +223,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
                     // gathered target rows (stage s) and the sub-block's raw rows
                     if (!mbar_wait(BAR_R_FULL(s), (li >> 1) & 1, abort_flag, args.status)) goto loader_done;
                     if (!waited_b) {
-                        if (!mbar_wait(BAR_B_FULL, lb & 1, abort_flag, args.status)) goto loader_done;
+                        if (!mbar_wait(BAR_B_FULL(lb & 1), (lb >> 1) & 1, abort_flag, args.status)) goto loader_done;
                         waited_b = true;
                     }
                     const float *raw = reinterpret_cast<const float *>(sm + S::RAW + s * S::RAWSTAGE);
@@ -486,25 +493,25 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
             const bool far = first.nrows < 0;
             if (!mbar_wait(BAR_B_EMPTY, (lb & 1) ^ 1, abort_flag, args.status)) goto mma_done;
             b_issued = lb + 1;
-            mbar_expect_tx(BAR_B_FULL, TX);
+            mbar_expect_tx(BAR_B_FULL(lb & 1), TX);
             const CUtensorMap *mh = far ? &map_s_hi : &map_t_hi;
             const CUtensorMap *ml = far ? &map_s_lo : &map_t_lo;
 #pragma unroll
             for (int g = 0; g < NREG; ++g) {
                 const int x = g * (128 / EB);      // first element of swizzle region g
-                tma_load_2d(sbase + S::B_HI + g * REGION, mh, x, first.row0, BAR_B_FULL);
-                tma_load_2d(sbase + S::B_LO + g * REGION, ml, x, first.row0, BAR_B_FULL);
+                tma_load_2d(sbase + S::B_HI + g * REGION, mh, x, first.row0, BAR_B_FULL(lb & 1));
+                tma_load_2d(sbase + S::B_LO + g * REGION, ml, x, first.row0, BAR_B_FULL(lb & 1));
             }
             if constexpr (S::GATHER) {
-                tma_load_2d(sbase + S::RAWB, far ? &map_rs : &map_rt, 0, first.row0, BAR_B_FULL);
-                bulk_copy(sbase + S::CENT, args.cent + (int64_t)first.cidx * TC_K, TC_K * 4, BAR_B_FULL);
+                tma_load_2d(sbase + S::RAWB, far ? &map_rs : &map_rt, 0, first.row0, BAR_B_FULL(lb & 1));
+                bulk_copy(sbase + S::CENT, args.cent + (int64_t)first.cidx * TC_K, TC_K * 4, BAR_B_FULL(lb & 1));
             }
             const int i0 = args.block_off[b], i1 = args.block_off[b + 1];
             for (int it = i0; it < i1; ++it, ++li) {
                 const int s = li & 1;
                 const uint32_t par = (li >> 1) & 1;
                 if (!mbar_wait(BAR_A_FULL(s), par, abort_flag, args.status)) goto mma_done;
-                if (it == i0 && !mbar_wait(BAR_B_FULL, lb & 1, abort_flag, args.status)) goto mma_done;
+                if (it == i0 && !mbar_wait(BAR_B_FULL(lb & 1), (lb >> 1) & 1, abort_flag, args.status)) goto mma_done;
                 if (!mbar_wait(BAR_T_EMPTY(s), par ^ 1, abort_flag, args.status)) goto mma_done;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + (uint32_t)(s * 128);
@@ -532,7 +539,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
         }
     mma_done:
         // the last sub-block's copies may still be landing after an abort
-        if (b_issued > 0) mbar_drain(BAR_B_FULL, (b_issued - 1) & 1);
+        if (b_issued > 0) mbar_drain(BAR_B_FULL((b_issued - 1) & 1), ((b_issued - 1) >> 1) & 1);
     }
     tc_fence_before();
     __syncthreads();
