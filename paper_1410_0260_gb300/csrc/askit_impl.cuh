@@ -77,8 +77,7 @@ constexpr int ASK_TILE_M = 128;
 // Source rows per sub-block (one tensor-core N tile); leaves and skeletons
 // longer than this are split into consecutive sub-blocks.
 constexpr int ASK_BLK_N = 128;
-// Items per segment of a sub-block's items (schedule of the K-chunked kernel's
-// paired items).
+// Items of one run of a sub-block's items with wide rows (d > TC_K).
 constexpr int ASK_SEG_ITEMS = 8;
 // Columns of the tensor-core operand arrays (d <= TC_K).
 constexpr int TC_K = 64;
@@ -155,29 +154,26 @@ struct WorkLists {
     int32_t *slot_of_emit = nullptr; // [n_entries] sorted position of each emitted entry
     int32_t *tgt = nullptr;          // [n_entries] target slot of each sorted entry
     EvalItem *items = nullptr;       // [n_items], grouped by sub-block
-    int32_t *block_off = nullptr;    // [n_blocks + 1] items of each sub-block
-    int32_t *block_order = nullptr;  // [n_blocks] heaviest first
-    // persistent-kernel schedule: sub-blocks dealt to n_ctas CTAs, heaviest
-    // first, each to the CTA with the least work so far
-    int n_ctas = 0;
-    int32_t *cta_off = nullptr;      // [n_ctas + 1] the schedule in use (one of the two below)
-    int32_t *cta_blocks = nullptr;   // [n_blocks]
-    // 0: longest first (LPT), 1: tree-order ranges, 2: LPT over sub-block
-    // pairs (the leader of each pair; followers are processed with it)
-    int32_t *sched_off[3] = {nullptr, nullptr, nullptr};
-    int32_t *sched_blocks[3] = {nullptr, nullptr, nullptr};
-    int n_ctas_sched[3] = {0, 0, 0};
-    int32_t *partner = nullptr;      // [n_blocks] the paired follower of a leader block, else -1
-    int64_t n_pairs = 0;
-    // segments: every sub-block's items cut into runs of at most
-    // ASK_SEG_ITEMS (a follower at its leader's cuts), the leaders' segments
-    // dealt block by block, heaviest first, to the least-loaded CTA (the
-    // K-chunked kernel's paired items: the CTAs work on few blocks at a time)
-    int64_t n_seg = 0;
-    int32_t *seg_off = nullptr;      // [n_seg + 1] items of each segment
-    int32_t *seg_partner = nullptr;  // [n_seg] the follower's segment, else -1
-    int32_t *seg_sched_off = nullptr;   // [n_ctas + 1]
-    int32_t *seg_sched = nullptr;       // [leader segments]
+    const int32_t *block_off = nullptr;    // [n_blocks + 1] items of each sub-block
+    const int32_t *block_order = nullptr;  // [n_blocks] heaviest first
+    // Schedules of the persistent kernels.  Every sub-block's items are cut into
+    // runs (a paired follower's at its leader's cuts), and the runs are dealt to
+    // n_ctas CTAs.  [0]: heaviest sub-block first, its runs one after another,
+    // each to the CTA with the least work so far; [1]: the same in tree order;
+    // [2]: paired -- the leaders' and the single sub-blocks' runs, partner the
+    // follower's run of each run (else -1).  A schedule that was not built
+    // (out-of-sample lists have those that a kernel may take) has n_ctas = 0.
+    struct Sched {
+        int n_ctas = 0;
+        const int32_t *run_off = nullptr;    // [runs + 1] items of each run
+        const int32_t *partner = nullptr;    // [runs] ([2] only)
+        const int32_t *cta_off = nullptr;    // [n_ctas + 1]
+        const int32_t *cta_runs = nullptr;   // runs of each CTA, in order
+    } sched[3];
+    int32_t *plan = nullptr;         // the device array that holds the above, block_off and block_order
+    int use = 0;                     // schedule in use without pairs: 0 or 1
+    int64_t n_pairs = 0;             // leader sub-blocks with a paired follower
+    int64_t pair_items = 0;          // their items (a follower has as many)
     int64_t pairs_alg = 0, pairs_cmp = 0, near_tot = 0, far_tot = 0;
 };
 
@@ -310,9 +306,9 @@ struct askit_tree_s {
     std::vector<int64_t> h_sub_node; // [n_sub] heap index of each sub-block's node
     // launch configuration of the evaluation kernels (askit_autotune)
     int tune_sched = 0;            // block-to-CTA schedule: 0 LPT, 1 tree-order ranges
-    int tune_stages = 3;           // gathered target-row stages of the FP16x3 kernel (2 or 3)
+    int tune_stages = 0;           // target-row stages of the FP16x3 kernels (2 to 4; 0: each kernel's default)
     int tune_runs = 1;             // 8-row tiled loads for runs of consecutive targets
-    int tune_pairs = 0;            // FP16x3: items over two sub-blocks of a node (256 columns)
+    int tune_pairs = -1;           // items over two sub-blocks of a node (256 columns): 0, 1, or -1 (take_pairs)
     int spin_limit = 0;            // polls of the FP16x3 kernel's bounded waits (0: default)
     // refinements of the pruning (askit_set_pruning): skeletons only for nodes
     // at most far_height levels above the leaves (-1: all), and the kernel cut
@@ -331,6 +327,16 @@ struct askit_tree_s {
         size_t used = 0;
     } kt;
 };
+
+// Whether the global-centered and the K-chunked kernel take paired items.  An item
+// costs them about the same with one sub-block or two, so by default pairs are
+// taken where most items have a partner: 1M x 64 3.94 ms an Evaluate against 4.37
+// unpaired, 64K x 64 165 us against 182, 10K x 1000 888 us against 1090; but 6K x
+// 700 with single-block skeletons, more singles than pairs, 230 us against 201.
+inline bool take_pairs(const askit_tree_s *t, const WorkLists &w) {
+    if (t->tune_pairs == 0) return false;
+    return t->tune_pairs == 1 || w.pair_items > w.n_items - 2 * w.pair_items;
+}
 
 // Records the begin (end = false) or end event of one evaluation-kernel
 // launch on stream s while the tree's kernel timer is on; a no-op otherwise
@@ -424,10 +430,9 @@ askit_status seg_sort_i32_f64(const int32_t *kin, int32_t *kout, const double *v
 askit_status seg_sort_i32(const int32_t *kin, int32_t *kout, int64_t n, int nseg,
                           const int32_t *beg, const int32_t *end, void *tmp, size_t *tmp_bytes,
                           cudaStream_t s);
-askit_status sort_u64_i32(const uint64_t *kin, uint64_t *kout, const int32_t *vin, int32_t *vout,
-                          int64_t n, void *tmp, size_t *tmp_bytes, cudaStream_t s);
-askit_status sort_u64_i64(const uint64_t *kin, uint64_t *kout, const int64_t *vin, int64_t *vout,
-                          int64_t n, void *tmp, size_t *tmp_bytes, cudaStream_t s);
+// stable, keys below 2^bits
+askit_status sort_u32_i32(const uint32_t *kin, uint32_t *kout, const int32_t *vin, int32_t *vout,
+                          int64_t n, int bits, void *tmp, size_t *tmp_bytes, cudaStream_t s);
 askit_status scan_i64(const int64_t *in, int64_t *out, int64_t n, void *tmp, size_t *tmp_bytes,
                       cudaStream_t s);
 
@@ -464,7 +469,7 @@ void free_prune_sets(PruneSets &ps);
 askit_status build_insample_lists(askit_tree t, const PruneSets &ps, cudaStream_t s);
 void use_schedule(askit_tree t);
 askit_status build_work_lists(askit_tree t, const int32_t *sets, int stride, const int32_t *set_row, int64_t T,
-                              WorkLists &w, DevArena &arena, cudaStream_t s);
+                              WorkLists &w, DevArena &arena, bool all_schedules, cudaStream_t s);
 askit_status reduce_partials(const WorkLists &w, const float *partial, int r, const int32_t *out_rows,
                              float *U, int64_t ldu, cudaStream_t s);
 askit_status insample_prune_sets(askit_tree t, PruneSets &ps, cudaStream_t s);

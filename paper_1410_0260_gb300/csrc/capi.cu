@@ -60,12 +60,12 @@ __global__ void pos_kernel(const int32_t *perm, int64_t N, int32_t *pos) {
 }
 
 // Order out-of-sample queries by the tree position of their nearest source
-// (so a tile's targets share near and far blocks): key (pos << 32) | q.
+// (so a tile's targets share near and far blocks), ties by q (a stable sort).
 __global__ void oos_keys_kernel(const int32_t *knn, int kappa, const int32_t *pos, int64_t T,
-                                uint64_t *keys, int32_t *vals) {
+                                uint32_t *keys, int32_t *vals) {
     int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= T) return;
-    keys[q] = ((uint64_t)pos[knn[q * kappa]] << 32) | (uint64_t)q;
+    keys[q] = (uint32_t)pos[knn[q * kappa]];
     vals[q] = (int32_t)q;
 }
 
@@ -78,18 +78,12 @@ __global__ void gather_knn_kernel(const V *knn, int kappa, const int32_t *order,
 }
 
 __global__ void gather_y_kernel(const float *Y, int64_t ldy, int d, int d_pad, const int32_t *order,
-                                int64_t T, int64_t T_pad, float *out, float *nrm) {
-    int64_t row = blockIdx.x;
+                                int64_t T, int64_t T_pad, float *out) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t row = e / d_pad;
+    const int k = (int)(e % d_pad);
     if (row >= T_pad) return;
-    int64_t q = row < T ? order[row] : -1;
-    for (int k = threadIdx.x; k < d_pad; k += blockDim.x)
-        out[row * d_pad + k] = (q >= 0 && k < d) ? Y[q * ldy + k] : 0.f;
-    if (threadIdx.x == 0) {
-        double acc = 0.0;
-        if (q >= 0)
-            for (int k = 0; k < d; ++k) acc += (double)Y[q * ldy + k] * Y[q * ldy + k];
-        nrm[row] = (float)acc;
-    }
+    out[e] = (row < T && k < d) ? Y[(int64_t)order[row] * ldy + k] : 0.f;
 }
 
 // Rows X[ids[q]] of the caller-order points; an id out of range sets *bad
@@ -460,10 +454,10 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     DevArena tmp;
     tmp.async = true;
     tmp.stream = s;
-    float *Yc = nullptr, *Yt = nullptr, *nrm = nullptr;
+    float *Yc = nullptr, *Yt = nullptr;
     int32_t *ids = nullptr, *ids_s = nullptr, *order = nullptr, *vals = nullptr, *sets = nullptr;
     double *dist = nullptr, *dist_s = nullptr;
-    uint64_t *keys = nullptr, *keys_s = nullptr;
+    uint32_t *keys = nullptr, *keys_s = nullptr;
     void *cub = nullptr;
     size_t cb = 0;
     WorkLists w;
@@ -472,6 +466,8 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     int *yg_flag = nullptr;
     QuerySplit qs;
     int64_t T_pad = (T + ASK_TILE_M - 1) / ASK_TILE_M * ASK_TILE_M;
+    int pos_bits = 1;
+    while (((int64_t)1 << pos_bits) < t->N) ++pos_bits;
     askit_status rc = ASKIT_OK;
 #define OTRY(x) do { rc = (x); if (rc != ASKIT_OK) goto out; } while (0)
     OTRY(tmp.alloc(&Yc, (size_t)T * d));
@@ -483,19 +479,18 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     OTRY(tmp.alloc(&keys, T)); OTRY(tmp.alloc(&keys_s, T));
     OTRY(tmp.alloc(&vals, T)); OTRY(tmp.alloc(&order, T));
     oos_keys_kernel<<<nblk(T, 256), 256, 0, s>>>(ids, kappa, t->pos, T, keys, vals);
-    OTRY(sort_u64_i32(nullptr, nullptr, nullptr, nullptr, T, nullptr, &cb, s));
+    OTRY(sort_u32_i32(nullptr, nullptr, nullptr, nullptr, T, pos_bits, nullptr, &cb, s));
     OTRY(tmp.alloc((char **)&cub, cb));
-    OTRY(sort_u64_i32(keys, keys_s, vals, order, T, cub, &cb, s));
+    OTRY(sort_u32_i32(keys, keys_s, vals, order, T, pos_bits, cub, &cb, s));
     OTRY(tmp.alloc(&ids_s, (size_t)T * kappa));
     OTRY(tmp.alloc(&dist_s, (size_t)T * kappa));
     gather_knn_kernel<<<nblk(T * kappa, 256), 256, 0, s>>>(ids, kappa, order, T, ids_s);
     gather_knn_kernel<<<nblk(T * kappa, 256), 256, 0, s>>>(dist, kappa, order, T, dist_s);
     OTRY(tmp.alloc(&Yt, (size_t)T_pad * t->d_pad));
-    OTRY(tmp.alloc(&nrm, T_pad));
-    gather_y_kernel<<<(unsigned)T_pad, 128, 0, s>>>(Yc, d, d, t->d_pad, order, T, T_pad, Yt, nrm);
+    gather_y_kernel<<<nblk(T_pad * t->d_pad, 256), 256, 0, s>>>(Yc, d, d, t->d_pad, order, T, T_pad, Yt);
     OTRY(tmp.alloc(&sets, (size_t)T * kappa));
     OTRY(oos_prune_sets(t, ids_s, dist_s, T, kappa, sets, s));
-    OTRY(build_work_lists(t, sets, kappa, nullptr, T, w, tmp, s));
+    OTRY(build_work_lists(t, sets, kappa, nullptr, T, w, tmp, false, s));
     OTRY(tmp.alloc(&partial, (size_t)w.n_entries * c.r));
     if (t->precision == ASKIT_PREC_FP16X3 && t->d <= TC_K && use_g16(t)) {
         // the targets in the global-centered FP16x3 form; a batch reaching
@@ -844,8 +839,9 @@ askit_status askit_autotune(askit_tree t, int32_t reps, void *stream, askit_tune
     // rows without TMA (no tiled runs); the per-sub-block kernel 2 or 3 stages
     // (two with paired items) and tiled runs on or off
     const bool g16 = fp16 && use_g16(t);
-    const int st_lo = fp16 ? (g16 ? 3 : 2) : t->tune_stages;
-    const int st_hi = fp16 ? (g16 ? 4 : 3) : t->tune_stages;
+    const int st_fix = t->tune_stages > 0 ? t->tune_stages : 3;
+    const int st_lo = fp16 ? (g16 ? 3 : 2) : st_fix;
+    const int st_hi = fp16 ? (g16 ? 4 : 3) : st_fix;
     const int ru_lo = fp16 && !g16 ? 0 : t->tune_runs, ru_hi = fp16 && !g16 ? 1 : t->tune_runs;
     for (int sc = 0; sc < (tc ? 2 : 1); ++sc)
         for (int st = st_lo; st <= st_hi; ++st)
@@ -860,7 +856,7 @@ askit_status askit_autotune(askit_tree t, int32_t reps, void *stream, askit_tune
     // the K-chunked kernel (d > TC_K, 16-bit splits) pairs at any r; its
     // stages and runs are fixed
     const bool wide = t->d > TC_K && (t->precision == ASKIT_PREC_FP16X3 || t->precision == ASKIT_PREC_BF16X3);
-    if (wide && n_pairs > 0) cand.push_back({2, t->tune_stages, t->tune_runs, 1, 0.0});
+    if (wide && n_pairs > 0) cand.push_back({2, st_fix, t->tune_runs, 1, 0.0});
     float *U = nullptr;
     ASK_CUDA(cudaMallocAsync(&U, sizeof(float) * (size_t)t->N * std::max(1, t->dw.r), s));
     cudaEvent_t e0 = nullptr, e1 = nullptr;

@@ -812,18 +812,23 @@ askit_status run_g16(askit_tree t, const WeightCtx &c, G16State *st, G16Args a, 
     // paired 256-column items up to r = 4
     bool done = false;
     if constexpr (RC <= 4) {
-        if (t->tune_pairs && w.sched_off[2]) {
-            a.cta_off = w.sched_off[2];
-            a.cta_blocks = w.sched_blocks[2];
-            a.partner = w.partner;
-            if (t->tune_stages <= 3) ASK_TRY((launch_g16<RC, 3, 2>(st, a, w.n_ctas, s)));
-            else ASK_TRY((launch_g16<RC, 4, 2>(st, a, w.n_ctas, s)));
+        if (take_pairs(t, w)) {
+            const WorkLists::Sched &p = w.sched[2];
+            a.block_off = p.run_off;
+            a.partner = p.partner;
+            a.cta_off = p.cta_off;
+            a.cta_blocks = p.cta_runs;
+            if (t->tune_stages <= 3) ASK_TRY((launch_g16<RC, 3, 2>(st, a, p.n_ctas, s)));
+            else ASK_TRY((launch_g16<RC, 4, 2>(st, a, p.n_ctas, s)));
             done = true;
         }
     }
     if (!done) {
-        if (t->tune_stages <= 3) ASK_TRY((launch_g16<RC, 3, 1>(st, a, w.n_ctas, s)));
-        else ASK_TRY((launch_g16<RC, 4, 1>(st, a, w.n_ctas, s)));
+        // by default four stages for r = 1 (1M x 64: 4.37 ms an Evaluate against
+        // 5.60 with three), three above (50K, r = 3: 309 us against 320)
+        const int st_n = t->tune_stages > 0 ? t->tune_stages : (RC == 1 ? 4 : 3);
+        if (st_n <= 3) ASK_TRY((launch_g16<RC, 3, 1>(st, a, w.sched[w.use].n_ctas, s)));
+        else ASK_TRY((launch_g16<RC, 4, 1>(st, a, w.sched[w.use].n_ctas, s)));
     }
     return ktimer_mark(t, s, true);
 }
@@ -845,9 +850,9 @@ askit_status eval_g16(askit_tree t, const WeightCtx &c, const QuerySplit &q, con
     ASK_TRY(g16_state(t, &st));
     G16Args a;
     a.items = w.items;
-    a.block_off = w.block_off;
-    a.cta_off = w.cta_off;
-    a.cta_blocks = w.cta_blocks;
+    a.block_off = w.sched[w.use].run_off;
+    a.cta_off = w.sched[w.use].cta_off;
+    a.cta_blocks = w.sched[w.use].cta_runs;
     a.tgt = w.tgt;
     a.q_hi = q.hi;
     a.q_lo = q.lo;

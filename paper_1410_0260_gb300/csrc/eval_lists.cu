@@ -18,6 +18,9 @@
 #include <math.h>
 
 #include <algorithm>
+#include <functional>
+#include <queue>
+#include <vector>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -180,145 +183,167 @@ __global__ void oos_sets_kernel(const int32_t *leafof, const int32_t *knn, const
     for (int u = n; u < stride; ++u) o[u] = INT_MAX;
 }
 
-// Near and Far sets of one target from its sorted prune leaves.  Near =
-// the leaves; Far = for each depth, the sibling of every distinct ancestor
-// at that depth when the sibling is not itself an ancestor of a near leaf.
-// With a height limit fh >= 0 (skeletons only for nodes at most fh levels
-// above the leaves, Section 3's level restriction), a higher Far node is
-// replaced by its descendants fh levels above the leaves (none holds a near
-// leaf).  emit(node, far) is called once per node of Near(i) and Far(i).
-template <class F>
-__device__ __forceinline__ void walk_lists(const int32_t *set, int stride, int L, int fh, F emit) {
-    int n = 0;
-    while (n < stride && set[n] != INT_MAX) ++n;
-    for (int u = 0; u < n; ++u) emit(set[u], false);
-    for (int depth = L; depth >= 1; --depth) {
-        int sh = L - depth;
-        for (int u = 0; u < n; ++u) {
-            int32_t b = set[u] >> sh;
-            if (u > 0 && (set[u - 1] >> sh) == b) continue;   // ancestor already handled
-            int32_t sib = b ^ 1;
-            // the set is sorted, so the leaves under sib form one run: find
-            // the first leaf >= sib's first leaf
-            const int32_t lo = sib << sh;
-            int a = 0, z = n;
-            while (a < z) {
-                const int mid = (a + z) >> 1;
-                if (set[mid] < lo) a = mid + 1; else z = mid;
-            }
-            const bool inU = a < n && (set[a] >> sh) == sib;
-            if (inU) continue;
-            if (fh >= 0 && sh > fh) {
-                const int down = sh - fh;
-                for (int32_t k = 0; k < ((int32_t)1 << down); ++k) emit((sib << down) + k, true);
-            } else {
-                emit(sib, true);
-            }
-        }
-    }
-}
-
-// Source rows of a node's block: a leaf's points (near) or its skeleton (far).
-__device__ __forceinline__ int block_rows(int32_t node, bool far, const int32_t *nsize, const int32_t *s) {
-    return far ? s[node] : nsize[node];
-}
-
-// Entries are (target, source sub-block of <= ASK_BLK_N rows) pairs; the key
-// of a sub-block is (node << 5) | (chunk << 1) | far.
-__device__ __forceinline__ uint32_t sub_key(int32_t node, int chunk, bool far) {
-    return ((uint32_t)node << 5) | ((uint32_t)chunk << 1) | (far ? 1u : 0u);
-}
-
 // Prune-set row of target q: its own row, or a shared one (leaf-grouped).
 __device__ __forceinline__ const int32_t *set_of(const int32_t *sets, int stride, const int32_t *set_row, int64_t q) {
     return sets + (set_row ? (int64_t)set_row[q] : q) * stride;
 }
 
-__global__ void count_kernel(const int32_t *sets, int stride, const int32_t *set_row, int64_t T, int L, int fh,
-                             const int32_t *nsize, const int32_t *s, int64_t *cnt, int64_t *nearc, int64_t *farc,
-                             int64_t *pairs) {
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= T) return;
-    int64_t c = 0, nf = 0, nn = 0, pr = 0;
-    walk_lists(set_of(sets, stride, set_row, q), stride, L, fh, [&](int32_t node, bool far) {
-        int rows = block_rows(node, far, nsize, s);
-        c += (rows + ASK_BLK_N - 1) / ASK_BLK_N;
-        pr += rows;
-        if (far) ++nf; else ++nn;
-    });
-    cnt[q] = c;
-    nearc[q] = nn;
-    farc[q] = nf;
-    pairs[q] = pr;
-}
-
-__global__ void emit_kernel(const int32_t *sets, int stride, const int32_t *set_row, int64_t T, int L, int fh,
-                            const int32_t *nsize, const int32_t *s, const int64_t *off, uint64_t *keys,
-                            int64_t *vals) {
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= T) return;
-    int64_t o = off[q];
-    walk_lists(set_of(sets, stride, set_row, q), stride, L, fh, [&](int32_t node, bool far) {
-        int rows = block_rows(node, far, nsize, s);
-        for (int ch = 0; ch * ASK_BLK_N < rows; ++ch) {
-            keys[o] = ((uint64_t)sub_key(node, ch, far) << 32) | (uint64_t)q;
-            vals[o] = o;
-            ++o;
+// Near and Far sets of one target from its sorted prune leaves, a warp per
+// target.  Near = the leaves; Far = for each depth, the sibling of every distinct
+// ancestor at that depth when the sibling is not itself an ancestor of a near
+// leaf.  With a height limit fh >= 0 (skeletons only for nodes at most fh levels
+// above the leaves, Section 3's level restriction), a higher Far node is replaced
+// by its descendants fh levels above the leaves (none holds a near leaf).
+// Every sub-block (<= ASK_BLK_N rows) of a Near or Far node is an entry; entries
+// are in the order near leaves ascending, then far nodes from the deepest level
+// up, which fixes the order their partial sums are added in.  EMIT false: counts
+// the target's entries into cnt and adds the near nodes, far nodes and pairs to
+// tot[0 .. 2]; EMIT true: writes the entries from off[q] on: key = sub-block
+// index, val = the entry's own position, tq = the target.
+// The lanes take 32 leaves at a time: a thread a target spent 70 us on 100
+// targets (each walk a chain of dependent loads), a warp 10.
+template <bool EMIT>
+__global__ void __launch_bounds__(256) lists_kernel(const int32_t *sets, int stride, const int32_t *set_row, int64_t T,
+                                                    int L, int fh, const int32_t *nsize, const int32_t *s,
+                                                    const int32_t *leaf_cbase, const int32_t *node_cbase,
+                                                    const int64_t *off, int64_t *cnt, unsigned long long *tot,
+                                                    uint32_t *keys, int32_t *vals, int32_t *tq) {
+    __shared__ unsigned long long sum[3];
+    const int lane = threadIdx.x & 31;
+    const int64_t q = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (!EMIT) {
+        if (threadIdx.x < 3) sum[threadIdx.x] = 0;
+        __syncthreads();
+    }
+    if (q < T) {                                           // warp-uniform
+        const int32_t *set = set_of(sets, stride, set_row, q);
+        const int32_t leaf0 = (int32_t)1 << L;
+        int n = 0;
+        for (int b = 0; b < stride; b += 32) {
+            const unsigned m = __ballot_sync(0xffffffffu, b + lane < stride && set[b + lane] != INT_MAX);
+            n += __popc(m);
+            if (m != 0xffffffffu) break;
         }
-    });
+        int64_t run = EMIT ? off[q] : 0;
+        unsigned long long c_near = 0, c_far = 0, c_pairs = 0;
+        // this lane's nodes first .. first + k - 1 (none for k = 0)
+        auto take = [&](int32_t first, int32_t k, bool far) {
+            int c = 0;
+            for (int32_t i = 0; i < k; ++i) {
+                const int rows = far ? s[first + i] : nsize[first + i];
+                c += (rows + ASK_BLK_N - 1) / ASK_BLK_N;
+                c_pairs += rows;
+            }
+            (far ? c_far : c_near) += k;
+            int incl = c;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (EMIT) {
+                int64_t o = run + incl - c;
+                for (int32_t i = 0; i < k; ++i) {
+                    const int32_t node = first + i;
+                    const int rows = far ? s[node] : nsize[node];
+                    const int32_t c0 = far ? node_cbase[node] : leaf_cbase[node - leaf0];
+                    for (int ch = 0; ch * ASK_BLK_N < rows; ++ch, ++o) {
+                        keys[o] = (uint32_t)(c0 + ch);
+                        vals[o] = (int32_t)o;
+                        tq[o] = (int32_t)q;
+                    }
+                }
+            }
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        };
+        for (int b = 0; b < n; b += 32) {
+            const int u = b + lane;
+            take(u < n ? set[u] : 0, u < n ? 1 : 0, false);
+        }
+        for (int depth = L; depth >= 1; --depth) {
+            const int sh = L - depth;
+            for (int b = 0; b < n; b += 32) {
+                const int u = b + lane;
+                int32_t first = 0, k = 0;
+                if (u < n) {
+                    const int32_t anc = set[u] >> sh;
+                    if (u == 0 || (set[u - 1] >> sh) != anc) {       // the first leaf below its ancestor
+                        const int32_t sib = anc ^ 1, lo = sib << sh;
+                        // the leaves under sib form one run of the sorted set
+                        int x = 0, z = n;
+                        while (x < z) {
+                            const int mid = (x + z) >> 1;
+                            if (set[mid] < lo) x = mid + 1; else z = mid;
+                        }
+                        if (!(x < n && (set[x] >> sh) == sib)) {
+                            const int down = fh >= 0 && sh > fh ? sh - fh : 0;
+                            first = sib << down;
+                            k = (int32_t)1 << down;
+                        }
+                    }
+                }
+                take(first, k, true);
+            }
+        }
+        if (!EMIT) {
+            for (int o = 16; o > 0; o >>= 1) {
+                c_near += __shfl_xor_sync(0xffffffffu, c_near, o);
+                c_far += __shfl_xor_sync(0xffffffffu, c_far, o);
+                c_pairs += __shfl_xor_sync(0xffffffffu, c_pairs, o);
+            }
+            if (lane == 0) {
+                cnt[q] = run;
+                if (tot) {
+                    atomicAdd(&sum[0], c_near);
+                    atomicAdd(&sum[1], c_far);
+                    atomicAdd(&sum[2], c_pairs);
+                }
+            }
+        }
+    }
+    if (!EMIT && tot) {
+        __syncthreads();
+        if (threadIdx.x < 3) atomicAdd(tot + threadIdx.x, sum[threadIdx.x]);
+    }
 }
 
-// After sorting by (sub-block, target): slot of every emitted entry, the
-// target of every sorted entry, and the first entry of every sub-block.
-__global__ void scatter_kernel(const uint64_t *keys, const int64_t *emit_of, int64_t n, int32_t *slot_of_emit,
-                               int32_t *tgt, int64_t *bflag) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// After the stable sort by sub-block: slot of every emitted entry and the target
+// of every sorted entry.
+__global__ void scatter_kernel(const int32_t *emit_of, const int32_t *tq, int64_t n, int32_t *slot_of_emit,
+                               int32_t *tgt) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= n) return;
-    slot_of_emit[emit_of[e]] = (int32_t)e;
-    tgt[e] = (int32_t)(uint32_t)keys[e];
-    bflag[e] = (e == 0 || (keys[e] >> 32) != (keys[e - 1] >> 32)) ? 1 : 0;
+    const int32_t o = emit_of[e];
+    slot_of_emit[o] = (int32_t)e;
+    tgt[e] = tq[o];
 }
 
-// Block index (inclusive scan of bflag minus one) and block starts.
-__global__ void block_start_kernel(const int64_t *bflag, const int64_t *bidx_excl, int64_t n, int64_t *bstart) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    if (bflag[e]) bstart[bidx_excl[e]] = e;
+// First entry of every sub-block c (the number of smaller keys), c = 0 .. n_sub.
+__global__ void sub_start_kernel(const uint32_t *keys, int64_t n, int64_t n_sub, int32_t *start) {
+    const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (c > n_sub) return;
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (keys[mid] < (uint32_t)c) lo = mid + 1; else hi = mid;
+    }
+    start[c] = (int32_t)lo;
 }
 
-__global__ void item_flag_kernel(const int64_t *bflag, const int64_t *bidx_excl, const int64_t *bstart, int64_t n,
-                                 int64_t *iflag) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    int64_t b = bidx_excl[e] + bflag[e] - 1;
-    iflag[e] = ((e - bstart[b]) % ASK_TILE_M) == 0 ? 1 : 0;
-}
-
-__global__ void build_items_kernel(const uint64_t *keys, const int64_t *bflag, const int64_t *bidx_excl,
-                                   const int64_t *iflag, const int64_t *iidx_excl, int64_t n, int64_t nb,
-                                   const int64_t *bstart, const int32_t *nstart, const int32_t *nsize,
-                                   const int64_t *spool, const int32_t *s, const int32_t *leaf_cbase,
-                                   const int32_t *node_cbase, int64_t leaf0, EvalItem *items, int32_t *block_off) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    int64_t b = bidx_excl[e] + bflag[e] - 1;
-    if (bflag[e]) block_off[b] = (int32_t)iidx_excl[e];
-    if (e == 0) block_off[nb] = (int32_t)(iidx_excl[n - 1] + iflag[n - 1]);
-    if (!iflag[e]) return;
-    uint32_t key = (uint32_t)(keys[e] >> 32);
-    int32_t node = (int32_t)(key >> 5);
-    int chunk = (int)((key >> 1) & 15);
-    bool far = key & 1;
-    int rows = far ? s[node] : nsize[node];
-    int64_t bend = (b + 1 < nb) ? bstart[b + 1] : n;
-    EvalItem x;
-    x.row0 = (far ? (int32_t)spool[node] : nstart[node]) + chunk * ASK_BLK_N;
-    x.nrows = min(ASK_BLK_N, rows - chunk * ASK_BLK_N) | (far ? (int32_t)0x80000000 : 0);
-    x.e0 = (int32_t)e;
-    x.cnt = (int32_t)((bend - e) < ASK_TILE_M ? (bend - e) : ASK_TILE_M);
-    x.cidx = (far ? node_cbase[node] : leaf_cbase[node - leaf0]) + chunk;
-    x.pad_[0] = x.pad_[1] = x.pad_[2] = 0;
-    items[iidx_excl[e]] = x;
+// Items of block b = sub-block blk_sub[b]: its entries in runs of ASK_TILE_M.
+__global__ void build_items_kernel(const int32_t *blk_sub, const int32_t *block_off, const int32_t *start,
+                                   const int64_t *sb_row0, const int32_t *sb_nr, int64_t n_leaf_sub, EvalItem *items) {
+    const int b = blockIdx.x;
+    const int32_t c = blk_sub[b], i0 = block_off[b], n = block_off[b + 1] - i0;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        EvalItem x;
+        x.row0 = (int32_t)sb_row0[c];
+        x.nrows = sb_nr[c] | (c >= n_leaf_sub ? (int32_t)0x80000000 : 0);
+        x.e0 = start[c] + k * ASK_TILE_M;
+        x.cnt = min(ASK_TILE_M, start[c + 1] - x.e0);
+        x.cidx = c;
+        x.pad_[0] = x.pad_[1] = x.pad_[2] = 0;
+        items[i0 + k] = x;
+    }
 }
 
 // U of target q = the sum of its entries' partials in emission order; a thread
@@ -524,13 +549,16 @@ askit_status build_tc_operands(askit_tree t, cudaStream_t s) {
     // wide kernel) and get the 16-bit splits only
     const bool wide = t->d > TC_K;
     const int kw = wide ? t->d_pad : TC_K;
-    if (kw > 8192) return ASKIT_OK;     // no tensor-core operands (plain FP32 path only)
-    t->kw = kw;
     ASK_TRY(t->arena.alloc(&t->sb_row0, std::max<int64_t>(1, t->n_sub)));
     ASK_TRY(t->arena.alloc(&t->sb_nr, std::max<int64_t>(1, t->n_sub)));
     ASK_CUDA(cudaMemcpyAsync(t->sb_row0, r0.data(), sizeof(int64_t) * t->n_sub, cudaMemcpyHostToDevice, s));
     ASK_CUDA(cudaMemcpyAsync(t->sb_nr, nr.data(), sizeof(int32_t) * t->n_sub, cudaMemcpyHostToDevice, s));
     t->n_leaf_sub = n_leaf_sub;
+    if (kw > 8192) {                    // no tensor-core operands (plain FP32 path only)
+        ASK_CUDA(cudaStreamSynchronize(s));
+        return ASKIT_OK;
+    }
+    t->kw = kw;
     int64_t *d_r0 = t->sb_row0;
     int32_t *d_nr = t->sb_nr;
     int64_t *d_nd0 = nullptr;
@@ -680,6 +708,39 @@ askit_status oos_prune_sets(askit_tree t, const int32_t *knn, const double *dist
     return ASKIT_OK;
 }
 
+namespace {
+
+// Deals runs with the given costs, in order, each to the CTA with the least work
+// so far (ties to the lowest): cta_off [nc + 1] and the runs of each CTA.
+void deal(const std::vector<std::pair<int32_t, int64_t>> &runs, int nc, std::vector<int32_t> &cta_off,
+          std::vector<int32_t> &cta_runs) {
+    std::vector<int32_t> cta(runs.size());
+    bool equal = true;
+    for (size_t k = 1; k < runs.size(); ++k) equal = equal && runs[k].second == runs[0].second;
+    if (equal) {
+        for (size_t k = 0; k < runs.size(); ++k) cta[k] = (int32_t)(k % nc);
+    } else {
+        typedef std::pair<int64_t, int> Load;   // (work, CTA)
+        std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
+        for (int c = 0; c < nc; ++c) heap.push({0, c});
+        for (size_t k = 0; k < runs.size(); ++k) {
+            Load top = heap.top();
+            heap.pop();
+            cta[k] = top.second;
+            top.first += runs[k].second;
+            heap.push(top);
+        }
+    }
+    cta_off.assign(nc + 1, 0);
+    for (int32_t c : cta) ++cta_off[c + 1];
+    for (int c = 0; c < nc; ++c) cta_off[c + 1] += cta_off[c];
+    cta_runs.resize(runs.size());
+    std::vector<int32_t> at(cta_off.begin(), cta_off.end() - 1);
+    for (size_t k = 0; k < runs.size(); ++k) cta_runs[at[cta[k]]++] = runs[k].first;
+}
+
+}  // namespace
+
 // Work lists for T targets (slot order) with the given prune sets: every
 // (target, source sub-block) pair becomes an entry; entries are sorted by
 // (sub-block, target); each sub-block's entries are cut into items of up to
@@ -687,38 +748,44 @@ askit_status oos_prune_sets(askit_tree t, const int32_t *knn, const double *dist
 // the entry's target; reduce() then sums each target's entries in emission
 // order (Near leaves ascending, then Far nodes from the deepest level up),
 // which is fixed, so the result does not depend on scheduling.
+// Emission is in target order, so a stable sort by the sub-block index alone (two
+// passes of 32-bit keys and values up to 65,536 sub-blocks; a 64-bit sort of
+// (sub-block, target) took eight) gives the order, and the sub-blocks' first
+// entries follow from binary searches.  The host reads those starts back, makes
+// the schedules from them and uploads one array.
 askit_status build_work_lists(askit_tree t, const int32_t *sets, int stride, const int32_t *set_row, int64_t T,
-                              WorkLists &wlst, DevArena &arena, cudaStream_t s) {
-    int64_t *cnt = nullptr, *nearc = nullptr, *farc = nullptr, *pairs = nullptr, *vals = nullptr, *emit_of = nullptr;
-    int64_t *bflag = nullptr, *bidx = nullptr, *bstart = nullptr, *iflag = nullptr, *iidx = nullptr;
-    uint64_t *keys = nullptr, *keys_s = nullptr;
+                              WorkLists &wlst, DevArena &arena, bool all_schedules, cudaStream_t s) {
+    int64_t *cnt = nullptr;
+    unsigned long long *tot = nullptr;
+    uint32_t *keys = nullptr, *keys_s = nullptr;
+    int32_t *vals = nullptr, *emit_of = nullptr, *tq = nullptr, *start = nullptr;
     void *tmp = nullptr;
     size_t tb = 0, tb2 = 0;
     askit_status rc = ASKIT_OK;
     cudaError_t e = cudaSuccess;
-    int64_t total = 0, nb = 0, nit = 0;
-    std::vector<int64_t> h_near(T), h_far(T), h_pairs(T);
+    int64_t total = 0;
+    const int64_t n_sub = t->n_sub;
+    unsigned long long h_tot[3] = {0, 0, 0};
+    int bits = 1;
+    while (((int64_t)1 << bits) < n_sub) ++bits;
     WorkLists &w = wlst;
     w.T = T;
 #define WCHK(x) do { e = (x); if (e != cudaSuccess) goto fail; } while (0)
 #define WTRY(x) do { rc = (x); if (rc != ASKIT_OK) goto out; } while (0)
     WCHK(cudaMallocAsync(&cnt, sizeof(int64_t) * (T + 1), s));
-    WCHK(cudaMallocAsync(&nearc, sizeof(int64_t) * T, s));
-    WCHK(cudaMallocAsync(&farc, sizeof(int64_t) * T, s));
-    WCHK(cudaMallocAsync(&pairs, sizeof(int64_t) * T, s));
+    WCHK(cudaMallocAsync(&tot, sizeof(unsigned long long) * 3, s));
     WTRY(arena.alloc(&w.off, T + 1));
     WCHK(cudaMemsetAsync(cnt + T, 0, sizeof(int64_t), s));
-    count_kernel<<<nblk(T, 128), 128, 0, s>>>(sets, stride, set_row, T, t->L, t->far_height, t->nsize, t->d_s, cnt,
-                                              nearc, farc,
-                                              pairs);
+    WCHK(cudaMemsetAsync(tot, 0, sizeof(unsigned long long) * 3, s));
+    lists_kernel<false><<<nblk(T, 8), 256, 0, s>>>(sets, stride, set_row, T, t->L, t->far_height, t->nsize, t->d_s,
+                                                   t->leaf_cbase, t->node_cbase, nullptr, cnt, tot, nullptr, nullptr,
+                                                   nullptr);
     WCHK(cudaGetLastError());
     WTRY(scan_i64(nullptr, nullptr, T + 1, nullptr, &tb, s));
     WCHK(cudaMallocAsync(&tmp, tb, s));
     WTRY(scan_i64(cnt, w.off, T + 1, tmp, &tb, s));
     WCHK(cudaMemcpyAsync(&total, w.off + T, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    WCHK(cudaMemcpyAsync(h_near.data(), nearc, sizeof(int64_t) * T, cudaMemcpyDeviceToHost, s));
-    WCHK(cudaMemcpyAsync(h_far.data(), farc, sizeof(int64_t) * T, cudaMemcpyDeviceToHost, s));
-    WCHK(cudaMemcpyAsync(h_pairs.data(), pairs, sizeof(int64_t) * T, cudaMemcpyDeviceToHost, s));
+    WCHK(cudaMemcpyAsync(h_tot, tot, sizeof h_tot, cudaMemcpyDeviceToHost, s));
     WCHK(cudaStreamSynchronize(s));
     cudaFreeAsync(tmp, s);
     tmp = nullptr;
@@ -730,271 +797,172 @@ askit_status build_work_lists(askit_tree t, const int32_t *sets, int stride, con
         rc = ASKIT_ERR_UNSUPPORTED;
         goto out;
     }
-    WCHK(cudaMallocAsync(&keys, sizeof(uint64_t) * total, s));
-    WCHK(cudaMallocAsync(&keys_s, sizeof(uint64_t) * total, s));
-    WCHK(cudaMallocAsync(&vals, sizeof(int64_t) * total, s));
-    WCHK(cudaMallocAsync(&emit_of, sizeof(int64_t) * total, s));
-    emit_kernel<<<nblk(T, 128), 128, 0, s>>>(sets, stride, set_row, T, t->L, t->far_height, t->nsize, t->d_s, w.off,
-                                             keys, vals);
+    WCHK(cudaMallocAsync(&keys, sizeof(uint32_t) * std::max<int64_t>(1, total), s));
+    WCHK(cudaMallocAsync(&keys_s, sizeof(uint32_t) * std::max<int64_t>(1, total), s));
+    WCHK(cudaMallocAsync(&vals, sizeof(int32_t) * std::max<int64_t>(1, total), s));
+    WCHK(cudaMallocAsync(&emit_of, sizeof(int32_t) * std::max<int64_t>(1, total), s));
+    WCHK(cudaMallocAsync(&tq, sizeof(int32_t) * std::max<int64_t>(1, total), s));
+    WCHK(cudaMallocAsync(&start, sizeof(int32_t) * (n_sub + 1), s));
+    lists_kernel<true><<<nblk(T, 8), 256, 0, s>>>(sets, stride, set_row, T, t->L, t->far_height, t->nsize, t->d_s,
+                                                  t->leaf_cbase, t->node_cbase, w.off, nullptr, nullptr, keys, vals, tq);
     WCHK(cudaGetLastError());
-    WTRY(sort_u64_i64(nullptr, nullptr, nullptr, nullptr, total, nullptr, &tb, s));
-    WTRY(scan_i64(nullptr, nullptr, total, nullptr, &tb2, s));
-    tb = std::max(tb, tb2);
-    WCHK(cudaMallocAsync(&tmp, tb, s));
-    WTRY(sort_u64_i64(keys, keys_s, vals, emit_of, total, tmp, &tb, s));
-    WTRY(arena.alloc(&w.slot_of_emit, total + 4));   // read in groups of 4
-    WTRY(arena.alloc(&w.tgt, total));
-    WCHK(cudaMallocAsync(&bflag, sizeof(int64_t) * total, s));
-    WCHK(cudaMallocAsync(&bidx, sizeof(int64_t) * total, s));
-    WCHK(cudaMallocAsync(&iflag, sizeof(int64_t) * total, s));
-    WCHK(cudaMallocAsync(&iidx, sizeof(int64_t) * total, s));
-    scatter_kernel<<<nblk(total, 256), 256, 0, s>>>(keys_s, emit_of, total, w.slot_of_emit, w.tgt, bflag);
-    WCHK(cudaGetLastError());
-    WTRY(scan_i64(bflag, bidx, total, tmp, &tb, s));
-    {
-        int64_t lastb = 0, lastf = 0;
-        WCHK(cudaMemcpyAsync(&lastb, bidx + total - 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        WCHK(cudaMemcpyAsync(&lastf, bflag + total - 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        WCHK(cudaStreamSynchronize(s));
-        nb = lastb + lastf;
-    }
-    WCHK(cudaMallocAsync(&bstart, sizeof(int64_t) * nb, s));
-    block_start_kernel<<<nblk(total, 256), 256, 0, s>>>(bflag, bidx, total, bstart);
-    item_flag_kernel<<<nblk(total, 256), 256, 0, s>>>(bflag, bidx, bstart, total, iflag);
-    WCHK(cudaGetLastError());
-    WTRY(scan_i64(iflag, iidx, total, tmp, &tb, s));
-    {
-        int64_t lasti = 0, lastf = 0;
-        WCHK(cudaMemcpyAsync(&lasti, iidx + total - 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        WCHK(cudaMemcpyAsync(&lastf, iflag + total - 1, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        WCHK(cudaStreamSynchronize(s));
-        nit = lasti + lastf;
-    }
-    WTRY(arena.alloc(&w.items, nit));
-    WTRY(arena.alloc(&w.block_off, nb + 1));
-    build_items_kernel<<<nblk(total, 256), 256, 0, s>>>(keys_s, bflag, bidx, iflag, iidx, total, nb, bstart, t->nstart,
-                                                        t->nsize, t->d_spool, t->d_s, t->leaf_cbase, t->node_cbase,
-                                                        (int64_t)1 << t->L, w.items, w.block_off);
+    WTRY(sort_u32_i32(nullptr, nullptr, nullptr, nullptr, total, bits, nullptr, &tb2, s));
+    WCHK(cudaMallocAsync(&tmp, tb2, s));
+    WTRY(sort_u32_i32(keys, keys_s, vals, emit_of, total, bits, tmp, &tb2, s));
+    sub_start_kernel<<<nblk(n_sub + 1, 128), 128, 0, s>>>(keys_s, total, n_sub, start);
     WCHK(cudaGetLastError());
     {
-        std::vector<EvalItem> hi(nit);
-        std::vector<int32_t> boff(nb + 1);
-        WCHK(cudaMemcpyAsync(hi.data(), w.items, sizeof(EvalItem) * nit, cudaMemcpyDeviceToHost, s));
-        WCHK(cudaMemcpyAsync(boff.data(), w.block_off, sizeof(int32_t) * (nb + 1), cudaMemcpyDeviceToHost, s));
-        WCHK(cudaStreamSynchronize(s));
-        std::vector<int64_t> cost(nb, 0);
-        int64_t pc = 0;
-        for (int64_t b = 0; b < nb; ++b)
-            for (int32_t it = boff[b]; it < boff[b + 1]; ++it) {
-                cost[b] += ASK_TILE_M * ASK_BLK_N;
-                pc += (int64_t)ASK_TILE_M * ASK_BLK_N;
+        std::vector<int32_t> h_start(n_sub + 1);
+        WCHK(cudaMemcpyAsync(h_start.data(), start, sizeof(int32_t) * (n_sub + 1), cudaMemcpyDeviceToHost, s));
+        // the copy above comes first on the stream, so the host works while the
+        // entries are scattered
+        cudaEvent_t ev = nullptr;
+        WCHK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        e = cudaEventRecord(ev, s);
+        if (e == cudaSuccess) {
+            rc = arena.alloc(&w.slot_of_emit, total + 4);   // read in groups of 4
+            if (rc == ASKIT_OK) rc = arena.alloc(&w.tgt, total);
+            if (rc == ASKIT_OK) {
+                if (total > 0)
+                    scatter_kernel<<<nblk(total, 256), 256, 0, s>>>(emit_of, tq, total, w.slot_of_emit, w.tgt);
+                e = cudaGetLastError();
             }
+            const cudaError_t es = cudaEventSynchronize(ev);
+            if (e == cudaSuccess) e = es;
+        }
+        cudaEventDestroy(ev);
+        if (rc != ASKIT_OK) goto out;
+        if (e != cudaSuccess) goto fail;
+        // blocks: the sub-blocks with entries, in index order
+        std::vector<int32_t> blk_sub, boff(1, 0);
+        for (int64_t c = 0; c < n_sub; ++c) {
+            const int32_t n = h_start[c + 1] - h_start[c];
+            if (n == 0) continue;
+            blk_sub.push_back((int32_t)c);
+            boff.push_back(boff.back() + (n + ASK_TILE_M - 1) / ASK_TILE_M);
+        }
+        const int64_t nb = (int64_t)blk_sub.size(), nit = boff.back();
+        auto n_items = [&](int32_t b) { return boff[b + 1] - boff[b]; };
         std::vector<int32_t> order(nb);
         for (int64_t b = 0; b < nb; ++b) order[b] = (int32_t)b;
-        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return cost[x] > cost[y]; });
-        WTRY(arena.alloc(&w.block_order, nb));
-        WCHK(cudaMemcpyAsync(w.block_order, order.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice, s));
-        // Two schedules over one persistent CTA per SM (a sub-block costs its
-        // items plus a fixed reload of its source tile); askit_autotune picks.
-        //  0: LPT -- heaviest first, each to the least-loaded CTA;
-        //  1: tree order -- sub-blocks taken in their node's tree order, each
-        //     to the least-loaded CTA: the CTAs advance through the tree
-        //     together, so the sub-blocks in flight at any time on all SMs
-        //     share most of their targets (L2 reuse of target rows).
+        std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return n_items(x) > n_items(y); });
+        // Pairs: sub-blocks 2k and 2k + 1 of one node need the same targets (a
+        // target needing a node needs all its sub-blocks), so their items match
+        // one to one and a kernel can take both in one 256-column item.  A leader
+        // is never the last sub-block of its node, so it is full and its
+        // follower's rows start ASK_BLK_N rows later.  The leader keeps its
+        // items, the follower's are skipped.
+        std::vector<int32_t> partner(nb, -1);
+        std::vector<char> follower(nb, 0);
+        w.n_pairs = w.pair_items = 0;
+        int64_t lead_items = 0;
+        for (int64_t b = 0, first = 0; b < nb; ++b) {
+            const int32_t c = blk_sub[b];
+            if (b > 0 && t->h_sub_node[c] != t->h_sub_node[blk_sub[b - 1]]) first = b;
+            if (follower[b]) continue;
+            lead_items += n_items(b);
+            if (!((b - first) & 1) && b + 1 < nb && blk_sub[b + 1] == c + 1 &&
+                t->h_sub_node[c + 1] == t->h_sub_node[c] && h_start[c + 2] - h_start[c + 1] == h_start[c + 1] - h_start[c]) {
+                partner[b] = (int32_t)(b + 1);
+                follower[b + 1] = 1;
+                ++w.n_pairs;
+                w.pair_items += n_items(b);
+            }
+        }
+        w.n_items = nit;
+        w.n_blocks = nb;
         int dev = 0, sms = 0;
         WCHK(cudaGetDevice(&dev));
         WCHK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int nc = (int)std::max<int64_t>(1, std::min<int64_t>(nb, sms));
-        auto bcost = [&](int32_t b) { return (int64_t)(boff[b + 1] - boff[b]) * 4 + 3; };
-        std::vector<int32_t> coff[3], cblk[3];
-        {
-            std::vector<std::vector<int32_t>> lists(nc);
-            std::vector<std::pair<int64_t, int>> heap;   // (load, cta), min-heap
-            for (int c = 0; c < nc; ++c) heap.push_back({0, c});
-            auto cmp = [](const std::pair<int64_t, int> &x, const std::pair<int64_t, int> &y) {
-                return x.first > y.first || (x.first == y.first && x.second > y.second);
-            };
-            std::make_heap(heap.begin(), heap.end(), cmp);
-            for (int64_t q = 0; q < nb; ++q) {
-                const int32_t bq = order[q];
-                std::pop_heap(heap.begin(), heap.end(), cmp);
-                auto top = heap.back();
-                heap.pop_back();
-                lists[top.second].push_back(bq);
-                top.first += bcost(bq);
-                heap.push_back(top);
-                std::push_heap(heap.begin(), heap.end(), cmp);
-            }
-            coff[0].assign(nc + 1, 0);
-            for (int c = 0; c < nc; ++c) {
-                coff[0][c + 1] = coff[0][c] + (int32_t)lists[c].size();
-                cblk[0].insert(cblk[0].end(), lists[c].begin(), lists[c].end());
-            }
-        }
-        {
-            std::vector<int64_t> bpos(nb, 0);
-            for (int64_t b = 0; b < nb; ++b) {
-                const int32_t cx = hi[boff[b]].cidx;
-                bpos[b] = (cx >= 0 && cx < (int32_t)t->h_sub_pos.size()) ? t->h_sub_pos[cx] : 0;
-            }
-            std::vector<int32_t> tord(nb);
-            for (int64_t b = 0; b < nb; ++b) tord[b] = (int32_t)b;
-            std::stable_sort(tord.begin(), tord.end(), [&](int32_t x, int32_t y) { return bpos[x] < bpos[y]; });
-            std::vector<std::vector<int32_t>> lists(nc);
-            std::vector<std::pair<int64_t, int>> heap;   // (load, cta), min-heap
-            for (int c = 0; c < nc; ++c) heap.push_back({0, c});
-            auto cmp = [](const std::pair<int64_t, int> &x, const std::pair<int64_t, int> &y) {
-                return x.first > y.first || (x.first == y.first && x.second > y.second);
-            };
-            std::make_heap(heap.begin(), heap.end(), cmp);
-            for (int64_t q = 0; q < nb; ++q) {
-                std::pop_heap(heap.begin(), heap.end(), cmp);
-                auto top = heap.back();
-                heap.pop_back();
-                lists[top.second].push_back(tord[q]);
-                top.first += bcost(tord[q]);
-                heap.push_back(top);
-                std::push_heap(heap.begin(), heap.end(), cmp);
-            }
-            coff[1].assign(nc + 1, 0);
-            for (int c = 0; c < nc; ++c) {
-                coff[1][c + 1] = coff[1][c] + (int32_t)lists[c].size();
-                cblk[1].insert(cblk[1].end(), lists[c].begin(), lists[c].end());
-            }
-        }
-        // Pairs: sub-blocks 2k and 2k+1 of one node need the same targets (a
-        // target needing a node needs all its sub-blocks), so their items
-        // match one to one; the FP16x3 kernel can take both in one 256-column
-        // item.  The leader keeps its items, the follower's are skipped.
-        std::vector<int32_t> partner(nb, -1);
-        std::vector<char> follower(nb, 0);
-        if (!t->h_sub_node.empty()) {
-            std::vector<int32_t> blk_of_sub(t->h_sub_node.size(), -1);
-            for (int64_t b = 0; b < nb; ++b) {
-                const int32_t cx = hi[boff[b]].cidx;
-                if (cx >= 0 && cx < (int32_t)blk_of_sub.size()) blk_of_sub[cx] = (int32_t)b;
-            }
-            for (int64_t b = 0; b < nb; ++b) {
-                const int32_t cx = hi[boff[b]].cidx;
-                if (cx < 0 || cx + 1 >= (int32_t)t->h_sub_node.size()) continue;
-                const int64_t node = t->h_sub_node[cx];
-                if (t->h_sub_node[cx + 1] != node) continue;
-                int32_t first = cx;
-                while (first > 0 && t->h_sub_node[first - 1] == node) --first;
-                if ((cx - first) & 1) continue;           // odd position in its node
-                const int32_t b2 = blk_of_sub[cx + 1];
-                if (b2 < 0 || boff[b2 + 1] - boff[b2] != boff[b + 1] - boff[b]) continue;
-                // a leader is never the last sub-block of its node, so it is
-                // full and its follower's rows start 128 rows later
-                bool same = (hi[boff[b]].nrows & 0x7fffffff) == ASK_BLK_N;
-                for (int32_t k = 0; same && k < boff[b + 1] - boff[b]; ++k)
-                    same = hi[boff[b] + k].cnt == hi[boff[b2] + k].cnt;
-                if (!same) continue;
-                partner[b] = b2;
-                follower[b2] = 1;
-            }
-        }
-        {
-            std::vector<std::vector<int32_t>> lists(nc);
-            std::vector<std::pair<int64_t, int>> heap;
-            for (int c = 0; c < nc; ++c) heap.push_back({0, c});
-            auto cmp = [](const std::pair<int64_t, int> &x, const std::pair<int64_t, int> &y) {
-                return x.first > y.first || (x.first == y.first && x.second > y.second);
-            };
-            std::make_heap(heap.begin(), heap.end(), cmp);
-            int64_t np = 0;
-            for (int64_t q = 0; q < nb; ++q) {
-                const int32_t bq = order[q];
-                if (follower[bq]) continue;
-                np += partner[bq] >= 0;
-                std::pop_heap(heap.begin(), heap.end(), cmp);
-                auto top = heap.back();
-                heap.pop_back();
-                lists[top.second].push_back(bq);
-                top.first += bcost(bq) * (partner[bq] >= 0 ? 2 : 1);
-                heap.push_back(top);
-                std::push_heap(heap.begin(), heap.end(), cmp);
-            }
-            coff[2].assign(nc + 1, 0);
-            for (int c = 0; c < nc; ++c) {
-                coff[2][c + 1] = coff[2][c] + (int32_t)lists[c].size();
-                cblk[2].insert(cblk[2].end(), lists[c].begin(), lists[c].end());
-            }
-            w.n_pairs = np;
-        }
-        {
-            std::vector<int32_t> soff, sfirst(nb + 1, 0);
-            for (int64_t b = 0; b < nb; ++b) {
-                sfirst[b] = (int32_t)soff.size();
-                for (int32_t i = boff[b]; i < boff[b + 1]; i += ASK_SEG_ITEMS) soff.push_back(i);
-            }
-            sfirst[nb] = (int32_t)soff.size();
-            const int64_t nseg = (int64_t)soff.size();
-            soff.push_back(boff[nb]);
-            std::vector<int32_t> spart(std::max<int64_t>(1, nseg), -1);
-            for (int64_t b = 0; b < nb; ++b)
-                if (partner[b] >= 0)
-                    for (int32_t k = 0; k < sfirst[b + 1] - sfirst[b]; ++k) spart[sfirst[b] + k] = sfirst[partner[b]] + k;
-            std::vector<std::vector<int32_t>> lists(nc);
-            std::vector<std::pair<int64_t, int>> heap;
-            for (int c = 0; c < nc; ++c) heap.push_back({0, c});
-            auto cmp = [](const std::pair<int64_t, int> &x, const std::pair<int64_t, int> &y) {
-                return x.first > y.first || (x.first == y.first && x.second > y.second);
-            };
-            std::make_heap(heap.begin(), heap.end(), cmp);
-            for (int64_t q = 0; q < nb; ++q) {
-                const int32_t bq = order[q];
-                if (follower[bq]) continue;
-                for (int32_t sg = sfirst[bq]; sg < sfirst[bq + 1]; ++sg) {
-                    std::pop_heap(heap.begin(), heap.end(), cmp);
-                    auto top = heap.back();
-                    heap.pop_back();
-                    lists[top.second].push_back(sg);
-                    top.first += ((int64_t)(soff[sg + 1] - soff[sg]) * 4 + 3) * (partner[bq] >= 0 ? 2 : 1);
-                    heap.push_back(top);
-                    std::push_heap(heap.begin(), heap.end(), cmp);
-                }
-            }
-            std::vector<int32_t> so(nc + 1, 0), sl;
-            for (int c = 0; c < nc; ++c) {
-                so[c + 1] = so[c] + (int32_t)lists[c].size();
-                sl.insert(sl.end(), lists[c].begin(), lists[c].end());
-            }
-            w.n_seg = nseg;
-            WTRY(arena.alloc(&w.seg_off, nseg + 1));
-            WTRY(arena.alloc(&w.seg_partner, std::max<int64_t>(1, nseg)));
-            WTRY(arena.alloc(&w.seg_sched_off, nc + 1));
-            WTRY(arena.alloc(&w.seg_sched, std::max<size_t>(1, sl.size())));
-            WCHK(cudaMemcpyAsync(w.seg_off, soff.data(), sizeof(int32_t) * (nseg + 1), cudaMemcpyHostToDevice, s));
-            WCHK(cudaMemcpyAsync(w.seg_partner, spart.data(), sizeof(int32_t) * spart.size(), cudaMemcpyHostToDevice, s));
-            WCHK(cudaMemcpyAsync(w.seg_sched_off, so.data(), sizeof(int32_t) * (nc + 1), cudaMemcpyHostToDevice, s));
-            if (!sl.empty())
-                WCHK(cudaMemcpyAsync(w.seg_sched, sl.data(), sizeof(int32_t) * sl.size(), cudaMemcpyHostToDevice, s));
-            // the host vectors must outlive the copies
-            WCHK(cudaStreamSynchronize(s));
-        }
-        w.n_ctas = nc;
+        // Items a run, narrow rows: about 24 runs a CTA, of 8 to 64 items -- short
+        // enough to deal the work evenly (64K x 64, paired: 165 us an Evaluate
+        // against 186 with whole blocks), long enough that the source tiles (74 KB
+        // a pair) are not reloaded all the time (1M x 64: 3.94 ms with whole
+        // blocks, 4.12 in runs of 8); fewer where that leaves CTAs without work.
+        // Wide rows, whose sub-blocks stream through shared memory for every item:
+        // ASK_SEG_ITEMS.
+        // Unpaired items take half as long, so a reload weighs more: 6 runs a CTA.
+        auto run_items = [&](int64_t items, bool pair) -> int32_t {
+            const int64_t least = std::max<int64_t>(1, std::min<int64_t>(8, (items + 2 * sms - 1) / (2 * sms)));
+            if (t->d > TC_K) return (int32_t)std::min<int64_t>(ASK_SEG_ITEMS, least);
+            return (int32_t)std::max<int64_t>(least, std::min<int64_t>(64, items / ((pair ? 24 : 6) * (int64_t)sms)));
+        };
+        // the upload: blk_sub, block_off, block_order, then each schedule's arrays
+        std::vector<int32_t> up(blk_sub);
+        const size_t o_boff = up.size();
+        up.insert(up.end(), boff.begin(), boff.end());
+        const size_t o_order = up.size();
+        up.insert(up.end(), order.begin(), order.end());
+        size_t o_run[3], o_part = 0, o_cta[3], o_list[3];
+        const bool paired = take_pairs(t, w);
         for (int k = 0; k < 3; ++k) {
-            WTRY(arena.alloc(&w.sched_off[k], nc + 1));
-            WTRY(arena.alloc(&w.sched_blocks[k], std::max<int64_t>(1, nb)));
-            WCHK(cudaMemcpyAsync(w.sched_off[k], coff[k].data(), sizeof(int32_t) * (nc + 1), cudaMemcpyHostToDevice, s));
-            WCHK(cudaMemcpyAsync(w.sched_blocks[k], cblk[k].data(), sizeof(int32_t) * cblk[k].size(),
-                                 cudaMemcpyHostToDevice, s));
-            w.n_ctas_sched[k] = nc;
+            w.sched[k] = WorkLists::Sched();
+            if (!all_schedules && k != (t->tune_sched & 1) && !(k == 2 && paired)) continue;
+            std::vector<int32_t> ord = order;
+            if (k == 1)
+                std::stable_sort(ord.begin(), ord.end(), [&](int32_t x, int32_t y) {
+                    const int64_t px = t->h_sub_pos[blk_sub[x]], py = t->h_sub_pos[blk_sub[y]];
+                    return px != py ? px < py : x < y;
+                });
+            const int32_t len = run_items(k == 2 ? lead_items : nit, k == 2);
+            std::vector<int32_t> roff, rfirst(nb), rpart;
+            for (int64_t b = 0; b < nb; ++b) {
+                rfirst[b] = (int32_t)roff.size();
+                for (int32_t i = boff[b]; i < boff[b + 1]; i += len) roff.push_back(i);
+            }
+            roff.push_back((int32_t)nit);
+            if (k == 2) {
+                rpart.assign(roff.size(), -1);
+                for (int64_t b = 0; b < nb; ++b)
+                    if (partner[b] >= 0)
+                        for (int32_t r = 0; r < (n_items(b) + len - 1) / len; ++r)
+                            rpart[rfirst[b] + r] = rfirst[partner[b]] + r;
+            }
+            // a run costs its items plus a fixed reload of its source tile
+            std::vector<std::pair<int32_t, int64_t>> runs;
+            for (int32_t b : ord) {
+                if (k == 2 && follower[b]) continue;
+                const int64_t f = k == 2 && partner[b] >= 0 ? 2 : 1;
+                for (int32_t r = rfirst[b]; roff[r] < boff[b + 1]; ++r)
+                    runs.push_back({r, ((int64_t)std::min(roff[r + 1], boff[b + 1]) - roff[r]) * 4 * f + 3 * f});
+            }
+            const int nc = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)runs.size(), sms));
+            std::vector<int32_t> cta_off, cta_runs;
+            deal(runs, nc, cta_off, cta_runs);
+            w.sched[k].n_ctas = nc;
+            o_run[k] = up.size();
+            up.insert(up.end(), roff.begin(), roff.end());
+            if (k == 2) {
+                o_part = up.size();
+                up.insert(up.end(), rpart.begin(), rpart.end());
+            }
+            o_cta[k] = up.size();
+            up.insert(up.end(), cta_off.begin(), cta_off.end());
+            o_list[k] = up.size();
+            up.insert(up.end(), cta_runs.begin(), cta_runs.end());
         }
-        WTRY(arena.alloc(&w.partner, std::max<int64_t>(1, nb)));
-        WCHK(cudaMemcpyAsync(w.partner, partner.data(), sizeof(int32_t) * nb, cudaMemcpyHostToDevice, s));
-        w.cta_off = w.sched_off[t->tune_sched & 1];
-        w.cta_blocks = w.sched_blocks[t->tune_sched & 1];
-        WCHK(cudaStreamSynchronize(s));
-        int64_t sn = 0, sf = 0, pa = 0;
-        for (int64_t q = 0; q < T; ++q) { sn += h_near[q]; sf += h_far[q]; pa += h_pairs[q]; }
-        w.n_items = nit;
-        w.n_blocks = nb;
-        w.pairs_alg = pa;
-        w.pairs_cmp = pc;
-        w.near_tot = sn;
-        w.far_tot = sf;
+        WTRY(arena.alloc(&w.plan, up.size()));
+        WTRY(arena.alloc(&w.items, nit));
+        WCHK(cudaMemcpyAsync(w.plan, up.data(), sizeof(int32_t) * up.size(), cudaMemcpyHostToDevice, s));
+        w.block_off = w.plan + o_boff;
+        w.block_order = w.plan + o_order;
+        for (int k = 0; k < 3; ++k) {
+            if (!w.sched[k].n_ctas) continue;
+            w.sched[k].run_off = w.plan + o_run[k];
+            w.sched[k].partner = k == 2 ? w.plan + o_part : nullptr;
+            w.sched[k].cta_off = w.plan + o_cta[k];
+            w.sched[k].cta_runs = w.plan + o_list[k];
+        }
+        w.use = t->tune_sched & 1;
+        if (nb > 0)
+            build_items_kernel<<<(unsigned)nb, 128, 0, s>>>(w.plan, w.block_off, start, t->sb_row0, t->sb_nr,
+                                                            t->n_leaf_sub, w.items);
+        WCHK(cudaGetLastError());
+        w.pairs_alg = (int64_t)h_tot[2];
+        w.pairs_cmp = nit * (int64_t)ASK_TILE_M * ASK_BLK_N;
+        w.near_tot = (int64_t)h_tot[0];
+        w.far_tot = (int64_t)h_tot[1];
+        WCHK(cudaStreamSynchronize(s));                     // the upload's source goes out of scope
     }
     goto out;
 fail:
@@ -1003,9 +971,9 @@ fail:
 out:
 #undef WCHK
 #undef WTRY
-    cudaStreamSynchronize(s);
-    for (void *q : {(void *)cnt, (void *)nearc, (void *)farc, (void *)pairs, (void *)vals, (void *)emit_of, (void *)bflag,
-                    (void *)bidx, (void *)bstart, (void *)iflag, (void *)iidx, (void *)keys, (void *)keys_s, tmp})
+    if (rc != ASKIT_OK) cudaStreamSynchronize(s);
+    for (void *q : {(void *)cnt, (void *)tot, (void *)vals, (void *)emit_of, (void *)tq, (void *)start, (void *)keys,
+                    (void *)keys_s, tmp})
         if (q) cudaFreeAsync(q, s);
     return rc;
 }
@@ -1023,9 +991,10 @@ askit_status build_insample_lists(askit_tree t, const PruneSets &ps, cudaStream_
     std::vector<int64_t> h_cnt(N);
     {
         int64_t *buf = nullptr;
-        ASK_CUDA(cudaMallocAsync(&buf, sizeof(int64_t) * 4 * N, s));
-        count_kernel<<<nblk(N, 128), 128, 0, s>>>(sets, stride, set_row, N, t->L, t->far_height, t->nsize, t->d_s, buf,
-                                                  buf + N, buf + 2 * N, buf + 3 * N);
+        ASK_CUDA(cudaMallocAsync(&buf, sizeof(int64_t) * N, s));
+        lists_kernel<false><<<nblk(N, 8), 256, 0, s>>>(sets, stride, set_row, N, t->L, t->far_height, t->nsize, t->d_s,
+                                                       t->leaf_cbase, t->node_cbase, nullptr, buf, nullptr, nullptr,
+                                                       nullptr, nullptr);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(h_cnt.data(), buf, sizeof(int64_t) * N, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1050,9 +1019,9 @@ askit_status build_insample_lists(askit_tree t, const PruneSets &ps, cudaStream_
         const int64_t t0 = t->wl_t0[b], T = t->wl_t0[b + 1] - t0;
         // a batch's targets start at t0: shift the shared-row index, or the rows
         if (set_row)
-            ASK_TRY(build_work_lists(t, sets, stride, set_row + t0, T, t->wl[b], t->arena, s));
+            ASK_TRY(build_work_lists(t, sets, stride, set_row + t0, T, t->wl[b], t->arena, true, s));
         else
-            ASK_TRY(build_work_lists(t, sets + t0 * stride, stride, nullptr, T, t->wl[b], t->arena, s));
+            ASK_TRY(build_work_lists(t, sets + t0 * stride, stride, nullptr, T, t->wl[b], t->arena, true, s));
         if (t->wl[b].n_entries >= ((int64_t)1 << 31)) {
             askit_set_error("a single target has more than 2^31 work entries");
             return ASKIT_ERR_UNSUPPORTED;
@@ -1064,21 +1033,16 @@ askit_status build_insample_lists(askit_tree t, const PruneSets &ps, cudaStream_
 }
 
 void free_work_lists(WorkLists &w, DevArena &arena) {
-    void *ptrs[] = {w.off, w.slot_of_emit, w.tgt, w.items, w.block_off, w.block_order, w.sched_off[0],
-                    w.sched_off[1], w.sched_off[2], w.sched_blocks[0], w.sched_blocks[1], w.sched_blocks[2],
-                    w.partner, w.seg_off, w.seg_partner, w.seg_sched_off, w.seg_sched};
+    void *ptrs[] = {w.off, w.slot_of_emit, w.tgt, w.items, w.plan};
     for (void *p : ptrs)
         if (p) arena.release(p);
     w = WorkLists();
 }
 
-// The CTA schedule the kernels use: LPT or tree order (askit_set_launch);
-// the paired schedule is taken by the FP16x3 kernel itself.
+// The CTA schedule the kernels use without pairs: heaviest first or tree order
+// (askit_set_launch).
 void use_schedule(askit_tree t) {
-    for (WorkLists &w : t->wl) {
-        w.cta_off = w.sched_off[t->tune_sched & 1];
-        w.cta_blocks = w.sched_blocks[t->tune_sched & 1];
-    }
+    for (WorkLists &w : t->wl) w.use = t->tune_sched & 1;
 }
 
 askit_status reduce_partials(const WorkLists &w, const float *partial, int r, const int32_t *out_rows, float *U,

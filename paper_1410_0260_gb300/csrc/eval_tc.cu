@@ -685,9 +685,9 @@ askit_status eval_tc(askit_tree t, const WeightCtx &c, int precision, const floa
     ASK_TRY(encode_raw((EncodeTiledFn)st->encode, &map_q, Xq, q_rows, t->d_pad, 1));
     TcArgs a;
     a.items = w.items;
-    a.block_off = w.block_off;
-    a.cta_off = w.cta_off;
-    a.cta_blocks = w.cta_blocks;
+    a.block_off = w.sched[w.use].run_off;
+    a.cta_off = w.sched[w.use].cta_off;
+    a.cta_blocks = w.sched[w.use].cta_runs;
     a.tgt = w.tgt;
     a.Xq = Xq;
     a.ldq = ldq;
@@ -705,14 +705,14 @@ askit_status eval_tc(askit_tree t, const WeightCtx &c, int precision, const floa
     a.f16_scale = 1.f;
     a.g_unscale = 1.f / (a.f16_scale * a.f16_scale);
     if (precision == ASKIT_PREC_TF32X3) {
-        if (c.r == 1) return launch<ASKIT_PREC_TF32X3, 1>(t, st, map_q, a, w.n_ctas, s);
-        if (c.r <= 4) return launch<ASKIT_PREC_TF32X3, 4>(t, st, map_q, a, w.n_ctas, s);
-        return launch<ASKIT_PREC_TF32X3, 16>(t, st, map_q, a, w.n_ctas, s);
+        if (c.r == 1) return launch<ASKIT_PREC_TF32X3, 1>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
+        if (c.r <= 4) return launch<ASKIT_PREC_TF32X3, 4>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
+        return launch<ASKIT_PREC_TF32X3, 16>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
     }
     if (precision == ASKIT_PREC_BF16X3) {
-        if (c.r == 1) return launch<ASKIT_PREC_BF16X3, 1>(t, st, map_q, a, w.n_ctas, s);
-        if (c.r <= 4) return launch<ASKIT_PREC_BF16X3, 4>(t, st, map_q, a, w.n_ctas, s);
-        return launch<ASKIT_PREC_BF16X3, 16>(t, st, map_q, a, w.n_ctas, s);
+        if (c.r == 1) return launch<ASKIT_PREC_BF16X3, 1>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
+        if (c.r <= 4) return launch<ASKIT_PREC_BF16X3, 4>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
+        return launch<ASKIT_PREC_BF16X3, 16>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
     }
     askit_set_error("unknown tensor-core precision %d", precision);
     return ASKIT_ERR_INVALID_ARG;

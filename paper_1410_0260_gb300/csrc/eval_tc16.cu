@@ -790,30 +790,33 @@ askit_status run16(askit_tree t, const WeightCtx &c, T16State *st, int pi, const
     }
     a.colv = c.colv;
     a.colw = c.colw;
+    const bool pairs = t->tune_pairs == 1 && w.sched[2].n_ctas > 0;
     auto go = [&]() -> askit_status {
         if constexpr (RC == 1) {
             if (uni) {
-                if (t->tune_pairs && w.sched_off[2]) {
-                    a.cta_off = w.sched_off[2];
-                    a.cta_blocks = w.sched_blocks[2];
-                    a.partner = w.partner;
-                    return launch16<P, RC, 2, 2, 1>(st, pi, map_q, map_q8, a, w.n_ctas, s);
+                if (pairs) {
+                    a.block_off = w.sched[2].run_off;
+                    a.partner = w.sched[2].partner;
+                    a.cta_off = w.sched[2].cta_off;
+                    a.cta_blocks = w.sched[2].cta_runs;
+                    return launch16<P, RC, 2, 2, 1>(st, pi, map_q, map_q8, a, w.sched[2].n_ctas, s);
                 }
-                if (t->tune_stages == 2) return launch16<P, RC, 2, 1, 1>(st, pi, map_q, map_q8, a, w.n_ctas, s);
-                return launch16<P, RC, 3, 1, 1>(st, pi, map_q, map_q8, a, w.n_ctas, s);
+                if (t->tune_stages == 2) return launch16<P, RC, 2, 1, 1>(st, pi, map_q, map_q8, a, w.sched[w.use].n_ctas, s);
+                return launch16<P, RC, 3, 1, 1>(st, pi, map_q, map_q8, a, w.sched[w.use].n_ctas, s);
             }
         }
         if constexpr (RC <= 4) {
             // paired 256-column items: two stages fit next to the 64 KB source tile
-            if (t->tune_pairs && w.sched_off[2]) {
-                a.cta_off = w.sched_off[2];
-                a.cta_blocks = w.sched_blocks[2];
-                a.partner = w.partner;
-                return launch16<P, RC, 2, 2, 0>(st, pi, map_q, map_q8, a, w.n_ctas, s);
+            if (pairs) {
+                a.block_off = w.sched[2].run_off;
+                a.partner = w.sched[2].partner;
+                a.cta_off = w.sched[2].cta_off;
+                a.cta_blocks = w.sched[2].cta_runs;
+                return launch16<P, RC, 2, 2, 0>(st, pi, map_q, map_q8, a, w.sched[2].n_ctas, s);
             }
         }
-        if (t->tune_stages == 2) return launch16<P, RC, 2, 1, 0>(st, pi, map_q, map_q8, a, w.n_ctas, s);
-        return launch16<P, RC, 3, 1, 0>(st, pi, map_q, map_q8, a, w.n_ctas, s);
+        if (t->tune_stages == 2) return launch16<P, RC, 2, 1, 0>(st, pi, map_q, map_q8, a, w.sched[w.use].n_ctas, s);
+        return launch16<P, RC, 3, 1, 0>(st, pi, map_q, map_q8, a, w.sched[w.use].n_ctas, s);
     };
     ASK_TRY(ktimer_mark(t, s, false));
     ASK_TRY(go());
@@ -852,9 +855,9 @@ askit_status eval_tc16(askit_tree t, const WeightCtx &c, int precision, const fl
                       CU_TENSOR_MAP_SWIZZLE_NONE));
     T16Args a;
     a.items = w.items;
-    a.block_off = w.block_off;
-    a.cta_off = w.cta_off;
-    a.cta_blocks = w.cta_blocks;
+    a.block_off = w.sched[w.use].run_off;
+    a.cta_off = w.sched[w.use].cta_off;
+    a.cta_blocks = w.sched[w.use].cta_runs;
     a.tgt = w.tgt;
     a.d_pad = t->d_pad;
     a.cent = t->cent;

@@ -671,16 +671,17 @@ askit_status launch_w(askit_tree t, TcwState *st, int pi, const TcwArgs &a, int 
 template <int P, int RC>
 askit_status run_w(askit_tree t, TcwState *st, int pi, TcwArgs a, const WorkLists &w, cudaStream_t s) {
     // paired items: the two sub-blocks of a node (same targets, same center)
-    // in one 256-column item, on the segments' schedule (several CTAs on one
-    // block at a time, so that its source rows stay in L2 across its items)
-    if (t->tune_pairs && w.seg_sched_off) {
-        a.block_off = w.seg_off;
-        a.partner = w.seg_partner;
-        a.cta_off = w.seg_sched_off;
-        a.cta_blocks = w.seg_sched;
-        return launch_w<P, RC, 2>(t, st, pi, a, w.n_ctas, s);
+    // in one 256-column item (several CTAs on one block at a time, so that its
+    // source rows stay in L2 across its items)
+    if (take_pairs(t, w)) {
+        const WorkLists::Sched &p = w.sched[2];
+        a.block_off = p.run_off;
+        a.partner = p.partner;
+        a.cta_off = p.cta_off;
+        a.cta_blocks = p.cta_runs;
+        return launch_w<P, RC, 2>(t, st, pi, a, p.n_ctas, s);
     }
-    return launch_w<P, RC, 1>(t, st, pi, a, w.n_ctas, s);
+    return launch_w<P, RC, 1>(t, st, pi, a, w.sched[w.use].n_ctas, s);
 }
 
 }  // namespace
@@ -712,9 +713,9 @@ askit_status eval_tc_wide(askit_tree t, const WeightCtx &c, int precision, const
     a.q = Xq;
     a.ldq = ldq;
     a.items = w.items;
-    a.block_off = w.block_off;
-    a.cta_off = w.cta_off;
-    a.cta_blocks = w.cta_blocks;
+    a.block_off = w.sched[w.use].run_off;
+    a.cta_off = w.sched[w.use].cta_off;
+    a.cta_blocks = w.sched[w.use].cta_runs;
     a.partner = nullptr;
     a.tgt = w.tgt;
     a.nkc = t->kw / W_KC;
