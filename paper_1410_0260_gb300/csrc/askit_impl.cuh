@@ -507,8 +507,7 @@ askit_status g16_split_rows(const float *X, int64_t ldx, int d, int64_t rows, co
 inline bool use_g16(const askit_tree_s *t) {
     return t->Xg_hi && (t->fp16_centering == 2 || (t->fp16_centering == 0 && t->g_ok));
 }
-askit_status knn_shortlist_tc16(askit_tree t, const float *Yp, int64_t T, const float *U, int *cnt, int32_t *cand,
-                                int cap, float eta, cudaStream_t s);
+// knn_oos.cu:
 // exact kNN of out-of-sample points Y [T, d] against the tree's points:
 // tensor-core shortlist + canonical FP64 re-rank where the operands exist,
 // else the tiled exhaustive search; ids / dist [T, kappa] as knn_exact_gpu

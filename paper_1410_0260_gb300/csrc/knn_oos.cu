@@ -1,0 +1,710 @@
+// Exact kappa nearest tree points of out-of-sample queries (d <= 64).
+//
+// 1. Home: the two leaves whose centers are nearest to each query (FP32 tiles).
+// 2. Seed: the kappa-th smallest FP32 distance over the points of those leaves,
+//    rounded up by the FP32 sum's error bound, is an upper bound U of the query's
+//    true kappa-th distance.
+// 3. Shortlist: every tree point against every query on the tensor cores, FP16x3;
+//    a point within U and the products' error margin becomes a candidate.
+// 4. Re-rank: FP32 distances of the candidates leave those that can be among the
+//    kappa nearest; only these get their canonical FP64 distance, ordered by
+//    (distance, id).
+// A query with more than KO_CAP candidates, or whose coordinates leave the
+// FP16-safe range, takes the exhaustive search.
+//
+// FP64 runs at 2 lanes an SM and clock here, so the FP64 distances are what the
+// steps avoid: seeding in FP64 over the two leaves took 74 of the 110 ms that
+// 100,000 queries spent against 131,072 points (d = 64), the FP64 re-rank of every
+// candidate 8.8 ms, the shortlist with operands split on the chip 18.6 ms.
+// Now, the same 100,000 queries: home 0.20, seed 1.8, shortlist 5.8, re-rank 2.4 ms.
+#include <cuda.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <mutex>
+
+#include "askit_impl.cuh"
+#include "knn_warp.cuh"
+#include "tc_ptx.cuh"
+
+namespace {
+
+using namespace tcx;
+
+inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
+
+constexpr int KO_CAP = 1024;                   // candidates a query keeps
+// The margin of the FP16x3 distance n_q + n_j - 2 a.b (both sides centered on the
+// data mean, a.b in three split products): the splits keep 22 significant bits and
+// the FP32 accumulation adds a few 2^-23 |a||b| a step, below 2^-18 (n_q + n_j)
+// together; eta = 2^-16.  Coordinates below 2^-13 of the scaled range lose bits of
+// their low half to the FP16 subnormal step 2^-24, an absolute error of at most
+// 2^-25 / sigma a coordinate; by the inequality of the means its share of the
+// distance is below eta/2 (n_q + n_j) + KO_ABS / sigma^2.
+constexpr float KO_ETA = 1.52587890625e-05f;
+constexpr float KO_ABS = 5.9604645e-08f;       // 2^-24
+
+// Relative bound of an FP32 sum of d squared differences, in any order.
+__host__ __device__ __forceinline__ float sum_gam(int d) { return (float)(d + 2) * 5.9604645e-8f * 1.25f + 1e-6f; }
+
+// Queries as FP16x3 operands of the shortlist: (y - xbar) sigma split hi + lo
+// [T_pad, 64], n = |y - xbar|^2; a query outside the FP16-safe range gets zero
+// rows and a full candidate count.  A warp per row; rows past T are zero.
+__global__ void ko_split_kernel(const float *Y, int d, int64_t T, int64_t T_pad, const float *xbar, float sigma,
+                                uint16_t *hi, uint16_t *lo, float *nq, int *cnt) {
+    const int lane = threadIdx.x & 31;
+    const int64_t row = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (row >= T_pad) return;                              // warp-uniform
+    float v[2], acc = 0.f;
+    bool bad = false;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int k = lane + 32 * h;
+        const float x = (row < T && k < d) ? Y[row * d + k] - xbar[k] : 0.f;
+        v[h] = x * sigma;
+        acc = fmaf(x, x, acc);
+        bad |= !(fabsf(v[h]) <= 30000.f);
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(FULL, acc, o);
+    bad = __any_sync(FULL, bad);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int64_t o = row * TC_K + lane + 32 * h;
+        const __half vh = __float2half_rn(bad ? 0.f : v[h]);
+        hi[o] = __half_as_ushort(vh);
+        lo[o] = __half_as_ushort(__float2half_rn(bad ? 0.f : v[h] - __half2float(vh)));
+    }
+    if (lane == 0) {
+        nq[row] = acc;
+        if (row < T) cnt[row] = bad ? KO_CAP + 1 : 0;
+    }
+}
+
+// Step 1.  Block (x, y): queries 64 x .. + 63 against the leaf centers of split y,
+// 64 at a time, FP32 differences from shared memory (4 queries x 8 centers a
+// thread: three 16-byte reads for 64 operations; a warp a query with scalar reads
+// of the centers took 5.5 ms at 100,000 queries and 256 leaves).  Writes the two
+// nearest centers of the split.
+constexpr int HO_T = 64, HO_LD = HO_T + 4;
+__global__ void __launch_bounds__(128) ko_home_kernel(const float *Y, int d, int64_t T, const float *cent,
+                                                      const int32_t *leaf_cbase, int64_t M, int64_t split_len,
+                                                      float *hd, int32_t *hi_) {
+    __shared__ __align__(16) float qs[TC_K][HO_LD], cs[TC_K][HO_LD];
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int64_t q0 = (int64_t)blockIdx.x * HO_T;
+    const int64_t l0 = (int64_t)blockIdx.y * split_len, l1 = min(M, l0 + split_len);
+    for (int e = tid; e < HO_T * TC_K; e += 128) {
+        const int q = e / TC_K, k = e % TC_K;
+        qs[k][q] = (q0 + q < T && k < d) ? Y[(q0 + q) * d + k] : 0.f;
+    }
+    float b0[4], b1[4];
+    int i0[4], i1[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { b0[i] = b1[i] = 3.4e38f; i0[i] = i1[i] = (int)l0; }
+    for (int64_t lb = l0; lb < l1; lb += HO_T) {
+        __syncthreads();
+        for (int e = tid; e < HO_T * TC_K; e += 128) {
+            const int c = e / TC_K, k = e % TC_K;
+            cs[k][c] = (lb + c < l1 && k < d) ? cent[(int64_t)leaf_cbase[lb + c] * TC_K + k] : 0.f;
+        }
+        __syncthreads();
+        float acc[4][8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+        for (int k = 0; k < d; ++k) {
+            const float4 q4 = *reinterpret_cast<const float4 *>(&qs[k][4 * ty]);
+            const float4 ca = *reinterpret_cast<const float4 *>(&cs[k][8 * tx]);
+            const float4 cb = *reinterpret_cast<const float4 *>(&cs[k][8 * tx + 4]);
+            const float qv[4] = {q4.x, q4.y, q4.z, q4.w};
+            const float cv[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float t = qv[i] - cv[j];
+                    acc[i][j] = fmaf(t, t, acc[i][j]);
+                }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int64_t l = lb + 8 * tx + j;
+            if (l >= l1) continue;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (acc[i][j] < b0[i]) { b1[i] = b0[i]; i1[i] = i0[i]; b0[i] = acc[i][j]; i0[i] = (int)l; }
+                else if (acc[i][j] < b1[i]) { b1[i] = acc[i][j]; i1[i] = (int)l; }
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        for (int o = 4; o > 0; o >>= 1) {                  // merge the 8 threads of a query
+            const float ob0 = __shfl_xor_sync(FULL, b0[i], o), ob1 = __shfl_xor_sync(FULL, b1[i], o);
+            const int oi0 = __shfl_xor_sync(FULL, i0[i], o), oi1 = __shfl_xor_sync(FULL, i1[i], o);
+            if (ob0 < b0[i]) {
+                const bool second = b0[i] < ob1;
+                b1[i] = second ? b0[i] : ob1;
+                i1[i] = second ? i0[i] : oi1;
+                b0[i] = ob0;
+                i0[i] = oi0;
+            } else if (ob0 < b1[i]) {
+                b1[i] = ob0;
+                i1[i] = oi0;
+            }
+        }
+        const int64_t q = q0 + 4 * ty + i;
+        if (tx == 0 && q < T) {
+            const int64_t o = ((int64_t)blockIdx.y * T + q) * 2;
+            hd[o] = b0[i];
+            hd[o + 1] = b1[i];
+            hi_[o] = i0[i];
+            hi_[o + 1] = i1[i];
+        }
+    }
+}
+
+// A warp's FP32 squared distances of 32 tree rows to its query: four lanes a row,
+// each with every fourth 16-byte piece (NJ pieces a lane, d_pad = 16 NJ), eight
+// rows at a time; lane l ends with the distance of pos(8 (l & 3) + (l >> 2)).
+template <int NJ, class F>
+__device__ __forceinline__ float rows32(const float *Xt, const float4 (&y)[NJ], int lane, F pos) {
+    const int sub = lane & 3, r8 = lane >> 2;
+    float4 x[4][NJ];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        const float4 *row = reinterpret_cast<const float4 *>(Xt + (int64_t)pos(8 * g + r8) * (16 * NJ)) + sub;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) x[g][j] = row[4 * j];
+    }
+    float v = 0.f;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        float a = 0.f;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const float t0 = y[j].x - x[g][j].x, t1 = y[j].y - x[g][j].y, t2 = y[j].z - x[g][j].z, t3 = y[j].w - x[g][j].w;
+            a = fmaf(t0, t0, a);
+            a = fmaf(t1, t1, a);
+            a = fmaf(t2, t2, a);
+            a = fmaf(t3, t3, a);
+        }
+        a += __shfl_xor_sync(FULL, a, 1);
+        a += __shfl_xor_sync(FULL, a, 2);
+        if (sub == g) v = a;
+    }
+    return v;
+}
+
+template <int NJ>
+__device__ __forceinline__ void load_query(const float *y, int d, int lane, float4 (&q)[NJ]) {
+    const int sub = lane & 3;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int k = 4 * (sub + 4 * j);
+        q[j] = make_float4(k < d ? y[k] : 0.f, k + 1 < d ? y[k + 1] : 0.f, k + 2 < d ? y[k + 2] : 0.f,
+                           k + 3 < d ? y[k + 3] : 0.f);
+    }
+}
+
+// Step 2, a warp per query: U.  The splits' candidates give the two home leaves;
+// their points' FP32 distances pass through a best-32 list.
+template <int NJ>
+__global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const float *Y, int d, int64_t T, const float *hd,
+                                                      const int32_t *hi_, int nsplit, int64_t M, const int32_t *nstart,
+                                                      const int32_t *nsize, int kappa, float *U) {
+    const int lane = threadIdx.x & 31;
+    const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (q >= T) return;                                    // warp-uniform
+    float bd = 3.4e38f;
+    int bi = 0;
+    if (lane < 2 * nsplit) {
+        const int64_t o = ((int64_t)(lane >> 1) * T + q) * 2 + (lane & 1);
+        bd = hd[o];
+        bi = hi_[o];
+    }
+    int leaf[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float m = bd;
+        int w = lane;
+        for (int o = 16; o > 0; o >>= 1) {
+            const float om = __shfl_xor_sync(FULL, m, o);
+            const int ow = __shfl_xor_sync(FULL, w, o);
+            if (om < m || (om == m && ow < w)) { m = om; w = ow; }
+        }
+        leaf[h] = __shfl_sync(FULL, bi, w);
+        if (lane == w) bd = 3.4e38f;
+    }
+    float4 y[NJ];
+    load_query<NJ>(Y + q * d, d, lane, y);
+    float l = 3.4e38f;
+    for (int h = 0; h < 2; ++h) {
+        if (h == 1 && leaf[1] == leaf[0]) break;
+        const int p0 = nstart[M + leaf[h]], np = nsize[M + leaf[h]];
+        for (int b = 0; b < np; b += 32) {
+            // rows past the leaf are other points or the zero rows past N
+            const float v = rows32<NJ>(Xt, y, lane, [&](int i) { return p0 + b + i; });
+            const int i = b + 8 * (lane & 3) + (lane >> 2);
+            warp_offer_f32(l, i < np ? v : 3.4e38f, kappa, lane);
+        }
+    }
+    const float kth = __shfl_sync(FULL, l, kappa - 1);
+    if (lane == 0) U[q] = kth < 3.0e38f ? __fadd_ru(__fmul_ru(kth, 1.f + 2.f * sum_gam(d)), 1e-37f) : 3.4e38f;
+}
+
+// Step 4, a warp per query.
+template <int NJ>
+__global__ void __launch_bounds__(256) ko_rerank_kernel(const float *Xt, const float *Y, int d, int64_t T,
+                                                        const int32_t *perm, const int *cnt, const int32_t *cand,
+                                                        int kappa, int32_t *ids, double *dist, int *n_ovf,
+                                                        int32_t *ovf) {
+    __shared__ float sd[8][KO_CAP];
+    __shared__ float sy[8][TC_K];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (q >= T) return;                                    // warp-uniform
+    const int n = cnt[q];
+    if (n > KO_CAP || n < kappa) {                         // (fewer cannot be: U bounds kappa points)
+        if (lane == 0) ovf[atomicAdd(n_ovf, 1)] = (int32_t)q;
+        return;
+    }
+    const int32_t *c = cand + q * KO_CAP;
+    float4 y[NJ];
+    load_query<NJ>(Y + q * d, d, lane, y);
+    for (int k = lane; k < d; k += 32) sy[warp][k] = Y[q * d + k];
+    float l = 3.4e38f;
+    for (int b = 0; b < n; b += 32) {
+        const int32_t mine = c[min(b + lane, n - 1)];
+        const float v = rows32<NJ>(Xt, y, lane, [&](int i) { return __shfl_sync(FULL, mine, i); });
+        const int i = b + 8 * (lane & 3) + (lane >> 2);
+        if (i < n) sd[warp][i] = v;
+        warp_offer_f32(l, i < n ? v : 3.4e38f, kappa, lane);
+    }
+    __syncwarp();
+    // a point among the kappa nearest has an FP32 distance within (1 + gam) /
+    // (1 - gam) of the kappa-th smallest one
+    const float lim = __shfl_sync(FULL, l, kappa - 1) * (1.f + 3.f * sum_gam(d)) + 1e-37f;
+    double ld = DBL_MAX;
+    int li = INT_MAX;
+    int have = 0;
+    int32_t held = 0;                                      // lane < have: a candidate's tree position
+    auto offer = [&]() {
+        double cd = DBL_MAX;
+        int ci = INT_MAX;
+        if (lane < have) {
+            ci = perm[held];
+            const float *x = Xt + (int64_t)held * (16 * NJ);
+            double acc = 0.0;
+            for (int k = 0; k < d; k += 4) {
+                const float4 xv = *reinterpret_cast<const float4 *>(x + k);
+                const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (k + e < d) {
+                        const double t = c_sub((double)sy[warp][k + e], (double)xs[e]);
+                        acc = c_add(acc, c_mul(t, t));
+                    }
+            }
+            cd = acc;
+        }
+        warp_offer(ld, li, cd, ci, kappa, false, lane);
+        have = 0;
+    };
+    for (int b = 0; b < n; b += 32) {
+        // not "above the limit", so a NaN distance stays in
+        const bool pass = b + lane < n && !(sd[warp][b + lane] > lim);
+        const unsigned m = __ballot_sync(FULL, pass);
+        const int32_t p = pass ? c[b + lane] : 0;
+        // the passing lanes' positions, in order, behind those held
+        const int k = __popc(m);
+        const int src = lane - have >= 0 && lane - have < k ? (int)__fns(m, 0, lane - have + 1) : 0;
+        const int32_t moved = __shfl_sync(FULL, p, src);
+        if (lane >= have && lane < have + k) held = moved;
+        if (have + k < 32) {
+            have += k;
+            continue;
+        }
+        const int rest = have + k - 32;
+        have = 32;
+        offer();
+        // the last `rest` of them start the next group
+        const int src2 = lane < rest ? (int)__fns(m, 0, k - rest + lane + 1) : 0;
+        held = __shfl_sync(FULL, p, src2);
+        have = rest;
+    }
+    if (have > 0) offer();
+    if (lane < kappa) {
+        ids[q * kappa + lane] = li;
+        dist[q * kappa + lane] = ld;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Step 3.  A tile of 256 tree positions stays in shared memory while tiles of 128
+// queries stream through four stages (TMA, 128-byte swizzled K-major FP16 hi and
+// lo); 12 tcgen05.mma (128 x 256 x 16) a tile pair leave sigma^2 a.b in one of two
+// 256-column TMEM accumulators; each of the two epilogue groups takes 128 columns:
+// n_j - 2 a.b / sigma^2 against the query's threshold, 32 columns' minimum first.
+// Bound by the tensor core (12 MMAs of 128 cycles a tile pair against about 1300
+// issue slots of the epilogue).  (source tile, query tile) pairs are dealt in
+// contiguous ranges of equal length, one CTA an SM.
+//   warps 0-7  epilogue, group = columns 128 g ..
+//   warp 8     TMA
+//   warp 9     TMEM allocation, MMA issue
+// Every wait is bounded (ASK_DEV_TIMEOUT).
+// ---------------------------------------------------------------------------
+constexpr int KS_REGION = 128 * 128;           // 128 rows x 64 FP16
+constexpr int KS_NA = 4;
+struct KS {
+    static constexpr int B_HI = 0, B_LO = 2 * KS_REGION;
+    static constexpr int A0 = 4 * KS_REGION;                   // stage: hi, lo
+    static constexpr int COL = A0 + KS_NA * 2 * KS_REGION;     // float [2][256] n_j
+    static constexpr int BAR = COL + 2 * 256 * 4;              // 20 mbarriers
+    static constexpr int MISC = BAR + 20 * 8;
+    static constexpr int BYTES = MISC + 16;
+    static constexpr int THREADS = 320;
+};
+struct KSArgs {
+    int64_t N, T, units;                       // units = source tiles x query tiles
+    int n_qt;
+    const float *nt;                           // [N_pad] |x - xbar|^2 of the tree rows
+    const float *nq, *U;                       // per query
+    float m2u, eta, abs;                       // -2 / sigma^2, KO_ETA, KO_ABS / sigma^2
+    int *cnt;
+    int32_t *cand;
+    int *status;
+};
+
+__global__ void __launch_bounds__(KS::THREADS, 1)
+ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_constant__ CUtensorMap map_ql,
+                    const __grid_constant__ CUtensorMap map_th, const __grid_constant__ CUtensorMap map_tl,
+                    const KSArgs args) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *sm = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const uint32_t sbase = smem_u32(sm), bar0 = sbase + KS::BAR;
+    auto BAR_A_FULL = [&](int s) { return bar0 + 8 * s; };
+    auto BAR_A_EMPTY = [&](int s) { return bar0 + 8 * (4 + s); };
+    const uint32_t BAR_B_FULL = bar0 + 8 * 8, BAR_B_EMPTY = bar0 + 8 * 9;
+    auto BAR_T_FULL = [&](int a) { return bar0 + 8 * (10 + a); };
+    auto BAR_T_EMPTY = [&](int a) { return bar0 + 8 * (12 + a); };
+    auto BAR_C_FULL = [&](int s) { return bar0 + 8 * (14 + s); };   // n_j of source tile (slot lb & 1)
+    auto BAR_C_EMPTY = [&](int s) { return bar0 + 8 * (16 + s); };
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sm + KS::MISC);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(sm + KS::MISC + 4);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int s = 0; s < KS_NA; ++s) {
+            mbar_init(BAR_A_FULL(s), 1);
+            mbar_init(BAR_A_EMPTY(s), 1);
+        }
+        mbar_init(BAR_B_FULL, 1);
+        mbar_init(BAR_B_EMPTY, 1);
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(BAR_T_FULL(a), 1);
+            mbar_init(BAR_T_EMPTY(a), 256);
+            mbar_init(BAR_C_FULL(a), 1);
+            mbar_init(BAR_C_EMPTY(a), 256);
+        }
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 9) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    // this CTA's units u0 .. u1 - 1; unit u: source tile u / n_qt, query tile u % n_qt
+    const int64_t u0 = args.units * blockIdx.x / gridDim.x, u1 = args.units * (blockIdx.x + 1) / gridDim.x;
+    const int n_qt = args.n_qt;
+
+    if (warp < 8) {
+        const int q4 = warp & 3, eg = warp >> 2, row = q4 * 32 + lane;
+        int li = 0, lb = -1;
+        int64_t bt = -1;
+        const float *col = nullptr;
+        const float m2 = args.m2u / (1.f - args.eta);
+        const float2 m22 = make_float2(m2, m2);
+        for (int64_t u = u0; u < u1; ++u, ++li) {
+            const int64_t b = u / n_qt;
+            const int qt = (int)(u - b * n_qt);
+            if (b != bt) {
+                if (lb >= 0) mbar_arrive(BAR_C_EMPTY(lb & 1));
+                ++lb;
+                bt = b;
+                if (!mbar_wait(BAR_C_FULL(lb & 1), (lb >> 1) & 1, abort_flag, args.status)) break;
+                col = reinterpret_cast<const float *>(sm + KS::COL) + (lb & 1) * 256 + 128 * eg;
+            }
+            const int64_t q = (int64_t)qt * 128 + row;
+            // n_j (1 - eta) - 2 a.b <= U (1 + eta) - n_q (1 - eta) + abs
+            const float thr = q < args.T ? (args.U[q] * (1.f + args.eta) + args.abs) / (1.f - args.eta) - args.nq[q]
+                                         : -INFINITY;
+            const int a = li & 1;
+            if (!mbar_wait(BAR_T_FULL(a), (li >> 1) & 1, abort_flag, args.status)) break;
+            tc_fence_after();
+            const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * 256 + 128 * eg);
+            const int64_t pos0 = b * 256 + 128 * eg;
+            auto chunk = [&](int c, const uint32_t (&g)[32]) {
+                float dd[32], m = INFINITY;
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) {
+                    const float4 n4 = *reinterpret_cast<const float4 *>(col + c * 32 + j);
+                    const float2 x = __ffma2_rn(make_float2(__uint_as_float(g[j]), __uint_as_float(g[j + 1])), m22,
+                                                make_float2(n4.x, n4.y));
+                    const float2 z = __ffma2_rn(make_float2(__uint_as_float(g[j + 2]), __uint_as_float(g[j + 3])), m22,
+                                                make_float2(n4.z, n4.w));
+                    dd[j] = x.x;
+                    dd[j + 1] = x.y;
+                    dd[j + 2] = z.x;
+                    dd[j + 3] = z.y;
+                    m = fminf(m, fminf(fminf(x.x, x.y), fminf(z.x, z.y)));
+                }
+                if (m <= thr) {
+                    uint32_t hit = 0;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) hit |= dd[j] <= thr ? 1u << j : 0u;
+                    const int64_t p0 = pos0 + c * 32;
+                    if (p0 + 32 > args.N) hit &= p0 < args.N ? (1u << (args.N - p0)) - 1u : 0u;   // rows past N
+                    int k = atomicAdd(args.cnt + q, __popc(hit));
+                    while (hit) {
+                        const int j = __ffs(hit) - 1;
+                        hit &= hit - 1;
+                        if (k < KO_CAP) args.cand[q * KO_CAP + k] = (int32_t)(p0 + j);
+                        ++k;
+                    }
+                }
+            };
+            uint32_t ga[32], gb[32];
+            tmem_ld32_async(tbase, ga);
+            tmem_wait_pin(ga);
+            tmem_ld32_async(tbase + 32, gb);
+            chunk(0, ga);
+            tmem_wait_pin(gb);
+            tmem_ld32_async(tbase + 64, ga);
+            chunk(1, gb);
+            tmem_wait_pin(ga);
+            tmem_ld32_async(tbase + 96, gb);
+            chunk(2, ga);
+            tmem_wait_pin(gb);
+            tc_fence_before();
+            mbar_arrive(BAR_T_EMPTY(a));       // all columns are in registers
+            chunk(3, gb);
+        }
+    } else if (warp == 8 && lane == 0) {
+        int li = 0, lb = -1;
+        int64_t bt = -1;
+        for (int64_t u = u0; u < u1; ++u, ++li) {
+            const int64_t b = u / n_qt;
+            const int qt = (int)(u - b * n_qt);
+            if (b != bt) {
+                ++lb;
+                bt = b;
+                const int cs = lb & 1;
+                if (!mbar_wait(BAR_C_EMPTY(cs), ((lb >> 1) & 1) ^ 1, abort_flag, args.status)) { --lb; goto tma_done; }
+                mbar_expect_tx(BAR_C_FULL(cs), 1024);
+                bulk_copy(sbase + KS::COL + cs * 1024, args.nt + b * 256, 1024, BAR_C_FULL(cs));
+                if (!mbar_wait(BAR_B_EMPTY, (lb & 1) ^ 1, abort_flag, args.status)) {
+                    mbar_drain(BAR_C_FULL(cs), (lb >> 1) & 1);
+                    --lb;
+                    goto tma_done;
+                }
+                mbar_expect_tx(BAR_B_FULL, 4 * KS_REGION);
+                for (int h = 0; h < 2; ++h) {
+                    tma_load_2d(sbase + KS::B_HI + h * KS_REGION, &map_th, 0, (int)(b * 256 + 128 * h), BAR_B_FULL);
+                    tma_load_2d(sbase + KS::B_LO + h * KS_REGION, &map_tl, 0, (int)(b * 256 + 128 * h), BAR_B_FULL);
+                }
+            }
+            const int s = li % KS_NA;
+            if (!mbar_wait(BAR_A_EMPTY(s), ((li / KS_NA) & 1) ^ 1, abort_flag, args.status)) goto tma_done;
+            const uint32_t st = sbase + KS::A0 + s * 2 * KS_REGION;
+            mbar_expect_tx(BAR_A_FULL(s), 2 * KS_REGION);
+            tma_load_2d(st, &map_qh, 0, qt * 128, BAR_A_FULL(s));
+            tma_load_2d(st + KS_REGION, &map_ql, 0, qt * 128, BAR_A_FULL(s));
+        }
+    tma_done:
+        // nothing may land in shared memory after the CTA has left (no-ops unless
+        // a wait gave up)
+        for (int k = li > KS_NA ? li - KS_NA : 0; k < li; ++k) mbar_drain(BAR_A_FULL(k % KS_NA), (k / KS_NA) & 1);
+        if (lb >= 0) {
+            mbar_drain(BAR_B_FULL, lb & 1);
+            mbar_drain(BAR_C_FULL(lb & 1), (lb >> 1) & 1);
+        }
+    } else if (warp == 9 && lane == 0) {
+        constexpr uint32_t IDESC = make_idesc(0u, 128, 256);
+        int li = 0, lb = -1, done = -1;
+        int64_t bt = -1;
+        for (int64_t u = u0; u < u1; ++u, ++li) {
+            const int64_t b = u / n_qt;
+            if (b != bt) {
+                if (lb >= 0) tc_commit(BAR_B_EMPTY);       // the last tile's MMAs have read it
+                ++lb;
+                bt = b;
+                if (!mbar_wait(BAR_B_FULL, lb & 1, abort_flag, args.status)) break;
+            }
+            const int s = li % KS_NA, a = li & 1;
+            if (!mbar_wait(BAR_A_FULL(s), (li / KS_NA) & 1, abort_flag, args.status)) break;
+            if (!mbar_wait(BAR_T_EMPTY(a), ((li >> 1) & 1) ^ 1, abort_flag, args.status)) break;
+            tc_fence_after();
+            const uint32_t dt = tmem + (uint32_t)(a * 256);
+            const uint32_t ah = sbase + KS::A0 + s * 2 * KS_REGION, al = ah + KS_REGION;
+            const uint32_t bh = sbase + KS::B_HI, bl = sbase + KS::B_LO;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {                  // the small cross terms first
+                const uint32_t off = (uint32_t)(k * 32);
+                tc_mma<ASKIT_PREC_FP16X3>(dt, sw128_desc(ah + off), sw128_desc(bl + off), IDESC, k > 0);
+                tc_mma<ASKIT_PREC_FP16X3>(dt, sw128_desc(al + off), sw128_desc(bh + off), IDESC, 1);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t off = (uint32_t)(k * 32);
+                tc_mma<ASKIT_PREC_FP16X3>(dt, sw128_desc(ah + off), sw128_desc(bh + off), IDESC, 1);
+            }
+            tc_commit(BAR_A_EMPTY(s));
+            tc_commit(BAR_T_FULL(a));
+            done = li;
+        }
+        // MMAs in flight after an abort end before TMEM is freed
+        if (done >= 0) mbar_drain(BAR_T_FULL(done & 1), (done >> 1) & 1);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 9) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    }
+}
+
+__global__ void ko_gather_kernel(const float *Y, int d, const int32_t *rows, int64_t n, float *out) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= n * d) return;
+    out[e] = Y[(int64_t)rows[e / d] * d + e % d];
+}
+
+__global__ void ko_scatter_kernel(const int32_t *ids_s, const double *dist_s, const int32_t *rows, int64_t n,
+                                  int kappa, int32_t *ids, double *dist) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= n * kappa) return;
+    const int64_t q = rows[e / kappa];
+    ids[q * kappa + e % kappa] = ids_s[e];
+    dist[q * kappa + e % kappa] = dist_s[e];
+}
+
+// Tensor maps of the tree's split target rows, here the shortlist's sources.
+askit_status tree_maps(askit_tree t, EncodeTiledFn fn, CUtensorMap *th, CUtensorMap *tl) {
+    ASK_TRY(encode_2d(fn, th, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, t->Xg_hi, t->N_pad, TC_K, 64, 128,
+                      CU_TENSOR_MAP_SWIZZLE_128B));
+    return encode_2d(fn, tl, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, t->Xg_lo, t->N_pad, TC_K, 64, 128,
+                     CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+}  // namespace
+
+askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t *ids, double *dist, cudaStream_t s) {
+    if (!t->Xg_hi || t->d > TC_K || kappa > 32)
+        return knn_exact_gpu(t->X, t->N, t->d, kappa, Y, T, ids, dist, s);
+    const int d = t->d;
+    const int64_t M = (int64_t)1 << t->L, N = t->N;
+    const int64_t T_pad = (T + 127) / 128 * 128;
+    // splits of the leaf centers, so that few queries still fill the GPU
+    int sms = 0, dev = 0;
+    ASK_CUDA(cudaGetDevice(&dev));
+    ASK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int64_t qb = (T + HO_T - 1) / HO_T;
+    int64_t nsplit = std::max<int64_t>(1, std::min<int64_t>(16, std::min<int64_t>((M + HO_T - 1) / HO_T, sms / qb)));
+    const int64_t split_len = ((M + nsplit - 1) / nsplit + HO_T - 1) / HO_T * HO_T;
+    nsplit = (M + split_len - 1) / split_len;
+    DevArena tmp;
+    tmp.async = true;
+    tmp.stream = s;
+    // one allocation: every part at a multiple of 256 bytes
+    size_t used = 0;
+    auto part = [&](size_t bytes) {
+        const size_t o = used;
+        used += (bytes + 255) / 256 * 256;
+        return o;
+    };
+    const size_t o_hi = part((size_t)T_pad * TC_K * 2), o_lo = part((size_t)T_pad * TC_K * 2), o_nq = part((size_t)T_pad * 4),
+                 o_hd = part((size_t)nsplit * T * 8), o_hx = part((size_t)nsplit * T * 8), o_u = part((size_t)T * 4),
+                 o_cnt = part((size_t)T * 4), o_ovf = part((size_t)(T + 1) * 4), o_cand = part((size_t)T * KO_CAP * 4);
+    uint8_t *buf = nullptr;
+    ASK_TRY(tmp.alloc(&buf, used));
+    uint16_t *qh = reinterpret_cast<uint16_t *>(buf + o_hi), *ql = reinterpret_cast<uint16_t *>(buf + o_lo);
+    float *nq = reinterpret_cast<float *>(buf + o_nq), *hd = reinterpret_cast<float *>(buf + o_hd),
+          *U = reinterpret_cast<float *>(buf + o_u);
+    int32_t *hx = reinterpret_cast<int32_t *>(buf + o_hx), *cand = reinterpret_cast<int32_t *>(buf + o_cand);
+    int *cnt = reinterpret_cast<int *>(buf + o_cnt), *n_ovf = reinterpret_cast<int *>(buf + o_ovf);
+    int32_t *ovf = n_ovf + 1;
+    int h_ovf = 0;
+    askit_status rc = ASKIT_OK;
+#define QTRY(x) do { rc = (x); if (rc != ASKIT_OK) goto out; } while (0)
+#define QCHK(x) do { const cudaError_t e_ = (x); if (e_ != cudaSuccess) { askit_set_error("out-of-sample kNN: %s", cudaGetErrorString(e_)); rc = e_ == cudaErrorMemoryAllocation ? ASKIT_ERR_OOM : ASKIT_ERR_CUDA; goto out; } } while (0)
+    QCHK(cudaMemsetAsync(n_ovf, 0, sizeof(int), s));
+    ko_split_kernel<<<nblk(T_pad, 8), 256, 0, s>>>(Y, d, T, T_pad, t->g_xbar, t->g_sigma, qh, ql, nq, cnt);
+    ko_home_kernel<<<dim3((unsigned)qb, (unsigned)nsplit), 128, 0, s>>>(Y, d, T, t->cent, t->leaf_cbase, M, split_len, hd,
+                                                                        hx);
+    if (t->d_pad == 32)
+        ko_seed_kernel<2><<<nblk(T, 8), 256, 0, s>>>(t->Xt, Y, d, T, hd, hx, (int)nsplit, M, t->nstart, t->nsize, kappa, U);
+    else
+        ko_seed_kernel<4><<<nblk(T, 8), 256, 0, s>>>(t->Xt, Y, d, T, hd, hx, (int)nsplit, M, t->nstart, t->nsize, kappa, U);
+    QCHK(cudaGetLastError());
+    {
+        EncodeTiledFn fn = nullptr;
+        CUtensorMap mth, mtl, mqh, mql;
+        QTRY(encode_fn(&fn));
+        QTRY(tree_maps(t, fn, &mth, &mtl));
+        QTRY(encode_2d(fn, &mqh, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, qh, T_pad, TC_K, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B));
+        QTRY(encode_2d(fn, &mql, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ql, T_pad, TC_K, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B));
+        KSArgs a;
+        a.N = N;
+        a.T = T;
+        a.n_qt = (int)(T_pad / 128);
+        a.units = (N + 255) / 256 * a.n_qt;
+        a.nt = t->ng_t;
+        a.nq = nq;
+        a.U = U;
+        a.m2u = -2.f / (t->g_sigma * t->g_sigma);
+        a.eta = KO_ETA;
+        a.abs = KO_ABS / (t->g_sigma * t->g_sigma);
+        a.cnt = cnt;
+        a.cand = cand;
+        a.status = t->d_status;
+        constexpr size_t smem = KS::BYTES + 1024;
+        static_assert(smem <= 232448, "shared-memory plan exceeds 227 KB");
+        static const cudaError_t attr =
+            cudaFuncSetAttribute(ko_shortlist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        QCHK(attr);
+        ko_shortlist_kernel<<<(unsigned)std::min<int64_t>(sms, a.units), KS::THREADS, smem, s>>>(mqh, mql, mth, mtl, a);
+        QCHK(cudaGetLastError());
+    }
+    if (t->d_pad == 32)
+        ko_rerank_kernel<2><<<nblk(T, 8), 256, 0, s>>>(t->Xt, Y, d, T, t->perm, cnt, cand, kappa, ids, dist, n_ovf, ovf);
+    else
+        ko_rerank_kernel<4><<<nblk(T, 8), 256, 0, s>>>(t->Xt, Y, d, T, t->perm, cnt, cand, kappa, ids, dist, n_ovf, ovf);
+    QCHK(cudaGetLastError());
+    QCHK(cudaMemcpyAsync(&h_ovf, n_ovf, sizeof(int), cudaMemcpyDeviceToHost, s));
+    QCHK(cudaStreamSynchronize(s));
+    if (h_ovf > 0) {
+        // the exhaustive search
+        float *Ys = nullptr;
+        int32_t *ids_s = nullptr;
+        double *dist_s = nullptr;
+        QTRY(tmp.alloc(&Ys, (size_t)h_ovf * d));
+        QTRY(tmp.alloc(&ids_s, (size_t)h_ovf * kappa));
+        QTRY(tmp.alloc(&dist_s, (size_t)h_ovf * kappa));
+        ko_gather_kernel<<<nblk((int64_t)h_ovf * d, 256), 256, 0, s>>>(Y, d, ovf, h_ovf, Ys);
+        QTRY(knn_exact_gpu(t->X, N, d, kappa, Ys, h_ovf, ids_s, dist_s, s));
+        ko_scatter_kernel<<<nblk((int64_t)h_ovf * kappa, 256), 256, 0, s>>>(ids_s, dist_s, ovf, h_ovf, kappa, ids, dist);
+        QCHK(cudaGetLastError());
+        QCHK(cudaStreamSynchronize(s));
+    }
+out:
+#undef QTRY
+#undef QCHK
+    tmp.free_all();
+    return rc;
+}
