@@ -138,6 +138,20 @@ askit_status validate(const askit_params *p, int64_t N, int32_t d, int64_t ldx, 
     return ASKIT_OK;
 }
 
+askit_status make_pool(askit_tree t) {
+    cudaMemPoolProps p = {};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.handleTypes = cudaMemHandleTypeNone;
+    p.location.type = cudaMemLocationTypeDevice;
+    ASK_CUDA(cudaGetDevice(&p.location.id));
+    ASK_CUDA(cudaMemPoolCreate(&t->pool, &p));
+    uint64_t keep = ASK_POOL_KEEP;
+    int no = 0;
+    ASK_CUDA(cudaMemPoolSetAttribute(t->pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    ASK_CUDA(cudaMemPoolSetAttribute(t->pool, cudaMemPoolReuseAllowInternalDependencies, &no));
+    return ASKIT_OK;
+}
+
 // Wall time of setup stage k (host clock, the stream drained at each mark).
 askit_status stage_mark(askit_tree t, int k, cudaStream_t s) {
     ASK_CUDA(cudaStreamSynchronize(s));
@@ -407,11 +421,13 @@ askit_status askit_setup(const float *X_dev, int64_t N, int32_t d, int64_t ldx, 
         return ASKIT_ERR_UNSUPPORTED;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    askit_status rc = setup_impl(t, X_dev, ldx, h_dev, knn_dev, s);
+    askit_status rc = make_pool(t);
+    if (rc == ASKIT_OK) rc = setup_impl(t, X_dev, ldx, h_dev, knn_dev, s);
     if (rc != ASKIT_OK) {
         cudaStreamSynchronize(s);
         eval_tc_free(t);
         t->arena.free_all();
+        if (t->pool) cudaMemPoolDestroy(t->pool);
         delete t;
         return rc;
     }
@@ -454,6 +470,7 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     DevArena tmp;
     tmp.async = true;
     tmp.stream = s;
+    tmp.pool = t->pool;
     float *Yc = nullptr, *Yt = nullptr;
     int32_t *ids = nullptr, *ids_s = nullptr, *order = nullptr, *vals = nullptr, *sets = nullptr;
     double *dist = nullptr, *dist_s = nullptr;
@@ -677,6 +694,7 @@ askit_status askit_destroy(askit_tree t) {
     eval_tc_free(t);
     t->dw.arena.free_all();
     t->arena.free_all();
+    if (t->pool) cudaMemPoolDestroy(t->pool);
     delete t;
     return ASKIT_OK;
 }

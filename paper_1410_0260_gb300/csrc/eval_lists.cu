@@ -161,26 +161,36 @@ __global__ void leaf_row_kernel(const int32_t *perm, const int32_t *leafof, int6
     row[q] = leafof[perm[q]] - M;
 }
 
-// Out-of-sample prune sets: distinct leaves of N_y (its first kappa_y
-// neighbors; no self term).
+// Out-of-sample prune sets: the sorted distinct leaves of N_y (its first kappa_y
+// neighbors; no self term), a warp per target, a neighbor per lane (kappa <= 32).
 __global__ void oos_sets_kernel(const int32_t *leafof, const int32_t *knn, const double *dist, const float *hsrc,
                                 double kscale, double cut, int64_t T, int kappa, int stride, int32_t *sets) {
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= T) return;
-    int32_t *o = sets + q * stride;
-    int n = 0;
-    const int ky = kappa_of(dist + q * kappa, knn + q * kappa, kappa, hsrc, kscale, cut);
-    for (int z = 0; z < ky; ++z) {
-        int32_t lf = leafof[knn[q * kappa + z]];
-        int p = n;
-        bool dup = false;
-        for (int u = 0; u < n; ++u) dup |= (o[u] == lf);
-        if (dup) continue;
-        while (p > 0 && o[p - 1] > lf) { o[p] = o[p - 1]; --p; }
-        o[p] = lf;
-        ++n;
+    const int lane = threadIdx.x & 31;
+    const int64_t q = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (q >= T) return;                                    // warp-uniform
+    const bool in = lane < kappa;
+    const int32_t id = in ? knn[q * kappa + lane] : 0;
+    int ky = kappa;                                        // kappa_of over the lanes
+    if (cut > 0.0) {
+        const double h = (double)hsrc[id];
+        const bool keep = in && c_div(c_mul(kscale, dist[q * kappa + lane]), c_mul(h, h)) < cut;
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        ky = m ? 32 - __clz(m) : 0;
     }
-    for (int u = n; u < stride; ++u) o[u] = INT_MAX;
+    int32_t v = in && lane < ky ? leafof[id] : INT_MAX;
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const int32_t o = __shfl_xor_sync(0xffffffffu, v, j);
+            v = (((lane & j) == 0) == ((lane & k) == 0)) ? min(v, o) : max(v, o);
+        }
+    const int32_t prev = __shfl_up_sync(0xffffffffu, v, 1);
+    const bool first = v != INT_MAX && (lane == 0 || v != prev);
+    const unsigned m = __ballot_sync(0xffffffffu, first);
+    int32_t *o = sets + q * stride;
+    if (first) o[__popc(m & ((1u << lane) - 1u))] = v;
+    for (int u = __popc(m) + lane; u < stride; u += 32) o[u] = INT_MAX;
 }
 
 // Prune-set row of target q: its own row, or a shared one (leaf-grouped).
@@ -702,7 +712,7 @@ askit_status insample_prune_sets(askit_tree t, PruneSets &ps, cudaStream_t s) {
 
 askit_status oos_prune_sets(askit_tree t, const int32_t *knn, const double *dist, int64_t T, int stride,
                             int32_t *sets, cudaStream_t s) {
-    oos_sets_kernel<<<nblk(T, 128), 128, 0, s>>>(t->leafof, knn, dist, t->hsrc, t->prm.kernel_scale, t->kappa_cut, T,
+    oos_sets_kernel<<<nblk(T, 8), 256, 0, s>>>(t->leafof, knn, dist, t->hsrc, t->prm.kernel_scale, t->kappa_cut, T,
                                                  t->kappa, stride, sets);
     ASK_LAUNCH();
     return ASKIT_OK;
@@ -770,10 +780,13 @@ askit_status build_work_lists(askit_tree t, const int32_t *sets, int stride, con
     while (((int64_t)1 << bits) < n_sub) ++bits;
     WorkLists &w = wlst;
     w.T = T;
+    auto temp = [&](void **p, size_t bytes) {
+        return arena.async ? cudaMallocFromPoolAsync(p, bytes, arena.pool, s) : cudaMallocAsync(p, bytes, s);
+    };
 #define WCHK(x) do { e = (x); if (e != cudaSuccess) goto fail; } while (0)
 #define WTRY(x) do { rc = (x); if (rc != ASKIT_OK) goto out; } while (0)
-    WCHK(cudaMallocAsync(&cnt, sizeof(int64_t) * (T + 1), s));
-    WCHK(cudaMallocAsync(&tot, sizeof(unsigned long long) * 3, s));
+    WCHK(temp((void **)&cnt, sizeof(int64_t) * (T + 1)));
+    WCHK(temp((void **)&tot, sizeof(unsigned long long) * 3));
     WTRY(arena.alloc(&w.off, T + 1));
     WCHK(cudaMemsetAsync(cnt + T, 0, sizeof(int64_t), s));
     WCHK(cudaMemsetAsync(tot, 0, sizeof(unsigned long long) * 3, s));
@@ -782,7 +795,7 @@ askit_status build_work_lists(askit_tree t, const int32_t *sets, int stride, con
                                                    nullptr);
     WCHK(cudaGetLastError());
     WTRY(scan_i64(nullptr, nullptr, T + 1, nullptr, &tb, s));
-    WCHK(cudaMallocAsync(&tmp, tb, s));
+    WCHK(temp((void **)&tmp, tb));
     WTRY(scan_i64(cnt, w.off, T + 1, tmp, &tb, s));
     WCHK(cudaMemcpyAsync(&total, w.off + T, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     WCHK(cudaMemcpyAsync(h_tot, tot, sizeof h_tot, cudaMemcpyDeviceToHost, s));
@@ -797,17 +810,17 @@ askit_status build_work_lists(askit_tree t, const int32_t *sets, int stride, con
         rc = ASKIT_ERR_UNSUPPORTED;
         goto out;
     }
-    WCHK(cudaMallocAsync(&keys, sizeof(uint32_t) * std::max<int64_t>(1, total), s));
-    WCHK(cudaMallocAsync(&keys_s, sizeof(uint32_t) * std::max<int64_t>(1, total), s));
-    WCHK(cudaMallocAsync(&vals, sizeof(int32_t) * std::max<int64_t>(1, total), s));
-    WCHK(cudaMallocAsync(&emit_of, sizeof(int32_t) * std::max<int64_t>(1, total), s));
-    WCHK(cudaMallocAsync(&tq, sizeof(int32_t) * std::max<int64_t>(1, total), s));
-    WCHK(cudaMallocAsync(&start, sizeof(int32_t) * (n_sub + 1), s));
+    WCHK(temp((void **)&keys, sizeof(uint32_t) * std::max<int64_t>(1, total)));
+    WCHK(temp((void **)&keys_s, sizeof(uint32_t) * std::max<int64_t>(1, total)));
+    WCHK(temp((void **)&vals, sizeof(int32_t) * std::max<int64_t>(1, total)));
+    WCHK(temp((void **)&emit_of, sizeof(int32_t) * std::max<int64_t>(1, total)));
+    WCHK(temp((void **)&tq, sizeof(int32_t) * std::max<int64_t>(1, total)));
+    WCHK(temp((void **)&start, sizeof(int32_t) * (n_sub + 1)));
     lists_kernel<true><<<nblk(T, 8), 256, 0, s>>>(sets, stride, set_row, T, t->L, t->far_height, t->nsize, t->d_s,
                                                   t->leaf_cbase, t->node_cbase, w.off, nullptr, nullptr, keys, vals, tq);
     WCHK(cudaGetLastError());
     WTRY(sort_u32_i32(nullptr, nullptr, nullptr, nullptr, total, bits, nullptr, &tb2, s));
-    WCHK(cudaMallocAsync(&tmp, tb2, s));
+    WCHK(temp((void **)&tmp, tb2));
     WTRY(sort_u32_i32(keys, keys_s, vals, emit_of, total, bits, tmp, &tb2, s));
     sub_start_kernel<<<nblk(n_sub + 1, 128), 128, 0, s>>>(keys_s, total, n_sub, start);
     WCHK(cudaGetLastError());

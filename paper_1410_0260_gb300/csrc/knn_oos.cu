@@ -16,7 +16,8 @@
 // steps avoid: seeding in FP64 over the two leaves took 74 of the 110 ms that
 // 100,000 queries spent against 131,072 points (d = 64), the FP64 re-rank of every
 // candidate 8.8 ms, the shortlist with operands split on the chip 18.6 ms.
-// Now, the same 100,000 queries: home 0.20, seed 1.8, shortlist 5.8, re-rank 2.4 ms.
+// Now, the same 100,000 queries: home 0.20, seed 1.7, shortlist
+// 4.8, re-rank 2.4 ms
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -208,15 +209,19 @@ __device__ __forceinline__ void load_query(const float *y, int d, int lane, floa
     }
 }
 
-// Step 2, a warp per query: U.  The splits' candidates give the two home leaves;
-// their points' FP32 distances pass through a best-32 list.
-template <int NJ>
+// Step 2, W warps per query: U.  The splits' candidates give the two home leaves;
+// their points' FP32 distances pass through the warps' best-32 lists, merged at
+// the end.  One warp a query where the queries fill the GPU, four below that (one
+// query is a chain of about 32 rounds of loads and merges: 51 us at 100 queries).
+template <int NJ, int W>
 __global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const float *Y, int d, int64_t T, const float *hd,
                                                       const int32_t *hi_, int nsplit, int64_t M, const int32_t *nstart,
                                                       const int32_t *nsize, int kappa, float *U) {
     const int lane = threadIdx.x & 31;
-    const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (q >= T) return;                                    // warp-uniform
+    const int warp = threadIdx.x >> 5;
+    const int64_t qw = blockIdx.x * (int64_t)(8 / W) + warp / W;
+    const int64_t q = qw < T ? qw : T - 1;                 // warps past T repeat the last query
+    __shared__ float lists[8][32];
     float bd = 3.4e38f;
     int bi = 0;
     if (lane < 2 * nsplit) {
@@ -243,15 +248,21 @@ __global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const flo
     for (int h = 0; h < 2; ++h) {
         if (h == 1 && leaf[1] == leaf[0]) break;
         const int p0 = nstart[M + leaf[h]], np = nsize[M + leaf[h]];
-        for (int b = 0; b < np; b += 32) {
+        for (int b = 32 * (warp % W); b < np; b += 32 * W) {
             // rows past the leaf are other points or the zero rows past N
             const float v = rows32<NJ>(Xt, y, lane, [&](int i) { return p0 + b + i; });
             const int i = b + 8 * (lane & 3) + (lane >> 2);
             warp_offer_f32(l, i < np ? v : 3.4e38f, kappa, lane);
         }
     }
+    if (W > 1) {
+        lists[warp][lane] = l;
+        __syncthreads();
+        if (warp % W) return;
+        for (int w = 1; w < W; ++w) warp_offer_f32(l, lists[warp + w][lane], kappa, lane);
+    }
     const float kth = __shfl_sync(FULL, l, kappa - 1);
-    if (lane == 0) U[q] = kth < 3.0e38f ? __fadd_ru(__fmul_ru(kth, 1.f + 2.f * sum_gam(d)), 1e-37f) : 3.4e38f;
+    if (lane == 0 && qw < T) U[q] = kth < 3.0e38f ? __fadd_ru(__fmul_ru(kth, 1.f + 2.f * sum_gam(d)), 1e-37f) : 3.4e38f;
 }
 
 // Step 4, a warp per query.
@@ -430,6 +441,34 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
         const float *col = nullptr;
         const float m2 = args.m2u / (1.f - args.eta);
         const float2 m22 = make_float2(m2, m2);
+        // this row's query of a unit: n_j (1 - eta) - 2 a.b <= U (1 + eta) - n_q (1 - eta) + abs
+        auto load = [&](int64_t u, float &un, float &nn) {
+            const int64_t q = u < u1 ? (u % n_qt) * 128 + row : args.T;
+            un = q < args.T ? args.U[q] : -INFINITY;
+            nn = q < args.T ? args.nq[q] : 0.f;
+        };
+        float un, nn;
+        load(u0, un, nn);
+        // A unit's hits stay in four masks; their places in the query's list come
+        // from one counter update a unit, whose answer is waited for only after the
+        // next unit (waiting for one a chunk made the epilogue three times as long
+        // as the MMAs)
+        uint32_t ph[4] = {0, 0, 0, 0};
+        int pk = 0;
+        int64_t pq = 0, pp = 0;
+        auto flush = [&]() {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint32_t m = ph[c];
+                while (m) {
+                    const int j = __ffs(m) - 1;
+                    m &= m - 1;
+                    if (pk < KO_CAP) args.cand[pq * KO_CAP + pk] = (int32_t)(pp + 32 * c + j);
+                    ++pk;
+                }
+            }
+            __syncwarp();
+        };
         for (int64_t u = u0; u < u1; ++u, ++li) {
             const int64_t b = u / n_qt;
             const int qt = (int)(u - b * n_qt);
@@ -441,15 +480,14 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
                 col = reinterpret_cast<const float *>(sm + KS::COL) + (lb & 1) * 256 + 128 * eg;
             }
             const int64_t q = (int64_t)qt * 128 + row;
-            // n_j (1 - eta) - 2 a.b <= U (1 + eta) - n_q (1 - eta) + abs
-            const float thr = q < args.T ? (args.U[q] * (1.f + args.eta) + args.abs) / (1.f - args.eta) - args.nq[q]
-                                         : -INFINITY;
+            const float thr = (un * (1.f + args.eta) + args.abs) / (1.f - args.eta) - nn;
+            load(u + 1, un, nn);
             const int a = li & 1;
             if (!mbar_wait(BAR_T_FULL(a), (li >> 1) & 1, abort_flag, args.status)) break;
             tc_fence_after();
             const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * 256 + 128 * eg);
             const int64_t pos0 = b * 256 + 128 * eg;
-            auto chunk = [&](int c, const uint32_t (&g)[32]) {
+            auto chunk = [&](int c, const uint32_t (&g)[32]) -> uint32_t {
                 float dd[32], m = INFINITY;
 #pragma unroll
                 for (int j = 0; j < 32; j += 4) {
@@ -464,37 +502,40 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
                     dd[j + 3] = z.y;
                     m = fminf(m, fminf(fminf(x.x, x.y), fminf(z.x, z.y)));
                 }
-                if (m <= thr) {
-                    uint32_t hit = 0;
+                uint32_t hit = 0;
+                if (__any_sync(FULL, m <= thr)) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) hit |= dd[j] <= thr ? 1u << j : 0u;
                     const int64_t p0 = pos0 + c * 32;
                     if (p0 + 32 > args.N) hit &= p0 < args.N ? (1u << (args.N - p0)) - 1u : 0u;   // rows past N
-                    int k = atomicAdd(args.cnt + q, __popc(hit));
-                    while (hit) {
-                        const int j = __ffs(hit) - 1;
-                        hit &= hit - 1;
-                        if (k < KO_CAP) args.cand[q * KO_CAP + k] = (int32_t)(p0 + j);
-                        ++k;
-                    }
                 }
+                return hit;
             };
-            uint32_t ga[32], gb[32];
+            uint32_t ga[32], gb[32], hit[4];
             tmem_ld32_async(tbase, ga);
             tmem_wait_pin(ga);
             tmem_ld32_async(tbase + 32, gb);
-            chunk(0, ga);
+            hit[0] = chunk(0, ga);
             tmem_wait_pin(gb);
             tmem_ld32_async(tbase + 64, ga);
-            chunk(1, gb);
+            hit[1] = chunk(1, gb);
             tmem_wait_pin(ga);
             tmem_ld32_async(tbase + 96, gb);
-            chunk(2, ga);
+            hit[2] = chunk(2, ga);
             tmem_wait_pin(gb);
             tc_fence_before();
             mbar_arrive(BAR_T_EMPTY(a));       // all columns are in registers
-            chunk(3, gb);
+            hit[3] = chunk(3, gb);
+            flush();
+            const int n = __popc(hit[0]) + __popc(hit[1]) + __popc(hit[2]) + __popc(hit[3]);
+            if (n) pk = atomicAdd(args.cnt + q, n);
+            __syncwarp();
+            pq = q;
+            pp = pos0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) ph[c] = hit[c];
         }
+        flush();
     } else if (warp == 8 && lane == 0) {
         int li = 0, lb = -1;
         int64_t bt = -1;
@@ -621,6 +662,7 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
     DevArena tmp;
     tmp.async = true;
     tmp.stream = s;
+    tmp.pool = t->pool;
     // one allocation: every part at a multiple of 256 bytes
     size_t used = 0;
     auto part = [&](size_t bytes) {
@@ -647,10 +689,12 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
     ko_split_kernel<<<nblk(T_pad, 8), 256, 0, s>>>(Y, d, T, T_pad, t->g_xbar, t->g_sigma, qh, ql, nq, cnt);
     ko_home_kernel<<<dim3((unsigned)qb, (unsigned)nsplit), 128, 0, s>>>(Y, d, T, t->cent, t->leaf_cbase, M, split_len, hd,
                                                                         hx);
-    if (t->d_pad == 32)
-        ko_seed_kernel<2><<<nblk(T, 8), 256, 0, s>>>(t->Xt, Y, d, T, hd, hx, (int)nsplit, M, t->nstart, t->nsize, kappa, U);
-    else
-        ko_seed_kernel<4><<<nblk(T, 8), 256, 0, s>>>(t->Xt, Y, d, T, hd, hx, (int)nsplit, M, t->nstart, t->nsize, kappa, U);
+    {
+        const bool few = T < 16 * sms;
+        auto seed = d <= 32 ? (few ? ko_seed_kernel<2, 4> : ko_seed_kernel<2, 1>)
+                            : (few ? ko_seed_kernel<4, 4> : ko_seed_kernel<4, 1>);
+        seed<<<nblk(T, few ? 2 : 8), 256, 0, s>>>(t->Xt, Y, d, T, hd, hx, (int)nsplit, M, t->nstart, t->nsize, kappa, U);
+    }
     QCHK(cudaGetLastError());
     {
         EncodeTiledFn fn = nullptr;
