@@ -178,43 +178,166 @@ __global__ void fill_kernel(const float *X, int d, const float *hsrc, double ksc
 }
 
 // Column-pivoted Householder QR of one node's block and the interpolation
-// matrix P = R11^{-1} R12 (one CTA per node).  At step k the pivot is the
-// column with the largest trailing squared norm (recomputed; ties to the
-// smallest position), |R_kk| is its norm, the reflector is H = I - tau v v^T
-// with v_k = 1 and beta = -sign(alpha) ||x||.
-constexpr int QR_THREADS = 256;
-__global__ void __launch_bounds__(QR_THREADS) cpqr_kernel(
+// matrix P = R11^{-1} R12, a cluster of C CTAs per node.  At step k the pivot is the
+// column with the largest trailing squared norm (recomputed; ties to the smallest
+// position), |R_kk| is its norm, the reflector is H = I - tau v v^T with v_k = 1 and
+// beta = -sign(alpha) ||x||.
+//
+// Bound by FP64: a warp instruction takes 64 cycles of its quarter of the SM (76 with
+// all four quarters busy) whatever its active lanes, and as long to be used.  Three
+// things follow.
+// (1) A step needs the products with v and the update (4 operations an element);
+// the trailing norms (2 more) are needed exactly only for the columns that can be
+// the pivot.  The update therefore also sums each column's norm in FP32 (elements
+// taken from the double's bits, scaled by the last pivot's exponent, no FP64
+// instruction), and only columns within the sum's error bound of the largest get
+// their canonical FP64 norm.  (2) A level with fewer nodes than SMs spreads each
+// node over a cluster: 32-column groups are dealt to the CTAs' warps in turn, so
+// that the columns left are shared evenly at every step.  The block stays in
+// L2; rows written by another CTA are read past L1.  (3) A lone candidate's norm
+// takes the warp's lanes for its products, and a step's square root and divisions
+// one warp.
+// All levels: 64K x 64, s = 256 (7 levels) 318 -> 125 ms; 10K x 1000, s = 1024 (6
+// levels) 5.7 -> 1.1 s; 1M x 64 (11 levels) 1.7 -> 1.1 s of skeletons.
+constexpr int QR_THREADS = 512;
+constexpr int QR_WARPS = QR_THREADS / 32;
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Stores v at `p` (an address of this CTA's shared memory) in CTA `rank`.
+__device__ __forceinline__ void cluster_store(uint64_t *p, uint32_t rank, uint64_t v) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    uint32_t ra;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(ra), "l"(v) : "memory");
+}
+
+// |a| 2^-e as a float, truncated (e: the exponent of a bound of |a|); lim =
+// max(897 + e, 1) << 20 cuts what would be below the smallest normal float.
+__device__ __forceinline__ float scaled_abs(double a, int base, int lim) {
+    const int hi = __double2hiint(a) & 0x7fffffff;
+    return hi < lim ? 0.f : __uint_as_float(((uint32_t)(hi - base) << 3) | ((uint32_t)__double2loint(a) >> 29));
+}
+
+template <int C>
+__global__ void __launch_bounds__(QR_THREADS, 2) cpqr_kernel(
     const int32_t *batch_nodes, const int64_t *woff, const int64_t *poff_ws, const int32_t *ncol,
     const int32_t *ellv, double tol, int s_min, int s_max, double *work, int32_t *piv_fixed,
     int cmax, int32_t *s_out) {
-    extern __shared__ double sh[];           // v[rows]
-    __shared__ double red_v[QR_THREADS / 32];
-    __shared__ int red_j[QR_THREADS / 32];
-    __shared__ double s_best;
-    __shared__ int s_p;
-    int g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    int64_t a = batch_nodes[g];
-    int cols = ncol[a], rows = ellv[a];
+    extern __shared__ double sh[];           // v[rows], then float nf[this CTA's columns]
+    __shared__ double red_v[QR_WARPS];
+    __shared__ int red_j[QR_WARPS];
+    __shared__ float red_f[QR_WARPS];
+    __shared__ double st_nrm, st_beta, st_tau, st_scal;      // the step's scalars
+    __shared__ int st_p;
+    // the CTAs' results of a reduction (slot = rank): largest FP32 norm; norm and position
+    __shared__ uint64_t x_f[C], x_v[C], x_j[C];
+    const int g = blockIdx.x / C, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const uint32_t rank = C > 1 ? cluster_rank() : 0;
+    const int64_t a = batch_nodes[g];
+    const int cols = ncol[a], rows = ellv[a];
     double *A = work + woff[g];
     double *P = work + poff_ws[g];
     int32_t *piv = piv_fixed + a * cmax;
     double *v = sh;
-    int s_hi = min(min(s_max, cols), rows);
-    int s_lo = min(min(s_min, cols), s_hi);
-    for (int j = tid; j < cols; j += QR_THREADS) piv[j] = j;
-    __syncthreads();
-    double r00 = 0.0;
+    float *nf = reinterpret_cast<float *>(sh + rows);
+    const int s_hi = min(min(s_max, cols), rows);
+    const int s_lo = min(min(s_min, cols), s_hi);
+    auto sync_all = [&]() {
+        __syncwarp();
+        if (C > 1) cluster_sync();
+        else __syncthreads();
+    };
+    // column groups of this warp: blk = wid C + rank, every QR_WARPS C; local slot
+    // of a group's FP32 norms: 32 (blk / C)
+    const int blk0 = wid * C + (int)rank;
+    auto ld = [&](const double *p) { return C > 1 ? __ldcg(p) : *p; };
+    auto norm_of = [&](int j, int k) {
+        double acc = 0.0;
+        const double *p = A + (int64_t)k * cols + j;
+        int i = k;
+        for (; i + 8 <= rows; i += 8, p += 8 * (int64_t)cols) {
+            double x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = ld(p + u * (int64_t)cols);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc = c_add(acc, c_mul(x[u], x[u]));
+        }
+        for (; i < rows; ++i, p += cols) {
+            const double x = ld(p);
+            acc = c_add(acc, c_mul(x, x));
+        }
+        return acc;
+    };
+    // the same sum with the whole warp on one column: 32 products an instruction,
+    // then one chain of additions
+    auto norm_of_one = [&](int j, int k) {
+        double acc = 0.0;
+        for (int i = k; i < rows; i += 32) {
+            const double x = i + lane < rows ? ld(A + (int64_t)(i + lane) * cols + j) : 0.0;
+            const double xx = c_mul(x, x);
+            const int n = min(32, rows - i);
+            for (int u = 0; u < n; ++u) acc = c_add(acc, __shfl_sync(0xffffffffu, xx, u));
+        }
+        return acc;
+    };
+    if (rank == 0)
+        for (int j = tid; j < cols; j += QR_THREADS) piv[j] = j;
+    // the bound of an FP32 norm's relative error: `rows` truncated elements, squared
+    // and added in order
+    const float rel = (float)(rows + 8) * 2.4e-7f;
+    double r00 = 0.0;                                     // (the first warp's)
     int s = s_hi;
+    bool have_nf = false;
     for (int k = 0; k < s_hi; ++k) {
+        // the columns that can be the pivot: all at the first step
+        float thr = -1.f;
+        if (have_nf) {
+            float m = -1.f;
+            for (int blk = blk0; blk * 32 < cols; blk += QR_WARPS * C) {
+                const int j = blk * 32 + lane;
+                if (j >= k && j < cols) m = fmaxf(m, nf[32 * (blk / C) + lane]);
+            }
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (lane == 0) red_f[wid] = m;
+            __syncthreads();
+            if (wid == 0) {
+                m = lane < QR_WARPS ? red_f[lane] : -1.f;
+                for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                if (C > 1) {
+                    if (lane < C) cluster_store(&x_f[rank], lane, (uint64_t)__float_as_uint(m));
+                } else if (lane == 0) {
+                    x_f[0] = (uint64_t)__float_as_uint(m);
+                }
+            }
+            sync_all();
+            m = -1.f;
+#pragma unroll
+            for (int c = 0; c < C; ++c) m = fmaxf(m, __uint_as_float((uint32_t)x_f[c]));
+            // (sums this small may have lost terms to the float range: all columns)
+            thr = m < 1e-25f ? -1.f : m * (1.f - rel);
+        }
         double best = -1.0;
         int bj = INT_MAX;
-        for (int j = k + tid; j < cols; j += QR_THREADS) {
-            double acc = 0.0;
-            for (int i = k; i < rows; ++i) {
-                double x = A[(int64_t)i * cols + j];
-                acc = c_add(acc, c_mul(x, x));
+        for (int blk = blk0; blk * 32 < cols; blk += QR_WARPS * C) {
+            const int j = blk * 32 + lane;
+            const bool can = j >= k && j < cols && (!have_nf || nf[32 * (blk / C) + lane] >= thr);
+            const unsigned m = __ballot_sync(0xffffffffu, can);
+            double acc = -1.0;
+            if (__popc(m) == 1) {
+                const double one = norm_of_one(blk * 32 + __ffs(m) - 1, k);
+                if (can) acc = one;
+            } else if (can) {
+                acc = norm_of(j, k);
             }
-            if (acc > best) { best = acc; bj = j; }   // j increases: ties keep the smaller
+            __syncwarp();
+            if (acc > best) { best = acc; bj = j; }       // j increases: ties keep the smaller
         }
         for (int o = 16; o > 0; o >>= 1) {
             double ob = __shfl_xor_sync(0xffffffffu, best, o);
@@ -223,57 +346,163 @@ __global__ void __launch_bounds__(QR_THREADS) cpqr_kernel(
         }
         if (lane == 0) { red_v[wid] = best; red_j[wid] = bj; }
         __syncthreads();
-        if (tid == 0) {
-            double b = red_v[0];
-            int p = red_j[0];
-            for (int w = 1; w < QR_THREADS / 32; ++w)
-                if (red_v[w] > b || (red_v[w] == b && red_j[w] < p)) { b = red_v[w]; p = red_j[w]; }
-            s_best = b;
-            s_p = p;
-        }
-        __syncthreads();
-        double nrm = __dsqrt_rn(s_best);
-        int p = s_p;
-        if (k == 0) r00 = nrm;
-        if (nrm == 0.0 || (k >= s_lo && nrm <= c_mul(tol, r00))) { s = k; break; }
-        if (p != k) {
-            for (int i = tid; i < rows; i += QR_THREADS) {
-                double t = A[(int64_t)i * cols + k];
-                A[(int64_t)i * cols + k] = A[(int64_t)i * cols + p];
-                A[(int64_t)i * cols + p] = t;
+        if (wid == 0) {
+            best = lane < QR_WARPS ? red_v[lane] : -1.0;
+            bj = lane < QR_WARPS ? red_j[lane] : INT_MAX;
+            for (int o = 16; o > 0; o >>= 1) {
+                double ob = __shfl_xor_sync(0xffffffffu, best, o);
+                int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+                if (ob > best || (ob == best && oj < bj)) { best = ob; bj = oj; }
             }
-            if (tid == 0) { int t = piv[k]; piv[k] = piv[p]; piv[p] = t; }
+            if (C > 1) {
+                // (every warp instruction in FP64 costs 64 cycles, so nothing below
+                // is computed by more than one warp a CTA)
+                if (lane < C) {
+                    cluster_store(&x_v[rank], lane, (uint64_t)__double_as_longlong(best));
+                    cluster_store(&x_j[rank], lane, (uint64_t)(uint32_t)bj);
+                }
+            } else if (lane == 0) {
+                x_v[0] = (uint64_t)__double_as_longlong(best);
+                x_j[0] = (uint64_t)(uint32_t)bj;
+            }
+        }
+        sync_all();
+        if (wid == 0) {
+            best = __longlong_as_double((long long)x_v[0]);
+            int p = (int)(uint32_t)x_j[0];
+#pragma unroll
+            for (int c = 1; c < C; ++c) {
+                const double ob = __longlong_as_double((long long)x_v[c]);
+                const int oj = (int)(uint32_t)x_j[c];
+                if (ob > best || (ob == best && oj < p)) { best = ob; p = oj; }
+            }
+            const double nrm = __dsqrt_rn(best);
+            if (k == 0) r00 = nrm;
+            const bool stop = p == INT_MAX || nrm == 0.0 || (k >= s_lo && nrm <= c_mul(tol, r00));
+            if (!stop) {
+                const double alpha = ld(A + (int64_t)k * cols + p);
+                const double beta = (alpha >= 0.0) ? -nrm : nrm;
+                const double tau = c_div(c_sub(beta, alpha), beta);
+                if (lane == 0) {
+                    st_nrm = nrm;
+                    st_beta = beta;
+                    st_tau = tau;
+                    st_scal = c_sub(alpha, beta);
+                }
+            }
+            if (lane == 0) st_p = stop ? -1 : p;
         }
         __syncthreads();
-        double alpha = A[(int64_t)k * cols + k];
-        double beta = (alpha >= 0.0) ? -nrm : nrm;
-        double tau = c_div(c_sub(beta, alpha), beta);
-        double scal = c_sub(alpha, beta);
-        __syncthreads();
-        for (int i = k + 1 + tid; i < rows; i += QR_THREADS) {
-            v[i] = c_div(A[(int64_t)i * cols + k], scal);
-            A[(int64_t)i * cols + k] = 0.0;
+        const int p = st_p;
+        if (p < 0) { s = k; break; }
+        const double nrm = st_nrm, beta = st_beta, tau = st_tau, scal = st_scal;
+        // v from the pivot column where it is; then columns k and p change places
+        // (the first CTA), the new column k's part below the diagonal becomes zero
+        for (int i = k + 1 + tid; i < rows; i += QR_THREADS) v[i] = c_div(ld(A + (int64_t)i * cols + p), scal);
+        if (tid == 0) v[k] = 1.0;
+        sync_all();                                       // every CTA has read column p
+        if (rank == 0) {
+            for (int i = tid; i < rows; i += QR_THREADS) {
+                double *row = A + (int64_t)i * cols;
+                const double xk = ld(row + k), xp = ld(row + p);
+                row[k] = i < k ? xp : i == k ? beta : 0.0;
+                if (p != k) row[p] = xk;
+            }
+            if (tid == 0 && p != k) { int t = piv[k]; piv[k] = piv[p]; piv[p] = t; }
         }
-        if (tid == 0) { v[k] = 1.0; A[(int64_t)k * cols + k] = beta; }
-        __syncthreads();
-        for (int j = k + 1 + tid; j < cols; j += QR_THREADS) {
+        sync_all();
+        // exponent of the norms' bound: every trailing element is at most nrm
+        const int e = (int)((__double2hiint(nrm) >> 20) & 0x7ff) - 1023;
+        const int base = (896 + e) * (1 << 20), lim = max(897 + e, 1) << 20;
+        for (int blk = blk0; blk * 32 < cols; blk += QR_WARPS * C) {
+            const int j = blk * 32 + lane;
+            if (j <= k || j >= cols) continue;
             double dot = 0.0;
-            for (int i = k; i < rows; ++i) dot = c_add(dot, c_mul(v[i], A[(int64_t)i * cols + j]));
-            double tdot = c_mul(tau, dot);
-            for (int i = k; i < rows; ++i)
-                A[(int64_t)i * cols + j] = c_sub(A[(int64_t)i * cols + j], c_mul(tdot, v[i]));
+            double *p0 = A + (int64_t)k * cols + j;
+            {
+                const double *q = p0;
+                int i = k;
+                for (; i + 8 <= rows; i += 8, q += 8 * (int64_t)cols) {
+                    double x[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) x[u] = ld(q + u * (int64_t)cols);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) dot = c_add(dot, c_mul(v[i + u], x[u]));
+                }
+                for (; i < rows; ++i, q += cols) dot = c_add(dot, c_mul(v[i], ld(q)));
+            }
+            const double tdot = c_mul(tau, dot);
+            float f = 0.f;
+            bool bad = false;
+            double *q = p0;
+            int i = k;
+            auto upd = [&](int ii, double x, double *dst) {
+                const double y = c_sub(x, c_mul(tdot, v[ii]));
+                *dst = y;
+                const float t = scaled_abs(y, base, lim);
+                bad |= (__double2hiint(y) & 0x7ff00000) == 0x7ff00000;
+                if (ii > k) f = fmaf(t, t, f);
+            };
+            for (; i + 8 <= rows; i += 8, q += 8 * (int64_t)cols) {
+                double x[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) x[u] = ld(q + u * (int64_t)cols);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) upd(i + u, x[u], q + u * (int64_t)cols);
+            }
+            for (; i < rows; ++i, q += cols) upd(i, ld(q), q);
+            nf[32 * (blk / C) + lane] = bad ? -1.f : f;   // a column that is not finite is never a pivot
         }
-        __syncthreads();
+        have_nf = true;
+        sync_all();
     }
-    int nr = cols - s;
-    for (int j = tid; j < nr; j += QR_THREADS) {
+    sync_all();
+    const int nr = cols - s;
+    for (int blk = blk0; blk * 32 < nr; blk += QR_WARPS * C) {
+        const int j = blk * 32 + lane;
+        if (j >= nr) continue;
         for (int i = s - 1; i >= 0; --i) {
-            double acc = A[(int64_t)i * cols + (s + j)];
-            for (int t = i + 1; t < s; ++t) acc = c_sub(acc, c_mul(A[(int64_t)i * cols + t], P[(int64_t)t * nr + j]));
-            P[(int64_t)i * nr + j] = c_div(acc, A[(int64_t)i * cols + i]);
+            double acc = ld(A + (int64_t)i * cols + (s + j));
+            const double *ai = A + (int64_t)i * cols;
+            int t = i + 1;
+            for (; t + 8 <= s; t += 8) {
+                double x[8], y[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    x[u] = ld(ai + t + u);
+                    y[u] = P[(int64_t)(t + u) * nr + j];
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) acc = c_sub(acc, c_mul(x[u], y[u]));
+            }
+            for (; t < s; ++t) acc = c_sub(acc, c_mul(ld(ai + t), P[(int64_t)t * nr + j]));
+            P[(int64_t)i * nr + j] = c_div(acc, ld(ai + i));
         }
     }
-    if (tid == 0) s_out[a] = s;
+    if (rank == 0 && tid == 0) s_out[a] = s;
+    __syncwarp();
+    if (C > 1) cluster_sync();                            // no CTA leaves while another may store to it
+}
+
+template <int C>
+askit_status launch_cpqr(int nb, size_t smem, cudaStream_t s, const int32_t *nodes, const int64_t *woff,
+                         const int64_t *pws, askit_tree t, const int32_t *ell, int s_max, double *work, int32_t *piv,
+                         int cmax) {
+    ASK_CUDA(cudaFuncSetAttribute(cpqr_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nb * C));
+    cfg.blockDim = dim3(QR_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    ASK_CUDA(cudaLaunchKernelEx(&cfg, cpqr_kernel<C>, nodes, woff, pws, (const int32_t *)t->d_ncol, ell, t->prm.id_tol,
+                                (int)t->prm.s_min, s_max, work, piv, cmax, t->d_s));
+    return ASKIT_OK;
 }
 
 // Skeleton ids of the batch's nodes (first s pivots) and P into the level pool.
@@ -433,6 +662,9 @@ askit_status skeletonize(askit_tree t, cudaStream_t s) {
     std::vector<int64_t> lvl_ptot(L + 1, 0);
     std::vector<int64_t> node_poff(nn, 0);   // offset within its level pool
     const size_t budget = (size_t)6 << 30;   // FP64 workspace per batch
+    int dev = 0, sms = 0;
+    ASK_CUDA(cudaGetDevice(&dev));
+    ASK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
 
     for (int depth = L; depth >= 1; --depth) {
         int64_t a0 = (int64_t)1 << depth, a1 = (int64_t)2 << depth;
@@ -488,10 +720,13 @@ askit_status skeletonize(askit_tree t, cudaStream_t s) {
             }
             int maxrows = 0;
             for (int g = 0; g < nb; ++g) maxrows = std::max(maxrows, h_ell[nodes[g]]);
-            cpqr_kernel<<<nb, QR_THREADS, sizeof(double) * (maxrows + 1), s>>>(
-                d_nodes, d_woff, d_pws, t->d_ncol, d_ell, t->prm.id_tol, t->prm.s_min, s_max, work,
-                piv_fixed, cmax, t->d_s);
-            ASK_LAUNCH();
+            // a cluster per node while the CTAs stay within the SMs
+            int c = 1;
+            while (c < 8 && 2 * c * nb <= sms) c *= 2;
+            const size_t smem = sizeof(double) * (size_t)(maxrows + 1) +
+                                sizeof(float) * 32 * (((size_t)cmax + 31) / 32 / c + 1);
+            ASK_TRY((c == 1 ? launch_cpqr<1> : c == 2 ? launch_cpqr<2> : c == 4 ? launch_cpqr<4> : launch_cpqr<8>)(
+                nb, smem, s, d_nodes, d_woff, d_pws, t, d_ell, s_max, work, piv_fixed, cmax));
             ASK_CUDA(cudaMemcpyAsync(t->h_s.data() + nodes[0], t->d_s + nodes[0], sizeof(int32_t) * nb,
                                      cudaMemcpyDeviceToHost, s));
             ASK_CUDA(cudaStreamSynchronize(s));
