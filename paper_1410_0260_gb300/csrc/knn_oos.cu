@@ -12,12 +12,11 @@
 // A query with more than KO_CAP candidates, or whose coordinates leave the
 // FP16-safe range, takes the exhaustive search.
 //
-// FP64 runs at 2 lanes an SM and clock here, so the FP64 distances are what the
-// steps avoid: seeding in FP64 over the two leaves took 74 of the 110 ms that
+// An FP64 warp instruction takes 64 cycles of its quarter of the SM here, so the FP64
+// distances are what the steps avoid: seeding in FP64 over the two leaves took 74 of the 110 ms that
 // 100,000 queries spent against 131,072 points (d = 64), the FP64 re-rank of every
 // candidate 8.8 ms, the shortlist with operands split on the chip 18.6 ms.
-// Now, the same 100,000 queries: home 0.20, seed 1.7, shortlist
-// 4.8, re-rank 2.4 ms
+// Now, the same 100,000 queries: home 0.20, seed 1.7, shortlist 4.8, re-rank 1.9 ms.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -314,7 +313,7 @@ __global__ void __launch_bounds__(256) ko_rerank_kernel(const float *Xt, const f
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     if (k + e < d) {
-                        const double t = c_sub((double)sy[warp][k + e], (double)xs[e]);
+                        const double t = c_sub(c_f2d(sy[warp][k + e]), c_f2d(xs[e]));
                         acc = c_add(acc, c_mul(t, t));
                     }
             }
@@ -329,21 +328,7 @@ __global__ void __launch_bounds__(256) ko_rerank_kernel(const float *Xt, const f
         const unsigned m = __ballot_sync(FULL, pass);
         const int32_t p = pass ? c[b + lane] : 0;
         // the passing lanes' positions, in order, behind those held
-        const int k = __popc(m);
-        const int src = lane - have >= 0 && lane - have < k ? (int)__fns(m, 0, lane - have + 1) : 0;
-        const int32_t moved = __shfl_sync(FULL, p, src);
-        if (lane >= have && lane < have + k) held = moved;
-        if (have + k < 32) {
-            have += k;
-            continue;
-        }
-        const int rest = have + k - 32;
-        have = 32;
-        offer();
-        // the last `rest` of them start the next group
-        const int src2 = lane < rest ? (int)__fns(m, 0, k - rest + lane + 1) : 0;
-        held = __shfl_sync(FULL, p, src2);
-        have = rest;
+        warp_collect(m, p, have, held, lane, offer);
     }
     if (have > 0) offer();
     if (lane < kappa) {

@@ -86,4 +86,25 @@ __device__ __forceinline__ void warp_offer_f32(float &l, float v, int kappa, int
     }
 }
 
+// Gathers the values p of the lanes in m, in lane order, behind the `have` values
+// already held one a lane; at 32 calls full() (which takes them and sets have = 0)
+// and the rest start the next group.
+template <class F>
+__device__ __forceinline__ void warp_collect(unsigned m, int32_t p, int &have, int32_t &held, int lane, F full) {
+    const int k = __popc(m);
+    const int src = lane >= have && lane < have + k ? (int)__fns(m, 0, lane - have + 1) : 0;
+    const int32_t moved = __shfl_sync(FULL, p, src);
+    if (lane >= have && lane < have + k) held = moved;
+    if (have + k < 32) {
+        have += k;
+        return;
+    }
+    const int rest = have + k - 32;
+    have = 32;
+    full();
+    const int src2 = lane < rest ? (int)__fns(m, 0, k - rest + lane + 1) : 0;
+    held = __shfl_sync(FULL, p, src2);
+    have = rest;
+}
+
 }  // namespace

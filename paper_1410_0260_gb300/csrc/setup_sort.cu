@@ -39,6 +39,12 @@ askit_status seg_sort_i32(const int32_t *kin, int32_t *kout, int64_t n, int nseg
     return ASKIT_OK;
 }
 
+askit_status sort_f64_i32(const double *kin, double *kout, const int32_t *vin, int32_t *vout, int64_t n, void *tmp,
+                          size_t *tmp_bytes, cudaStream_t s) {
+    CUB_CALL(cub::DeviceRadixSort::SortPairs(tmp, *tmp_bytes, kin, kout, vin, vout, (int64_t)n, 0, 64, s));
+    return ASKIT_OK;
+}
+
 askit_status sort_u32_i32(const uint32_t *kin, uint32_t *kout, const int32_t *vin, int32_t *vout,
                           int64_t n, int bits, void *tmp, size_t *tmp_bytes, cudaStream_t s) {
     CUB_CALL(cub::DeviceRadixSort::SortPairs(tmp, *tmp_bytes, kin, kout, vin, vout, (int64_t)n, 0, bits, s));

@@ -22,7 +22,7 @@ namespace {
 __device__ __forceinline__ double c_dist2_df(const double *x, const float *y, int d) {
     double acc = 0.0;
     for (int k = 0; k < d; ++k) {
-        double t = c_sub(x[k], (double)y[k]);
+        double t = c_sub(x[k], c_f2d(y[k]));
         acc = c_add(acc, c_mul(t, t));
     }
     return acc;
@@ -49,7 +49,26 @@ __global__ void center_kernel(const float *X, int d, const int32_t *order, const
     if (k >= d) return;
     int64_t b = lvl_start[node], n = lvl_size[node];
     double acc = 0.0;
-    for (int64_t q = 0; q < n; ++q) acc = c_add(acc, (double)X[(int64_t)order[b + q] * d + k]);
+    // one chain of additions a coordinate: the next 16 rows' loads are in flight
+    // during this group's
+    int64_t q = 0;
+    constexpr int G = 16;
+    float x[G];
+    if (n >= G) {
+#pragma unroll
+        for (int u = 0; u < G; ++u) x[u] = X[(int64_t)order[b + u] * d + k];
+    }
+    for (; q + G <= n; q += G) {
+        float y[G];
+        const bool more = q + 2 * G <= n;
+#pragma unroll
+        for (int u = 0; u < G; ++u) y[u] = more ? X[(int64_t)order[b + q + G + u] * d + k] : 0.f;
+#pragma unroll
+        for (int u = 0; u < G; ++u) acc = c_add(acc, c_f2d(x[u]));
+#pragma unroll
+        for (int u = 0; u < G; ++u) x[u] = y[u];
+    }
+    for (; q < n; ++q) acc = c_add(acc, c_f2d(X[(int64_t)order[b + q] * d + k]));
     xc[(int64_t)node * d + k] = c_div(acc, (double)n);
 }
 
@@ -89,8 +108,8 @@ __global__ void proj_line_kernel(const float *X, int d, const int32_t *order, co
     const float *b = X + (int64_t)xr[node] * d;
     double acc = 0.0;
     for (int k = 0; k < d; ++k) {
-        double u = c_sub((double)xj[k], (double)a[k]);
-        double v = c_sub((double)b[k], (double)a[k]);
+        double u = c_sub(c_f2d(xj[k]), c_f2d(a[k]));
+        double v = c_sub(c_f2d(b[k]), c_f2d(a[k]));
         acc = c_add(acc, c_mul(u, v));
     }
     p[q] = acc;
@@ -108,8 +127,8 @@ __global__ void proj_rp_kernel(const float *X, int d, const int32_t *order, cons
     uint64_t w = 0;
     for (int k = 0; k < d; ++k) {
         if ((k & 63) == 0) w = philox_word(seed, (uint64_t)iter + 1, (uint64_t)node, (uint64_t)(k >> 6));
-        double v = ((w >> (k & 63)) & 1) ? -1.0 : 1.0;
-        acc = c_add(acc, c_mul(v, (double)xj[k]));
+        // +-1 times the coordinate: its sign
+        acc = c_add(acc, c_f2d(((w >> (k & 63)) & 1) ? -xj[k] : xj[k]));
     }
     p[q] = acc;
 }
@@ -127,69 +146,141 @@ __global__ void fill_kernel(T *a, int64_t n, T v) {
 
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
-// Exhaustive search of a candidate range for a set of queries; one warp per
-// query.  Candidates are rows cand[c0 .. c1) of X (ids), queries are ids
-// (self excluded) or rows of Y (qid < 0 marks out-of-sample).
-// The list of each query lives in (bd, bi)[q * 32 + lane].
-__global__ void knn_block_kernel(const float *X, int d, const int32_t *cand, const int32_t *cbeg,
-                                 const int32_t *cend, const int32_t *qids, const float *Y,
-                                 int64_t nq_total, const int32_t *qbeg, const int32_t *qend,
-                                 double *bd, int *bi, int kappa, bool dedup) {
-    extern __shared__ float sq[];   // one query row per warp
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int seg = blockIdx.x;
-    int64_t c0 = cbeg[seg], c1 = cend[seg];
-    float *myq = sq + (int64_t)warp * d;
-    for (int64_t q = qbeg[seg] + warp; q < qend[seg]; q += nw) {
-        int self = qids ? qids[q] : -1;
-        const float *xq = qids ? X + (int64_t)self * d : Y + q * d;
-        for (int k = lane; k < d; k += 32) myq[k] = xq[k];
-        __syncwarp();
-        int64_t slot = (qids ? (int64_t)self : q) * 32 + lane;
-        double ld = bd[slot];
-        int li = bi[slot];
-        // FP32 pre-filter: the FP32 difference-form sum of d squares is within a
-        // factor (1 +- gam) of the exact value, gam = (d + 2) 2^-24 (plus slack),
-        // so a candidate whose FP32 distance exceeds the current kappa-th FP64
-        // distance by that factor cannot enter the list and needs no FP64 work.
-        const float gam = (float)(d + 2) * 5.9604645e-8f * 1.25f + 1e-6f;
-        for (int64_t cb = c0; cb < c1; cb += 32) {
-            double cd = DBL_MAX;
-            int ci = INT_MAX;
-            int j = -1;
-            float d32 = 3.4e38f;
-            if (cb + lane < c1) {
-                j = cand ? cand[cb + lane] : (int)(cb + lane);
-                if (j != self) {
-                    const float *xj = X + (int64_t)j * d;
-                    float a = 0.f;
-                    for (int k = 0; k < d; ++k) {
-                        const float t = myq[k] - xj[k];
-                        a = fmaf(t, t, a);
-                    }
-                    d32 = a;
-                } else {
-                    j = -1;
+// Every point of an RP-tree leaf against its leaf-mates: block (leaf, y) takes the
+// leaf's points 64 y .. + 63 as queries, the leaf as candidates, 512 at a time.
+// FP32 squared distances (difference form) in 64 x 128 tiles from shared memory, 4 x 8
+// pairs a thread; a warp then takes a query's 512 distances: the kappa-th smallest
+// (a best-32 list of floats) and the list so far bound what can be among the
+// kappa nearest -- an FP32 distance is within (1 +- gam) of the exact one -- and
+// only those get their canonical FP64 distance, 32 to a batch.  An FP64
+// warp instruction takes 64 cycles of its quarter of the SM for one lane as for
+// 32: with the candidates tested 32 at a time against the FP64 list nearly every
+// group had a survivor and paid a batch (22.7 ms a tree of 64K x 64, leaves of
+// 512; now 1.8).  The list of each point lives in (bd, bi)[point * 32 + lane].
+constexpr int KL_Q = 64, KL_C = 512, KL_TILE = 128, KL_K = 32;
+constexpr int KL_DT = KL_C + 4, KL_QS = KL_Q + 4, KL_CS = KL_TILE + 4;
+constexpr size_t KL_SMEM = sizeof(float) * (KL_Q * KL_DT + KL_K * (KL_QS + KL_CS));
+
+__global__ void __launch_bounds__(256) knn_leaf_kernel(const float *X, int d, const int32_t *order, const int32_t *beg,
+                                                       const int32_t *end, int kappa, double *bd, int *bi) {
+    extern __shared__ __align__(16) float kl[];
+    float *dt = kl, *qs = kl + KL_Q * KL_DT, *cs = qs + KL_K * KL_QS;   // [query][candidate], [k][query], [k][candidate]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tx = tid & 15, ty = tid >> 4;                // pairs: queries 4 ty .., candidates 4 tx .. and 64 + 4 tx ..
+    const int b0 = beg[blockIdx.x], n = end[blockIdx.x] - b0, q0 = blockIdx.y * KL_Q;
+    if (q0 >= n) return;                                   // block-uniform
+    const int nq = min(KL_Q, n - q0);
+    const int32_t *ids = order + b0;
+    const float gam = (float)(d + 2) * 5.9604645e-8f * 1.25f + 1e-6f;
+    const bool vec = (d & 3) == 0;
+    for (int c0 = 0; c0 < n; c0 += KL_C) {
+        const int nc = min(KL_C, n - c0);
+        for (int t0 = 0; t0 < nc; t0 += KL_TILE) {
+            float acc[4][8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+            for (int k0 = 0; k0 < d; k0 += KL_K) {
+                __syncthreads();                           // the last slice, or the last chunk's distances, are read
+                for (int e = tid; e < KL_Q * KL_K; e += 256) {
+                    const int q = e / KL_K, k = e % KL_K;
+                    qs[k * KL_QS + q] = (q < nq && k0 + k < d) ? X[(int64_t)ids[q0 + q] * d + k0 + k] : 0.f;
+                }
+                for (int e = tid; e < KL_TILE * KL_K; e += 256) {
+                    const int c = e / KL_K, k = e % KL_K;
+                    cs[k * KL_CS + c] = (t0 + c < nc && k0 + k < d) ? X[(int64_t)ids[c0 + t0 + c] * d + k0 + k] : 0.f;
+                }
+                __syncthreads();
+                const int kn = min(KL_K, d - k0);
+                for (int k = 0; k < kn; ++k) {
+                    const float4 q4 = *reinterpret_cast<const float4 *>(qs + k * KL_QS + 4 * ty);
+                    const float4 ca = *reinterpret_cast<const float4 *>(cs + k * KL_CS + 4 * tx);
+                    const float4 cb = *reinterpret_cast<const float4 *>(cs + k * KL_CS + 64 + 4 * tx);
+                    const float qv[4] = {q4.x, q4.y, q4.z, q4.w};
+                    const float cv[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float t = qv[i] - cv[j];
+                            acc[i][j] = fmaf(t, t, acc[i][j]);
+                        }
                 }
             }
-            const double kth = __shfl_sync(FULL, ld, kappa - 1);
-            const bool need = j >= 0 && (!(d32 < 3.0e38f) || (double)d32 * (1.0 - (double)gam) <= kth);
-            if (!__ballot_sync(FULL, need)) continue;
-            if (need) {
-                const float *xj = X + (int64_t)j * d;
-                double acc = 0.0;
-                for (int k = 0; k < d; ++k) {
-                    double t = c_sub((double)myq[k], (double)xj[k]);
-                    acc = c_add(acc, c_mul(t, t));
-                }
-                cd = acc;
-                ci = j;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float *o = dt + (4 * ty + i) * KL_DT + t0 + 4 * tx;
+                *reinterpret_cast<float4 *>(o) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+                *reinterpret_cast<float4 *>(o + 64) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
             }
-            warp_offer(ld, li, cd, ci, kappa, dedup, lane);
         }
-        bd[slot] = ld;
-        bi[slot] = li;
-        __syncwarp();
+        __syncthreads();
+        for (int u = warp; u < nq; u += 8) {
+            const int self = ids[q0 + u];
+            const int64_t slot = (int64_t)self * 32 + lane;
+            double ld = bd[slot];
+            int li = bi[slot];
+            const float *row = dt + u * KL_DT;
+            const double kth = __shfl_sync(FULL, ld, kappa - 1);
+            // above this an exact distance exceeds the list's kappa-th
+            float lim = kth < 1e38 ? __double2float_ru(kth) * (1.f + 2.f * gam) + 1e-37f : INFINITY;
+            float l = 3.4e38f;
+            const int me = q0 + u - c0;                    // the query's own place among the candidates
+            for (int b = 0; b < nc; b += 32) {
+                const float v = b + lane < nc && b + lane != me ? row[b + lane] : 3.4e38f;
+                warp_offer_f32(l, v <= lim ? v : 3.4e38f, kappa, lane);
+            }
+            lim = fminf(lim, __shfl_sync(FULL, l, kappa - 1) * (1.f + 3.f * gam) + 1e-37f);
+            int have = 0;
+            int32_t held = 0;
+            auto offer = [&]() {
+                // not listed yet (every lane takes part in the exchange)
+                bool fresh = lane < have;
+#pragma unroll 8
+                for (int z = 0; z < 32; ++z) {
+                    const int listed = __shfl_sync(FULL, li, z);
+                    if (listed == held) fresh = false;
+                }
+                double cd = DBL_MAX;
+                int ci = INT_MAX;
+                if (fresh) {
+                    const float *xq = X + (int64_t)self * d, *xj = X + (int64_t)held * d;
+                    double acc = 0.0;
+                    if (vec) {
+                        for (int k = 0; k < d; k += 4) {
+                            const float4 xa = *reinterpret_cast<const float4 *>(xq + k);
+                            const float4 xb = *reinterpret_cast<const float4 *>(xj + k);
+                            double t = c_sub(c_f2d(xa.x), c_f2d(xb.x));
+                            acc = c_add(acc, c_mul(t, t));
+                            t = c_sub(c_f2d(xa.y), c_f2d(xb.y));
+                            acc = c_add(acc, c_mul(t, t));
+                            t = c_sub(c_f2d(xa.z), c_f2d(xb.z));
+                            acc = c_add(acc, c_mul(t, t));
+                            t = c_sub(c_f2d(xa.w), c_f2d(xb.w));
+                            acc = c_add(acc, c_mul(t, t));
+                        }
+                    } else {
+                        acc = c_dist2(xq, xj, d);
+                    }
+                    cd = acc;
+                    ci = held;
+                }
+                warp_offer(ld, li, cd, ci, kappa, false, lane);
+                have = 0;
+            };
+            for (int b = 0; b < nc; b += 32) {
+                // not "above the limit", so a distance that is no number stays in
+                const bool pass = b + lane < nc && b + lane != me && !(row[b + lane] > lim);
+                const unsigned m = __ballot_sync(FULL, pass);
+                if (!m) continue;
+                const int32_t p = pass ? ids[c0 + b + lane] : 0;
+                warp_collect(m, p, have, held, lane, offer);
+            }
+            if (have > 0) offer();
+            bd[slot] = ld;
+            bi[slot] = li;
+        }
     }
 }
 
@@ -201,6 +292,8 @@ __global__ void knn_block_kernel(const float *X, int d, const int32_t *cand, con
 // distance and recomputes the survivors in canonical FP64.  Each split
 // writes its own best-32 lists; knn_merge_kernel merges the splits.
 constexpr int KT_Q = 64, KT_C = 128, KT_K = 32;
+// points a segment above which a tree level is sorted as a whole
+constexpr int64_t TREE_RADIX = 2048;
 
 __global__ void __launch_bounds__(256) knn_tiled_kernel(const float *X, int64_t N, int d, const float *Y,
                                                          int64_t Q, int64_t split_len, int kappa, double *bd,
@@ -287,7 +380,7 @@ __global__ void __launch_bounds__(256) knn_tiled_kernel(const float *X, int64_t 
                     const float *xj = X + j * d;
                     double a = 0.0;
                     for (int k = 0; k < d; ++k) {
-                        const double t = c_sub((double)xq[k], (double)xj[k]);
+                        const double t = c_sub(c_f2d(xq[k]), c_f2d(xj[k]));
                         a = c_add(a, c_mul(t, t));
                     }
                     cd = a;
@@ -345,8 +438,19 @@ __global__ void knn_dist_kernel(const float *X, int64_t N, int d, int kappa, con
     dist[t] = c_dist2(X + i * d, X + (int64_t)ids[t] * d, d);
 }
 
+// The sorted positions' segments and ids.
+__global__ void seg_gather_kernel(const int32_t *pos, const int32_t *seg, const int32_t *order, int64_t n,
+                                  uint32_t *skey, int32_t *ids) {
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    skey[q] = (uint32_t)seg[pos[q]];
+    ids[q] = order[pos[q]];
+}
+
 // Scratch shared by one tree build.
 struct TreeScratch {
+    int32_t *pos0 = nullptr, *pos1 = nullptr;
+    uint32_t *skey0 = nullptr, *skey1 = nullptr;
     int32_t *seg = nullptr, *tmp_ids = nullptr, *bid = nullptr, *xl = nullptr;
     double *keys = nullptr, *keys_out = nullptr, *xc = nullptr, *Dq = nullptr;
     unsigned long long *bbits = nullptr;
@@ -356,6 +460,7 @@ struct TreeScratch {
 };
 
 void free_scratch(TreeScratch &s) {
+    cudaFree(s.pos0); cudaFree(s.pos1); cudaFree(s.skey0); cudaFree(s.skey1);
     cudaFree(s.seg); cudaFree(s.tmp_ids); cudaFree(s.bid); cudaFree(s.xl); cudaFree(s.keys);
     cudaFree(s.keys_out); cudaFree(s.xc); cudaFree(s.Dq); cudaFree(s.bbits); cudaFree(s.lvl_start);
     cudaFree(s.lvl_end); cudaFree(s.lvl_size); cudaFree(s.cub);
@@ -424,9 +529,18 @@ askit_status build_tree_gpu(const float *X, int64_t N, int d, int L, int kind, u
         if ((rc = seg_sort_f64_i32(nullptr, nullptr, nullptr, nullptr, N, (int)half, nullptr, nullptr, nullptr, &b1, s)) != ASKIT_OK) goto done;
         if ((rc = seg_sort_i32(nullptr, nullptr, N, (int)(2 * half), nullptr, nullptr, nullptr, &b2, s)) != ASKIT_OK) goto done;
         sc.cub_bytes = b1 > b2 ? b1 : b2;
+        if ((rc = sort_f64_i32(nullptr, nullptr, nullptr, nullptr, N, nullptr, &b1, s)) != ASKIT_OK) goto done;
+        if ((rc = sort_u32_i32(nullptr, nullptr, nullptr, nullptr, N, 32, nullptr, &b2, s)) != ASKIT_OK) goto done;
+        sc.cub_bytes = std::max(sc.cub_bytes, b1 > b2 ? b1 : b2);
+        TCHK(cudaMalloc(&sc.pos0, sizeof(int32_t) * N), "alloc");
+        TCHK(cudaMalloc(&sc.pos1, sizeof(int32_t) * N), "alloc");
+        TCHK(cudaMalloc(&sc.skey0, sizeof(uint32_t) * N), "alloc");
+        TCHK(cudaMalloc(&sc.skey1, sizeof(uint32_t) * N), "alloc");
         TCHK(cudaMalloc(&sc.cub, sc.cub_bytes), "alloc");
 
         iota_kernel<<<nblk(N, 256), 256, 0, s>>>(order, N);
+        int id_bits = 1;
+        while (((int64_t)1 << id_bits) < N) ++id_bits;
         for (int t = 0; t < L; ++t) {
             int64_t a0 = (int64_t)1 << t;
             int nseg = (int)a0;
@@ -450,6 +564,21 @@ askit_status build_tree_gpu(const float *X, int64_t N, int d, int L, int kind, u
                 proj_rp_kernel<<<nblk(N, 256), 256, 0, s>>>(X, d, order, sc.seg, N, a0, seed, iter, sc.keys);
             }
             TCHK(cudaGetLastError(), "projection kernels");
+            if (N / nseg > TREE_RADIX) {
+                // Few large segments: the segmented sort takes one block for each
+                // (a 64K segment about 1 ms, a 1M one 16 ms), so the whole level is
+                // radix-sorted by key, then stably by segment.
+                iota_kernel<<<nblk(N, 256), 256, 0, s>>>(sc.pos0, N);
+                if ((rc = sort_f64_i32(sc.keys, sc.keys_out, sc.pos0, sc.pos1, N, sc.cub, &sc.cub_bytes, s)) != ASKIT_OK) goto done;
+                seg_gather_kernel<<<nblk(N, 256), 256, 0, s>>>(sc.pos1, sc.seg, order, N, sc.skey0, sc.pos0);
+                if ((rc = sort_u32_i32(sc.skey0, sc.skey1, sc.pos0, sc.tmp_ids, N, t + 1, sc.cub, &sc.cub_bytes, s)) != ASKIT_OK) goto done;
+                // children back to ascending id: by id, then stably by child
+                seg_of_pos_kernel<<<nblk(N, 256), 256, 0, s>>>(sc.lvl_start + 2 * a0, 2 * nseg, N, sc.pos0);
+                if ((rc = sort_u32_i32(reinterpret_cast<uint32_t *>(sc.tmp_ids), sc.skey0, sc.pos0, sc.pos1, N, id_bits, sc.cub, &sc.cub_bytes, s)) != ASKIT_OK) goto done;
+                if ((rc = sort_u32_i32(reinterpret_cast<uint32_t *>(sc.pos1), sc.skey1, reinterpret_cast<int32_t *>(sc.skey0), order, N, t + 2, sc.cub, &sc.cub_bytes, s)) != ASKIT_OK) goto done;
+                TCHK(cudaGetLastError(), "level sort");
+                continue;
+            }
             // (key, id) order inside every node: stable sort of an id-ascending segment
             if ((rc = seg_sort_f64_i32(sc.keys, sc.keys_out, order, sc.tmp_ids, N, nseg, ls, le, sc.cub, &sc.cub_bytes, s)) != ASKIT_OK) goto done;
             // children back to ascending id
@@ -521,6 +650,10 @@ askit_status knn_rp_gpu(const float *X, int64_t N, int d, int kappa, int iters, 
         h[a] = (int32_t)st[nleaf + a];
         h[nleaf + a] = (int32_t)(st[nleaf + a] + sz[nleaf + a]);
     }
+    const int64_t max_leaf = sz[nleaf];                    // the first leaf is the largest
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(knn_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KL_SMEM);
+    ASK_CUDA(attr);
     double *bd = nullptr;
     int *bi = nullptr;
     int32_t *order = nullptr, *segs = nullptr;
@@ -534,9 +667,8 @@ askit_status knn_rp_gpu(const float *X, int64_t N, int d, int kappa, int iters, 
     for (int it = 0; rc == ASKIT_OK && e == cudaSuccess && it < iters; ++it) {
         rc = build_tree_gpu(X, N, d, L, 1, seed, it, order, s);
         if (rc != ASKIT_OK) break;
-        // queries of leaf b = its own points (ids in `order`), candidates = the same range
-        knn_block_kernel<<<(unsigned)nleaf, 256, 8 * d * sizeof(float), s>>>(
-            X, d, order, segs, segs + nleaf, order, nullptr, N, segs, segs + nleaf, bd, bi, kappa, true);
+        knn_leaf_kernel<<<dim3((unsigned)nleaf, nblk(max_leaf, KL_Q)), 256, KL_SMEM, s>>>(X, d, order, segs, segs + nleaf,
+                                                                                         kappa, bd, bi);
         e = cudaGetLastError();
     }
     if (rc == ASKIT_OK && e == cudaSuccess) {
@@ -625,7 +757,7 @@ __global__ void knn_noalloc_kernel(const float *X, int64_t N, int d, const float
                 const float *xj = X + (cb + lane) * d;
                 double acc = 0.0;
                 for (int k = 0; k < d; ++k) {
-                    double t = c_sub((double)myq[k], (double)xj[k]);
+                    double t = c_sub(c_f2d(myq[k]), c_f2d(xj[k]));
                     acc = c_add(acc, c_mul(t, t));
                 }
                 cd = acc;
