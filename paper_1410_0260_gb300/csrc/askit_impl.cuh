@@ -309,6 +309,7 @@ struct askit_tree_s {
     void *tc = nullptr;            // tensor-core kernel state (tensor maps)
     void *tcw = nullptr;           // the same for the wide (d > TC_K) kernel
     void *tc16 = nullptr;          // the same for the 16-bit narrow kernel
+    void *tf32 = nullptr;          // the same for the 3xTF32 kernel
     int64_t *sb_row0 = nullptr;    // [n_sub] first row of each sub-block (Xt rows, then Xs rows)
     int32_t *sb_nr = nullptr;      // [n_sub] rows of each sub-block
     int64_t n_leaf_sub = 0;        // sub-blocks of leaves (the rest are skeleton sub-blocks)
@@ -517,6 +518,14 @@ void eval_tc_wide_free(askit_tree t);
 askit_status eval_tc16(askit_tree t, const WeightCtx &c, int precision, const float *Xq, int64_t ldq, int64_t q_rows,
                        const WorkLists &w, float *partial, cudaStream_t s);
 void eval_tc16_free(askit_tree t);
+// Column data {A, B, C, w} of every sub-block into c.colv (and, rc = 4 or 16, the
+// weights into c.colw): A = 2 sc g_unscale, B = -sc |b|^2, C = -sc; uni (rc = 1):
+// {B, w} alone
+askit_status block_columns(askit_tree t, const WeightCtx &c, int rc, bool uni, float g_unscale, cudaStream_t s);
+// eval_tf32.cu: 3xTF32, r <= 4
+askit_status eval_tf32(askit_tree t, const WeightCtx &c, const float *Xq, int64_t ldq, const WorkLists &w,
+                       float *partial, cudaStream_t s);
+void eval_tf32_free(askit_tree t);
 // eval_g16.cu: the global-centered FP16x3 kernel (targets pre-split in q)
 askit_status eval_g16(askit_tree t, const WeightCtx &c, const QuerySplit &q, const WorkLists &w, float *partial,
                       cudaStream_t s);

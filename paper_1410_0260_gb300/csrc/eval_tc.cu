@@ -673,6 +673,9 @@ askit_status eval_tc(askit_tree t, const WeightCtx &c, int precision, const floa
         askit_set_error("tensor-core evaluation covers r <= %d; use ASKIT_PREC_SIMT_FP32", Smem<ASKIT_PREC_TF32X3>::RC_MAX);
         return ASKIT_ERR_UNSUPPORTED;
     }
+    // 3xTF32 up to four vectors: both sides centered on the sub-block, the targets'
+    // split rows in TMEM (eval_tf32.cu); more vectors' FP32 sums are made here
+    if (precision == ASKIT_PREC_TF32X3 && c.r <= 4) return eval_tf32(t, c, Xq, ldq, w, partial, s);
     if (w.n_blocks == 0) return ASKIT_OK;
     if (ldq != t->d_pad) {
         askit_set_error("target rows must have d_pad columns");
@@ -705,8 +708,6 @@ askit_status eval_tc(askit_tree t, const WeightCtx &c, int precision, const floa
     a.f16_scale = 1.f;
     a.g_unscale = 1.f / (a.f16_scale * a.f16_scale);
     if (precision == ASKIT_PREC_TF32X3) {
-        if (c.r == 1) return launch<ASKIT_PREC_TF32X3, 1>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
-        if (c.r <= 4) return launch<ASKIT_PREC_TF32X3, 4>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
         return launch<ASKIT_PREC_TF32X3, 16>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
     }
     if (precision == ASKIT_PREC_BF16X3) {
@@ -723,5 +724,6 @@ void eval_tc_free(askit_tree t) {
     t->tc = nullptr;
     eval_tc_wide_free(t);
     eval_tc16_free(t);
+    eval_tf32_free(t);
     eval_g16_free(t);
 }

@@ -716,14 +716,8 @@ askit_status run16(askit_tree t, const WeightCtx &c, T16State *st, int pi, const
         const float sc = (float)(t->prm.kernel_scale * 1.4426950408889634 / (hf * hf));
         a.uni_a = 2.f * g_unscale * sc;
         a.uni_c = -sc;
-        ASK_TRY(launch_pdl(tc16_cols_kernel<RC, 1>, dim3((unsigned)t->n_sub), dim3(128), 0, s, t->sb_row0, t->sb_nr,
-                           t->n_leaf_sub, t->sc_t, t->sc_s, t->nrmc_t, t->nrmc_s, c.Wt, c.Ws, c.r, g_unscale, c.colv,
-                           c.colw));
-    } else {
-        ASK_TRY(launch_pdl(tc16_cols_kernel<RC, 0>, dim3((unsigned)t->n_sub), dim3(128), 0, s, t->sb_row0, t->sb_nr,
-                           t->n_leaf_sub, t->sc_t, t->sc_s, t->nrmc_t, t->nrmc_s, c.Wt, c.Ws, c.r, g_unscale, c.colv,
-                           c.colw));
     }
+    ASK_TRY(block_columns(t, c, RC, uni, g_unscale, s));
     a.colv = c.colv;
     a.colw = c.colw;
     const bool pairs = t->tune_pairs == 1 && w.sched[2].n_ctas > 0;
@@ -768,6 +762,12 @@ askit_status dispatch16(askit_tree t, const WeightCtx &c, T16State *st, int pi, 
 }
 
 }  // namespace
+
+askit_status block_columns(askit_tree t, const WeightCtx &c, int rc, bool uni, float g_unscale, cudaStream_t s) {
+    auto k = rc == 1 ? (uni ? tc16_cols_kernel<1, 1> : tc16_cols_kernel<1, 0>) : rc == 4 ? tc16_cols_kernel<4, 0> : tc16_cols_kernel<16, 0>;
+    return launch_pdl(k, dim3((unsigned)t->n_sub), dim3(128), 0, s, t->sb_row0, t->sb_nr, t->n_leaf_sub, t->sc_t,
+                      t->sc_s, t->nrmc_t, t->nrmc_s, c.Wt, c.Ws, c.r, g_unscale, c.colv, c.colw);
+}
 
 askit_status eval_tc16(askit_tree t, const WeightCtx &c, int precision, const float *Xq, int64_t ldq, int64_t q_rows,
                        const WorkLists &w, float *partial, cudaStream_t s) {
