@@ -497,8 +497,8 @@ askit_status build_work_lists(askit_tree t, const int32_t *sets, int stride, con
 askit_status reduce_partials(const WorkLists &w, const float *partial, int r, const int32_t *out_rows,
                              float *U, int64_t ldu, cudaStream_t s);
 askit_status insample_prune_sets(askit_tree t, PruneSets &ps, cudaStream_t s);
-askit_status oos_prune_sets(askit_tree t, const int32_t *knn, const double *dist, int64_t T, int stride,
-                            int32_t *sets, cudaStream_t s);
+askit_status oos_prune_sets(askit_tree t, const int32_t *knn, const double *dist, const int32_t *order, int64_t T,
+                            int stride, int32_t *sets, cudaStream_t s);
 // every array of w back to the arena
 void free_work_lists(WorkLists &w, DevArena &arena);
 
@@ -522,7 +522,7 @@ void eval_tc16_free(askit_tree t);
 // weights into c.colw): A = 2 sc g_unscale, B = -sc |b|^2, C = -sc; uni (rc = 1):
 // {B, w} alone
 askit_status block_columns(askit_tree t, const WeightCtx &c, int rc, bool uni, float g_unscale, cudaStream_t s);
-// eval_tf32.cu: 3xTF32, r <= 4
+// eval_tf32.cu: 3xTF32
 askit_status eval_tf32(askit_tree t, const WeightCtx &c, const float *Xq, int64_t ldq, const WorkLists &w,
                        float *partial, cudaStream_t s);
 void eval_tf32_free(askit_tree t);
@@ -532,9 +532,11 @@ askit_status eval_g16(askit_tree t, const WeightCtx &c, const QuerySplit &q, con
 void eval_g16_free(askit_tree t);
 askit_status build_g16_operands(askit_tree t, cudaStream_t s);
 // target rows X [rows, ldx] (d columns) in the global-centered form of tree t;
-// *overflow (if given) is set when a value leaves the FP16-safe range
+// *overflow (if given) is set when a value leaves the FP16-safe range; with an
+// order, row i is X[order[i]] (zero from n_order on)
 askit_status g16_split_rows(const float *X, int64_t ldx, int d, int64_t rows, const askit_tree_s *t, uint16_t *hi,
-                            uint16_t *lo, uint16_t *nx, int *overflow, cudaStream_t s);
+                            uint16_t *lo, uint16_t *nx, int *overflow, cudaStream_t s,
+                            const int32_t *order = nullptr, int64_t n_order = 0);
 // whether FP16x3 evaluations of this tree take the global-centered kernel
 inline bool use_g16(const askit_tree_s *t) {
     return t->Xg_hi && (t->fp16_centering == 2 || (t->fp16_centering == 0 && t->g_ok));

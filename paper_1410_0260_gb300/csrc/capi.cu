@@ -69,14 +69,6 @@ __global__ void oos_keys_kernel(const int32_t *knn, int kappa, const int32_t *po
     vals[q] = (int32_t)q;
 }
 
-template <class V>
-__global__ void gather_knn_kernel(const V *knn, int kappa, const int32_t *order, int64_t T, V *out) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= T * kappa) return;
-    int64_t q = e / kappa;
-    out[e] = knn[(int64_t)order[q] * kappa + (e % kappa)];
-}
-
 __global__ void gather_y_kernel(const float *Y, int64_t ldy, int d, int d_pad, const int32_t *order,
                                 int64_t T, int64_t T_pad, float *out) {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -472,8 +464,9 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     tmp.stream = s;
     tmp.pool = t->pool;
     float *Yc = nullptr, *Yt = nullptr;
-    int32_t *ids = nullptr, *ids_s = nullptr, *order = nullptr, *vals = nullptr, *sets = nullptr;
-    double *dist = nullptr, *dist_s = nullptr;
+    int32_t *ids = nullptr, *order = nullptr, *vals = nullptr, *sets = nullptr;
+    double *dist = nullptr;
+    const bool g16 = t->precision == ASKIT_PREC_FP16X3 && t->d <= TC_K && use_g16(t);
     uint32_t *keys = nullptr, *keys_s = nullptr;
     void *cub = nullptr;
     size_t cb = 0;
@@ -499,26 +492,21 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     OTRY(sort_u32_i32(nullptr, nullptr, nullptr, nullptr, T, pos_bits, nullptr, &cb, s));
     OTRY(tmp.alloc((char **)&cub, cb));
     OTRY(sort_u32_i32(keys, keys_s, vals, order, T, pos_bits, cub, &cb, s));
-    OTRY(tmp.alloc(&ids_s, (size_t)T * kappa));
-    OTRY(tmp.alloc(&dist_s, (size_t)T * kappa));
-    gather_knn_kernel<<<nblk(T * kappa, 256), 256, 0, s>>>(ids, kappa, order, T, ids_s);
-    gather_knn_kernel<<<nblk(T * kappa, 256), 256, 0, s>>>(dist, kappa, order, T, dist_s);
-    OTRY(tmp.alloc(&Yt, (size_t)T_pad * t->d_pad));
-    gather_y_kernel<<<nblk(T_pad * t->d_pad, 256), 256, 0, s>>>(Yc, d, d, t->d_pad, order, T, T_pad, Yt);
-    OTRY(tmp.alloc(&sets, (size_t)T * kappa));
-    OTRY(oos_prune_sets(t, ids_s, dist_s, T, kappa, sets, s));
-    OTRY(build_work_lists(t, sets, kappa, nullptr, T, w, tmp, false, s));
-    OTRY(tmp.alloc(&partial, (size_t)w.n_entries * c.r));
-    if (t->precision == ASKIT_PREC_FP16X3 && t->d <= TC_K && use_g16(t)) {
-        // the targets in the global-centered FP16x3 form; a batch reaching
-        // outside the FP16-safe range (far from the data) takes the
-        // per-sub-block centered kernel instead
+    if (g16) {
+        // the targets in the global-centered FP16x3 form
         OTRY(tmp.alloc(&yg_hi, (size_t)T_pad * TC_K));
         OTRY(tmp.alloc(&yg_lo, (size_t)T_pad * TC_K));
         OTRY(tmp.alloc(&yg_x, (size_t)T_pad * 16));
         OTRY(tmp.alloc(&yg_flag, 1));
         if (cudaMemsetAsync(yg_flag, 0, sizeof(int), s) != cudaSuccess) { askit_set_error("flag"); rc = ASKIT_ERR_CUDA; goto out; }
-        OTRY(g16_split_rows(Yt, t->d_pad, d, T_pad, t, yg_hi, yg_lo, yg_x, yg_flag, s));
+        OTRY(g16_split_rows(Yc, d, d, T_pad, t, yg_hi, yg_lo, yg_x, yg_flag, s, order, T));
+    }
+    OTRY(tmp.alloc(&sets, (size_t)T * kappa));
+    OTRY(oos_prune_sets(t, ids, dist, order, T, kappa, sets, s));
+    OTRY(build_work_lists(t, sets, kappa, nullptr, T, w, tmp, false, s));
+    OTRY(tmp.alloc(&partial, (size_t)w.n_entries * c.r));
+    if (g16) {
+        // (the lists' last synchronization has covered the split)
         int flag = 0;
         if (cudaMemcpyAsync(&flag, yg_flag, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) { askit_set_error("range flag"); rc = ASKIT_ERR_CUDA; goto out; }
@@ -528,6 +516,12 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
             qs.x = yg_x;
             qs.rows = T_pad;
         }
+    }
+    if (!qs.hi) {
+        // FP32 rows for the other kernels: other precisions, or a batch that
+        // reaches outside the FP16-safe range (far from the data)
+        OTRY(tmp.alloc(&Yt, (size_t)T_pad * t->d_pad));
+        gather_y_kernel<<<nblk(T_pad * t->d_pad, 256), 256, 0, s>>>(Yc, d, d, t->d_pad, order, T, T_pad, Yt);
     }
     OTRY(run_eval(t, c, t->precision, Yt, t->d_pad, T_pad, qs.hi ? &qs : nullptr, w, partial, order, U_dev, ldu, s));
     if (cudaStreamSynchronize(s) != cudaSuccess) { askit_set_error("out-of-sample evaluate: %s", cudaGetErrorString(cudaGetLastError())); rc = ASKIT_ERR_CUDA; }

@@ -892,16 +892,17 @@ __device__ __forceinline__ void split16(float v, uint16_t &h, uint16_t &l) {
 // FP16-safe range raises *overflow.
 __global__ void gsplit_targets_kernel(const float *X, int64_t ldx, int d, int64_t rows, const float *xbar, float sigma,
                                       float tau, float kappa, uint16_t *hi, uint16_t *lo, uint16_t *nx,
-                                      int *overflow) {
+                                      int *overflow, const int32_t *order, int64_t n_order) {
     const int lane = threadIdx.x & 31;
     const int64_t row = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
+    const int64_t src = !order ? row : row < n_order ? order[row] : -1;    // -1: a zero row
     double acc = 0.0;
     bool bad = false;
 #pragma unroll
     for (int h = 0; h < TC_K / 32; ++h) {
         const int k = lane + 32 * h;
-        const float x = k < d ? X[row * ldx + k] - xbar[k] : 0.f;
+        const float x = k < d ? (src >= 0 ? X[src * ldx + k] : 0.f) - xbar[k] : 0.f;
         acc += (double)x * (double)x;
         const float v = x * sigma;
         bad |= !(fabsf(v) <= 30000.f);
@@ -1025,10 +1026,11 @@ float pow2_near(double v) {
 }  // namespace
 
 askit_status g16_split_rows(const float *X, int64_t ldx, int d, int64_t rows, const askit_tree_s *t, uint16_t *hi,
-                            uint16_t *lo, uint16_t *nx, int *overflow, cudaStream_t s) {
+                            uint16_t *lo, uint16_t *nx, int *overflow, cudaStream_t s, const int32_t *order,
+                            int64_t n_order) {
     if (rows <= 0) return ASKIT_OK;
     gsplit_targets_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(X, ldx, d, rows, t->g_xbar, t->g_sigma, t->g_tau,
-                                                                    t->g_kappa, hi, lo, nx, overflow);
+                                                                    t->g_kappa, hi, lo, nx, overflow, order, n_order);
     ASK_LAUNCH();
     return ASKIT_OK;
 }

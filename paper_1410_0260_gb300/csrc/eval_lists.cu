@@ -163,17 +163,18 @@ __global__ void leaf_row_kernel(const int32_t *perm, const int32_t *leafof, int6
 
 // Out-of-sample prune sets: the sorted distinct leaves of N_y (its first kappa_y
 // neighbors; no self term), a warp per target, a neighbor per lane (kappa <= 32).
-__global__ void oos_sets_kernel(const int32_t *leafof, const int32_t *knn, const double *dist, const float *hsrc,
-                                double kscale, double cut, int64_t T, int kappa, int stride, int32_t *sets) {
+__global__ void oos_sets_kernel(const int32_t *leafof, const int32_t *knn, const double *dist, const int32_t *order,
+                                const float *hsrc, double kscale, double cut, int64_t T, int kappa, int stride, int32_t *sets) {
     const int lane = threadIdx.x & 31;
     const int64_t q = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
     if (q >= T) return;                                    // warp-uniform
     const bool in = lane < kappa;
-    const int32_t id = in ? knn[q * kappa + lane] : 0;
+    const int64_t src = (int64_t)order[q] * kappa + lane;  // target q's neighbors: the caller's row order[q]
+    const int32_t id = in ? knn[src] : 0;
     int ky = kappa;                                        // kappa_of over the lanes
     if (cut > 0.0) {
         const double h = (double)hsrc[id];
-        const bool keep = in && c_div(c_mul(kscale, dist[q * kappa + lane]), c_mul(h, h)) < cut;
+        const bool keep = in && c_div(c_mul(kscale, dist[src]), c_mul(h, h)) < cut;
         const unsigned m = __ballot_sync(0xffffffffu, keep);
         ky = m ? 32 - __clz(m) : 0;
     }
@@ -710,9 +711,9 @@ askit_status insample_prune_sets(askit_tree t, PruneSets &ps, cudaStream_t s) {
     return ASKIT_OK;
 }
 
-askit_status oos_prune_sets(askit_tree t, const int32_t *knn, const double *dist, int64_t T, int stride,
-                            int32_t *sets, cudaStream_t s) {
-    oos_sets_kernel<<<nblk(T, 8), 256, 0, s>>>(t->leafof, knn, dist, t->hsrc, t->prm.kernel_scale, t->kappa_cut, T,
+askit_status oos_prune_sets(askit_tree t, const int32_t *knn, const double *dist, const int32_t *order, int64_t T,
+                            int stride, int32_t *sets, cudaStream_t s) {
+    oos_sets_kernel<<<nblk(T, 8), 256, 0, s>>>(t->leafof, knn, dist, order, t->hsrc, t->prm.kernel_scale, t->kappa_cut, T,
                                                  t->kappa, stride, sets);
     ASK_LAUNCH();
     return ASKIT_OK;

@@ -673,9 +673,8 @@ askit_status eval_tc(askit_tree t, const WeightCtx &c, int precision, const floa
         askit_set_error("tensor-core evaluation covers r <= %d; use ASKIT_PREC_SIMT_FP32", Smem<ASKIT_PREC_TF32X3>::RC_MAX);
         return ASKIT_ERR_UNSUPPORTED;
     }
-    // 3xTF32 up to four vectors: both sides centered on the sub-block, the targets'
-    // split rows in TMEM (eval_tf32.cu); more vectors' FP32 sums are made here
-    if (precision == ASKIT_PREC_TF32X3 && c.r <= 4) return eval_tf32(t, c, Xq, ldq, w, partial, s);
+    // 3xTF32: both sides centered on the sub-block, the targets' split rows in TMEM
+    if (precision == ASKIT_PREC_TF32X3) return eval_tf32(t, c, Xq, ldq, w, partial, s);
     if (w.n_blocks == 0) return ASKIT_OK;
     if (ldq != t->d_pad) {
         askit_set_error("target rows must have d_pad columns");

@@ -1,4 +1,4 @@
-// Evaluate (Algorithm 4) on the tcgen05 tensor cores in 3xTF32, d <= 64, r <= 4.
+// Evaluate (Algorithm 4) on the tcgen05 tensor cores in 3xTF32, d <= 64.
 //
 // Work item = one source sub-block (<= 128 rows of a leaf or a skeleton) against up
 // to 128 targets that need it.  Both sides are centered on the sub-block's mean c_B
@@ -223,7 +223,9 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
 #pragma unroll
                 for (int z = 0; z < RC; ++z) acc[z] = 0.f;
                 float2 acc2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-                float2 accw[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                float2 accw[RC > 1 ? RC / 2 : 1];
+#pragma unroll
+                for (int z = 0; z < (RC > 1 ? RC / 2 : 1); ++z) accw[z] = make_float2(0.f, 0.f);
                 if (q * 32 < item.cnt) {                           // warp-uniform
                     const float2 pt2 = make_float2(pt, pt);
                     // arg = g A + (C p + B) = -sc (p + q - 2 g); columns past the rows
@@ -248,12 +250,17 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                             if constexpr (RC == 1) {
                                 acc2[(jj >> 1) & 1] = __ffma2_rn(k, make_float2(cw.z, cw.w), acc2[(jj >> 1) & 1]);
                             } else {
-                                const float4 *w4 = reinterpret_cast<const float4 *>(cwp + (c * 32 + jj) * RC);
-                                const float4 wa = w4[0], wb = w4[1];
-                                accw[0] = __ffma2_rn(make_float2(k.x, k.x), make_float2(wa.x, wa.y), accw[0]);
-                                accw[1] = __ffma2_rn(make_float2(k.x, k.x), make_float2(wa.z, wa.w), accw[1]);
-                                accw[0] = __ffma2_rn(make_float2(k.y, k.y), make_float2(wb.x, wb.y), accw[0]);
-                                accw[1] = __ffma2_rn(make_float2(k.y, k.y), make_float2(wb.z, wb.w), accw[1]);
+                                const float2 ka = make_float2(k.x, k.x), kb = make_float2(k.y, k.y);
+                                const float4 *wa = reinterpret_cast<const float4 *>(cwp + (c * 32 + jj) * RC);
+                                const float4 *wb = wa + RC / 4;
+#pragma unroll
+                                for (int z = 0; z < RC / 4; ++z) {
+                                    const float4 va = wa[z], vb = wb[z];
+                                    accw[2 * z] = __ffma2_rn(ka, make_float2(va.x, va.y), accw[2 * z]);
+                                    accw[2 * z + 1] = __ffma2_rn(ka, make_float2(va.z, va.w), accw[2 * z + 1]);
+                                    accw[2 * z] = __ffma2_rn(kb, make_float2(vb.x, vb.y), accw[2 * z]);
+                                    accw[2 * z + 1] = __ffma2_rn(kb, make_float2(vb.z, vb.w), accw[2 * z + 1]);
+                                }
                             }
                         }
                     };
@@ -268,10 +275,11 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                     if constexpr (RC == 1) {
                         acc[0] = (acc2[0].x + acc2[0].y) + (acc2[1].x + acc2[1].y);
                     } else {
-                        acc[0] = accw[0].x;
-                        acc[1] = accw[0].y;
-                        acc[2] = accw[1].x;
-                        acc[3] = accw[1].y;
+#pragma unroll
+                        for (int z = 0; z < RC / 2; ++z) {
+                            acc[2 * z] = accw[z].x;
+                            acc[2 * z + 1] = accw[z].y;
+                        }
                     }
                 }
                 tc_fence_before();
@@ -505,7 +513,8 @@ askit_status eval_tf32(askit_tree t, const WeightCtx &c, const float *Xq, int64_
         return run_tf32<1, true>(t, c, st, a, sc.n_ctas, s);
     }
     if (c.r == 1) return run_tf32<1, false>(t, c, st, a, sc.n_ctas, s);
-    return run_tf32<4, false>(t, c, st, a, sc.n_ctas, s);
+    if (c.r <= 4) return run_tf32<4, false>(t, c, st, a, sc.n_ctas, s);
+    return run_tf32<16, false>(t, c, st, a, sc.n_ctas, s);
 }
 
 void eval_tf32_free(askit_tree t) {

@@ -341,14 +341,15 @@ __global__ void __launch_bounds__(256) ko_rerank_kernel(const float *Xt, const f
 // Step 3.  A tile of 256 tree positions stays in shared memory while tiles of 128
 // queries stream through four stages (TMA, 128-byte swizzled K-major FP16 hi and
 // lo); 12 tcgen05.mma (128 x 256 x 16) a tile pair leave sigma^2 a.b in one of two
-// 256-column TMEM accumulators; each of the two epilogue groups takes 128 columns:
+// 256-column TMEM accumulators; each of the four epilogue groups takes 64 columns:
 // n_j - 2 a.b / sigma^2 against the query's threshold, 32 columns' minimum first.
-// Bound by the tensor core (12 MMAs of 128 cycles a tile pair against about 1300
-// issue slots of the epilogue).  (source tile, query tile) pairs are dealt in
-// contiguous ranges of equal length, one CTA an SM.
-//   warps 0-7  epilogue, group = columns 128 g ..
-//   warp 8     TMA
-//   warp 9     TMEM allocation, MMA issue
+// 12 MMAs of 128 cycles a tile pair against about 1300 issue slots of the epilogue:
+// with two groups the epilogue's latency bound it (tensor pipe 43 %, issue 36 %).
+// (source tile, query tile) pairs are dealt in contiguous ranges of equal length,
+// one CTA an SM.
+//   warps 0-15 epilogue, group g = columns 64 g ..
+//   warp 16    TMA
+//   warp 17    TMEM allocation, MMA issue
 // Every wait is bounded (ASK_DEV_TIMEOUT).
 // ---------------------------------------------------------------------------
 constexpr int KS_REGION = 128 * 128;           // 128 rows x 64 FP16
@@ -360,7 +361,7 @@ struct KS {
     static constexpr int BAR = COL + 2 * 256 * 4;              // 20 mbarriers
     static constexpr int MISC = BAR + 20 * 8;
     static constexpr int BYTES = MISC + 16;
-    static constexpr int THREADS = 320;
+    static constexpr int THREADS = 576;
 };
 struct KSArgs {
     int64_t N, T, units;                       // units = source tiles x query tiles
@@ -399,14 +400,14 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
         mbar_init(BAR_B_EMPTY, 1);
         for (int a = 0; a < 2; ++a) {
             mbar_init(BAR_T_FULL(a), 1);
-            mbar_init(BAR_T_EMPTY(a), 256);
+            mbar_init(BAR_T_EMPTY(a), 512);
             mbar_init(BAR_C_FULL(a), 1);
-            mbar_init(BAR_C_EMPTY(a), 256);
+            mbar_init(BAR_C_EMPTY(a), 512);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 9) {
+    if (warp == 17) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -419,7 +420,7 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
     const int64_t u0 = args.units * blockIdx.x / gridDim.x, u1 = args.units * (blockIdx.x + 1) / gridDim.x;
     const int n_qt = args.n_qt;
 
-    if (warp < 8) {
+    if (warp < 16) {
         const int q4 = warp & 3, eg = warp >> 2, row = q4 * 32 + lane;
         int li = 0, lb = -1;
         int64_t bt = -1;
@@ -434,16 +435,16 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
         };
         float un, nn;
         load(u0, un, nn);
-        // A unit's hits stay in four masks; their places in the query's list come
+        // A unit's hits stay in two masks; their places in the query's list come
         // from one counter update a unit, whose answer is waited for only after the
         // next unit (waiting for one a chunk made the epilogue three times as long
         // as the MMAs)
-        uint32_t ph[4] = {0, 0, 0, 0};
+        uint32_t ph[2] = {0, 0};
         int pk = 0;
         int64_t pq = 0, pp = 0;
         auto flush = [&]() {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < 2; ++c) {
                 uint32_t m = ph[c];
                 while (m) {
                     const int j = __ffs(m) - 1;
@@ -462,7 +463,7 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
                 ++lb;
                 bt = b;
                 if (!mbar_wait(BAR_C_FULL(lb & 1), (lb >> 1) & 1, abort_flag, args.status)) break;
-                col = reinterpret_cast<const float *>(sm + KS::COL) + (lb & 1) * 256 + 128 * eg;
+                col = reinterpret_cast<const float *>(sm + KS::COL) + (lb & 1) * 256 + 64 * eg;
             }
             const int64_t q = (int64_t)qt * 128 + row;
             const float thr = (un * (1.f + args.eta) + args.abs) / (1.f - args.eta) - nn;
@@ -470,10 +471,10 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
             const int a = li & 1;
             if (!mbar_wait(BAR_T_FULL(a), (li >> 1) & 1, abort_flag, args.status)) break;
             tc_fence_after();
-            const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * 256 + 128 * eg);
-            const int64_t pos0 = b * 256 + 128 * eg;
+            const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(a * 256 + 64 * eg);
+            const int64_t pos0 = b * 256 + 64 * eg;
             auto chunk = [&](int c, const uint32_t (&g)[32]) -> uint32_t {
-                float dd[32], m = INFINITY;
+                float dd[32], m4[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
 #pragma unroll
                 for (int j = 0; j < 32; j += 4) {
                     const float4 n4 = *reinterpret_cast<const float4 *>(col + c * 32 + j);
@@ -485,43 +486,40 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
                     dd[j + 1] = x.y;
                     dd[j + 2] = z.x;
                     dd[j + 3] = z.y;
-                    m = fminf(m, fminf(fminf(x.x, x.y), fminf(z.x, z.y)));
+                    m4[(j >> 2) & 3] = fminf(m4[(j >> 2) & 3], fminf(fminf(x.x, x.y), fminf(z.x, z.y)));
                 }
+                const float m = fminf(fminf(m4[0], m4[1]), fminf(m4[2], m4[3]));
                 uint32_t hit = 0;
                 if (__any_sync(FULL, m <= thr)) {
+                    uint32_t h4[4] = {0, 0, 0, 0};         // four chains instead of one of 32
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) hit |= dd[j] <= thr ? 1u << j : 0u;
+                    for (int j = 0; j < 32; ++j) h4[j & 3] |= dd[j] <= thr ? 1u << j : 0u;
+                    hit = (h4[0] | h4[1]) | (h4[2] | h4[3]);
                     const int64_t p0 = pos0 + c * 32;
                     if (p0 + 32 > args.N) hit &= p0 < args.N ? (1u << (args.N - p0)) - 1u : 0u;   // rows past N
                 }
                 return hit;
             };
-            uint32_t ga[32], gb[32], hit[4];
+            uint32_t ga[32], gb[32], hit[2];
             tmem_ld32_async(tbase, ga);
             tmem_wait_pin(ga);
             tmem_ld32_async(tbase + 32, gb);
             hit[0] = chunk(0, ga);
             tmem_wait_pin(gb);
-            tmem_ld32_async(tbase + 64, ga);
-            hit[1] = chunk(1, gb);
-            tmem_wait_pin(ga);
-            tmem_ld32_async(tbase + 96, gb);
-            hit[2] = chunk(2, ga);
-            tmem_wait_pin(gb);
             tc_fence_before();
             mbar_arrive(BAR_T_EMPTY(a));       // all columns are in registers
-            hit[3] = chunk(3, gb);
+            hit[1] = chunk(1, gb);
             flush();
-            const int n = __popc(hit[0]) + __popc(hit[1]) + __popc(hit[2]) + __popc(hit[3]);
+            const int n = __popc(hit[0]) + __popc(hit[1]);
             if (n) pk = atomicAdd(args.cnt + q, n);
             __syncwarp();
             pq = q;
             pp = pos0;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) ph[c] = hit[c];
+            for (int c = 0; c < 2; ++c) ph[c] = hit[c];
         }
         flush();
-    } else if (warp == 8 && lane == 0) {
+    } else if (warp == 16 && lane == 0) {
         int li = 0, lb = -1;
         int64_t bt = -1;
         for (int64_t u = u0; u < u1; ++u, ++li) {
@@ -560,7 +558,7 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
             mbar_drain(BAR_B_FULL, lb & 1);
             mbar_drain(BAR_C_FULL(lb & 1), (lb >> 1) & 1);
         }
-    } else if (warp == 9 && lane == 0) {
+    } else if (warp == 17 && lane == 0) {
         constexpr uint32_t IDESC = make_idesc(0u, 128, 256);
         int li = 0, lb = -1, done = -1;
         int64_t bt = -1;
@@ -599,7 +597,7 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 9) {
+    if (warp == 17) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
     }
