@@ -225,8 +225,43 @@ __device__ __forceinline__ float scaled_abs(double a, int base, int lim) {
     return hi < lim ? 0.f : __uint_as_float(((uint32_t)(hi - base) << 3) | ((uint32_t)__double2loint(a) >> 29));
 }
 
+// f(i, x, p) for rows i .. rows - 1 of a column (p: its element of row i, rows
+// `cols` apart), eight loads at a time; AHEAD: the next eight in flight during these.
+template <bool AHEAD, class L, class F>
+__device__ __forceinline__ void walk_column(double *p, int64_t cols, int i, int rows, L ld, F f) {
+    double x[8];
+    if (AHEAD && i + 8 <= rows) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = ld(p + u * cols);
+    }
+    for (; i + 8 <= rows; i += 8, p += 8 * cols) {
+        double y[8];
+        if (AHEAD) {
+            const bool more = i + 16 <= rows;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) y[u] = more ? ld(p + (8 + u) * cols) : 0.0;
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = ld(p + u * cols);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f(i + u, x[u], p + u * cols);
+        if (AHEAD) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = y[u];
+        }
+    }
+    for (; i < rows; ++i, p += cols) f(i, ld(p), p);
+}
+
+// With two or four CTAs a node a column's chain is short of warps to hide the loads
+// behind, so they run ahead, at one CTA an SM; clusters of eight CTAs that each need
+// an SM do not all fit the GPCs at once (16 nodes: two waves), so those stay at two.
 template <int C>
-__global__ void __launch_bounds__(QR_THREADS, 2) cpqr_kernel(
+constexpr bool QR_AHEAD = C == 2 || C == 4;
+
+template <int C>
+__global__ void __launch_bounds__(QR_THREADS, QR_AHEAD<C> ? 1 : 2) cpqr_kernel(
     const int32_t *batch_nodes, const int64_t *woff, const int64_t *poff_ws, const int32_t *ncol,
     const int32_t *ellv, double tol, int s_min, int s_max, double *work, int32_t *piv_fixed,
     int cmax, int32_t *s_out) {
@@ -260,30 +295,21 @@ __global__ void __launch_bounds__(QR_THREADS, 2) cpqr_kernel(
     auto ld = [&](const double *p) { return C > 1 ? __ldcg(p) : *p; };
     auto norm_of = [&](int j, int k) {
         double acc = 0.0;
-        const double *p = A + (int64_t)k * cols + j;
-        int i = k;
-        for (; i + 8 <= rows; i += 8, p += 8 * (int64_t)cols) {
-            double x[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) x[u] = ld(p + u * (int64_t)cols);
-#pragma unroll
-            for (int u = 0; u < 8; ++u) acc = c_add(acc, c_mul(x[u], x[u]));
-        }
-        for (; i < rows; ++i, p += cols) {
-            const double x = ld(p);
-            acc = c_add(acc, c_mul(x, x));
-        }
+        walk_column<QR_AHEAD<C>>(A + (int64_t)k * cols + j, cols, k, rows, ld,
+                             [&](int, double x, double *) { acc = c_add(acc, c_mul(x, x)); });
         return acc;
     };
     // the same sum with the whole warp on one column: 32 products an instruction,
     // then one chain of additions
     auto norm_of_one = [&](int j, int k) {
         double acc = 0.0;
+        auto row = [&](int i) { return i + lane < rows ? ld(A + (int64_t)(i + lane) * cols + j) : 0.0; };
+        double x = row(k);
         for (int i = k; i < rows; i += 32) {
-            const double x = i + lane < rows ? ld(A + (int64_t)(i + lane) * cols + j) : 0.0;
-            const double xx = c_mul(x, x);
+            const double next = row(i + 32), xx = c_mul(x, x);
             const int n = min(32, rows - i);
             for (int u = 0; u < n; ++u) acc = c_add(acc, __shfl_sync(0xffffffffu, xx, u));
+            x = next;
         }
         return acc;
     };
@@ -419,38 +445,18 @@ __global__ void __launch_bounds__(QR_THREADS, 2) cpqr_kernel(
             if (j <= k || j >= cols) continue;
             double dot = 0.0;
             double *p0 = A + (int64_t)k * cols + j;
-            {
-                const double *q = p0;
-                int i = k;
-                for (; i + 8 <= rows; i += 8, q += 8 * (int64_t)cols) {
-                    double x[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) x[u] = ld(q + u * (int64_t)cols);
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) dot = c_add(dot, c_mul(v[i + u], x[u]));
-                }
-                for (; i < rows; ++i, q += cols) dot = c_add(dot, c_mul(v[i], ld(q)));
-            }
+            walk_column<QR_AHEAD<C>>(p0, cols, k, rows, ld,
+                                 [&](int i, double x, double *) { dot = c_add(dot, c_mul(v[i], x)); });
             const double tdot = c_mul(tau, dot);
             float f = 0.f;
             bool bad = false;
-            double *q = p0;
-            int i = k;
-            auto upd = [&](int ii, double x, double *dst) {
-                const double y = c_sub(x, c_mul(tdot, v[ii]));
+            walk_column<QR_AHEAD<C>>(p0, cols, k, rows, ld, [&](int i, double x, double *dst) {
+                const double y = c_sub(x, c_mul(tdot, v[i]));
                 *dst = y;
                 const float t = scaled_abs(y, base, lim);
                 bad |= (__double2hiint(y) & 0x7ff00000) == 0x7ff00000;
-                if (ii > k) f = fmaf(t, t, f);
-            };
-            for (; i + 8 <= rows; i += 8, q += 8 * (int64_t)cols) {
-                double x[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) x[u] = ld(q + u * (int64_t)cols);
-#pragma unroll
-                for (int u = 0; u < 8; ++u) upd(i + u, x[u], q + u * (int64_t)cols);
-            }
-            for (; i < rows; ++i, q += cols) upd(i, ld(q), q);
+                if (i > k) f = fmaf(t, t, f);
+            });
             nf[32 * (blk / C) + lane] = bad ? -1.f : f;   // a column that is not finite is never a pivot
         }
         have_nf = true;
@@ -465,15 +471,31 @@ __global__ void __launch_bounds__(QR_THREADS, 2) cpqr_kernel(
             double acc = ld(A + (int64_t)i * cols + (s + j));
             const double *ai = A + (int64_t)i * cols;
             int t = i + 1;
-            for (; t + 8 <= s; t += 8) {
-                double x[8], y[8];
+            double x[8], y[8];
+            auto rows8 = [&](int t0, double (&xx)[8], double (&yy)[8]) {
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    x[u] = ld(ai + t + u);
-                    y[u] = P[(int64_t)(t + u) * nr + j];
+                    xx[u] = ld(ai + t0 + u);
+                    yy[u] = P[(int64_t)(t0 + u) * nr + j];
+                }
+            };
+            if (QR_AHEAD<C> && t + 8 <= s) rows8(t, x, y);
+            for (; t + 8 <= s; t += 8) {
+                double xn[8], yn[8];
+                if (QR_AHEAD<C>) {
+                    if (t + 16 <= s) rows8(t + 8, xn, yn);
+                } else {
+                    rows8(t, x, y);
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) acc = c_sub(acc, c_mul(x[u], y[u]));
+                if (QR_AHEAD<C>) {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        x[u] = xn[u];
+                        y[u] = yn[u];
+                    }
+                }
             }
             for (; t < s; ++t) acc = c_sub(acc, c_mul(ld(ai + t), P[(int64_t)t * nr + j]));
             P[(int64_t)i * nr + j] = c_div(acc, ld(ai + i));
@@ -720,9 +742,13 @@ askit_status skeletonize(askit_tree t, cudaStream_t s) {
             }
             int maxrows = 0;
             for (int g = 0; g < nb; ++g) maxrows = std::max(maxrows, h_ell[nodes[g]]);
-            // a cluster per node while the CTAs stay within the SMs
+            // a cluster per node while the CTAs stay within the SMs and each has four
+            // column groups, one for every quarter of its SM (64K x 64, 512 columns:
+            // a level takes 14.7 ms with four CTAs a node, 15.5 with eight)
+            int maxcols = 0;
+            for (int g = 0; g < nb; ++g) maxcols = std::max(maxcols, t->h_ncol[nodes[g]]);
             int c = 1;
-            while (c < 8 && 2 * c * nb <= sms) c *= 2;
+            while (c < 8 && 2 * c * nb <= sms && 2 * c * 128 <= maxcols) c *= 2;
             const size_t smem = sizeof(double) * (size_t)(maxrows + 1) +
                                 sizeof(float) * 32 * (((size_t)cmax + 31) / 32 / c + 1);
             ASK_TRY((c == 1 ? launch_cpqr<1> : c == 2 ? launch_cpqr<2> : c == 4 ? launch_cpqr<4> : launch_cpqr<8>)(

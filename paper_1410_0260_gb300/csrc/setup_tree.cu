@@ -49,20 +49,27 @@ __global__ void center_kernel(const float *X, int d, const int32_t *order, const
     if (k >= d) return;
     int64_t b = lvl_start[node], n = lvl_size[node];
     double acc = 0.0;
-    // one chain of additions a coordinate: the next 16 rows' loads are in flight
-    // during this group's
+    // one chain of additions a coordinate, 64 cycles each: the next 16 rows' loads,
+    // and the ids of the 16 after them, are in flight during this group's
     int64_t q = 0;
     constexpr int G = 16;
     float x[G];
-    if (n >= G) {
+    int32_t id[G];
+    auto ids = [&](int64_t q0) {
 #pragma unroll
-        for (int u = 0; u < G; ++u) x[u] = X[(int64_t)order[b + u] * d + k];
+        for (int u = 0; u < G; ++u) id[u] = q0 + G <= n ? order[b + q0 + u] : 0;
+    };
+    if (n >= G) {
+        ids(0);
+#pragma unroll
+        for (int u = 0; u < G; ++u) x[u] = X[(int64_t)id[u] * d + k];
+        ids(G);
     }
     for (; q + G <= n; q += G) {
         float y[G];
-        const bool more = q + 2 * G <= n;
 #pragma unroll
-        for (int u = 0; u < G; ++u) y[u] = more ? X[(int64_t)order[b + q + G + u] * d + k] : 0.f;
+        for (int u = 0; u < G; ++u) y[u] = X[(int64_t)id[u] * d + k];     // (row 0 past the last group)
+        ids(q + 2 * G);
 #pragma unroll
         for (int u = 0; u < G; ++u) acc = c_add(acc, c_f2d(x[u]));
 #pragma unroll
