@@ -751,7 +751,8 @@ def main():
     roof["kernel"] = ("eval_simt_kernel" if args.precision == "simt_fp32" else
                       "eval_tcw_kernel" if d > 64 else
                       ("eval_g16_kernel" if info["fp16_centering"] == 2 else "eval_tc16_kernel")
-                      if args.precision == "fp16x3" else "eval_tc_kernel")
+                      if args.precision == "fp16x3" else
+                      "eval_tf32_kernel" if args.precision == "tf32x3" else "eval_tc_kernel")
     roof["ms_per_launch"] = k_ms / max(1, k_launches)
     roof["launches_per_evaluate"] = k_launches // args.steps
     roof["evaluate_ms"] = ms_eval

@@ -1,4 +1,4 @@
-// Evaluate (Algorithm 4) on the tcgen05 tensor cores.
+// Evaluate (Algorithm 4) on the tcgen05 tensor cores in BF16x3, d <= 64.
 //
 // Work item = one source sub-block (<= 128 rows of a leaf's points for the
 // direct near field, or of a node's skeleton for the far field) against up
@@ -14,7 +14,7 @@
 // is bounded by the spread of the item's targets or by |x - y| itself, so
 // the FP32 rounding of the norm expansion stays at that scale even for the
 // wide skeletons of high tree nodes.  The contraction is split in three
-// products (hi*hi + hi*lo + lo*hi) of TF32 or BF16 parts with FP32
+// products (hi*hi + hi*lo + lo*hi) of BF16 parts with FP32
 // accumulation.
 //
 // One CTA per SM, warp-specialized, 416 threads:
@@ -52,10 +52,6 @@ constexpr uint32_t TMEM_COLS = 256;             // two 128-column FP32 accumulat
 // Precision traits: element bytes, swizzle regions per operand (TC_K
 // elements x element bytes / 128), MMA K steps, tcgen05 operand format.
 template <int P> struct Prec;
-template <> struct Prec<ASKIT_PREC_TF32X3> {
-    static constexpr int EB = 4, NREG = 2, KSTEPS = 8;   // K = 8 per MMA
-    static constexpr uint32_t FMT = 2;                   // TF32 in .kind::tf32
-};
 template <> struct Prec<ASKIT_PREC_BF16X3> {
     static constexpr int EB = 2, NREG = 1, KSTEPS = 4;   // K = 16 per MMA
     static constexpr uint32_t FMT = 1;                   // BF16 in .kind::f16
@@ -64,17 +60,16 @@ template <> struct Prec<ASKIT_PREC_BF16X3> {
 // Shared-memory plan (offsets from a 1024-byte aligned base).
 template <int P>
 struct Smem {
-    // the 16-bit splits have room to stage raw rows: targets are then gathered
-    // by TMA (tile::gather4) and the loaders work from shared memory only
-    static constexpr bool GATHER = P != ASKIT_PREC_TF32X3;
+    // targets are gathered by TMA (tile::gather4) and the loaders work from shared
+    // memory only
     static constexpr int OPB = Prec<P>::NREG * REGION;    // one operand (hi or lo) of one tile
     static constexpr int B_HI = 0, B_LO = OPB;
     static constexpr int A0 = 2 * OPB;                     // stage s: hi at A0 + s*2*OPB, lo at + OPB
     static constexpr int TILES = 6 * OPB;
     static constexpr int RAWSTAGE = TILE_ROWS * TC_K * 4;  // one stage of gathered FP32 target rows
-    static constexpr int RAW = TILES;                      // [2] stages (GATHER)
-    static constexpr int RAWB = RAW + (GATHER ? 2 * RAWSTAGE : 0);        // raw FP32 source rows (GATHER)
-    static constexpr int CENT = RAWB + (GATHER ? RAWSTAGE : 0);           // float [TC_K] c_B of the sub-block
+    static constexpr int RAW = TILES;                      // [2] stages
+    static constexpr int RAWB = RAW + 2 * RAWSTAGE;        // raw FP32 source rows
+    static constexpr int CENT = RAWB + RAWSTAGE;           // float [TC_K] c_B of the sub-block
     static constexpr int ANORM = CENT + TC_K * 4;                         // float [2][128] |a|^2 + 2 a.delta
     static constexpr int COLV = ANORM + 2 * 128 * 4;       // float4 [2][128]: per source pair {A, B}, {C, w} (see loader)
     static constexpr int RC_MAX = 16;
@@ -89,15 +84,12 @@ struct TcArgs {
     const int32_t *block_off;
     const int32_t *cta_off, *cta_blocks;   // this CTA's sub-blocks: cta_blocks[cta_off[c] .. cta_off[c+1])
     const int32_t *tgt;       // entry -> target slot
-    const float *Xq;          // target coordinates [*, ldq]
-    int64_t ldq;
     int d_pad;
     const float *cent;        // [n_sub, TC_K]
     const float *sc_t, *sc_s; // c log2(e) / h^2 per source row
-    const float *Xt, *Xs;     // raw source coordinates [*, d_pad] (column terms)
     const float *Wt, *Ws;
     int r;
-    float f16_scale;          // prescale of the 16-bit operands (1: BF16 and TF32 are not prescaled)
+    float f16_scale;          // prescale of the 16-bit operands (1: BF16 is not prescaled)
     float g_unscale;          // 1 / f16_scale^2
     float *partial;
     int *status;
@@ -183,8 +175,6 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
             const int nrows = item.nrows & 0x7fffffff;
             const bool has_src = t < nrows;
             const int64_t srow = (int64_t)item.row0 + t;
-            const float *ysrc = (far ? args.Xs : args.Xt) + srow * args.d_pad;
-            const float *cB = args.cent + (int64_t)item.cidx * TC_K;
             // block-constant column data of source row t: c log2(e) / h^2 and w
             const float sc = has_src ? __ldg((far ? args.sc_s : args.sc_t) + srow) : 0.f;
             const float *wrow = (far ? args.Ws : args.Wt) + srow * args.r;
@@ -193,33 +183,24 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
             // this group's first item of the block
             int it = i0 + (((li & 1) ^ grp) & 1);
             if (it < i1) item = args.items[it];
-            int slot = (it < i1 && t < item.cnt) ? (S::GATHER ? 0 : args.tgt[item.e0 + t]) : -1;
-            int first = (it < i1 && !S::GATHER) ? args.tgt[item.e0] : 0;
+            bool next_tgt = it < i1 && t < item.cnt;
             li += ((li & 1) ^ grp) & 1;
             for (; it < i1; it += 2, li += 2) {
                 const int s = li & 1;
                 const uint32_t par = ((li >> 1) & 1) ^ 1;
-                const int cnt = item.cnt;
-                const float *xrow = args.Xq + (int64_t)(slot >= 0 ? slot : 0) * args.ldq;
-                const float *xt0 = args.Xq + (int64_t)first * args.ldq;
-                const bool has_tgt = slot >= 0;
-                // prefetch this group's next item of the block (the gather path
-                // needs only its size: the gather warp fetches the rows)
+                const bool has_tgt = next_tgt;
+                // this group's next item of the block, ahead (only its size: the
+                // gather warp fetches the rows)
                 if (it + 2 < i1) {
                     item = args.items[it + 2];
-                    if constexpr (!S::GATHER) {
-                        slot = t < item.cnt ? args.tgt[item.e0 + t] : -1;
-                        first = args.tgt[item.e0];
-                    } else {
-                        slot = t < item.cnt ? 0 : -1;
-                    }
+                    next_tgt = t < item.cnt;
                 }
                 if (!mbar_wait(BAR_A_EMPTY(s), par, abort_flag, args.status)) goto loader_done;
                 if (!mbar_wait(BAR_T_EMPTY(s), par, abort_flag, args.status)) goto loader_done;
                 uint8_t *ahi = sm + S::A0 + s * 2 * S::OPB;
                 uint8_t *alo = ahi + S::OPB;
                 float nn = 0.f, dd = 0.f, qq = 0.f;
-                if constexpr (S::GATHER) {
+                {
                     // gathered target rows (stage s) and the sub-block's raw rows
                     if (!mbar_wait(BAR_R_FULL(s), (li >> 1) & 1, abort_flag, args.status)) goto loader_done;
                     if (!waited_b) {
@@ -277,72 +258,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
                     dd = dd2.x + dd2.y;
                     qq = qq2.x + qq2.y;
                     if (!has_tgt) nn = dd = 0.f;
-                } else {
-                // two 4-column chunks per step: 32 contiguous bytes of a row
-#pragma unroll 4
-                for (int k8 = 0; k8 < TC_K / 8; ++k8) {
-                    float xa[8], ya[8];
-                    if (2 * k8 < nk4) {
-                        const float4 x0 = has_tgt ? __ldg(reinterpret_cast<const float4 *>(xrow + 8 * k8)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        const float4 x1 = has_tgt ? __ldg(reinterpret_cast<const float4 *>(xrow + 8 * k8 + 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        const float4 t0 = __ldg(reinterpret_cast<const float4 *>(xt0 + 8 * k8));
-                        const float4 t1 = __ldg(reinterpret_cast<const float4 *>(xt0 + 8 * k8 + 4));
-                        const float4 b0 = *reinterpret_cast<const float4 *>(cB + 8 * k8);
-                        const float4 b1 = *reinterpret_cast<const float4 *>(cB + 8 * k8 + 4);
-                        const float4 y0 = has_src ? __ldg(reinterpret_cast<const float4 *>(ysrc + 8 * k8)) : t0;
-                        const float4 y1 = has_src ? __ldg(reinterpret_cast<const float4 *>(ysrc + 8 * k8 + 4)) : t1;
-                        const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-                        const float ts[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-                        const float bs[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-                        const float ys[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            xa[e] = has_tgt ? xs[e] - ts[e] : 0.f;       // a = x - c_T
-                            nn = fmaf(xa[e], xa[e], nn);
-                            dd = fmaf(xa[e], ts[e] - bs[e], dd);          // a . delta
-                            ya[e] = ys[e] - ts[e];                        // y - c_T
-                            qq = fmaf(ya[e], ya[e], qq);
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) xa[e] = 0.f;
-                    }
-                    if constexpr (P == ASKIT_PREC_TF32X3) {
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int c4 = 2 * k8 + h, reg = c4 >> 3, chunk = c4 & 7;
-                            float4 hi, lo;
-                            hi.x = __uint_as_float(__float_as_uint(xa[4 * h + 0]) & 0xffffe000u);
-                            hi.y = __uint_as_float(__float_as_uint(xa[4 * h + 1]) & 0xffffe000u);
-                            hi.z = __uint_as_float(__float_as_uint(xa[4 * h + 2]) & 0xffffe000u);
-                            hi.w = __uint_as_float(__float_as_uint(xa[4 * h + 3]) & 0xffffe000u);
-                            lo.x = xa[4 * h + 0] - hi.x; lo.y = xa[4 * h + 1] - hi.y;
-                            lo.z = xa[4 * h + 2] - hi.z; lo.w = xa[4 * h + 3] - hi.w;
-                            const int off = reg * REGION + t * 128 + ((chunk ^ (t & 7)) << 4);
-                            *reinterpret_cast<float4 *>(ahi + off) = hi;
-                            *reinterpret_cast<float4 *>(alo + off) = lo;
-                        }
-                    } else {
-                        // 8 elements = one 16-byte chunk of the 128-byte row
-                        uint32_t hv[4], lv[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            float v0 = xa[2 * e], v1 = xa[2 * e + 1];
-                            uint16_t h0, h1, l0, l1;
-                            const __nv_bfloat16 a0 = __float2bfloat16_rn(v0), a1 = __float2bfloat16_rn(v1);
-                            h0 = __bfloat16_as_ushort(a0); h1 = __bfloat16_as_ushort(a1);
-                            l0 = __bfloat16_as_ushort(__float2bfloat16_rn(v0 - __bfloat162float(a0)));
-                            l1 = __bfloat16_as_ushort(__float2bfloat16_rn(v1 - __bfloat162float(a1)));
-                            hv[e] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-                            lv[e] = (uint32_t)l0 | ((uint32_t)l1 << 16);
-                        }
-                        const int off = t * 128 + ((k8 ^ (t & 7)) << 4);
-                        *reinterpret_cast<uint4 *>(ahi + off) = make_uint4(hv[0], hv[1], hv[2], hv[3]);
-                        *reinterpret_cast<uint4 *>(alo + off) = make_uint4(lv[0], lv[1], lv[2], lv[3]);
-                    }
                 }
-                }
-                (void)cnt;
                 // row term |a|^2 + 2 a.delta; column data of source row t:
                 // arg = g (2 u sc) + (-sc) p_t + (-sc q) = -sc (p_t + q - 2 u g)
                 a_norm[s * 128 + t] = nn + 2.f * dd;
@@ -363,7 +279,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
                 // generic-proxy stores -> visible to the tensor core's async proxy
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 mbar_arrive(BAR_A_FULL(s));
-                if constexpr (S::GATHER) mbar_arrive(BAR_R_EMPTY(s));
+                mbar_arrive(BAR_R_EMPTY(s));
             }
             // li now points past this block for this group; realign to the block end
             li = li_block_end;
@@ -455,7 +371,7 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
     epi_done:;
     } else if (warp == 13) {
         // ---------------------------------------------- target-row gatherer (warp 13)
-        if constexpr (S::GATHER) {
+        {
             const uint32_t bytes = (uint32_t)(TILE_ROWS * args.d_pad * 4);
             int li = 0, issued = 0;
             for (int ci = args.cta_off[blockIdx.x]; ci < args.cta_off[blockIdx.x + 1] && !*abort_flag; ++ci) {
@@ -484,8 +400,8 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
         }
     } else if (warp == 12 && lane == 0) {
         // ------------------------------------------------- TMA + MMA issuer
-        // hi + lo of one 128-row sub-block, and its raw FP32 rows (gather path)
-        const uint32_t TX = 2 * NREG * REGION + (S::GATHER ? (uint32_t)(TILE_ROWS * args.d_pad * 4 + TC_K * 4) : 0u);
+        // hi + lo of one 128-row sub-block, and its raw FP32 rows
+        const uint32_t TX = 2 * NREG * REGION + (uint32_t)(TILE_ROWS * args.d_pad * 4 + TC_K * 4);
         int li = 0, lb = 0, b_issued = 0;
         for (int ci = args.cta_off[blockIdx.x]; ci < args.cta_off[blockIdx.x + 1] && !*abort_flag; ++ci, ++lb) {
             const int b = args.cta_blocks[ci];
@@ -502,10 +418,8 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
                 tma_load_2d(sbase + S::B_HI + g * REGION, mh, x, first.row0, BAR_B_FULL(lb & 1));
                 tma_load_2d(sbase + S::B_LO + g * REGION, ml, x, first.row0, BAR_B_FULL(lb & 1));
             }
-            if constexpr (S::GATHER) {
-                tma_load_2d(sbase + S::RAWB, far ? &map_rs : &map_rt, 0, first.row0, BAR_B_FULL(lb & 1));
-                bulk_copy(sbase + S::CENT, args.cent + (int64_t)first.cidx * TC_K, TC_K * 4, BAR_B_FULL(lb & 1));
-            }
+            tma_load_2d(sbase + S::RAWB, far ? &map_rs : &map_rt, 0, first.row0, BAR_B_FULL(lb & 1));
+            bulk_copy(sbase + S::CENT, args.cent + (int64_t)first.cidx * TC_K, TC_K * 4, BAR_B_FULL(lb & 1));
             const int i0 = args.block_off[b], i1 = args.block_off[b + 1];
             for (int it = i0; it < i1; ++it, ++li) {
                 const int s = li & 1;
@@ -549,106 +463,45 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_consta
     }
 }
 
-// Tensor maps of the four source operand arrays for one precision.
+// Tensor maps: the split source rows (boxes of 64 x 128, 128-byte swizzle) [t_hi,
+// t_lo, s_hi, s_lo], and the raw FP32 source rows in 128-row boxes.
 struct TcState {
-    CUtensorMap map[2][4];   // [precision: 0 tf32, 1 bf16][t_hi, t_lo, s_hi, s_lo]
-    bool ready[2] = {false, false};
-    CUtensorMap raw_t, raw_s;   // raw FP32 source rows, 128-row boxes (gather path)
-    bool raw_ready = false;
-    void *encode = nullptr;     // cuTensorMapEncodeTiled
+    CUtensorMap map[4], raw_t, raw_s;
+    bool ready = false;
+    EncodeTiledFn encode = nullptr;
 };
 
-askit_status encode_map(EncodeTiledFn fn, CUtensorMap *m, void *base, int64_t rows, int ty) {
-    const bool f32 = ty == 0;
-    const int eb = f32 ? 4 : 2;
-    cuuint64_t dims[2] = {(cuuint64_t)TC_K, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)TC_K * eb};
-    cuuint32_t box[2] = {(cuuint32_t)(128 / eb), (cuuint32_t)TILE_ROWS};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = fn(m, ty == 0 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                       : ty == 1 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, base, dims,
-                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        askit_set_error("cuTensorMapEncodeTiled failed (%d)", (int)r);
-        return ASKIT_ERR_CUDA;
-    }
-    return ASKIT_OK;
-}
+std::mutex g_tc_mu;   // the tensor maps are built once, under a lock
 
-// Unswizzled FP32 map over [rows, cols] with boxes of box_rows full rows
-// (box_rows = 1 for tile::gather4).
-askit_status encode_raw(EncodeTiledFn fn, CUtensorMap *m, const void *base, int64_t rows, int cols, int box_rows) {
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
-    cuuint32_t box[2] = {(cuuint32_t)cols, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(base), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        askit_set_error("cuTensorMapEncodeTiled (raw rows) failed (%d)", (int)r);
-        return ASKIT_ERR_CUDA;
-    }
-    return ASKIT_OK;
-}
-
-std::mutex g_tc_mu;   // tensor-map state and launch attributes are built once, under a lock
-
-askit_status tc_state(askit_tree t, int pi, TcState **out) {
+askit_status tc_state(askit_tree t, TcState **out) {
     std::lock_guard<std::mutex> lock(g_tc_mu);
     if (!t->tc) t->tc = new TcState();
     TcState *st = (TcState *)t->tc;
-    if (!st->encode) {
-        void *fnp = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        ASK_CUDA(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fnp, 12000, cudaEnableDefault, &q));
-        if (!fnp || q != cudaDriverEntryPointSuccess) {
-            askit_set_error("cuTensorMapEncodeTiled not available");
-            return ASKIT_ERR_CUDA;
-        }
-        st->encode = fnp;
-    }
-    EncodeTiledFn fn = (EncodeTiledFn)st->encode;
-    if (!st->raw_ready) {
-        ASK_TRY(encode_raw(fn, &st->raw_t, t->Xt, t->N_pad, t->d_pad, TILE_ROWS));
-        ASK_TRY(encode_raw(fn, &st->raw_s, t->Xs, t->srows, t->d_pad, TILE_ROWS));
-        st->raw_ready = true;
-    }
-    if (!st->ready[pi]) {
-        const int ty = pi;   // 0 fp32 (tf32), 1 bf16
-        void *th = pi == 0 ? (void *)t->Xt_hi : (void *)t->Xt_bhi;
-        void *tl = pi == 0 ? (void *)t->Xt_lo : (void *)t->Xt_blo;
-        void *sh = pi == 0 ? (void *)t->Xs_hi : (void *)t->Xs_bhi;
-        void *sl = pi == 0 ? (void *)t->Xs_lo : (void *)t->Xs_blo;
-        ASK_TRY(encode_map(fn, &st->map[pi][0], th, t->N_pad, ty));
-        ASK_TRY(encode_map(fn, &st->map[pi][1], tl, t->N_pad, ty));
-        ASK_TRY(encode_map(fn, &st->map[pi][2], sh, t->srows, ty));
-        ASK_TRY(encode_map(fn, &st->map[pi][3], sl, t->srows, ty));
-        st->ready[pi] = true;
+    if (!st->ready) {
+        ASK_TRY(encode_fn(&st->encode));
+        const void *arr[4] = {t->Xt_bhi, t->Xt_blo, t->Xs_bhi, t->Xs_blo};
+        for (int i = 0; i < 4; ++i)
+            ASK_TRY(encode_2d(st->encode, &st->map[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, arr[i],
+                              i < 2 ? t->N_pad : t->srows, TC_K, 64, TILE_ROWS, CU_TENSOR_MAP_SWIZZLE_128B));
+        ASK_TRY(encode_2d(st->encode, &st->raw_t, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, t->Xt, t->N_pad, t->d_pad, t->d_pad,
+                          TILE_ROWS, CU_TENSOR_MAP_SWIZZLE_NONE));
+        ASK_TRY(encode_2d(st->encode, &st->raw_s, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, t->Xs, t->srows, t->d_pad, t->d_pad,
+                          TILE_ROWS, CU_TENSOR_MAP_SWIZZLE_NONE));
+        st->ready = true;
     }
     *out = st;
     return ASKIT_OK;
 }
 
 template <int P, int RC>
-askit_status launch(askit_tree t, TcState *st, const CUtensorMap &map_q, const TcArgs &a, int a_grid,
-                    cudaStream_t s) {
-    using S = Smem<P>;
-    const int pi = P == ASKIT_PREC_TF32X3 ? 0 : 1;
-    const size_t smem = S::BYTES + 1024;
-    static bool attr_set = false;
-    {
-        std::lock_guard<std::mutex> lock(g_tc_mu);
-        if (!attr_set) {
-            ASK_CUDA(cudaFuncSetAttribute(eval_tc_kernel<P, RC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            attr_set = true;
-        }
-    }
-    const unsigned grid = (unsigned)a_grid;
+askit_status launch(askit_tree t, TcState *st, const CUtensorMap &map_q, const TcArgs &a, int grid, cudaStream_t s) {
+    const size_t smem = Smem<P>::BYTES + 1024;
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(eval_tc_kernel<P, RC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    ASK_CUDA(attr);
     ASK_TRY(ktimer_mark(t, s, false));
-    ASK_TRY(launch_pdl(eval_tc_kernel<P, RC>, dim3(grid), dim3(TC_THREADS), smem, s, st->map[pi][0], st->map[pi][1],
-                       st->map[pi][2], st->map[pi][3], map_q, st->raw_t, st->raw_s, a));
+    ASK_TRY(launch_pdl(eval_tc_kernel<P, RC>, dim3((unsigned)grid), dim3(TC_THREADS), smem, s, st->map[0], st->map[1],
+                       st->map[2], st->map[3], map_q, st->raw_t, st->raw_s, a));
     return ktimer_mark(t, s, true);
 }
 
@@ -660,45 +513,43 @@ askit_status eval_tc(askit_tree t, const WeightCtx &c, int precision, const floa
     // FP16x3 with pre-split, globally centered targets where that keeps FP32
     // grade (eval_g16.cu)
     if (precision == ASKIT_PREC_FP16X3 && qs && use_g16(t)) return eval_g16(t, c, *qs, w, partial, s);
-    // FP16x3 centers both sides on the sub-block mean (eval_tc16.cu); BF16x3
-    // keeps the per-item target centering below: its 8-bit significands leave
-    // a residual of about 2^-17 of |a| |b| per product, so the smaller |a| of
-    // the per-item center is what keeps it within the split-path tolerance
+    // FP16x3 and 3xTF32 center both sides on the sub-block mean (eval_tc16.cu,
+    // eval_tf32.cu); BF16x3 keeps the per-item target centering below: its 8-bit
+    // significands leave a residual of about 2^-17 of |a| |b| per product, so the
+    // smaller |a| of the per-item center is what keeps it within the split-path
+    // tolerance
     if (precision == ASKIT_PREC_FP16X3) return eval_tc16(t, c, precision, Xq, ldq, q_rows, w, partial, s);
     if (precision != ASKIT_PREC_TF32X3 && precision != ASKIT_PREC_BF16X3) {
         askit_set_error("unknown tensor-core precision %d", precision);
         return ASKIT_ERR_INVALID_ARG;
     }
-    if (c.r > Smem<ASKIT_PREC_TF32X3>::RC_MAX) {
-        askit_set_error("tensor-core evaluation covers r <= %d; use ASKIT_PREC_SIMT_FP32", Smem<ASKIT_PREC_TF32X3>::RC_MAX);
+    if (c.r > Smem<ASKIT_PREC_BF16X3>::RC_MAX) {
+        askit_set_error("tensor-core evaluation covers r <= %d; use ASKIT_PREC_SIMT_FP32", Smem<ASKIT_PREC_BF16X3>::RC_MAX);
         return ASKIT_ERR_UNSUPPORTED;
     }
-    // 3xTF32: both sides centered on the sub-block, the targets' split rows in TMEM
-    if (precision == ASKIT_PREC_TF32X3) return eval_tf32(t, c, Xq, ldq, w, partial, s);
     if (w.n_blocks == 0) return ASKIT_OK;
     if (ldq != t->d_pad) {
         askit_set_error("target rows must have d_pad columns");
         return ASKIT_ERR_INVALID_ARG;
     }
+    if (precision == ASKIT_PREC_TF32X3) return eval_tf32(t, c, Xq, ldq, w, partial, s);
     TcState *st = nullptr;
-    ASK_TRY(tc_state(t, precision == ASKIT_PREC_TF32X3 ? 0 : 1, &st));
+    ASK_TRY(tc_state(t, &st));
     // gather map over this call's target rows (one box row per gathered row)
     CUtensorMap map_q;
-    ASK_TRY(encode_raw((EncodeTiledFn)st->encode, &map_q, Xq, q_rows, t->d_pad, 1));
+    ASK_TRY(encode_2d(st->encode, &map_q, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, Xq, q_rows, t->d_pad, t->d_pad, 1,
+                      CU_TENSOR_MAP_SWIZZLE_NONE));
+    const WorkLists::Sched &sc = w.sched[w.use];
     TcArgs a;
     a.items = w.items;
-    a.block_off = w.sched[w.use].run_off;
-    a.cta_off = w.sched[w.use].cta_off;
-    a.cta_blocks = w.sched[w.use].cta_runs;
+    a.block_off = sc.run_off;
+    a.cta_off = sc.cta_off;
+    a.cta_blocks = sc.cta_runs;
     a.tgt = w.tgt;
-    a.Xq = Xq;
-    a.ldq = ldq;
     a.d_pad = t->d_pad;
     a.cent = t->cent;
     a.sc_t = t->sc_t;
     a.sc_s = t->sc_s;
-    a.Xt = t->Xt;
-    a.Xs = t->Xs;
     a.Wt = c.Wt;
     a.Ws = c.Ws;
     a.r = c.r;
@@ -706,16 +557,9 @@ askit_status eval_tc(askit_tree t, const WeightCtx &c, int precision, const floa
     a.status = t->d_status;
     a.f16_scale = 1.f;
     a.g_unscale = 1.f / (a.f16_scale * a.f16_scale);
-    if (precision == ASKIT_PREC_TF32X3) {
-        return launch<ASKIT_PREC_TF32X3, 16>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
-    }
-    if (precision == ASKIT_PREC_BF16X3) {
-        if (c.r == 1) return launch<ASKIT_PREC_BF16X3, 1>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
-        if (c.r <= 4) return launch<ASKIT_PREC_BF16X3, 4>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
-        return launch<ASKIT_PREC_BF16X3, 16>(t, st, map_q, a, w.sched[w.use].n_ctas, s);
-    }
-    askit_set_error("unknown tensor-core precision %d", precision);
-    return ASKIT_ERR_INVALID_ARG;
+    if (c.r == 1) return launch<ASKIT_PREC_BF16X3, 1>(t, st, map_q, a, sc.n_ctas, s);
+    if (c.r <= 4) return launch<ASKIT_PREC_BF16X3, 4>(t, st, map_q, a, sc.n_ctas, s);
+    return launch<ASKIT_PREC_BF16X3, 16>(t, st, map_q, a, sc.n_ctas, s);
 }
 
 void eval_tc_free(askit_tree t) {
