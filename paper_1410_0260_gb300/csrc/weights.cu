@@ -27,16 +27,16 @@ __global__ void permute_in_kernel(const float *W, int64_t ldw, int r, const int3
 // products), and every load of a v(R) value from shared memory serves R rows.
 // The row sums are reduced over the lanes by a transposing butterfly (R RC sums
 // in about R RC shuffles).  R = 8 (r <= 4) or 4 (r > 4: R RC accumulators in
-// registers) where a level has 64 nodes or more, 2 near the root, whose few
-// nodes would otherwise leave most SMs idle; a row's sum is formed in the same
-// order for every R.  Levels are launched with programmatic serialization: a
+// registers) at every level: R = 2 near the root, for more blocks there, was no
+// faster at 4K, 64K or 1M points and cost 1-4 us a call at 50K, r = 3, where every
+// block stages its own v(R).  Levels are launched with programmatic serialization: a
 // level's blocks resolve their pivots and read their first P rows while the
 // level below still runs.
 // Measured (a set_weights call with its permutation, GB300; before: one row a
 // warp, 4-byte loads, r > 4 bound by its shared-memory loads):
 //   1M x 64, s = 256, r = 1     398 -> 275 us (1.07 GB of P: 158 us at the copy rate)
-//   64K x 64, s = 512, r = 16  2587 -> 147 us
-//   50K x 64, s = 256, r = 3    163 ->  32 us
+//   64K x 64, s = 512, r = 16  2587 -> 107 us (147 with 4-byte loads of v)
+//   50K x 64, s = 256, r = 3    163 ->  39 us
 constexpr int UP_KU = 1024;      // columns of P staged at a time
 constexpr int UP_WARPS = 8;
 
@@ -107,22 +107,41 @@ __global__ void __launch_bounds__(32 * UP_WARPS) upward_kernel(
                 waited = true;
             }
             __syncthreads();
-            // UB gathered values in flight a thread
-            constexpr int UB = RC == 1 ? 4 : 8;
-            for (int e0 = threadIdx.x; e0 < 128 * ni * RC; e0 += UB * 32 * UP_WARPS) {
-                float x[UB];
+            // column 128 i + 4 l + c at slot (4 i + c) 32 + l; eight gathered loads
+            // in flight a thread, 16 bytes each where the rows allow it
+            auto slot_of = [](int u) { return ((u >> 7) * 4 + (u & 3)) * 32 + ((u >> 2) & 31); };
+            constexpr int UB = 8;
+            if (RC > 1 && (r & 3) == 0) {
+                constexpr int Q = RC > 1 ? RC / 4 : 1;             // 16-byte pieces of a column
+                for (int e0 = threadIdx.x; e0 < 128 * ni * Q; e0 += UB * 32 * UP_WARPS) {
+                    float4 x[UB];
 #pragma unroll
-                for (int b = 0; b < UB; ++b) {
-                    const int e = e0 + b * 32 * UP_WARPS, z = z0 + e % RC;
-                    const int32_t row = e < 128 * ni * RC ? vrows[e / RC] : -1;
-                    x[b] = (row >= 0 && z < r) ? src[(int64_t)row * r + z] : 0.f;
+                    for (int b = 0; b < UB; ++b) {
+                        const int e = e0 + b * 32 * UP_WARPS, z = z0 + 4 * (e % Q);
+                        const int32_t row = e < 128 * ni * Q ? vrows[e / Q] : -1;
+                        x[b] = (row >= 0 && z < r) ? *reinterpret_cast<const float4 *>(src + (int64_t)row * r + z)
+                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+#pragma unroll
+                    for (int b = 0; b < UB; ++b) {
+                        const int e = e0 + b * 32 * UP_WARPS;
+                        if (e < 128 * ni * Q) *reinterpret_cast<float4 *>(vs + slot_of(e / Q) * STR + 4 * (e % Q)) = x[b];
+                    }
                 }
+            } else {
+                for (int e0 = threadIdx.x; e0 < 128 * ni * RC; e0 += UB * 32 * UP_WARPS) {
+                    float x[UB];
 #pragma unroll
-                for (int b = 0; b < UB; ++b) {
-                    const int e = e0 + b * 32 * UP_WARPS, u = e / RC;
-                    // column 128 i + 4 l + c at slot (4 i + c) 32 + l
-                    const int slot = ((u >> 7) * 4 + (u & 3)) * 32 + ((u >> 2) & 31);
-                    if (e < 128 * ni * RC) vs[slot * STR + e % RC] = x[b];
+                    for (int b = 0; b < UB; ++b) {
+                        const int e = e0 + b * 32 * UP_WARPS, z = z0 + e % RC;
+                        const int32_t row = e < 128 * ni * RC ? vrows[e / RC] : -1;
+                        x[b] = (row >= 0 && z < r) ? src[(int64_t)row * r + z] : 0.f;
+                    }
+#pragma unroll
+                    for (int b = 0; b < UB; ++b) {
+                        const int e = e0 + b * 32 * UP_WARPS;
+                        if (e < 128 * ni * RC) vs[slot_of(e / RC) * STR + e % RC] = x[b];
+                    }
                 }
             }
             __syncthreads();
@@ -195,9 +214,9 @@ __global__ void __launch_bounds__(32 * UP_WARPS) upward_kernel(
     }
 }
 
-template <int RC, int R>
-askit_status launch_upward_r(askit_tree t, WeightCtx &c, int depth, int r, cudaStream_t s) {
-    constexpr int STR = up_stride<RC>();
+template <int RC>
+askit_status launch_upward(askit_tree t, WeightCtx &c, int depth, int r, cudaStream_t s) {
+    constexpr int STR = up_stride<RC>(), R = RC <= 4 ? 8 : 4;
     // set once per kernel instance (thread-safe static initialisation)
     static const cudaError_t attr =
         cudaFuncSetAttribute(upward_kernel<RC, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -210,12 +229,6 @@ askit_status launch_upward_r(askit_tree t, WeightCtx &c, int depth, int r, cudaS
     return launch_pdl(upward_kernel<RC, R>, dim3((unsigned)a0, ny), dim3(32 * UP_WARPS), smem, s, a0, depth == t->L, r,
                       ku_max, t->nstart, t->d_s, t->d_ncol, t->d_pivoff, t->piv, t->d_p32off, t->P32, t->d_spool, c.Wt,
                       c.Ws);
-}
-
-template <int RC>
-askit_status launch_upward(askit_tree t, WeightCtx &c, int depth, int r, cudaStream_t s) {
-    if (depth < 6) return launch_upward_r<RC, 2>(t, c, depth, r, s);
-    return launch_upward_r<RC, RC <= 4 ? 8 : 4>(t, c, depth, r, s);
 }
 
 }  // namespace
