@@ -137,7 +137,6 @@ eval_tcw_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_const
     using S = WSmem<RC, NB>;
     constexpr int NSLOT = S::NSLOT, NCOL = S::NCOL, NSA = S::NSA, NSB = S::NSB, NRAW = S::NRAW;
     constexpr uint32_t FMT = P == ASKIT_PREC_BF16X3 ? 1u : 0u;
-    constexpr uint32_t IDESC = make_idesc(FMT, W_ROWS, NCOL);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
     const uint32_t sbase = smem_u32(sm);
@@ -563,6 +562,15 @@ eval_tcw_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_const
         int g = 0, li = 0;
         for (int ci = c_begin; ci < c_end && !*abort_flag; ++ci) {
             const int b = args.cta_blocks[ci];
+            // N covers the columns the epilogue reads (steps of 16 for r = 1, of 32
+            // above): sub-blocks of fewer than 128 rows, and single ones in the
+            // paired layout, cost what they have (10K x 1000, leaves of 157 rows:
+            // 900 -> 886 us a launch)
+            int f0 = 0;
+            const int nf = follower_rows(b, f0);
+            const int ncols = nf > 0 ? W_ROWS + nf : (args.items[args.block_off[b]].nrows & 0x7fffffff);
+            constexpr int STEP = RC == 1 ? 16 : 32;
+            const uint32_t idesc = make_idesc(FMT, W_ROWS, (ncols + STEP - 1) / STEP * STEP);
             for (int it = args.block_off[b]; it < args.block_off[b + 1]; ++it, ++li) {
                 const int a = li % NSLOT;
                 const uint32_t d_main = tmem + (uint32_t)(a * NCOL), d_cross = tmem + (uint32_t)(256 + a * NCOL);
@@ -579,9 +587,9 @@ eval_tcw_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_const
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {   // K = 16 per MMA: two K groups
                         const uint32_t oa = (uint32_t)(2 * k) * LA, ob = (uint32_t)(2 * k) * LB;
-                        tc_mma<P>(d_cross, nsw_desc(a_hi + oa, LA), nsw_desc(b_lo + ob, LB), IDESC, (kc | k) != 0);
-                        tc_mma<P>(d_cross, nsw_desc(a_lo + oa, LA), nsw_desc(b_hi + ob, LB), IDESC, 1);
-                        tc_mma<P>(d_main, nsw_desc(a_hi + oa, LA), nsw_desc(b_hi + ob, LB), IDESC, (kc | k) != 0);
+                        tc_mma<P>(d_cross, nsw_desc(a_hi + oa, LA), nsw_desc(b_lo + ob, LB), idesc, (kc | k) != 0);
+                        tc_mma<P>(d_cross, nsw_desc(a_lo + oa, LA), nsw_desc(b_hi + ob, LB), idesc, 1);
+                        tc_mma<P>(d_main, nsw_desc(a_hi + oa, LA), nsw_desc(b_hi + ob, LB), idesc, (kc | k) != 0);
                     }
                     tc_commit(BAR_A_FREE(sa));
                     tc_commit(BAR_B_FREE(sb));
