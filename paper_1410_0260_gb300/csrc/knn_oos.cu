@@ -16,7 +16,7 @@
 // distances are what the steps avoid: seeding in FP64 over the two leaves took 74 of the 110 ms that
 // 100,000 queries spent against 131,072 points (d = 64), the FP64 re-rank of every
 // candidate 8.8 ms, the shortlist with operands split on the chip 18.6 ms.
-// Now, the same 100,000 queries: home 0.20, seed 1.7, shortlist 4.8, re-rank 1.9 ms.
+// Now, the same 100,000 queries: home 0.20, seed 1.2, shortlist 4.3, re-rank 1.2 ms.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -165,53 +165,83 @@ __global__ void __launch_bounds__(128) ko_home_kernel(const float *Y, int d, int
     }
 }
 
-// A warp's FP32 squared distances of 32 tree rows to its query: four lanes a row,
-// each with every fourth 16-byte piece (NJ pieces a lane, d_pad = 16 NJ), eight
-// rows at a time; lane l ends with the distance of pos(8 (l & 3) + (l >> 2)).
+// A warp's FP32 squared distances of 32 tree rows to its query: eight lanes a row,
+// each with every eighth 16-byte piece (NJ pieces a lane, d_pad = 32 NJ), four rows
+// a load, so that a load takes whole 128-byte lines (with four lanes a row it took
+// halves of eight lines, twice the cycles in the load unit, which bound the seed at
+// 91 %: 1.74 ms for 100,000 queries, 1.17 with this and the gathered offers below); the lanes' sums meet in a transposing butterfly.  Lane l ends with the
+// distance of pos(4 (l & 7) + (l >> 3)).
 template <int NJ, class F>
 __device__ __forceinline__ float rows32(const float *Xt, const float4 (&y)[NJ], int lane, F pos) {
-    const int sub = lane & 3, r8 = lane >> 2;
-    float4 x[4][NJ];
+    const int sub = lane & 7, r4 = lane >> 3;
+    float4 x[8][NJ];
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        const float4 *row = reinterpret_cast<const float4 *>(Xt + (int64_t)pos(8 * g + r8) * (16 * NJ)) + sub;
+    for (int g = 0; g < 8; ++g) {
+        const float4 *row = reinterpret_cast<const float4 *>(Xt + (int64_t)pos(4 * g + r4) * (32 * NJ)) + sub;
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) x[g][j] = row[4 * j];
+        for (int j = 0; j < NJ; ++j) x[g][j] = row[8 * j];
     }
-    float v = 0.f;
+    float a[8];
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        float a = 0.f;
+    for (int g = 0; g < 8; ++g) {
+        a[g] = 0.f;
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
             const float t0 = y[j].x - x[g][j].x, t1 = y[j].y - x[g][j].y, t2 = y[j].z - x[g][j].z, t3 = y[j].w - x[g][j].w;
-            a = fmaf(t0, t0, a);
-            a = fmaf(t1, t1, a);
-            a = fmaf(t2, t2, a);
-            a = fmaf(t3, t3, a);
+            a[g] = fmaf(t0, t0, a[g]);
+            a[g] = fmaf(t1, t1, a[g]);
+            a[g] = fmaf(t2, t2, a[g]);
+            a[g] = fmaf(t3, t3, a[g]);
         }
-        a += __shfl_xor_sync(FULL, a, 1);
-        a += __shfl_xor_sync(FULL, a, 2);
-        if (sub == g) v = a;
     }
-    return v;
+    // lanes with bit m of sub set keep the upper half of the values left
+#pragma unroll
+    for (int m = 4; m >= 1; m >>= 1) {
+        const bool up = sub & m;
+#pragma unroll
+        for (int k = 0; k < m; ++k) {
+            const float keep = up ? a[k + m] : a[k], give = up ? a[k] : a[k + m];
+            a[k] = keep + __shfl_xor_sync(FULL, give, m);
+        }
+    }
+    return a[0];
 }
 
 template <int NJ>
 __device__ __forceinline__ void load_query(const float *y, int d, int lane, float4 (&q)[NJ]) {
-    const int sub = lane & 3;
+    const int sub = lane & 7;
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
-        const int k = 4 * (sub + 4 * j);
+        const int k = 4 * (sub + 8 * j);
         q[j] = make_float4(k < d ? y[k] : 0.f, k + 1 < d ? y[k + 1] : 0.f, k + 2 < d ? y[k + 2] : 0.f,
                            k + 3 < d ? y[k + 3] : 0.f);
     }
 }
 
+// Offers one value per lane to the list l by way of buf (64 floats of the warp,
+// `have` < 32 of them waiting): only values below the list's kappa-th are taken,
+// and 32 of them are sorted and merged at a time (22 shuffles, otherwise spent on
+// nearly every batch of 32 for the few values that still enter).
+__device__ __forceinline__ void gather_f32(float &l, float v, float *buf, int &have, int kappa, int lane) {
+    const bool useful = v < __shfl_sync(FULL, l, kappa - 1);
+    const unsigned m = __ballot_sync(FULL, useful);
+    if (!m) return;
+    if (useful) buf[have + __popc(m & ((1u << lane) - 1u))] = v;
+    have += __popc(m);
+    __syncwarp();
+    if (have < 32) return;
+    have -= 32;
+    const float first = buf[lane], rest = buf[32 + (lane < have ? lane : 0)];
+    __syncwarp();
+    if (lane < have) buf[lane] = rest;
+    __syncwarp();
+    warp_offer_f32(l, first, kappa, lane);
+}
+
 // Step 2, W warps per query: U.  The splits' candidates give the two home leaves;
 // their points' FP32 distances pass through the warps' best-32 lists, merged at
 // the end.  One warp a query where the queries fill the GPU, four below that (one
-// query is a chain of about 32 rounds of loads and merges: 51 us at 100 queries).
+// query is a chain of about 32 rounds of loads and merges: 51 us at 100 queries with one warp, 24 with four).
 template <int NJ, int W>
 __global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const float *Y, int d, int64_t T, const float *hd,
                                                       const int32_t *hi_, int nsplit, int64_t M, const int32_t *nstart,
@@ -220,7 +250,8 @@ __global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const flo
     const int warp = threadIdx.x >> 5;
     const int64_t qw = blockIdx.x * (int64_t)(8 / W) + warp / W;
     const int64_t q = qw < T ? qw : T - 1;                 // warps past T repeat the last query
-    __shared__ float lists[8][32];
+    __shared__ float lists[8][64];
+    int have = 0;
     float bd = 3.4e38f;
     int bi = 0;
     if (lane < 2 * nsplit) {
@@ -250,11 +281,13 @@ __global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const flo
         for (int b = 32 * (warp % W); b < np; b += 32 * W) {
             // rows past the leaf are other points or the zero rows past N
             const float v = rows32<NJ>(Xt, y, lane, [&](int i) { return p0 + b + i; });
-            const int i = b + 8 * (lane & 3) + (lane >> 2);
-            warp_offer_f32(l, i < np ? v : 3.4e38f, kappa, lane);
+            const int i = b + 4 * (lane & 7) + (lane >> 3);
+            gather_f32(l, i < np ? v : 3.4e38f, lists[warp], have, kappa, lane);
         }
     }
+    warp_offer_f32(l, lane < have ? lists[warp][lane] : 3.4e38f, kappa, lane);
     if (W > 1) {
+        __syncwarp();
         lists[warp][lane] = l;
         __syncthreads();
         if (warp % W) return;
@@ -264,14 +297,20 @@ __global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const flo
     if (lane == 0 && qw < T) U[q] = kth < 3.0e38f ? __fadd_ru(__fmul_ru(kth, 1.f + 2.f * sum_gam(d)), 1e-37f) : 3.4e38f;
 }
 
-// Step 4, a warp per query.
-template <int NJ>
-__global__ void __launch_bounds__(256) ko_rerank_kernel(const float *Xt, const float *Y, int d, int64_t T,
+// Step 4, a warp per query, W warps a block: eight where the queries fill the GPU,
+// one below that (a query is a chain of about 20 loads and 200 FP64 instructions, so
+// few queries are spread over as many SMs as they can reach: 54 -> 39 us at 100
+// queries).  100,000 queries 1.73 -> 1.22 ms with the lists ordered by integer
+// comparisons; the FP64 distances of 32 candidates a query alone take 0.98.
+template <int NJ, int W>
+__global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, const float *Y, int d, int64_t T,
                                                         const int32_t *perm, const int *cnt, const int32_t *cand,
                                                         int kappa, int32_t *ids, double *dist, int *n_ovf,
                                                         int32_t *ovf) {
-    __shared__ float sd[8][KO_CAP];
-    __shared__ float sy[8][TC_K];
+    __shared__ float sd[W][KO_CAP];
+    __shared__ float sy[W][TC_K];
+    __shared__ float sl[W][64];
+    int have_l = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (q >= T) return;                                    // warp-uniform
@@ -288,10 +327,11 @@ __global__ void __launch_bounds__(256) ko_rerank_kernel(const float *Xt, const f
     for (int b = 0; b < n; b += 32) {
         const int32_t mine = c[min(b + lane, n - 1)];
         const float v = rows32<NJ>(Xt, y, lane, [&](int i) { return __shfl_sync(FULL, mine, i); });
-        const int i = b + 8 * (lane & 3) + (lane >> 2);
+        const int i = b + 4 * (lane & 7) + (lane >> 3);
         if (i < n) sd[warp][i] = v;
-        warp_offer_f32(l, i < n ? v : 3.4e38f, kappa, lane);
+        gather_f32(l, i < n ? v : 3.4e38f, sl[warp], have_l, kappa, lane);
     }
+    warp_offer_f32(l, lane < have_l ? sl[warp][lane] : 3.4e38f, kappa, lane);
     __syncwarp();
     // a point among the kappa nearest has an FP32 distance within (1 + gam) /
     // (1 - gam) of the kappa-th smallest one
@@ -305,10 +345,12 @@ __global__ void __launch_bounds__(256) ko_rerank_kernel(const float *Xt, const f
         int ci = INT_MAX;
         if (lane < have) {
             ci = perm[held];
-            const float *x = Xt + (int64_t)held * (16 * NJ);
+            const float *x = Xt + (int64_t)held * (32 * NJ);
             double acc = 0.0;
+            float4 nx = *reinterpret_cast<const float4 *>(x);
             for (int k = 0; k < d; k += 4) {
-                const float4 xv = *reinterpret_cast<const float4 *>(x + k);
+                const float4 xv = nx;
+                nx = *reinterpret_cast<const float4 *>(x + min(k + 4, 32 * NJ - 4));
                 const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
@@ -674,8 +716,8 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
                                                                         hx);
     {
         const bool few = T < 16 * sms;
-        auto seed = d <= 32 ? (few ? ko_seed_kernel<2, 4> : ko_seed_kernel<2, 1>)
-                            : (few ? ko_seed_kernel<4, 4> : ko_seed_kernel<4, 1>);
+        auto seed = d <= 32 ? (few ? ko_seed_kernel<1, 4> : ko_seed_kernel<1, 1>)
+                            : (few ? ko_seed_kernel<2, 4> : ko_seed_kernel<2, 1>);
         seed<<<nblk(T, few ? 2 : 8), 256, 0, s>>>(t->Xt, Y, d, T, hd, hx, (int)nsplit, M, t->nstart, t->nsize, kappa, U);
     }
     QCHK(cudaGetLastError());
@@ -708,10 +750,13 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
         ko_shortlist_kernel<<<(unsigned)std::min<int64_t>(sms, a.units), KS::THREADS, smem, s>>>(mqh, mql, mth, mtl, a);
         QCHK(cudaGetLastError());
     }
-    if (t->d_pad == 32)
-        ko_rerank_kernel<2><<<nblk(T, 8), 256, 0, s>>>(t->Xt, Y, d, T, t->perm, cnt, cand, kappa, ids, dist, n_ovf, ovf);
-    else
-        ko_rerank_kernel<4><<<nblk(T, 8), 256, 0, s>>>(t->Xt, Y, d, T, t->perm, cnt, cand, kappa, ids, dist, n_ovf, ovf);
+    {
+        const bool few = T < 16 * sms;
+        auto rerank = t->d_pad == 32 ? (few ? ko_rerank_kernel<1, 1> : ko_rerank_kernel<1, 8>)
+                                     : (few ? ko_rerank_kernel<2, 1> : ko_rerank_kernel<2, 8>);
+        rerank<<<nblk(T, few ? 1 : 8), few ? 32 : 256, 0, s>>>(t->Xt, Y, d, T, t->perm, cnt, cand, kappa, ids, dist,
+                                                              n_ovf, ovf);
+    }
     QCHK(cudaGetLastError());
     QCHK(cudaMemcpyAsync(&h_ovf, n_ovf, sizeof(int), cudaMemcpyDeviceToHost, s));
     QCHK(cudaStreamSynchronize(s));

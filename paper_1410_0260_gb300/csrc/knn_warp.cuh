@@ -9,8 +9,13 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 
+// Order by (D, id).  Distances are sums of squares, never negative nor -0, so their
+// bits order them as integers (a NaN behind every number): two FP64 comparisons would
+// hold the warp's quarter of the SM for 128 cycles.
 __device__ __forceinline__ bool kv_less(double da, int ia, double db, int ib) {
-    return da < db || (da == db && ia < ib);
+    const unsigned long long a = (unsigned long long)__double_as_longlong(da);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(db);
+    return a < b || (a == b && ia < ib);
 }
 
 // ---------------------------------------------------------------------------
