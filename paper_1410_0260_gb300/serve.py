@@ -143,32 +143,42 @@ class Server:
 
     def _schedule_loop(self):
         while True:
-            with self.cv:
-                while not self.stop and (not self.queue or not any(not s.busy for s in self.slots)):
-                    self.cv.wait()
-                if self.stop and not self.queue:
-                    return
-                batch, need = self._take_batch()
-                if need > self.budget:
-                    # can never fit: reject the oldest request
-                    r = self.queue.popleft()
-                    r.error = f"request needs {need} device bytes, budget is {self.budget}"
-                    r.t_done = time.perf_counter()
-                    r.done.set()
-                    continue
-                while need > self.free_bytes and not self.stop:
-                    self.cv.wait()        # admission: wait for memory to free up
-                t = time.perf_counter()
-                taken = {id(r) for r in batch}
-                self.queue = deque(q for q in self.queue if id(q) not in taken)
-                for r in batch:
-                    r.t_start = t
-                slot = next(s for s in self.slots if not s.busy)
-                slot.busy = True
-                self.n_batches += 1
-                self.free_bytes -= need
-                self.peak_concurrency = max(self.peak_concurrency, sum(s.busy for s in self.slots))
-            threading.Thread(target=self._run, args=(slot, batch, need), daemon=True).start()
+            started = []
+            try:
+                with self.cv:
+                    while not self.stop and (not self.queue or not any(not s.busy for s in self.slots)):
+                        self.cv.wait()
+                    if self.stop and not self.queue:
+                        return
+                    # a batch for every free slot before any of them runs: a short batch
+                    # would otherwise be over before the next one is formed
+                    while self.queue and any(not s.busy for s in self.slots):
+                        batch, need = self._take_batch()
+                        if need > self.budget:
+                            # can never fit: reject the oldest request
+                            r = self.queue.popleft()
+                            r.error = f"request needs {need} device bytes, budget is {self.budget}"
+                            r.t_done = time.perf_counter()
+                            r.done.set()
+                            continue
+                        if need > self.free_bytes and started:
+                            break                 # the memory may be held by those not yet started
+                        while need > self.free_bytes and not self.stop:
+                            self.cv.wait()        # admission: wait for memory to free up
+                        t = time.perf_counter()
+                        taken = {id(r) for r in batch}
+                        self.queue = deque(q for q in self.queue if id(q) not in taken)
+                        for r in batch:
+                            r.t_start = t
+                        slot = next(s for s in self.slots if not s.busy)
+                        slot.busy = True
+                        self.n_batches += 1
+                        self.free_bytes -= need
+                        self.peak_concurrency = max(self.peak_concurrency, sum(s.busy for s in self.slots))
+                        started.append((slot, batch, need))
+            finally:                          # also where forming a further batch fails
+                for args in started:
+                    threading.Thread(target=self._run, args=args, daemon=True).start()
 
     def _run(self, slot: _Slot, batch: list[Request], need: int):
         try:
