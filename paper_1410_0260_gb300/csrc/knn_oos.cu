@@ -16,7 +16,7 @@
 // distances are what the steps avoid: seeding in FP64 over the two leaves took 74 of the 110 ms that
 // 100,000 queries spent against 131,072 points (d = 64), the FP64 re-rank of every
 // candidate 8.8 ms, the shortlist with operands split on the chip 18.6 ms.
-// Now, the same 100,000 queries: home 0.20, seed 1.2, shortlist 4.3, re-rank 1.2 ms.
+// Now, the same 100,000 queries: home 0.19, seed 0.96, shortlist 3.8, re-rank 1.2 ms.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -49,18 +49,20 @@ __host__ __device__ __forceinline__ float sum_gam(int d) { return (float)(d + 2)
 
 // Queries as FP16x3 operands of the shortlist: (y - xbar) sigma split hi + lo
 // [T_pad, 64], n = |y - xbar|^2; a query outside the FP16-safe range gets zero
-// rows and a full candidate count.  A warp per row; rows past T are zero.
-__global__ void ko_split_kernel(const float *Y, int d, int64_t T, int64_t T_pad, const float *xbar, float sigma,
+// rows and a full candidate count.  A warp per row; rows past T are zero.  Row i is
+// query order[i] (order null: query i), here and in the steps that follow.
+__global__ void ko_split_kernel(const float *Y, int d, const int32_t *order, int64_t T, int64_t T_pad, const float *xbar, float sigma,
                                 uint16_t *hi, uint16_t *lo, float *nq, int *cnt) {
     const int lane = threadIdx.x & 31;
     const int64_t row = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= T_pad) return;                              // warp-uniform
+    const int64_t src = order && row < T ? order[row] : row;
     float v[2], acc = 0.f;
     bool bad = false;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int k = lane + 32 * h;
-        const float x = (row < T && k < d) ? Y[row * d + k] - xbar[k] : 0.f;
+        const float x = (row < T && k < d) ? Y[src * d + k] - xbar[k] : 0.f;
         v[h] = x * sigma;
         acc = fmaf(x, x, acc);
         bad |= !(fabsf(v[h]) <= 30000.f);
@@ -165,6 +167,23 @@ __global__ void __launch_bounds__(128) ko_home_kernel(const float *Y, int d, int
     }
 }
 
+// The nearest home leaf of each query, the key of the queries' order, and 0 .. T - 1.
+__global__ void ko_key_kernel(const float *hd, const int32_t *hi_, int nsplit, int64_t T, uint32_t *key, int32_t *iota) {
+    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (q >= T) return;
+    float m = 3.4e38f;
+    int32_t leaf = 0;
+    for (int p = 0; p < nsplit; ++p) {
+        const int64_t o = ((int64_t)p * T + q) * 2;
+        if (hd[o] < m) {
+            m = hd[o];
+            leaf = hi_[o];
+        }
+    }
+    key[q] = (uint32_t)leaf;
+    iota[q] = (int32_t)q;
+}
+
 // A warp's FP32 squared distances of 32 tree rows to its query: eight lanes a row,
 // each with every eighth 16-byte piece (NJ pieces a lane, d_pad = 32 NJ), four rows
 // a load, so that a load takes whole 128-byte lines (with four lanes a row it took
@@ -243,19 +262,21 @@ __device__ __forceinline__ void gather_f32(float &l, float v, float *buf, int &h
 // the end.  One warp a query where the queries fill the GPU, four below that (one
 // query is a chain of about 32 rounds of loads and merges: 51 us at 100 queries with one warp, 24 with four).
 template <int NJ, int W>
-__global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const float *Y, int d, int64_t T, const float *hd,
+__global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const float *Y, int d, const int32_t *order,
+                                                      int64_t T, const float *hd,
                                                       const int32_t *hi_, int nsplit, int64_t M, const int32_t *nstart,
                                                       const int32_t *nsize, int kappa, float *U) {
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int64_t qw = blockIdx.x * (int64_t)(8 / W) + warp / W;
     const int64_t q = qw < T ? qw : T - 1;                 // warps past T repeat the last query
+    const int64_t src = order ? order[q] : q;
     __shared__ float lists[8][64];
     int have = 0;
     float bd = 3.4e38f;
     int bi = 0;
     if (lane < 2 * nsplit) {
-        const int64_t o = ((int64_t)(lane >> 1) * T + q) * 2 + (lane & 1);
+        const int64_t o = ((int64_t)(lane >> 1) * T + src) * 2 + (lane & 1);
         bd = hd[o];
         bi = hi_[o];
     }
@@ -273,7 +294,7 @@ __global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const flo
         if (lane == w) bd = 3.4e38f;
     }
     float4 y[NJ];
-    load_query<NJ>(Y + q * d, d, lane, y);
+    load_query<NJ>(Y + src * d, d, lane, y);
     float l = 3.4e38f;
     for (int h = 0; h < 2; ++h) {
         if (h == 1 && leaf[1] == leaf[0]) break;
@@ -303,10 +324,10 @@ __global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const flo
 // queries).  100,000 queries 1.73 -> 1.22 ms with the lists ordered by integer
 // comparisons; the FP64 distances of 32 candidates a query alone take 0.98.
 template <int NJ, int W>
-__global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, const float *Y, int d, int64_t T,
-                                                        const int32_t *perm, const int *cnt, const int32_t *cand,
-                                                        int kappa, int32_t *ids, double *dist, int *n_ovf,
-                                                        int32_t *ovf) {
+__global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, const float *Y, int d,
+                                                           const int32_t *order, int64_t T, const int32_t *perm,
+                                                           const int *cnt, const int32_t *cand, int kappa,
+                                                           int32_t *ids, double *dist, int *n_ovf, int32_t *ovf) {
     __shared__ float sd[W][KO_CAP];
     __shared__ float sy[W][TC_K];
     __shared__ float sl[W][64];
@@ -314,15 +335,16 @@ __global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, cons
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (q >= T) return;                                    // warp-uniform
+    const int64_t src = order ? order[q] : q;
     const int n = cnt[q];
     if (n > KO_CAP || n < kappa) {                         // (fewer cannot be: U bounds kappa points)
-        if (lane == 0) ovf[atomicAdd(n_ovf, 1)] = (int32_t)q;
+        if (lane == 0) ovf[atomicAdd(n_ovf, 1)] = (int32_t)src;
         return;
     }
     const int32_t *c = cand + q * KO_CAP;
     float4 y[NJ];
-    load_query<NJ>(Y + q * d, d, lane, y);
-    for (int k = lane; k < d; k += 32) sy[warp][k] = Y[q * d + k];
+    load_query<NJ>(Y + src * d, d, lane, y);
+    for (int k = lane; k < d; k += 32) sy[warp][k] = Y[src * d + k];
     float l = 3.4e38f;
     for (int b = 0; b < n; b += 32) {
         const int32_t mine = c[min(b + lane, n - 1)];
@@ -374,8 +396,8 @@ __global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, cons
     }
     if (have > 0) offer();
     if (lane < kappa) {
-        ids[q * kappa + lane] = li;
-        dist[q * kappa + lane] = ld;
+        ids[src * kappa + lane] = li;
+        dist[src * kappa + lane] = ld;
     }
 }
 
@@ -697,7 +719,7 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
     };
     const size_t o_hi = part((size_t)T_pad * TC_K * 2), o_lo = part((size_t)T_pad * TC_K * 2), o_nq = part((size_t)T_pad * 4),
                  o_hd = part((size_t)nsplit * T * 8), o_hx = part((size_t)nsplit * T * 8), o_u = part((size_t)T * 4),
-                 o_cnt = part((size_t)T * 4), o_ovf = part((size_t)(T + 1) * 4), o_cand = part((size_t)T * KO_CAP * 4);
+                 o_cnt = part((size_t)T * 4), o_ord = part((size_t)T * 4), o_ovf = part((size_t)(T + 1) * 4), o_cand = part((size_t)T * KO_CAP * 4);
     uint8_t *buf = nullptr;
     ASK_TRY(tmp.alloc(&buf, used));
     uint16_t *qh = reinterpret_cast<uint16_t *>(buf + o_hi), *ql = reinterpret_cast<uint16_t *>(buf + o_lo);
@@ -706,19 +728,41 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
     int32_t *hx = reinterpret_cast<int32_t *>(buf + o_hx), *cand = reinterpret_cast<int32_t *>(buf + o_cand);
     int *cnt = reinterpret_cast<int *>(buf + o_cnt), *n_ovf = reinterpret_cast<int *>(buf + o_ovf);
     int32_t *ovf = n_ovf + 1;
+    const int32_t *order = nullptr;
     int h_ovf = 0;
     askit_status rc = ASKIT_OK;
 #define QTRY(x) do { rc = (x); if (rc != ASKIT_OK) goto out; } while (0)
 #define QCHK(x) do { const cudaError_t e_ = (x); if (e_ != cudaSuccess) { askit_set_error("out-of-sample kNN: %s", cudaGetErrorString(e_)); rc = e_ == cudaErrorMemoryAllocation ? ASKIT_ERR_OOM : ASKIT_ERR_CUDA; goto out; } } while (0)
     QCHK(cudaMemsetAsync(n_ovf, 0, sizeof(int), s));
-    ko_split_kernel<<<nblk(T_pad, 8), 256, 0, s>>>(Y, d, T, T_pad, t->g_xbar, t->g_sigma, qh, ql, nq, cnt);
     ko_home_kernel<<<dim3((unsigned)qb, (unsigned)nsplit), 128, 0, s>>>(Y, d, T, t->cent, t->leaf_cbase, M, split_len, hd,
                                                                         hx);
+    // Queries in the order of their home leaves: the 128 of a tile then have their
+    // candidates in the same few source tiles, and nearly all other tile pairs skip
+    // the hit path; the seed's leaves are shared by neighboring warps.  Worth it from
+    // 2^31 (query, point) pairs: 100,000 x 131,072 saves 0.65 ms (shortlist 4.27 ->
+    // 3.80, seed 1.17 -> 0.99) for a sort of about 20 us, and the saving is in
+    // proportion to the pairs, the sort's few launches are not.
+    if (t->L > 0 && T >= 16 * sms && T * N >= (int64_t)1 << 31) {
+        // the sort's buffers lie in the candidate lists, which are written later
+        const size_t T4 = ((size_t)T * 4 + 255) / 256 * 256;
+        uint8_t *sb = buf + o_cand;
+        uint32_t *key = reinterpret_cast<uint32_t *>(sb), *key2 = reinterpret_cast<uint32_t *>(sb + T4);
+        int32_t *iota = reinterpret_cast<int32_t *>(sb + 2 * T4);
+        size_t tb = 0;
+        QTRY(sort_u32_i32(key, key2, iota, iota, T, t->L, nullptr, &tb, s));
+        if (3 * T4 + tb <= (size_t)T * KO_CAP * 4) {
+            int32_t *ord = reinterpret_cast<int32_t *>(buf + o_ord);
+            ko_key_kernel<<<nblk(T, 256), 256, 0, s>>>(hd, hx, (int)nsplit, T, key, iota);
+            QTRY(sort_u32_i32(key, key2, iota, ord, T, t->L, sb + 3 * T4, &tb, s));
+            order = ord;
+        }
+    }
+    ko_split_kernel<<<nblk(T_pad, 8), 256, 0, s>>>(Y, d, order, T, T_pad, t->g_xbar, t->g_sigma, qh, ql, nq, cnt);
     {
         const bool few = T < 16 * sms;
         auto seed = d <= 32 ? (few ? ko_seed_kernel<1, 4> : ko_seed_kernel<1, 1>)
                             : (few ? ko_seed_kernel<2, 4> : ko_seed_kernel<2, 1>);
-        seed<<<nblk(T, few ? 2 : 8), 256, 0, s>>>(t->Xt, Y, d, T, hd, hx, (int)nsplit, M, t->nstart, t->nsize, kappa, U);
+        seed<<<nblk(T, few ? 2 : 8), 256, 0, s>>>(t->Xt, Y, d, order, T, hd, hx, (int)nsplit, M, t->nstart, t->nsize, kappa, U);
     }
     QCHK(cudaGetLastError());
     {
@@ -754,7 +798,7 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
         const bool few = T < 16 * sms;
         auto rerank = t->d_pad == 32 ? (few ? ko_rerank_kernel<1, 1> : ko_rerank_kernel<1, 8>)
                                      : (few ? ko_rerank_kernel<2, 1> : ko_rerank_kernel<2, 8>);
-        rerank<<<nblk(T, few ? 1 : 8), few ? 32 : 256, 0, s>>>(t->Xt, Y, d, T, t->perm, cnt, cand, kappa, ids, dist,
+        rerank<<<nblk(T, few ? 1 : 8), few ? 32 : 256, 0, s>>>(t->Xt, Y, d, order, T, t->perm, cnt, cand, kappa, ids, dist,
                                                               n_ovf, ovf);
     }
     QCHK(cudaGetLastError());
