@@ -296,7 +296,9 @@ askit_status askit_graph_destroy(askit_graph g);
  * kernels; the plain FP32 kernel has one configuration.  Schedules, stages and tiled runs change no
  * result bit (every work item is computed the same way; partials are reduced
  * in a fixed order); paired items sum both sub-blocks' columns in one
- * accumulator, which changes the FP32 summation order only.  `reps` timed evaluations per candidate after one warm-up; at most
+ * accumulator, which changes the FP32 summation order only.  Until this or
+ * askit_set_launch is called, lists are dealt heaviest first and paired items
+ * are taken where most items have a partner.  `reps` timed evaluations per candidate after one warm-up; at most
  * `max_out` entries are written to `out`, the count to `n_out`.  Blocks.
  */
 typedef struct {

@@ -17,17 +17,18 @@
 // products (hi*hi + hi*lo + lo*hi) of BF16 parts with FP32
 // accumulation.
 //
-// One CTA per SM, warp-specialized, 416 threads:
-//   warps 0-7  loaders, two groups taking alternate items: thread t gathers
-//              the item's target row t, centers and splits it, and stores it
-//              in the 128-byte-swizzled K-major layout the tensor core reads
+// One CTA per SM, warp-specialized, 448 threads:
+//   warps 0-7  loaders, two groups taking alternate items: thread t centers
+//              and splits the item's gathered target row t and stores it in
+//              the 128-byte-swizzled K-major layout the tensor core reads
 //              (stage = group); it also forms the row term of target t and
 //              the column data of source row t;
 //   warps 8-11 epilogue: tcgen05.ld of their 32 TMEM lanes (one row each),
 //              exponent on MUFU.EX2, reduction against the weights;
 //   warp 12    one thread issues the TMA loads of the sub-block (centered,
 //              pre-split rows) and the tcgen05.mma instructions, and commits
-//              them to mbarriers.
+//              them to mbarriers;
+//   warp 13    gathers the items' target rows (TMA tile::gather4).
 // Two TMEM accumulators (2 x 128 columns) let the MMAs of item i+1 run
 // while the epilogue drains item i.  Every mbarrier wait is bounded: on
 // timeout the kernel records ASK_DEV_TIMEOUT, all roles leave their loops,
