@@ -79,6 +79,13 @@ constexpr int ASK_TILE_M = 128;
 constexpr int ASK_BLK_N = 128;
 // Items of one run of a sub-block's items with wide rows (d > TC_K).
 constexpr int ASK_SEG_ITEMS = 8;
+// Sub-blocks past this value of rho = sc_max max |y - c_B|^2 (sc = c log2(e) / h^2)
+// are too wide for the 3xTF32 kernel's common center c_B: the exponent's rounding
+// error is about 1.6e-7 rho where a target meets near points far from c_B (a node
+// that median splits left with parts of two clusters, or with an outlier), 2e-5 at
+// this line, a fifth of the split products' tolerance.  Points without gaps stay
+// below it: at most 106 over the leaves and skeletons of 64K x 64 manifold points.
+constexpr float ASK_WIDE_RHO = 128.f;
 // Columns of the tensor-core operand arrays (d <= TC_K).
 constexpr int TC_K = 64;
 // Default and largest entries of one in-sample work-list batch (entry
@@ -138,7 +145,8 @@ struct __align__(16) EvalItem {
     int32_t e0;      // first entry
     int32_t cnt;     // targets (entries) of this item
     int32_t cidx;    // sub-block index (its center in the centered operand arrays)
-    int32_t pad_[3];
+    int32_t wide;    // 1: the 3xTF32 kernel centers this item on its targets (sb_wide)
+    int32_t pad_[2];
 };
 
 // Target rows of one evaluation in the global-centered FP16x3 form: hi / lo
@@ -312,6 +320,10 @@ struct askit_tree_s {
     void *tf32 = nullptr;          // the same for the 3xTF32 kernel
     int64_t *sb_row0 = nullptr;    // [n_sub] first row of each sub-block (Xt rows, then Xs rows)
     int32_t *sb_nr = nullptr;      // [n_sub] rows of each sub-block
+    // [n_sub] (d <= TC_K) 1 where sc_max max |y - c_B|^2 over the sub-block's rows
+    // exceeds ASK_WIDE_RHO: too wide for 3xTF32 with both sides centered on c_B
+    int32_t *sb_wide = nullptr;
+    bool any_wide = false;         // one at least
     int64_t n_leaf_sub = 0;        // sub-blocks of leaves (the rest are skeleton sub-blocks)
     std::vector<int64_t> h_sub_pos; // [n_sub] tree position of each sub-block's node (schedule order)
     std::vector<int64_t> h_sub_node; // [n_sub] heap index of each sub-block's node

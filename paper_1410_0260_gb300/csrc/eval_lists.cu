@@ -342,7 +342,8 @@ __global__ void sub_start_kernel(const uint32_t *keys, int64_t n, int64_t n_sub,
 
 // Items of block b = sub-block blk_sub[b]: its entries in runs of ASK_TILE_M.
 __global__ void build_items_kernel(const int32_t *blk_sub, const int32_t *block_off, const int32_t *start,
-                                   const int64_t *sb_row0, const int32_t *sb_nr, int64_t n_leaf_sub, EvalItem *items) {
+                                   const int64_t *sb_row0, const int32_t *sb_nr, const int32_t *sb_wide, int64_t n_leaf_sub,
+                                   EvalItem *items) {
     const int b = blockIdx.x;
     const int32_t c = blk_sub[b], i0 = block_off[b], n = block_off[b + 1] - i0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
@@ -352,7 +353,8 @@ __global__ void build_items_kernel(const int32_t *blk_sub, const int32_t *block_
         x.e0 = start[c] + k * ASK_TILE_M;
         x.cnt = min(ASK_TILE_M, start[c + 1] - x.e0);
         x.cidx = c;
-        x.pad_[0] = x.pad_[1] = x.pad_[2] = 0;
+        x.wide = sb_wide ? sb_wide[c] : 0;
+        x.pad_[0] = x.pad_[1] = 0;
         items[i0 + k] = x;
     }
 }
@@ -503,6 +505,30 @@ __global__ void tc_prep_kernel(const float *X, int d_pad, int kw, bool kgplanes,
     }
 }
 
+// Sub-blocks too wide for 3xTF32 on their common center (ASK_WIDE_RHO); a norm
+// that is no number or infinite counts as wide.
+__global__ void wide_kernel(const int64_t *sb_row0, const int32_t *sb_nr, int64_t n_leaf_sub, const float *sc_t,
+                            const float *sc_s, const float *nrm_t, const float *nrm_s, int32_t *wide) {
+    const int64_t b = blockIdx.x;
+    const int lane = threadIdx.x;
+    const bool far = b >= n_leaf_sub;
+    float sc = 0.f, n = 0.f;
+    bool bad = false;
+    for (int q = lane; q < sb_nr[b]; q += 32) {
+        const int64_t row = sb_row0[b] + q;
+        const float v = (far ? nrm_s : nrm_t)[row];
+        bad |= !(v <= 3.4e38f);
+        n = fmaxf(n, v);
+        sc = fmaxf(sc, (far ? sc_s : sc_t)[row]);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        sc = fmaxf(sc, __shfl_xor_sync(0xffffffffu, sc, o));
+        n = fmaxf(n, __shfl_xor_sync(0xffffffffu, n, o));
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) wide[b] = bad || !(sc * n <= ASK_WIDE_RHO);
+}
+
 // Largest |x_k| over the data (bounds every centered coordinate by twice it).
 __global__ void extent_kernel(const float *X, int64_t N, int d, float *ext) {
     int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -627,10 +653,19 @@ askit_status build_tc_operands(askit_tree t, cudaStream_t s) {
             t->Xs, t->d_pad, kw, wide, d_r0 + n_leaf_sub, d_nr + n_leaf_sub, d_nd0 + n_leaf_sub, d_ndn + n_leaf_sub,
             t->srows, t->f16_scale, t->cent + n_leaf_sub * kw, t->Xs_hi, t->Xs_lo, t->Xs_bhi, t->Xs_blo, t->Xs_hhi,
             t->Xs_hlo, t->nrmc_s);
+    if (!wide && t->n_sub > 0) {
+        ASK_TRY(t->arena.alloc(&t->sb_wide, t->n_sub));
+        wide_kernel<<<(unsigned)t->n_sub, 32, 0, s>>>(t->sb_row0, t->sb_nr, n_leaf_sub, t->sc_t, t->sc_s, t->nrmc_t,
+                                                      t->nrmc_s, t->sb_wide);
+    }
     ASK_LAUNCH();
     cudaFreeAsync(d_nd0, s);
     cudaFreeAsync(d_ndn, s);
+    std::vector<int32_t> h_wide(t->sb_wide ? t->n_sub : 0);
+    if (t->sb_wide)
+        ASK_CUDA(cudaMemcpyAsync(h_wide.data(), t->sb_wide, sizeof(int32_t) * t->n_sub, cudaMemcpyDeviceToHost, s));
     ASK_CUDA(cudaStreamSynchronize(s));
+    t->any_wide = std::find(h_wide.begin(), h_wide.end(), 1) != h_wide.end();
     if (!wide) ASK_TRY(build_g16_operands(t, s));
     return ASKIT_OK;
 }
@@ -970,7 +1005,7 @@ askit_status build_work_lists(askit_tree t, const int32_t *sets, int stride, con
         w.use = t->tune_sched & 1;
         if (nb > 0)
             build_items_kernel<<<(unsigned)nb, 128, 0, s>>>(w.plan, w.block_off, start, t->sb_row0, t->sb_nr,
-                                                            t->n_leaf_sub, w.items);
+                                                            t->sb_wide, t->n_leaf_sub, w.items);
         WCHK(cudaGetLastError());
         w.pairs_alg = (int64_t)h_tot[2];
         w.pairs_cmp = nit * (int64_t)ASK_TILE_M * ASK_BLK_N;

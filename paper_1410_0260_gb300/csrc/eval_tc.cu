@@ -515,7 +515,7 @@ askit_status eval_tc(askit_tree t, const WeightCtx &c, int precision, const floa
     // grade (eval_g16.cu)
     if (precision == ASKIT_PREC_FP16X3 && qs && use_g16(t)) return eval_g16(t, c, *qs, w, partial, s);
     // FP16x3 and 3xTF32 center both sides on the sub-block mean (eval_tc16.cu,
-    // eval_tf32.cu); BF16x3 keeps the per-item target centering below: its 8-bit
+    // eval_tf32.cu, there except in sub-blocks that are too wide for it); BF16x3 keeps the per-item target centering below: its 8-bit
     // significands leave a residual of about 2^-17 of |a| |b| per product, so the
     // smaller |a| of the per-item center is what keeps it within the split-path
     // tolerance

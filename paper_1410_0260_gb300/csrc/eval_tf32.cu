@@ -8,6 +8,17 @@
 // with a.b from three TF32 split products, the small cross terms first, FP32
 // accumulation.
 //
+// A sub-block whose rows reach far from c_B (EvalItem::wide) centers each target row on
+// the nearest of four of the item's targets instead (the first, the last and two
+// between), with the exact rewriting
+//     a = x - c,  r^2 = |a|^2 + 2 a.(c - c_B) + |y - c|^2 - 2 a.b
+// Around c_B the norms of near points in a far cluster cancel; these terms stay at the
+// scale of |a|, which is small also where an item's targets (in tree order) lie in
+// several clusters.  Three clusters in 4 dimensions, centers in a box of 100 h,
+// relative error: 1.6e-4 on c_B, 8.9e-5 on the first target alone, 2.0e-6 on the nearest
+// of four.  The column terms -sc |y - c|^2 belong to the item then: the loader thread of
+// target row t forms those of source row t, one a center, from the FP32 rows.
+//
 // The targets' split rows are the MMA's A operand in TMEM: a loader thread owns a
 // row, so it centers, splits and stores it (tcgen05.st) without a layout in shared
 // memory, and the tensor core reads only B there (an item's 24 MMAs of 128 x 128 x 8
@@ -31,6 +42,7 @@
 #include <cuda.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "askit_impl.cuh"
 #include "tc_ptx.cuh"
@@ -42,6 +54,7 @@ using namespace tcx;
 constexpr int F_REGION = 128 * 128;            // 128 rows x 32 TF32, 128-byte swizzle
 constexpr int F_NRAW = 3;
 constexpr int F_THREADS = 640;
+constexpr int F_NCEN = 4;                      // centers of a wide item's targets
 
 template <int RC>
 struct SF {
@@ -52,7 +65,9 @@ struct SF {
     static constexpr int BLK_COLV = 256, BLK_COLW = BLK_COLV + 128 * 16;
     static constexpr int BLKSLOT = BLK_COLW + (RC > 1 ? 128 * RC * 4 : 0);
     static constexpr int ANORM = BLK + 2 * BLKSLOT;            // float [2][128]
-    static constexpr int BAR = ANORM + 2 * 128 * 4;            // 24 mbarriers
+    static constexpr int BITEM = ANORM + 2 * 128 * 4;          // float [2][F_NCEN][128]: B of a wide item's columns by center
+    static constexpr int PICK = BITEM + 2 * F_NCEN * 128 * 4;  // int [2][128]: center of a wide item's row
+    static constexpr int BAR = PICK + 2 * 128 * 4;             // 24 mbarriers
     static constexpr int MISC = BAR + 24 * 8;
     static constexpr int BYTES = MISC + 16;
 };
@@ -62,6 +77,8 @@ struct FArgs {
     const int32_t *block_off, *cta_off, *cta_blocks;
     const int32_t *tgt;
     const float *q;                // target rows [*, d_pad]
+    const float *Xt, *Xs;          // source rows [*, d_pad] and their c log2(e) / h^2 (wide items)
+    const float *sc_t, *sc_s;
     int d_pad;
     const float *cent;             // [n_sub, TC_K]
     const float4 *colv;            // [n_sub, 128] {A_j, A_j+1, B_j, B_j+1}, {C_j, C_j+1, w_j, w_j+1}
@@ -84,8 +101,9 @@ __device__ __forceinline__ void mma_tf32_ts(uint32_t d, uint32_t a, uint64_t b, 
 
 // UNI (r = 1): one bandwidth for all sources; the column data is {B_j, B_j+1, w_j,
 // w_j+1} a pair, and A and C are scalars, which halves the epilogue's shared-memory
-// reads (two reads a pair: 484 us at 64K x 64).
-template <int RC, bool UNI>
+// reads (two reads a pair: 484 us at 64K x 64).  WIDE: the tree has wide sub-blocks
+// (64K x 64 without any: 429 us, 444 with the test in every item).
+template <int RC, bool UNI, bool WIDE>
 __global__ void __launch_bounds__(F_THREADS, 1)
 eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_constant__ CUtensorMap map_t_lo,
                  const __grid_constant__ CUtensorMap map_s_hi, const __grid_constant__ CUtensorMap map_s_lo,
@@ -96,14 +114,15 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t sbase = smem_u32(sm), bar0 = sbase + S::BAR;
-    float *a_norm = reinterpret_cast<float *>(sm + S::ANORM);
+    float *a_norm = reinterpret_cast<float *>(sm + S::ANORM), *b_item = reinterpret_cast<float *>(sm + S::BITEM);
+    int *pick = reinterpret_cast<int *>(sm + S::PICK);
     auto BAR_R_FULL = [&](int s) { return bar0 + 8 * s; };            // raw rows of stage s landed (64)
     auto BAR_R_EMPTY = [&](int s) { return bar0 + 8 * (3 + s); };     // loaders done with stage s (128)
     auto BAR_A_FULL = [&](int g) { return bar0 + 8 * (6 + g); };      // split rows of side g in TMEM (128)
     auto BAR_A_EMPTY = [&](int g) { return bar0 + 8 * (8 + g); };     // MMAs read them (commit)
     auto BAR_T_FULL = [&](int g) { return bar0 + 8 * (10 + g); };     // accumulator g complete (commit)
     auto BAR_T_EMPTY = [&](int g) { return bar0 + 8 * (12 + g); };    // drained (128)
-    auto BAR_N_EMPTY = [&](int g) { return bar0 + 8 * (14 + g); };    // |a|^2 of side g read (128)
+    auto BAR_N_EMPTY = [&](int g) { return bar0 + 8 * (14 + g); };    // row terms of side g, a wide item's B, read (128)
     auto BAR_BLK_FULL = [&](int s) { return bar0 + 8 * (16 + s); };   // c_B, column data of slot s landed
     auto BAR_BLK_EMPTY = [&](int s) { return bar0 + 8 * (18 + s); };  // epilogue done with slot s (256)
     const uint32_t BAR_B_FULL = bar0 + 8 * 20, BAR_B_EMPTY = bar0 + 8 * 21;
@@ -154,7 +173,8 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
             bool need_blk = true;
             for (int it = i0; it < i1; ++it, ++li) {
                 if ((li & 1) != g) continue;
-                const int cnt = args.items[it].cnt;
+                const EvalItem item = args.items[it];
+                const int cnt = item.cnt;
                 const int sr = li % F_NRAW, par = ((li >> 1) & 1) ^ 1;
                 if (need_blk) {
                     if (!mbar_wait(BAR_BLK_FULL(lb & 1), (lb >> 1) & 1, abort_flag, args.status, args.spin)) goto loader_done;
@@ -166,15 +186,61 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                 tc_fence_after();
                 const uint8_t *x = sm + S::RAW + sr * S::RAWSTAGE + row * rst;
                 const float4 *cb = reinterpret_cast<const float4 *>(sm + S::BLK + (lb & 1) * S::BLKSLOT);
-                const bool mine = row < cnt;
+                const bool mine = row < cnt, wide = WIDE && item.wide != 0;   // (wide: warp-uniform)
                 float2 nn = make_float2(0.f, 0.f);
                 const float2 m1 = make_float2(-1.f, -1.f);
+                const float4 *ctr = cb;
+                if (wide) {
+                    const float4 *ct[F_NCEN];
+#pragma unroll
+                    for (int k = 0; k < F_NCEN; ++k)
+                        ct[k] = reinterpret_cast<const float4 *>(sm + S::RAW + sr * S::RAWSTAGE +
+                                                                 k * (cnt - 1) / (F_NCEN - 1) * rst);
+                    const bool far = item.nrows < 0;
+                    const bool src = row < (item.nrows & 0x7fffffff);
+                    const int64_t srow = (int64_t)item.row0 + (src ? row : 0);
+                    const float4 *yr = reinterpret_cast<const float4 *>((far ? args.Xs : args.Xt) + srow * args.d_pad);
+                    const float msc = -(far ? args.sc_s : args.sc_t)[srow];
+                    float2 dx[F_NCEN], dy[F_NCEN];
+#pragma unroll
+                    for (int k = 0; k < F_NCEN; ++k) dx[k] = dy[k] = make_float2(0.f, 0.f);
+                    for (int j = 0; j < args.d_pad / 4; ++j) {
+                        const float4 xv = *reinterpret_cast<const float4 *>(x + 16 * j), yv = yr[j];
+#pragma unroll
+                        for (int k = 0; k < F_NCEN; ++k) {
+                            const float4 tv = ct[k][j];
+                            const float2 t0 = make_float2(tv.x, tv.y), t1 = make_float2(tv.z, tv.w);
+                            float2 u = __ffma2_rn(t0, m1, make_float2(xv.x, xv.y));
+                            dx[k] = __ffma2_rn(u, u, dx[k]);
+                            u = __ffma2_rn(t1, m1, make_float2(xv.z, xv.w));
+                            dx[k] = __ffma2_rn(u, u, dx[k]);
+                            u = __ffma2_rn(t0, m1, make_float2(yv.x, yv.y));
+                            dy[k] = __ffma2_rn(u, u, dy[k]);
+                            u = __ffma2_rn(t1, m1, make_float2(yv.z, yv.w));
+                            dy[k] = __ffma2_rn(u, u, dy[k]);
+                        }
+                    }
+                    int pk = 0;
+                    float near = dx[0].x + dx[0].y;
+                    ctr = ct[0];
+#pragma unroll
+                    for (int k = 0; k < F_NCEN; ++k) {
+                        const float dk = dx[k].x + dx[k].y;
+                        if (dk < near) {
+                            near = dk;
+                            pk = k;
+                            ctr = ct[k];
+                        }
+                        b_item[(F_NCEN * g + k) * 128 + row] = src ? msc * (dy[k].x + dy[k].y) : UNI ? -INFINITY : 0.f;
+                    }
+                    pick[g * 128 + row] = pk;
+                }
                 for (int c = 0; c < args.d_pad / 16; ++c) {        // 16 columns at a time
                     uint32_t hi[16], lo[16];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const float4 xv = *reinterpret_cast<const float4 *>(x + 64 * c + 16 * j);
-                        const float4 mv = cb[4 * c + j];
+                        const float4 mv = ctr[4 * c + j];
                         float2 a[2] = {__ffma2_rn(make_float2(mv.x, mv.y), m1, make_float2(xv.x, xv.y)),
                                        __ffma2_rn(make_float2(mv.z, mv.w), m1, make_float2(xv.z, xv.w))};
 #pragma unroll
@@ -192,7 +258,20 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                     tmem_st16(ta + 16 * c, hi);
                     tmem_st16(ta + 64 + 16 * c, lo);
                 }
-                a_norm[g * 128 + row] = nn.x + nn.y;
+                float rowterm = nn.x + nn.y;
+                if (wide) {
+                    float2 dd = make_float2(0.f, 0.f);             // a.(c - c_B)
+                    for (int j = 0; j < args.d_pad / 4; ++j) {
+                        const float4 xv = *reinterpret_cast<const float4 *>(x + 16 * j), tv = ctr[j], bv = cb[j];
+                        const float2 t0 = make_float2(tv.x, tv.y), t1 = make_float2(tv.z, tv.w);
+                        dd = __ffma2_rn(__ffma2_rn(t0, m1, make_float2(xv.x, xv.y)),
+                                        __ffma2_rn(make_float2(bv.x, bv.y), m1, t0), dd);
+                        dd = __ffma2_rn(__ffma2_rn(t1, m1, make_float2(xv.z, xv.w)),
+                                        __ffma2_rn(make_float2(bv.z, bv.w), m1, t1), dd);
+                    }
+                    rowterm = mine ? fmaf(2.f, dd.x + dd.y, rowterm) : 0.f;
+                }
+                a_norm[g * 128 + row] = rowterm;
                 mbar_arrive(BAR_R_EMPTY(sr));
                 tmem_st_wait();
                 tc_fence_before();
@@ -218,7 +297,9 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                 if (!mbar_wait(BAR_T_FULL(g), (li >> 1) & 1, abort_flag, args.status, args.spin)) goto epi_done;
                 tc_fence_after();
                 const float pt = a_norm[g * 128 + row];
-                mbar_arrive(BAR_N_EMPTY(g));
+                const bool wide = WIDE && item.wide != 0;
+                const float2 *bi = reinterpret_cast<const float2 *>(b_item + (F_NCEN * g + (wide ? pick[g * 128 + row] : 0)) * 128);
+                if (!wide) mbar_arrive(BAR_N_EMPTY(g));
                 float acc[RC];
 #pragma unroll
                 for (int z = 0; z < RC; ++z) acc[z] = 0.f;
@@ -230,11 +311,16 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                     const float2 pt2 = make_float2(pt, pt);
                     // arg = g A + (C p + B) = -sc (p + q - 2 g); columns past the rows
                     // carry A = B = C = w = 0
-                    auto cols = [&](int c, const uint32_t (&gr)[32]) {
+                    auto cols = [&](int c, const uint32_t (&gr)[32], auto is_wide) {
 #pragma unroll
                         for (int jj = 0; jj < 32; jj += 2) {
                             if constexpr (UNI) {
-                                const float4 bw = cv4[(c * 32 + jj) >> 1];
+                                float4 bw = cv4[(c * 32 + jj) >> 1];
+                                if constexpr (decltype(is_wide)::value) {
+                                    const float2 b2 = bi[(c * 32 + jj) >> 1];
+                                    bw.x = b2.x;
+                                    bw.y = b2.y;
+                                }
                                 const float2 in = __ffma2_rn(make_float2(args.uni_c, args.uni_c), pt2, make_float2(bw.x, bw.y));
                                 const float2 ag = __ffma2_rn(make_float2(__uint_as_float(gr[jj]), __uint_as_float(gr[jj + 1])),
                                                              make_float2(args.uni_a, args.uni_a), in);
@@ -242,7 +328,13 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                                 acc2[(jj >> 1) & 1] = __ffma2_rn(kk, make_float2(bw.z, bw.w), acc2[(jj >> 1) & 1]);
                                 continue;
                             }
-                            const float4 ab = cv4[c * 32 + jj], cw = cv4[c * 32 + jj + 1];
+                            float4 ab = cv4[c * 32 + jj];
+                            const float4 cw = cv4[c * 32 + jj + 1];
+                            if constexpr (decltype(is_wide)::value) {
+                                const float2 b2 = bi[(c * 32 + jj) >> 1];
+                                ab.z = b2.x;
+                                ab.w = b2.y;
+                            }
                             const float2 inner = __ffma2_rn(make_float2(cw.x, cw.y), pt2, make_float2(ab.z, ab.w));
                             const float2 arg = __ffma2_rn(make_float2(__uint_as_float(gr[jj]), __uint_as_float(gr[jj + 1])),
                                                           make_float2(ab.x, ab.y), inner);
@@ -270,7 +362,13 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                         uint32_t ga[32];
                         tmem_ld32_async(tbase + (uint32_t)(c * 32), ga);
                         tmem_wait_pin(ga);
-                        cols(c, ga);
+                        if constexpr (WIDE) {
+                            if (wide) {
+                                cols(c, ga, std::true_type());
+                                continue;
+                            }
+                        }
+                        cols(c, ga, std::false_type());
                     }
                     if constexpr (RC == 1) {
                         acc[0] = (acc2[0].x + acc2[0].y) + (acc2[1].x + acc2[1].y);
@@ -283,6 +381,7 @@ eval_tf32_kernel(const __grid_constant__ CUtensorMap map_t_hi, const __grid_cons
                     }
                 }
                 tc_fence_before();
+                if (wide) mbar_arrive(BAR_N_EMPTY(g));
                 mbar_arrive(BAR_T_EMPTY(g));
                 if (row < item.cnt) {
                     float *p = args.partial + (int64_t)(item.e0 + row) * args.r;
@@ -459,21 +558,26 @@ askit_status f_state(askit_tree t, FState **out) {
     return ASKIT_OK;
 }
 
-template <int RC, bool UNI>
+template <int RC, bool UNI, bool WIDE>
 askit_status run_tf32(askit_tree t, const WeightCtx &c, FState *st, FArgs a, int grid, cudaStream_t s) {
     using S = SF<RC>;
     constexpr size_t smem = S::BYTES + 1024;
     static_assert(smem <= 232448, "shared-memory plan exceeds 227 KB");
     static const cudaError_t attr =
-        cudaFuncSetAttribute(eval_tf32_kernel<RC, UNI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(eval_tf32_kernel<RC, UNI, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     ASK_CUDA(attr);
     ASK_TRY(block_columns(t, c, RC, UNI, 1.f, s));
     a.colv = c.colv;
     a.colw = c.colw;
     ASK_TRY(ktimer_mark(t, s, false));
-    ASK_TRY(launch_pdl(eval_tf32_kernel<RC, UNI>, dim3((unsigned)grid), dim3(F_THREADS), smem, s, st->map[0], st->map[1],
+    ASK_TRY(launch_pdl(eval_tf32_kernel<RC, UNI, WIDE>, dim3((unsigned)grid), dim3(F_THREADS), smem, s, st->map[0], st->map[1],
                        st->map[2], st->map[3], a));
     return ktimer_mark(t, s, true);
+}
+
+template <int RC, bool UNI>
+askit_status run_tf32(askit_tree t, const WeightCtx &c, FState *st, const FArgs &a, int grid, cudaStream_t s) {
+    return t->any_wide ? run_tf32<RC, UNI, true>(t, c, st, a, grid, s) : run_tf32<RC, UNI, false>(t, c, st, a, grid, s);
 }
 
 }  // namespace
@@ -496,6 +600,10 @@ askit_status eval_tf32(askit_tree t, const WeightCtx &c, const float *Xq, int64_
     a.tgt = w.tgt;
     a.q = Xq;
     a.d_pad = t->d_pad;
+    a.Xt = t->Xt;
+    a.Xs = t->Xs;
+    a.sc_t = t->sc_t;
+    a.sc_s = t->sc_s;
     a.cent = t->cent;
     a.colv = nullptr;
     a.colw = nullptr;
