@@ -238,7 +238,10 @@ __global__ void __launch_bounds__(256) knn_leaf_kernel(const float *X, int d, co
                 const float v = b + lane < nc && b + lane != me ? row[b + lane] : 3.4e38f;
                 warp_offer_f32(l, v <= lim ? v : 3.4e38f, kappa, lane);
             }
-            lim = fminf(lim, __shfl_sync(FULL, l, kappa - 1) * (1.f + 3.f * gam) + 1e-37f);
+            // only a real distance bounds: fewer than kappa below FP32's range leave the
+            // limit as it is, and distances past that range (+inf here) stay in
+            const float lk = __shfl_sync(FULL, l, kappa - 1);
+            if (lk < 3.0e38f) lim = fminf(lim, lk * (1.f + 3.f * gam) + 1e-37f);
             int have = 0;
             int32_t held = 0;
             auto offer = [&]() {
@@ -277,7 +280,7 @@ __global__ void __launch_bounds__(256) knn_leaf_kernel(const float *X, int d, co
                 have = 0;
             };
             for (int b = 0; b < nc; b += 32) {
-                // not "above the limit", so a distance that is no number stays in
+                // not "above the limit", so a distance that is no number, or infinite, stays in
                 const bool pass = b + lane < nc && b + lane != me && !(row[b + lane] > lim);
                 const unsigned m = __ballot_sync(FULL, pass);
                 if (!m) continue;
