@@ -382,7 +382,8 @@ __global__ void __launch_bounds__(256) knn_tiled_kernel(const float *X, int64_t 
                 const bool valid = j < c1 && (self ? j != self[q] : (Y || j != q));
                 const float d32 = dt[qq][rr * 32 + lane];
                 const double kth = __shfl_sync(FULL, ld[u], kappa - 1);
-                const bool need = valid && (double)d32 * (1.0 - (double)gam) <= kth;
+                // (a distance past FP32's range, or no number, is left to FP64)
+                const bool need = valid && (!(d32 < 3.0e38f) || (double)d32 * (1.0 - (double)gam) <= kth);
                 if (!__ballot_sync(FULL, need)) continue;
                 double cd = DBL_MAX;
                 int ci = INT_MAX;

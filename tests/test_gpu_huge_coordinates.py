@@ -40,3 +40,22 @@ def _lists(X, **kw):
 def test_random_projection_lists_past_the_fp32_range(N, d, leaf, kappa, kind):
     X = _points(N, d, kind, np.random.default_rng(N + d))
     _lists(X, leaf_size=leaf, kappa=kappa, knn_mode=1, rp_iters=3, s_max=8, id_tol=0.0, h=1.0, seed=4).close()
+
+
+@pytest.mark.parametrize("N,d,kappa,kind", [(300, 5, 8, "outliers"), (700, 8, 32, "marker"), (1300, 70, 16, "all")])
+def test_exhaustive_lists_past_the_fp32_range(N, d, kappa, kind):
+    import oracle
+    rng = np.random.default_rng(N + d)
+    X = _points(N, d, kind, rng)
+    g = _lists(X, leaf_size=64, kappa=kappa, knn_mode=0, s_max=8, id_tol=0.0, h=1.0, seed=4)
+    # the tree's own points as queries, and (d > 64) new points
+    rows = np.arange(0, N, 7, dtype=np.int32)
+    ids, dist = g.knn_points(torch.from_numpy(rows).cuda())
+    oi, od = oracle.knn_exact(X, kappa, rows=rows.astype(np.int64))
+    assert np.array_equal(ids.cpu().numpy(), oi) and np.array_equal(dist.cpu().numpy(), od)
+    if d > 64:
+        Y = _points(40, d, kind, rng)
+        ids, dist = g.knn_targets(torch.from_numpy(Y).cuda())
+        oi, od = oracle.knn_exact(X, kappa, Y=Y)
+        assert np.array_equal(ids.cpu().numpy(), oi) and np.array_equal(dist.cpu().numpy(), od)
+    g.close()
