@@ -298,7 +298,7 @@ struct askit_tree_s {
     // centered on the data mean g_xbar; targets (x - xbar) g_sigma and
     // sources (y - xbar) 2 sc_j / g_sigma split into FP16 hi + lo; the norm
     // blocks of targets [rows, 16] and of every source sub-block (scales
-    // g_tau, g_kappa); n = |x - xbar|^2.  g_rho = max_j sc_j * max_i n_i
+    // g_tau, g_kappa); n = |x - xbar|^2, g_r2max the largest.  g_rho = max_j sc_j * max_i n_i
     // decides the automatic choice (g_ok)
     uint16_t *Xg_hi = nullptr, *Xg_lo = nullptr, *Xg_x = nullptr;   // tree points as targets
     uint16_t *Xb_hi = nullptr, *Xb_lo = nullptr;                    // tree points as sources
@@ -307,7 +307,7 @@ struct askit_tree_s {
     float *ng_t = nullptr, *ng_s = nullptr;
     float *g_xbar = nullptr;       // [TC_K] device
     float g_sigma = 1.f, g_tau = 1.f, g_kappa = 1.f;
-    double g_rho = 0.0;
+    double g_rho = 0.0, g_r2max = 0.0;
     bool g_ok = false;
     int fp16_centering = 0;        // 0 automatic (global when g_ok), 1 per sub-block, 2 global
     void *g16 = nullptr;           // tensor maps of the global-centered kernel

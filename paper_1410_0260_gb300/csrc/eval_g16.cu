@@ -1089,6 +1089,7 @@ askit_status build_g16_operands(askit_tree t, cudaStream_t s) {
     const double r2max = hred[1];
     t->g_tau = pow2_near(r2max > 0.0 ? sqrt(sc_max / r2max) : 1.0);
     t->g_kappa = pow2_near(sqrt(sc_max * r2max));
+    t->g_r2max = r2max;
     t->g_rho = sc_max * r2max;
     t->g_ok = t->g_rho <= RHO_MAX;
     // the tree points as targets, and the sources' norm blocks

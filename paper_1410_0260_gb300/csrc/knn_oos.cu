@@ -10,7 +10,8 @@
 //    kappa nearest; only these get their canonical FP64 distance, ordered by
 //    (distance, id).
 // A query with more than KO_CAP candidates, or whose coordinates leave the
-// FP16-safe range, takes the exhaustive search.
+// FP16-safe range, takes the exhaustive search, and every query does where norms or
+// scales would leave FP32's range (fp32_safe): no FP32 distance below overflows.
 //
 // An FP64 warp instruction takes 64 cycles of its quarter of the SM here, so the FP64
 // distances are what the steps avoid: seeding in FP64 over the two leaves took 74 of the 110 ms that
@@ -690,10 +691,19 @@ askit_status tree_maps(askit_tree t, EncodeTiledFn fn, CUtensorMap *th, CUtensor
                      CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
+// Whether the shortlist's FP32 figures stay finite and normal: the tree's norms below
+// 1e37, those of queries in the FP16-safe range (|y_k - xbar_k| sigma <= 30000) at most
+// 5.8e10 / sigma^2 < 6e36, so every squared distance below 3.2e37; and 2 / sigma^2,
+// KO_ABS / sigma^2 normal.
+bool fp32_safe(const askit_tree_s *t) {
+    const double s2 = (double)t->g_sigma * t->g_sigma;
+    return t->g_r2max < 1e37 && s2 > 1e-26 && s2 < 1e30;
+}
+
 }  // namespace
 
 askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t *ids, double *dist, cudaStream_t s) {
-    if (!t->Xg_hi || t->d > TC_K || kappa > 32)
+    if (!t->Xg_hi || t->d > TC_K || kappa > 32 || !fp32_safe(t))
         return knn_exact_gpu(t->X, t->N, t->d, kappa, Y, T, ids, dist, s);
     const int d = t->d;
     const int64_t M = (int64_t)1 << t->L, N = t->N;

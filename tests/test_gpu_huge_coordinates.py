@@ -59,3 +59,18 @@ def test_exhaustive_lists_past_the_fp32_range(N, d, kappa, kind):
         oi, od = oracle.knn_exact(X, kappa, Y=Y)
         assert np.array_equal(ids.cpu().numpy(), oi) and np.array_equal(dist.cpu().numpy(), od)
     g.close()
+
+
+@pytest.mark.parametrize("scale", [4e18, 1e-19])
+def test_new_points_at_the_ends_of_the_fp32_range(scale):
+    """Norms around the mean overflow for some points (4e18), or the tensor-core
+    scale's square does (1e-19), while the neighbors themselves are ordinary."""
+    import oracle
+    rng = np.random.default_rng(3)
+    X = (rng.standard_normal((5000, 8)) * scale).astype(np.float32)
+    Y = (rng.standard_normal((500, 8)) * 1.2 * scale).astype(np.float32)
+    g = _lists(X, leaf_size=128, kappa=8, knn_mode=0, s_max=8, id_tol=0.0, h=scale, seed=4)
+    ids, dist = g.knn_targets(torch.from_numpy(Y).cuda())
+    oi, od = oracle.knn_exact(X, 8, Y=Y)
+    assert np.array_equal(ids.cpu().numpy(), oi) and np.array_equal(dist.cpu().numpy(), od)
+    g.close()
