@@ -113,7 +113,7 @@ void askit_default_params(askit_params *p);
  *           N(X) argument of Algorithm 5, self excluded), or NULL to compute.
  *   out     receives the tree handle (library-owned; askit_destroy frees it).
  * Errors: INVALID_ARG for N < 1, d < 1, m < 2, kappa outside 1..min(32, N-1),
- * s_max < 1, non-positive h or id_tol < 0; OOM when device memory runs out;
+ * s_max < 1, non-positive h, id_tol < 0 or a coordinate that is not finite; OOM when device memory runs out;
  * UNSUPPORTED for N >= 2^31, leaf_size or s_max above 2048 (16 sub-blocks
  * of 128 rows) or a tree deeper than 25 levels.  Blocks until the setup is
  * complete.
@@ -148,7 +148,8 @@ askit_status askit_evaluate(askit_tree t, float *U_dev, int64_t ldu, void *strea
  * here the prune set of y is its exact kappa nearest sources, eq. (2.5)
  * with {i} replaced by nothing).  Y_dev [T, d] FP32 (stride ldy),
  * U_dev [T, r] FP32 (stride ldu).  Allocates per-call work lists and
- * blocks the host until they are built.
+ * blocks the host until they are built.  INVALID_ARG, with U_dev untouched, when a
+ * target has a coordinate that is not finite.
  */
 askit_status askit_evaluate_targets(askit_tree t, const float *Y_dev, int64_t T, int64_t ldy,
                                     float *U_dev, int64_t ldu, void *stream);

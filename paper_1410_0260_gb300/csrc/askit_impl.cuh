@@ -510,7 +510,7 @@ askit_status reduce_partials(const WorkLists &w, const float *partial, int r, co
                              float *U, int64_t ldu, cudaStream_t s);
 askit_status insample_prune_sets(askit_tree t, PruneSets &ps, cudaStream_t s);
 askit_status oos_prune_sets(askit_tree t, const int32_t *knn, const double *dist, const int32_t *order, int64_t T,
-                            int stride, int32_t *sets, cudaStream_t s);
+                            int stride, int32_t *sets, int *bad, cudaStream_t s);
 // every array of w back to the arena
 void free_work_lists(WorkLists &w, DevArena &arena);
 

@@ -46,7 +46,13 @@ __global__ void leafof_kernel(const int32_t *perm, const int32_t *nstart, const 
     for (int q = threadIdx.x; q < nsize[a]; q += blockDim.x) leafof[perm[nstart[a] + q]] = (int32_t)a;
 }
 
-// Caller-given neighbor ids must lie in [0, N) and exclude the point itself.
+// Coordinates must be finite: the sorts and lists order by distances and projections.
+__global__ void check_finite_kernel(const float *X, int64_t n, int *bad) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e < n && !(fabsf(X[e]) <= FLT_MAX)) *bad = 1;
+}
+
+// Neighbor ids must lie in [0, N) and exclude the point itself.
 __global__ void check_knn_kernel(const int32_t *knn, int64_t N, int kappa, int *bad) {
     int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e >= N * kappa) return;
@@ -61,11 +67,14 @@ __global__ void pos_kernel(const int32_t *perm, int64_t N, int32_t *pos) {
 
 // Order out-of-sample queries by the tree position of their nearest source
 // (so a tile's targets share near and far blocks), ties by q (a stable sort).
-__global__ void oos_keys_kernel(const int32_t *knn, int kappa, const int32_t *pos, int64_t T,
+// A list that was not filled (a query at no finite distance from kappa points) holds
+// ids past N: key 0 (oos_prune_sets reports it).
+__global__ void oos_keys_kernel(const int32_t *knn, int kappa, const int32_t *pos, int64_t N, int64_t T,
                                 uint32_t *keys, int32_t *vals) {
     int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= T) return;
-    keys[q] = (uint32_t)pos[knn[q * kappa]];
+    const int32_t j = knn[q * kappa];
+    keys[q] = j >= 0 && j < N ? (uint32_t)pos[j] : 0u;
     vals[q] = (int32_t)q;
 }
 
@@ -161,26 +170,36 @@ askit_status setup_impl(askit_tree t, const float *X_dev, int64_t ldx, const flo
     ASK_TRY(t->arena.alloc(&t->X, (size_t)N * d));
     ASK_CUDA(cudaMemcpy2DAsync(t->X, sizeof(float) * d, X_dev, sizeof(float) * ldx, sizeof(float) * d, N,
                                cudaMemcpyDeviceToDevice, s));
+    int *bad = nullptr, hbad = 0;
+    ASK_TRY(t->arena.alloc(&bad, 1));
+    ASK_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
+    check_finite_kernel<<<nblk(N * d, 256), 256, 0, s>>>(t->X, N * d, bad);
+    ASK_LAUNCH();
+    ASK_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+    ASK_CUDA(cudaStreamSynchronize(s));
+    if (hbad) { askit_set_error("a point has a coordinate that is not finite"); return ASKIT_ERR_INVALID_ARG; }
     // nearest neighbors (Section 2.2)
     ASK_TRY(t->arena.alloc(&t->knn, (size_t)N * kappa));
     ASK_TRY(t->arena.alloc(&t->knnd, (size_t)N * kappa));
     if (knn_dev) {
         ASK_CUDA(cudaMemcpyAsync(t->knn, knn_dev, sizeof(int32_t) * N * kappa, cudaMemcpyDeviceToDevice, s));
-        int *bad = nullptr, hbad = 0;
-        ASK_TRY(t->arena.alloc(&bad, 1));
-        ASK_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
-        check_knn_kernel<<<nblk(N * kappa, 256), 256, 0, s>>>(t->knn, N, kappa, bad);
-        ASK_LAUNCH();
-        ASK_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
-        ASK_CUDA(cudaStreamSynchronize(s));
-        t->arena.release(bad);
-        if (hbad) { askit_set_error("knn_dev holds an id outside [0, N) or the point itself"); return ASKIT_ERR_INVALID_ARG; }
-        ASK_TRY(knn_dist_gpu(t->X, N, d, kappa, t->knn, t->knnd, s));
     } else if (t->prm.knn_mode == 0) {
         ASK_TRY(knn_exact_gpu(t->X, N, d, kappa, nullptr, N, t->knn, t->knnd, s));
     } else {
         ASK_TRY(knn_rp_gpu(t->X, N, d, kappa, t->prm.rp_iters, t->rp_leaf, t->prm.seed, t->knn, t->knnd, s));
     }
+    // every later stage indexes by these ids, the computed ones too
+    check_knn_kernel<<<nblk(N * kappa, 256), 256, 0, s>>>(t->knn, N, kappa, bad);
+    ASK_LAUNCH();
+    ASK_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+    ASK_CUDA(cudaStreamSynchronize(s));
+    t->arena.release(bad);
+    if (hbad) {
+        askit_set_error(knn_dev ? "knn_dev holds an id outside [0, N) or the point itself"
+                                : "the neighbor search left a list unfilled");
+        return ASKIT_ERR_INVALID_ARG;
+    }
+    if (knn_dev) ASK_TRY(knn_dist_gpu(t->X, N, d, kappa, t->knn, t->knnd, s));
     ASK_TRY(stage_mark(t, 0, s));
     // bandwidth of every source point (Section 4)
     ASK_TRY(t->arena.alloc(&t->hsrc, N));
@@ -473,7 +492,7 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     WorkLists w;
     float *partial = nullptr;
     uint16_t *yg_hi = nullptr, *yg_lo = nullptr, *yg_x = nullptr;
-    int *yg_flag = nullptr;
+    int *flags = nullptr, h_flags[2] = {0, 0};     // target outside the FP16-safe range; list not filled
     QuerySplit qs;
     int64_t T_pad = (T + ASK_TILE_M - 1) / ASK_TILE_M * ASK_TILE_M;
     int pos_bits = 1;
@@ -486,9 +505,11 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     OTRY(tmp.alloc(&ids, (size_t)T * kappa));
     OTRY(tmp.alloc(&dist, (size_t)T * kappa));
     OTRY(knn_oos(t, Yc, T, kappa, ids, dist, s));
+    OTRY(tmp.alloc(&flags, 2));
+    if (cudaMemsetAsync(flags, 0, 2 * sizeof(int), s) != cudaSuccess) { askit_set_error("flags"); rc = ASKIT_ERR_CUDA; goto out; }
     OTRY(tmp.alloc(&keys, T)); OTRY(tmp.alloc(&keys_s, T));
     OTRY(tmp.alloc(&vals, T)); OTRY(tmp.alloc(&order, T));
-    oos_keys_kernel<<<nblk(T, 256), 256, 0, s>>>(ids, kappa, t->pos, T, keys, vals);
+    oos_keys_kernel<<<nblk(T, 256), 256, 0, s>>>(ids, kappa, t->pos, t->N, T, keys, vals);
     OTRY(sort_u32_i32(nullptr, nullptr, nullptr, nullptr, T, pos_bits, nullptr, &cb, s));
     OTRY(tmp.alloc((char **)&cub, cb));
     OTRY(sort_u32_i32(keys, keys_s, vals, order, T, pos_bits, cub, &cb, s));
@@ -497,20 +518,22 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
         OTRY(tmp.alloc(&yg_hi, (size_t)T_pad * TC_K));
         OTRY(tmp.alloc(&yg_lo, (size_t)T_pad * TC_K));
         OTRY(tmp.alloc(&yg_x, (size_t)T_pad * 16));
-        OTRY(tmp.alloc(&yg_flag, 1));
-        if (cudaMemsetAsync(yg_flag, 0, sizeof(int), s) != cudaSuccess) { askit_set_error("flag"); rc = ASKIT_ERR_CUDA; goto out; }
-        OTRY(g16_split_rows(Yc, d, d, T_pad, t, yg_hi, yg_lo, yg_x, yg_flag, s, order, T));
+        OTRY(g16_split_rows(Yc, d, d, T_pad, t, yg_hi, yg_lo, yg_x, flags, s, order, T));
     }
     OTRY(tmp.alloc(&sets, (size_t)T * kappa));
-    OTRY(oos_prune_sets(t, ids, dist, order, T, kappa, sets, s));
+    OTRY(oos_prune_sets(t, ids, dist, order, T, kappa, sets, flags + 1, s));
     OTRY(build_work_lists(t, sets, kappa, nullptr, T, w, tmp, false, s));
     OTRY(tmp.alloc(&partial, (size_t)w.n_entries * c.r));
+    // (the lists' last synchronization has covered both)
+    if (cudaMemcpyAsync(h_flags, flags, sizeof h_flags, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess) { askit_set_error("target flags"); rc = ASKIT_ERR_CUDA; goto out; }
+    if (h_flags[1]) {
+        askit_set_error("a target has a coordinate that is not finite");
+        rc = ASKIT_ERR_INVALID_ARG;
+        goto out;
+    }
     if (g16) {
-        // (the lists' last synchronization has covered the split)
-        int flag = 0;
-        if (cudaMemcpyAsync(&flag, yg_flag, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) { askit_set_error("range flag"); rc = ASKIT_ERR_CUDA; goto out; }
-        if (!flag) {
+        if (!h_flags[0]) {
             qs.hi = yg_hi;
             qs.lo = yg_lo;
             qs.x = yg_x;

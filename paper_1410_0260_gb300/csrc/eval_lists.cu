@@ -162,15 +162,19 @@ __global__ void leaf_row_kernel(const int32_t *perm, const int32_t *leafof, int6
 }
 
 // Out-of-sample prune sets: the sorted distinct leaves of N_y (its first kappa_y
-// neighbors; no self term), a warp per target, a neighbor per lane (kappa <= 32).
+// neighbors; no self term), a warp per target, a neighbor per lane (kappa <= 32).  A
+// list that was not filled (ids past N) sets *bad.
 __global__ void oos_sets_kernel(const int32_t *leafof, const int32_t *knn, const double *dist, const int32_t *order,
-                                const float *hsrc, double kscale, double cut, int64_t T, int kappa, int stride, int32_t *sets) {
+                                const float *hsrc, double kscale, double cut, int64_t N, int64_t T, int kappa, int stride,
+                                int32_t *sets, int *bad) {
     const int lane = threadIdx.x & 31;
     const int64_t q = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
     if (q >= T) return;                                    // warp-uniform
-    const bool in = lane < kappa;
     const int64_t src = (int64_t)order[q] * kappa + lane;  // target q's neighbors: the caller's row order[q]
-    const int32_t id = in ? knn[src] : 0;
+    const int32_t j = lane < kappa ? knn[src] : 0;
+    const bool in = lane < kappa && j >= 0 && j < N;
+    const int32_t id = in ? j : 0;
+    if (lane < kappa && !in) *bad = 1;
     int ky = kappa;                                        // kappa_of over the lanes
     if (cut > 0.0) {
         const double h = (double)hsrc[id];
@@ -747,9 +751,9 @@ askit_status insample_prune_sets(askit_tree t, PruneSets &ps, cudaStream_t s) {
 }
 
 askit_status oos_prune_sets(askit_tree t, const int32_t *knn, const double *dist, const int32_t *order, int64_t T,
-                            int stride, int32_t *sets, cudaStream_t s) {
-    oos_sets_kernel<<<nblk(T, 8), 256, 0, s>>>(t->leafof, knn, dist, order, t->hsrc, t->prm.kernel_scale, t->kappa_cut, T,
-                                                 t->kappa, stride, sets);
+                            int stride, int32_t *sets, int *bad, cudaStream_t s) {
+    oos_sets_kernel<<<nblk(T, 8), 256, 0, s>>>(t->leafof, knn, dist, order, t->hsrc, t->prm.kernel_scale, t->kappa_cut, t->N, T,
+                                                 t->kappa, stride, sets, bad);
     ASK_LAUNCH();
     return ASKIT_OK;
 }
