@@ -153,8 +153,9 @@ __global__ void fill_kernel(T *a, int64_t n, T v) {
 
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
-// Every point of an RP-tree leaf against its leaf-mates: block (leaf, y) takes the
-// leaf's points 64 y .. + 63 as queries, the leaf as candidates, 512 at a time.
+// Every point of an RP-tree leaf against its leaf-mates: block y nleaf + leaf takes the
+// leaf's points 64 y .. + 63 as queries, the leaf as candidates, 512 at a time (one grid
+// dimension: a leaf may have more query blocks than the second one allows).
 // FP32 squared distances (difference form) in 64 x 128 tiles from shared memory, 4 x 8
 // pairs a thread; a warp then takes a query's 512 distances: the kappa-th smallest
 // (a best-32 list of floats) and the list so far bound what can be among the
@@ -169,12 +170,14 @@ constexpr int KL_DT = KL_C + 4, KL_QS = KL_Q + 4, KL_CS = KL_TILE + 4;
 constexpr size_t KL_SMEM = sizeof(float) * (KL_Q * KL_DT + KL_K * (KL_QS + KL_CS));
 
 __global__ void __launch_bounds__(256) knn_leaf_kernel(const float *X, int d, const int32_t *order, const int32_t *beg,
-                                                       const int32_t *end, int kappa, double *bd, int *bi) {
+                                                       const int32_t *end, unsigned nleaf, int kappa, double *bd,
+                                                       int *bi) {
     extern __shared__ __align__(16) float kl[];
     float *dt = kl, *qs = kl + KL_Q * KL_DT, *cs = qs + KL_K * KL_QS;   // [query][candidate], [k][query], [k][candidate]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx = tid & 15, ty = tid >> 4;                // pairs: queries 4 ty .., candidates 4 tx .. and 64 + 4 tx ..
-    const int b0 = beg[blockIdx.x], n = end[blockIdx.x] - b0, q0 = blockIdx.y * KL_Q;
+    const unsigned leaf = blockIdx.x % nleaf;
+    const int b0 = beg[leaf], n = end[leaf] - b0, q0 = (int)(blockIdx.x / nleaf) * KL_Q;
     if (q0 >= n) return;                                   // block-uniform
     const int nq = min(KL_Q, n - q0);
     const int32_t *ids = order + b0;
@@ -678,8 +681,8 @@ askit_status knn_rp_gpu(const float *X, int64_t N, int d, int kappa, int iters, 
     for (int it = 0; rc == ASKIT_OK && e == cudaSuccess && it < iters; ++it) {
         rc = build_tree_gpu(X, N, d, L, 1, seed, it, order, s);
         if (rc != ASKIT_OK) break;
-        knn_leaf_kernel<<<dim3((unsigned)nleaf, nblk(max_leaf, KL_Q)), 256, KL_SMEM, s>>>(X, d, order, segs, segs + nleaf,
-                                                                                         kappa, bd, bi);
+        knn_leaf_kernel<<<(unsigned)(nleaf * nblk(max_leaf, KL_Q)), 256, KL_SMEM, s>>>(
+            X, d, order, segs, segs + nleaf, (unsigned)nleaf, kappa, bd, bi);
         e = cudaGetLastError();
     }
     if (rc == ASKIT_OK && e == cudaSuccess) {
