@@ -172,8 +172,9 @@ askit_status askit_evaluate_host(askit_tree t, const float *W_host, int32_t r, i
  *   double squared distances.  Blocks until done.
  * For d <= 64 a tensor-core FP16x3 shortlist (every point within a bound of
  * each query's k-th distance, with a margin five times the arithmetic's error)
- * is re-ranked in FP64; queries whose shortlist overflows take the exhaustive
- * search.
+ * is re-ranked in FP64; queries whose shortlist overflows scan the leaves that
+ * can hold a point within the bound, and queries far outside the data take the
+ * exhaustive search.
  */
 askit_status askit_knn_targets(askit_tree t, const float *Y_dev, int64_t T, int64_t ldy, int32_t *ids_dev,
                                double *dist_dev, void *stream);

@@ -9,8 +9,11 @@
 // 4. Re-rank: FP32 distances of the candidates leave those that can be among the
 //    kappa nearest; only these get their canonical FP64 distance, ordered by
 //    (distance, id).
-// A query with more than KO_CAP candidates, or whose coordinates leave the
-// FP16-safe range, takes the exhaustive search, and every query does where norms or
+// A query with more than KO_CAP candidates -- the margin, in proportion to the squared
+// distance from the data mean, takes in whole clusters or stretches of a curve where
+// points lie that close -- scans the leaves whose ball around their center can hold a
+// point within U.  A query whose coordinates leave the FP16-safe range takes the
+// exhaustive search, and every query does where norms or
 // scales would leave FP32's range (fp32_safe): no FP32 distance below overflows.
 //
 // An FP64 warp instruction takes 64 cycles of its quarter of the SM here, so the FP64
@@ -35,6 +38,7 @@ using namespace tcx;
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 constexpr int KO_CAP = 1024;                   // candidates a query keeps
+constexpr int KO_BAD = 1 << 30;                // count of a query outside the FP16-safe range
 // The margin of the FP16x3 distance n_q + n_j - 2 a.b (both sides centered on the
 // data mean, a.b in three split products): the splits keep 22 significant bits and
 // the FP32 accumulation adds a few 2^-23 |a||b| a step, below 2^-18 (n_q + n_j)
@@ -50,7 +54,7 @@ __host__ __device__ __forceinline__ float sum_gam(int d) { return (float)(d + 2)
 
 // Queries as FP16x3 operands of the shortlist: (y - xbar) sigma split hi + lo
 // [T_pad, 64], n = |y - xbar|^2; a query outside the FP16-safe range gets zero
-// rows and a full candidate count.  A warp per row; rows past T are zero.  Row i is
+// rows and the count KO_BAD (hits on the zero rows add to it: N < 2^30 here).  A warp per row; rows past T are zero.  Row i is
 // query order[i] (order null: query i), here and in the steps that follow.
 __global__ void ko_split_kernel(const float *Y, int d, const int32_t *order, int64_t T, int64_t T_pad, const float *xbar, float sigma,
                                 uint16_t *hi, uint16_t *lo, float *nq, int *cnt) {
@@ -79,7 +83,7 @@ __global__ void ko_split_kernel(const float *Y, int d, const int32_t *order, int
     }
     if (lane == 0) {
         nq[row] = acc;
-        if (row < T) cnt[row] = bad ? KO_CAP + 1 : 0;
+        if (row < T) cnt[row] = bad ? KO_BAD : 0;
     }
 }
 
@@ -328,7 +332,8 @@ template <int NJ, int W>
 __global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, const float *Y, int d,
                                                            const int32_t *order, int64_t T, const int32_t *perm,
                                                            const int *cnt, const int32_t *cand, int kappa,
-                                                           int32_t *ids, double *dist, int *n_ovf, int32_t *ovf) {
+                                                           int32_t *ids, double *dist, int *n_ovf, int32_t *ovf,
+                                                           int32_t *wide) {
     __shared__ float sd[W][KO_CAP];
     __shared__ float sy[W][TC_K];
     __shared__ float sl[W][64];
@@ -338,8 +343,12 @@ __global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, cons
     if (q >= T) return;                                    // warp-uniform
     const int64_t src = order ? order[q] : q;
     const int n = cnt[q];
-    if (n > KO_CAP || n < kappa) {                         // (fewer cannot be: U bounds kappa points)
+    if (n >= KO_BAD || n < kappa) {                        // (fewer cannot be: U bounds kappa points)
         if (lane == 0) ovf[atomicAdd(n_ovf, 1)] = (int32_t)src;
+        return;
+    }
+    if (n > KO_CAP) {
+        if (lane == 0) wide[atomicAdd(n_ovf + 1, 1)] = (int32_t)q;
         return;
     }
     const int32_t *c = cand + q * KO_CAP;
@@ -396,6 +405,104 @@ __global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, cons
         warp_collect(m, p, have, held, lane, offer);
     }
     if (have > 0) offer();
+    if (lane < kappa) {
+        ids[src * kappa + lane] = li;
+        dist[src * kappa + lane] = ld;
+    }
+}
+
+// Radius of every leaf's ball around its center, rounded up, from the squared norms of
+// its centered rows (FP64 sums of FP32 differences, rounded).
+__global__ void ko_radius_kernel(const float *nrmc, const int32_t *nstart, const int32_t *nsize, int64_t M, float *rad) {
+    const int lane = threadIdx.x & 31;
+    const int64_t l = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (l >= M) return;                                    // warp-uniform
+    float m = 0.f;
+    for (int i = lane; i < nsize[M + l]; i += 32) m = fmaxf(m, nrmc[nstart[M + l] + i]);
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
+    if (lane == 0) rad[l] = sqrtf(m) * (1.f + 2e-6f) + 1e-18f;
+}
+
+// A query with too many candidates, a block per query: its warps take the leaves in
+// turn, 32 centers at a time (a lane each), and scan those that |y - c| - radius leaves
+// within sqrt(U).  FP32 distances within U, and within the warp's kappa-th FP64 one so
+// far, get their FP64 distance, 32 to a batch; the warps' lists are merged at the end.
+// Overflow comes with tight clusters or few intrinsic dimensions, where the balls rule
+// out nearly all leaves: 3,001 queries against 1M points of a curve in 3 dimensions
+// took 38.4 ms with the exhaustive search here, 1.7 so; 50,000 against 64 clusters of
+// 2,048 points 88.3 ms and 8.2.
+constexpr int BA_WARPS = 8;
+template <int NJ>
+__global__ void __launch_bounds__(32 * BA_WARPS) ko_ball_kernel(const float *Xt, const float *Y, int d,
+                                                                const int32_t *order, const int32_t *rows,
+                                                                const int32_t *perm, const float *U, const float *cent,
+                                                                const int32_t *leaf_cbase, const float *rad, int64_t M,
+                                                                const int32_t *nstart, const int32_t *nsize, int kappa,
+                                                                int32_t *ids, double *dist) {
+    __shared__ float sy[TC_K];
+    __shared__ double sd[BA_WARPS][32];
+    __shared__ int si[BA_WARPS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t q = rows[blockIdx.x], src = order ? order[q] : q;
+    for (int k = threadIdx.x; k < TC_K; k += 32 * BA_WARPS) sy[k] = k < d ? Y[src * d + k] : 0.f;
+    float4 y[NJ];
+    load_query<NJ>(Y + src * d, d, lane, y);
+    __syncthreads();
+    const float gam = sum_gam(d), su = sqrtf(U[q]) * (1.f + 2e-6f);
+    const float u = U[q] * (1.f + gam) + 1e-37f;           // FP32 distances of the kappa nearest are within this
+    double ld = DBL_MAX;
+    int li = INT_MAX, have = 0;
+    int32_t held = 0;                                      // lane < have: a candidate's tree position
+    auto offer = [&]() {
+        double cd = DBL_MAX;
+        int ci = INT_MAX;
+        if (lane < have) {
+            ci = perm[held];
+            cd = c_dist2(sy, Xt + (int64_t)held * (32 * NJ), d);
+        }
+        warp_offer(ld, li, cd, ci, kappa, false, lane);
+        have = 0;
+    };
+    for (int64_t l0 = 32 * (int64_t)warp; l0 < M; l0 += 32 * BA_WARPS) {
+        const int64_t l = l0 + lane;
+        bool in = l < M;
+        if (in) {
+            const float4 *c = reinterpret_cast<const float4 *>(cent + (int64_t)leaf_cbase[l] * TC_K);
+            float acc = 0.f;
+#pragma unroll 4
+            for (int k = 0; k < 8 * NJ; ++k) {
+                const float4 v = c[k];
+                const float t0 = sy[4 * k] - v.x, t1 = sy[4 * k + 1] - v.y, t2 = sy[4 * k + 2] - v.z, t3 = sy[4 * k + 3] - v.w;
+                acc = fmaf(t0, t0, acc);
+                acc = fmaf(t1, t1, acc);
+                acc = fmaf(t2, t2, acc);
+                acc = fmaf(t3, t3, acc);
+            }
+            in = !(sqrtf(acc) * (1.f - gam - 4e-6f) - rad[l] > su);
+        }
+        unsigned m = __ballot_sync(FULL, in);
+        while (m) {
+            const int64_t leaf = l0 + __ffs(m) - 1;
+            m &= m - 1;
+            const int p0 = nstart[M + leaf], np = nsize[M + leaf];
+            for (int b = 0; b < np; b += 32) {
+                // rows past the leaf are other points or the zero rows past N
+                const float v = rows32<NJ>(Xt, y, lane, [&](int i) { return p0 + b + i; });
+                const int i = b + 4 * (lane & 7) + (lane >> 3);
+                const double kth = __shfl_sync(FULL, ld, kappa - 1);
+                const float lim = kth < 1e38 ? fminf(u, __double2float_ru(kth) * (1.f + 2.f * gam) + 1e-37f) : u;
+                const unsigned hit = __ballot_sync(FULL, i < np && v <= lim);
+                // the lanes' rows are not in lane order: positions travel with the hits
+                if (hit) warp_collect(hit, p0 + i, have, held, lane, offer);
+            }
+        }
+    }
+    if (have > 0) offer();
+    sd[warp][lane] = ld;
+    si[warp][lane] = li;
+    __syncthreads();
+    if (warp) return;
+    for (int w = 1; w < BA_WARPS; ++w) warp_offer(ld, li, sd[w][lane], si[w][lane], kappa, false, lane);
     if (lane < kappa) {
         ids[src * kappa + lane] = li;
         dist[src * kappa + lane] = ld;
@@ -729,7 +836,8 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
     };
     const size_t o_hi = part((size_t)T_pad * TC_K * 2), o_lo = part((size_t)T_pad * TC_K * 2), o_nq = part((size_t)T_pad * 4),
                  o_hd = part((size_t)nsplit * T * 8), o_hx = part((size_t)nsplit * T * 8), o_u = part((size_t)T * 4),
-                 o_cnt = part((size_t)T * 4), o_ord = part((size_t)T * 4), o_ovf = part((size_t)(T + 1) * 4), o_cand = part((size_t)T * KO_CAP * 4);
+                 o_cnt = part((size_t)T * 4), o_ord = part((size_t)T * 4), o_ovf = part((size_t)(2 * T + 2) * 4),
+                 o_rad = part((size_t)M * 4), o_cand = part((size_t)T * KO_CAP * 4);
     uint8_t *buf = nullptr;
     ASK_TRY(tmp.alloc(&buf, used));
     uint16_t *qh = reinterpret_cast<uint16_t *>(buf + o_hi), *ql = reinterpret_cast<uint16_t *>(buf + o_lo);
@@ -737,13 +845,14 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
           *U = reinterpret_cast<float *>(buf + o_u);
     int32_t *hx = reinterpret_cast<int32_t *>(buf + o_hx), *cand = reinterpret_cast<int32_t *>(buf + o_cand);
     int *cnt = reinterpret_cast<int *>(buf + o_cnt), *n_ovf = reinterpret_cast<int *>(buf + o_ovf);
-    int32_t *ovf = n_ovf + 1;
+    int32_t *ovf = n_ovf + 2, *wide = ovf + T;
+    float *rad = reinterpret_cast<float *>(buf + o_rad);
     const int32_t *order = nullptr;
-    int h_ovf = 0;
+    int h_n[2] = {0, 0}, h_ovf = 0;
     askit_status rc = ASKIT_OK;
 #define QTRY(x) do { rc = (x); if (rc != ASKIT_OK) goto out; } while (0)
 #define QCHK(x) do { const cudaError_t e_ = (x); if (e_ != cudaSuccess) { askit_set_error("out-of-sample kNN: %s", cudaGetErrorString(e_)); rc = e_ == cudaErrorMemoryAllocation ? ASKIT_ERR_OOM : ASKIT_ERR_CUDA; goto out; } } while (0)
-    QCHK(cudaMemsetAsync(n_ovf, 0, sizeof(int), s));
+    QCHK(cudaMemsetAsync(n_ovf, 0, 2 * sizeof(int), s));
     ko_home_kernel<<<dim3((unsigned)qb, (unsigned)nsplit), 128, 0, s>>>(Y, d, T, t->cent, t->leaf_cbase, M, split_len, hd,
                                                                         hx);
     // Queries in the order of their home leaves: the 128 of a tile then have their
@@ -809,11 +918,20 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
         auto rerank = t->d_pad == 32 ? (few ? ko_rerank_kernel<1, 1> : ko_rerank_kernel<1, 8>)
                                      : (few ? ko_rerank_kernel<2, 1> : ko_rerank_kernel<2, 8>);
         rerank<<<nblk(T, few ? 1 : 8), few ? 32 : 256, 0, s>>>(t->Xt, Y, d, order, T, t->perm, cnt, cand, kappa, ids, dist,
-                                                              n_ovf, ovf);
+                                                              n_ovf, ovf, wide);
     }
     QCHK(cudaGetLastError());
-    QCHK(cudaMemcpyAsync(&h_ovf, n_ovf, sizeof(int), cudaMemcpyDeviceToHost, s));
+    QCHK(cudaMemcpyAsync(h_n, n_ovf, sizeof h_n, cudaMemcpyDeviceToHost, s));
     QCHK(cudaStreamSynchronize(s));
+    h_ovf = h_n[0];
+    if (h_n[1] > 0) {
+        ko_radius_kernel<<<nblk(M, 8), 256, 0, s>>>(t->nrmc_t, t->nstart, t->nsize, M, rad);
+        auto ball = t->d_pad == 32 ? ko_ball_kernel<1> : ko_ball_kernel<2>;
+        ball<<<(unsigned)h_n[1], 32 * BA_WARPS, 0, s>>>(t->Xt, Y, d, order, wide, t->perm, U, t->cent, t->leaf_cbase, rad, M,
+                                                       t->nstart, t->nsize, kappa, ids, dist);
+        QCHK(cudaGetLastError());
+        if (h_ovf == 0) QCHK(cudaStreamSynchronize(s));
+    }
     if (h_ovf > 0) {
         // the exhaustive search
         float *Ys = nullptr;
