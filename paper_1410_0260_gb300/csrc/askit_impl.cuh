@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <chrono>
 #include <string>
 #include <vector>
@@ -37,6 +38,20 @@ void askit_set_error(const char *fmt, ...);
     do {                                             \
         ASK_CUDA(cudaGetLastError());                \
     } while (0)
+
+// Lets kernel k take `bytes` of dynamic shared memory.  The attribute belongs to a
+// device, so it is set at the first launch on each; `opted` (static at the caller, one a
+// kernel) has the bits of those where it is.
+template <class... KArgs>
+inline askit_status opt_in_smem(void (*k)(KArgs...), size_t bytes, std::atomic<uint64_t> &opted) {
+    int dev = 0;
+    ASK_CUDA(cudaGetDevice(&dev));
+    const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
+    if (opted.load() & bit) return ASKIT_OK;
+    ASK_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    opted.fetch_or(bit);
+    return ASKIT_OK;
+}
 
 // Launches kernel k so that it may start while the kernel before it on the
 // stream still runs (programmatic stream serialization).  Every kernel launched

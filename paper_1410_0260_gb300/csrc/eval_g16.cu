@@ -786,9 +786,8 @@ askit_status launch_g16(G16State *st, const G16Args &a, int grid, cudaStream_t s
     using S = SG<RC, NA, NB>;
     constexpr size_t smem = S::BYTES + 1024;
     static_assert(smem <= 232448, "shared-memory plan exceeds 227 KB");
-    static const cudaError_t attr = cudaFuncSetAttribute(eval_g16_kernel<RC, NA, NB>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    ASK_CUDA(attr);
+    static std::atomic<uint64_t> opted{0};
+    ASK_TRY(opt_in_smem(eval_g16_kernel<RC, NA, NB>, smem, opted));
     return launch_pdl(eval_g16_kernel<RC, NA, NB>, dim3((unsigned)grid), dim3(S::THREADS), smem, s, st->map[0],
                       st->map[1], st->map[2], st->map[3], a);
 }

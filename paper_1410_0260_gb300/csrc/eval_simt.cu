@@ -209,9 +209,8 @@ askit_status launch_simt(askit_tree t, const WeightCtx &c, const float *Xq, int6
     const size_t smem = sizeof(float) * (size_t)(SI_W + ASK_BLK_N * rz + ASK_TILE_M * ZC);
     constexpr int SMEM_MAX = (int)sizeof(float) * (SI_W + ASK_BLK_N * 64 + ASK_TILE_M * 16);
     static_assert(SMEM_MAX <= 232448, "shared-memory plan exceeds 227 KB");
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(eval_simt_kernel<ZC, DEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
-    ASK_CUDA(attr);
+    static std::atomic<uint64_t> opted{0};
+    ASK_TRY(opt_in_smem(eval_simt_kernel<ZC, DEEP>, SMEM_MAX, opted));
     // a sub-block's items over several blocks where there are few sub-blocks:
     // about eight waves of two blocks an SM
     const int64_t split = std::max<int64_t>(1, std::min<int64_t>(64, 8 * 2 * 152 / w.n_blocks));

@@ -497,9 +497,8 @@ askit_status tc_state(askit_tree t, TcState **out) {
 template <int P, int RC>
 askit_status launch(askit_tree t, TcState *st, const CUtensorMap &map_q, const TcArgs &a, int grid, cudaStream_t s) {
     const size_t smem = Smem<P>::BYTES + 1024;
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(eval_tc_kernel<P, RC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    ASK_CUDA(attr);
+    static std::atomic<uint64_t> opted{0};
+    ASK_TRY(opt_in_smem(eval_tc_kernel<P, RC>, smem, opted));
     ASK_TRY(ktimer_mark(t, s, false));
     ASK_TRY(launch_pdl(eval_tc_kernel<P, RC>, dim3((unsigned)grid), dim3(TC_THREADS), smem, s, st->map[0], st->map[1],
                        st->map[2], st->map[3], map_q, st->raw_t, st->raw_s, a));

@@ -697,9 +697,8 @@ askit_status launch16(T16State *st, int pi, const CUtensorMap &map_q, const CUte
     using S = S16<RC, NRAW, NB>;
     const size_t smem = S::BYTES + 1024;
     static_assert(S::BYTES + 1024 <= 232448, "shared-memory plan exceeds 227 KB");
-    static const cudaError_t attr = cudaFuncSetAttribute(eval_tc16_kernel<P, RC, NRAW, NB, UNI>,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    ASK_CUDA(attr);
+    static std::atomic<uint64_t> opted{0};
+    ASK_TRY(opt_in_smem(eval_tc16_kernel<P, RC, NRAW, NB, UNI>, smem, opted));
     return launch_pdl(eval_tc16_kernel<P, RC, NRAW, NB, UNI>, dim3((unsigned)grid), dim3(S::THREADS), smem, s,
                       st->map[pi][0], st->map[pi][1], st->map[pi][2], st->map[pi][3], map_q, map_q8, a);
 }

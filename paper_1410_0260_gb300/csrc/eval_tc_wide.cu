@@ -666,9 +666,8 @@ askit_status launch_w(askit_tree t, TcwState *st, int pi, const TcwArgs &a, int 
     using S = WSmem<RC, NB>;
     constexpr size_t smem = S::BYTES + 128;
     static_assert(smem <= 232448, "shared-memory plan exceeds 227 KB");
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(eval_tcw_kernel<P, RC, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    ASK_CUDA(attr);
+    static std::atomic<uint64_t> opted{0};
+    ASK_TRY(opt_in_smem(eval_tcw_kernel<P, RC, NB>, smem, opted));
     ASK_TRY(ktimer_mark(t, s, false));
     const CUtensorMap *m = st->map[pi][NB - 1];
     ASK_TRY(launch_pdl(eval_tcw_kernel<P, RC, NB>, dim3((unsigned)grid), dim3(W_THREADS), smem, s, m[0], m[1], m[2],

@@ -563,9 +563,8 @@ askit_status run_tf32(askit_tree t, const WeightCtx &c, FState *st, FArgs a, int
     using S = SF<RC>;
     constexpr size_t smem = S::BYTES + 1024;
     static_assert(smem <= 232448, "shared-memory plan exceeds 227 KB");
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(eval_tf32_kernel<RC, UNI, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    ASK_CUDA(attr);
+    static std::atomic<uint64_t> opted{0};
+    ASK_TRY(opt_in_smem(eval_tf32_kernel<RC, UNI, WIDE>, smem, opted));
     ASK_TRY(block_columns(t, c, RC, UNI, 1.f, s));
     a.colv = c.colv;
     a.colw = c.colw;

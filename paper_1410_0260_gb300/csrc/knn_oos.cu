@@ -907,9 +907,8 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
         a.status = t->d_status;
         constexpr size_t smem = KS::BYTES + 1024;
         static_assert(smem <= 232448, "shared-memory plan exceeds 227 KB");
-        static const cudaError_t attr =
-            cudaFuncSetAttribute(ko_shortlist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        QCHK(attr);
+        static std::atomic<uint64_t> opted{0};
+        QTRY(opt_in_smem(ko_shortlist_kernel, smem, opted));
         ko_shortlist_kernel<<<(unsigned)std::min<int64_t>(sms, a.units), KS::THREADS, smem, s>>>(mqh, mql, mth, mtl, a);
         QCHK(cudaGetLastError());
     }

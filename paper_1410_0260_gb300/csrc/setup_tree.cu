@@ -665,9 +665,8 @@ askit_status knn_rp_gpu(const float *X, int64_t N, int d, int kappa, int iters, 
         h[nleaf + a] = (int32_t)(st[nleaf + a] + sz[nleaf + a]);
     }
     const int64_t max_leaf = sz[nleaf];                    // the first leaf is the largest
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(knn_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)KL_SMEM);
-    ASK_CUDA(attr);
+    static std::atomic<uint64_t> opted{0};
+    ASK_TRY(opt_in_smem(knn_leaf_kernel, KL_SMEM, opted));
     double *bd = nullptr;
     int *bi = nullptr;
     int32_t *order = nullptr, *segs = nullptr;

@@ -218,10 +218,8 @@ template <int RC>
 askit_status launch_upward(askit_tree t, WeightCtx &c, int depth, int r, cudaStream_t s) {
     constexpr int STR = up_stride<RC>(), R = RC <= 4 ? 8 : 4;
     // set once per kernel instance (thread-safe static initialisation)
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(upward_kernel<RC, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(UP_KU * (STR * sizeof(float) + sizeof(int32_t))));
-    ASK_CUDA(attr);
+    static std::atomic<uint64_t> opted{0};
+    ASK_TRY(opt_in_smem(upward_kernel<RC, R>, UP_KU * (STR * sizeof(float) + sizeof(int32_t)), opted));
     const int64_t a0 = (int64_t)1 << depth;
     const int ku_max = std::max(128, std::min(UP_KU, (t->lvl_nr[depth] + 127) / 128 * 128));
     const size_t smem = (size_t)ku_max * (STR * sizeof(float) + sizeof(int32_t));
