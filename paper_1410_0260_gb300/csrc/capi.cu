@@ -900,11 +900,14 @@ askit_status askit_autotune(askit_tree t, int32_t reps, void *stream, askit_tune
         askit_set_error("events");
         rc = ASKIT_ERR_CUDA;
     }
+    // what this precision and r do not vary keeps its value (the automatic choices
+    // among them), for the tree's other precisions
+    const bool set_pairs = n_pairs > 0 && (wide || (fp16 && t->dw.r <= 4));
     auto apply = [&](const Cand &c) {
         t->tune_sched = c.pairs ? 0 : c.sched;
-        t->tune_stages = c.stages;
+        if (fp16) t->tune_stages = c.stages;
         t->tune_runs = c.runs;
-        t->tune_pairs = c.pairs;
+        if (set_pairs) t->tune_pairs = c.pairs;
         use_schedule(t);
     };
     for (size_t k = 0; k < cand.size() && rc == ASKIT_OK; ++k) {
