@@ -387,7 +387,10 @@ typedef struct {
     int64_t pairs_algorithmic;/* sum over targets of near + far source points */
     int64_t pairs_computed;   /* 128 x 128 target-source slots the items cover */
     int64_t near_total, far_total; /* sum over targets of |Near(i)| and |Far(i)| */
-    int64_t device_bytes;     /* library-owned device memory */
+    int64_t device_bytes;     /* device memory of the tree's arrays and of the pool of
+                                 its out-of-sample calls (at most 1 GiB kept between
+                                 them, given back where an allocation of the tree or
+                                 of its weight contexts would fail otherwise) */
     int64_t n_batches;        /* in-sample target batches (askit_params.batch_entries) */
     double setup_ms[7];       /* askit_setup's wall time by stage: kNN, tree, node lists
                                  (Algorithm 2), sampled rows (eq. 2.4), skeletons and

@@ -120,12 +120,20 @@ struct DevArena {
     bool async = false;
     cudaStream_t stream = nullptr;
     cudaMemPool_t pool = nullptr;
+    // otherwise: a pool whose unused memory is given back before an allocation fails
+    cudaMemPool_t trim = nullptr;
     template <class T>
     askit_status alloc(T **p, size_t count) {
         *p = nullptr;
         if (count == 0) count = 1;
         void *q = nullptr;
         cudaError_t e = async ? cudaMallocFromPoolAsync(&q, count * sizeof(T), pool, stream) : cudaMalloc(&q, count * sizeof(T));
+        if (e == cudaErrorMemoryAllocation && !async && trim) {
+            cudaGetLastError();
+            cudaDeviceSynchronize();                       // frees still in their streams' order
+            cudaMemPoolTrimTo(trim, 0);
+            e = cudaMalloc(&q, count * sizeof(T));
+        }
         if (e != cudaSuccess) {
             askit_set_error("cudaMalloc(%zu bytes): %s", count * sizeof(T), cudaGetErrorString(e));
             return e == cudaErrorMemoryAllocation ? ASKIT_ERR_OOM : ASKIT_ERR_CUDA;

@@ -433,6 +433,7 @@ askit_status askit_setup(const float *X_dev, int64_t N, int32_t d, int64_t ldx, 
     }
     cudaStream_t s = (cudaStream_t)stream;
     askit_status rc = make_pool(t);
+    t->arena.trim = t->dw.arena.trim = t->pool;
     if (rc == ASKIT_OK) rc = setup_impl(t, X_dev, ldx, h_dev, knn_dev, s);
     if (rc != ASKIT_OK) {
         cudaStreamSynchronize(s);
@@ -604,7 +605,10 @@ askit_status askit_get_info(askit_tree t, askit_info *info) {
         info->near_total += w.near_tot;
         info->far_total += w.far_tot;
     }
-    info->device_bytes = (int64_t)t->arena.bytes;
+    // the out-of-sample pool too, with what it keeps for the next call
+    uint64_t pooled = 0;
+    ASK_CUDA(cudaMemPoolGetAttribute(t->pool, cudaMemPoolAttrReservedMemCurrent, &pooled));
+    info->device_bytes = (int64_t)(t->arena.bytes + pooled);
     info->n_batches = (int64_t)t->wl.size();
     info->fp16_centering = use_g16(t) ? 2 : 1;
     info->pad_ = 0;
@@ -720,6 +724,7 @@ askit_status askit_weights_create(askit_tree t, askit_weights *out) {
     if (!t || !out) { askit_set_error("tree and out must be non-NULL"); return ASKIT_ERR_INVALID_ARG; }
     askit_weights w = new askit_weights_s();
     w->t = t;
+    w->ctx.arena.trim = t->pool;
     *out = w;
     return ASKIT_OK;
 }
@@ -952,6 +957,7 @@ askit_status askit_graph_create(askit_tree t, const float *W_dev, int32_t r, int
     }
     askit_graph g = new askit_graph_s();
     g->t = t;
+    g->ctx.arena.trim = t->pool;
     askit_status rc = ASKIT_OK;
     cudaGraph_t graph = nullptr;
     // uncaptured step: grows the context's buffers, builds operand state
@@ -1031,15 +1037,18 @@ askit_status askit_footprint(askit_tree t, int32_t kind, int64_t n, int32_t r, s
         if (t->n_sub > 0 && t->d <= TC_K)
             b += sizeof(float4) * (size_t)t->n_sub * 128 + (r > 1 ? sizeof(float) * (size_t)t->n_sub * (128 * 16 + 16) : 0);
     } else {
-        // an out-of-sample batch of n targets: queries, kNN, prune sets and
-        // work lists (entries estimated from the in-sample rate, doubled)
+        // an out-of-sample batch of n targets (entries estimated from the in-sample
+        // rate, doubled).  Neighbors: 1024 candidates a query, the queries' split rows,
+        // bounds, counts and lists, the leaves' radii (d > 64: best-32 lists)
         const double ent = 2.0 * per_target * n + 1024;
-        // kNN shortlist: candidates (1024 a query), seed lists, padded rows, and
-        // the dense work items (every leaf sub-block against each 128 queries)
-        const double knn = (double)n * (1024 * 4 + 32 * 12 + (size_t)t->d_pad * 4 + 32) +
-                           (double)t->n_leaf_sub * ((n + 127) / 128) * sizeof(EvalItem);
-        b = (size_t)(n * ((size_t)t->d * 4 + (size_t)t->d_pad * 4 + (size_t)t->kappa * (4 + 8 + 4 + 4) + 64) +
-                     ent * (8 * 4 + 4 + 4 * r + 32 / 128.0) + knn + (1 << 20));
+        const bool narrow = t->d <= TC_K;
+        const double knn = narrow ? (double)n * (1024 * 4 + 2 * 2 * TC_K + 48) + 4.0 * ((int64_t)1 << t->L) : 32.0 * 12 * n;
+        // target rows, their split forms, neighbors, order and prune sets
+        const double rows = (double)n * ((size_t)t->d * 4 + (size_t)t->d_pad * 4 + (size_t)t->kappa * 16 + 48 +
+                                         (narrow ? 2 * 2 * TC_K + 32 : 0));
+        // an entry: five 32-bit values and the sort's two, slot and target, its partials,
+        // its share of an item
+        b = (size_t)(rows + knn + ent * (9 * 4 + 4 * r + 32 / 128.0) + (1 << 20));
     }
     *bytes = b;
     return ASKIT_OK;
