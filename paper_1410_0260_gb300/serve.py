@@ -97,6 +97,9 @@ class Server:
             self.stop = True
             self.cv.notify_all()
         self._sched.join()
+        with self.cv:                          # batches still running use their slots' contexts
+            while any(s.busy for s in self.slots):
+                self.cv.wait()
         for s in self.slots:
             if s.stream is not None:
                 s.stream.synchronize()
@@ -146,9 +149,10 @@ class Server:
             started = []
             try:
                 with self.cv:
-                    while not self.stop and (not self.queue or not any(not s.busy for s in self.slots)):
+                    # also while stopping: what waits is served when a slot gets free
+                    while (not self.queue and not self.stop) or (self.queue and all(s.busy for s in self.slots)):
                         self.cv.wait()
-                    if self.stop and not self.queue:
+                    if not self.queue:
                         return
                     # a batch for every free slot before any of them runs: a short batch
                     # would otherwise be over before the next one is formed
