@@ -349,8 +349,8 @@ def id_fp64_cost(tree, w, secs):
 def _id_fp64_cost(tree, w, secs):
     """FP64 operations of the skeletonization's ID (Section 2.1, as the
     kernels run it: every product and sum a separate rounded instruction, no
-    FMA, so the pivots match the oracle's) from the skeleton structure, and
-    their rate against GB300's FP64 instruction rate over `secs` seconds (the
+    FMA, so the pivots match the oracle's; exact norms only of possible pivots)
+    from the skeleton structure, and their rate against GB300's FP64 instruction rate over `secs` seconds (the
     setup's skeleton stage, which also builds the node lists' samples)."""
     from paper_1410_0260_gb300 import askit
     s = tree.structure(askit.STRUCT_SKEL_S).astype(np.int64)
@@ -364,9 +364,11 @@ def _id_fp64_cost(tree, w, secs):
         if ell <= 0 or c[a] <= 0:
             continue
         k = np.arange(min(s[a] + 1, ell, c[a]), dtype=np.float64)
-        # each pivot step: trailing norms (mul + add), and for the other
-        # columns the reflector's dot product and update (2 mul/add pairs)
-        ops += float(np.sum(2 * (ell - k) * (c[a] - k) + 4 * (ell - k) * np.maximum(c[a] - k - 1, 0)))
+        # the first step's norms of all columns (mul + add); each later step's of the
+        # columns that its FP32 norms leave as candidates, counted as one; and each
+        # step's dot product with the reflector and update of the other columns (2
+        # mul/add pairs)
+        ops += float(2 * ell * c[a] + np.sum(2 * (ell - k[1:])) + np.sum(4 * (ell - k) * np.maximum(c[a] - k - 1, 0)))
         ops += float(s[a] * s[a] * (c[a] - s[a]))      # back substitution for P
         ops += float(ell * c[a] * (3 * w.d + 30))      # the kernel block: distances and the exponential
     return {"id_fp64_ops": ops, "id_fp64_instr_per_s": ops / secs if secs > 0 else None,
