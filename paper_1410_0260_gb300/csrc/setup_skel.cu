@@ -510,7 +510,15 @@ template <int C>
 askit_status launch_cpqr(int nb, size_t smem, cudaStream_t s, const int32_t *nodes, const int64_t *woff,
                          const int64_t *pws, askit_tree t, const int32_t *ell, int s_max, double *work, int32_t *piv,
                          int cmax) {
-    ASK_CUDA(cudaFuncSetAttribute(cpqr_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the most a block can have, whatever this launch takes: setups of several threads
+    // share the attribute
+    static std::atomic<uint64_t> opted{0};
+    cudaFuncAttributes fa;
+    int dev = 0, most = 0;
+    ASK_CUDA(cudaFuncGetAttributes(&fa, cpqr_kernel<C>));
+    ASK_CUDA(cudaGetDevice(&dev));
+    ASK_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    ASK_TRY(opt_in_smem(cpqr_kernel<C>, (size_t)most - fa.sharedSizeBytes, opted));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(nb * C));
     cfg.blockDim = dim3(QR_THREADS);
