@@ -368,8 +368,8 @@ askit_status askit_set_precision(askit_tree t, int32_t precision);
  *     target rows reach the tensor cores without conversion (the fastest;
  *     relative error of u about 1e-5 against about 1e-6 for mode 1, both
  *     within the split-product tolerance 1e-4).
- * Out-of-sample batches with a target outside the FP16-safe range of mode 2
- * (beyond about 7 times the data's extent from its mean) take mode 1.
+ * Out-of-sample batches with a target outside the FP16-safe range (beyond about
+ * 7 times the data's extent) are evaluated in 3xTF32, for d > 64 in plain FP32.
  * Host call; applies to later evaluations.
  */
 askit_status askit_set_fp16_centering(askit_tree t, int32_t mode);

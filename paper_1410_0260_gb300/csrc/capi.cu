@@ -87,6 +87,13 @@ __global__ void gather_y_kernel(const float *Y, int64_t ldy, int d, int d_pad, c
     out[e] = (row < T && k < d) ? Y[(int64_t)order[row] * ldy + k] : 0.f;
 }
 
+// Whether a coordinate leaves the range that the sub-block-centered FP16 splits hold:
+// |x| scale <= 30000, with the centers' at most 8192 below FP16's 65504.
+__global__ void far_targets_kernel(const float *Y, int64_t n, float scale, int *far) {
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e < n && !(fabsf(Y[e]) * scale <= 30000.f)) *far = 1;
+}
+
 // Rows X[ids[q]] of the caller-order points; an id out of range sets *bad
 // and gives a zero row.
 __global__ void gather_points_kernel(const float *X, int64_t N, int d, const int32_t *ids, int64_t Q, float *Y,
@@ -496,7 +503,7 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     int *flags = nullptr, h_flags[2] = {0, 0};     // target outside the FP16-safe range; list not filled
     QuerySplit qs;
     int64_t T_pad = (T + ASK_TILE_M - 1) / ASK_TILE_M * ASK_TILE_M;
-    int pos_bits = 1;
+    int pos_bits = 1, prec = t->precision;
     while (((int64_t)1 << pos_bits) < t->N) ++pos_bits;
     askit_status rc = ASKIT_OK;
 #define OTRY(x) do { rc = (x); if (rc != ASKIT_OK) goto out; } while (0)
@@ -520,6 +527,8 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
         OTRY(tmp.alloc(&yg_lo, (size_t)T_pad * TC_K));
         OTRY(tmp.alloc(&yg_x, (size_t)T_pad * 16));
         OTRY(g16_split_rows(Yc, d, d, T_pad, t, yg_hi, yg_lo, yg_x, flags, s, order, T));
+    } else if (t->precision == ASKIT_PREC_FP16X3) {
+        far_targets_kernel<<<nblk(T * d, 256), 256, 0, s>>>(Yc, T * d, t->f16_scale, flags);
     }
     OTRY(tmp.alloc(&sets, (size_t)T * kappa));
     OTRY(oos_prune_sets(t, ids, dist, order, T, kappa, sets, flags + 1, s));
@@ -533,21 +542,23 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
         rc = ASKIT_ERR_INVALID_ARG;
         goto out;
     }
-    if (g16) {
-        if (!h_flags[0]) {
-            qs.hi = yg_hi;
-            qs.lo = yg_lo;
-            qs.x = yg_x;
-            qs.rows = T_pad;
-        }
+    // a batch that reaches outside the FP16-safe range (far from the data) takes a
+    // precision with FP32's range: its splits would be infinite, the result no number
+    // (what FP16x3 refuses, r > 16 and rows too wide to split, it refuses far out too)
+    if (h_flags[0] && c.r <= 16 && t->Xt_hhi) {
+        prec = d <= TC_K ? ASKIT_PREC_TF32X3 : ASKIT_PREC_SIMT_FP32;
+    } else if (g16 && !h_flags[0]) {
+        qs.hi = yg_hi;
+        qs.lo = yg_lo;
+        qs.x = yg_x;
+        qs.rows = T_pad;
     }
     if (!qs.hi) {
-        // FP32 rows for the other kernels: other precisions, or a batch that
-        // reaches outside the FP16-safe range (far from the data)
+        // FP32 rows for the other kernels
         OTRY(tmp.alloc(&Yt, (size_t)T_pad * t->d_pad));
         gather_y_kernel<<<nblk(T_pad * t->d_pad, 256), 256, 0, s>>>(Yc, d, d, t->d_pad, order, T, T_pad, Yt);
     }
-    OTRY(run_eval(t, c, t->precision, Yt, t->d_pad, T_pad, qs.hi ? &qs : nullptr, w, partial, order, U_dev, ldu, s));
+    OTRY(run_eval(t, c, prec, Yt, t->d_pad, T_pad, qs.hi ? &qs : nullptr, w, partial, order, U_dev, ldu, s));
     if (cudaStreamSynchronize(s) != cudaSuccess) { askit_set_error("out-of-sample evaluate: %s", cudaGetErrorString(cudaGetLastError())); rc = ASKIT_ERR_CUDA; }
 out:
 #undef OTRY
