@@ -498,6 +498,7 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
     void *cub = nullptr;
     size_t cb = 0;
     WorkLists w;
+    WeightCtx own;
     float *partial = nullptr;
     uint16_t *yg_hi = nullptr, *yg_lo = nullptr, *yg_x = nullptr;
     int *flags = nullptr, h_flags[2] = {0, 0};     // target outside the FP16-safe range; list not filled
@@ -558,7 +559,17 @@ askit_status evaluate_targets_ctx(askit_tree t, const WeightCtx &c, const float 
         OTRY(tmp.alloc(&Yt, (size_t)T_pad * t->d_pad));
         gather_y_kernel<<<nblk(T_pad * t->d_pad, 256), 256, 0, s>>>(Yc, d, d, t->d_pad, order, T, T_pad, Yt);
     }
-    OTRY(run_eval(t, c, prec, Yt, t->d_pad, T_pad, qs.hi ? &qs : nullptr, w, partial, order, U_dev, ldu, s));
+    if (prec != t->precision && d <= TC_K) {
+        // the other kernel's column data differ from what calls on other streams keep in
+        // the context: its own
+        own.Wt = c.Wt;
+        own.Ws = c.Ws;
+        own.r = c.r;
+        OTRY(tmp.alloc(&own.colv, (size_t)std::max<int64_t>(1, t->n_sub) * 128));
+        if (c.r > 1) OTRY(tmp.alloc(&own.colw, (size_t)std::max<int64_t>(1, t->n_sub) * 128 * (c.r <= 4 ? 4 : 16)));
+    }
+    OTRY(run_eval(t, own.colv ? own : c, prec, Yt, t->d_pad, T_pad, qs.hi ? &qs : nullptr, w, partial, order, U_dev, ldu,
+                  s));
     if (cudaStreamSynchronize(s) != cudaSuccess) { askit_set_error("out-of-sample evaluate: %s", cudaGetErrorString(cudaGetLastError())); rc = ASKIT_ERR_CUDA; }
 out:
 #undef OTRY
