@@ -295,13 +295,17 @@ askit_status askit_graph_destroy(askit_graph g);
  *               kernel for d > 64 (FP16x3 and BF16x3, any r <= 16), which
  *               then copies and splits each target row once for both.
  * Only the schedule (and, for d > 64, pairs) varies for the other tensor-core
- * kernels; the plain FP32 kernel has one configuration.  Schedules, stages and tiled runs change no
- * result bit (every work item is computed the same way; partials are reduced
- * in a fixed order); paired items sum both sub-blocks' columns in one
- * accumulator, which changes the FP32 summation order only.  Until this or
- * askit_set_launch is called, lists are dealt heaviest first and paired items
- * are taken where most items have a partner.  `reps` timed evaluations per candidate after one warm-up; at most
- * `max_out` entries are written to `out`, the count to `n_out`.  Blocks.
+ * kernels; the plain FP32 kernel has one configuration.  Schedules, stages
+ * and tiled runs change no result bit (every work item is computed the same
+ * way; partials are reduced in a fixed order), nor do the paired items of the
+ * global-centered and the K-chunked kernel (a partial sum a sub-block); those
+ * of the per-sub-block kernel sum both sub-blocks' columns in one accumulator,
+ * which changes the FP32 summation order only.  Until this or askit_set_launch
+ * is called, lists are dealt heaviest first, and the global-centered and the
+ * K-chunked kernel take paired items where most items have a partner.  What
+ * the tree's precision and r do not vary keeps its value.  `reps` timed
+ * evaluations per candidate after one warm-up; at most `max_out` entries are
+ * written to `out`, the count to `n_out`.  Blocks.
  */
 typedef struct {
     int32_t schedule, stages, tiled_runs, pairs, chosen;

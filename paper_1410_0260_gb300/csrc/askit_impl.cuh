@@ -58,7 +58,8 @@ inline askit_status opt_in_smem(void (*k)(KArgs...), size_t bytes, std::atomic<u
 // this way calls pdl_wait() in every thread before it reads or writes anything
 // that an earlier kernel of the stream touches; what it does before that
 // (barriers, TMEM, operands fixed at setup) overlaps the earlier kernel's tail.
-// The first kernel of a call is launched normally.
+// set_weights starts with a normal launch; Evaluate with its column data, launched this
+// way: before its wait that kernel reads constants of the tree alone.
 template <class... KArgs, class... Args>
 inline askit_status launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                const Args &...args) {

@@ -119,9 +119,8 @@ askit_status validate(const askit_params *p, int64_t N, int32_t d, int64_t ldx, 
         return ASKIT_ERR_INVALID_ARG;
     }
     if (p->s_max < 1 || p->s_min < 0 || p->ell_extra < 0) { askit_set_error("need s_max >= 1, s_min >= 0, ell_extra >= 0"); return ASKIT_ERR_INVALID_ARG; }
-    // a source block (a leaf's points or a skeleton) is cut into at most 16
-    // sub-blocks of ASK_BLK_N rows (the work lists keep the sub-block index in
-    // 4 bits), and a node's heap index must fit the lists' 27-bit node field
+    // a source block (a leaf's points or a skeleton) is cut into at most 16 sub-blocks
+    // of ASK_BLK_N rows; the work lists index sub-blocks and nodes in 32 bits
     if (p->leaf_size > 16 * ASK_BLK_N || p->s_max > 16 * ASK_BLK_N) {
         askit_set_error("leaf_size and s_max must be at most %d", 16 * ASK_BLK_N);
         return ASKIT_ERR_UNSUPPORTED;

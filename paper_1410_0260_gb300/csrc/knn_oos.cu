@@ -857,10 +857,13 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
                                                                         hx);
     // Queries in the order of their home leaves: the 128 of a tile then have their
     // candidates in the same few source tiles, and nearly all other tile pairs skip
-    // the hit path; the seed's leaves are shared by neighboring warps.  Worth it from
-    // 2^31 (query, point) pairs: 100,000 x 131,072 saves 0.65 ms (shortlist 4.27 ->
-    // 3.80, seed 1.17 -> 0.99) for a sort of about 20 us, and the saving is in
-    // proportion to the pairs, the sort's few launches are not.
+    // the hit path; the seed's leaves are shared by neighboring warps.  The saving is
+    // in proportion to the (query, point) pairs, the sort's few launches (about 20 us)
+    // are not.  knn_targets against 131,072 points of 64 dimensions, in the given order
+    // and sorted: 3,001 queries 557 and 567 us, 5,000 735 and 730, 10,000 (1.3e9 pairs)
+    // 1073 and 1026, 16,400 (2.1e9) 1510 and 1405, 100,000 7.15 and 6.43 ms; against
+    // 1M, 2,500 (2.6e9) 1343 and 1334 us, 20,000 15.05 and 14.86 ms.  It pays from
+    // about 10^9 pairs on; the line lies at 2^31, where it does at every size measured.
     if (t->L > 0 && T >= 16 * sms && T * N >= (int64_t)1 << 31) {
         // the sort's buffers lie in the candidate lists, which are written later
         const size_t T4 = ((size_t)T * 4 + 255) / 256 * 256;
@@ -878,6 +881,10 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
     }
     ko_split_kernel<<<nblk(T_pad, 8), 256, 0, s>>>(Y, d, order, T, T_pad, t->g_xbar, t->g_sigma, qh, ql, nq, cnt);
     {
+        // Below 16 queries an SM one warp a query leaves the GPU short of warps.  Against
+        // 131,072 points, four warps and one: 500 queries 373 and 393 us, 1,000 408 and
+        // 433, 1,500 444 and 454, 2,432 (the line) 505 and 502, 5,000 725 and 726,
+        // 16,400 1452 and 1402
         const bool few = T < 16 * sms;
         auto seed = d <= 32 ? (few ? ko_seed_kernel<1, 4> : ko_seed_kernel<1, 1>)
                             : (few ? ko_seed_kernel<2, 4> : ko_seed_kernel<2, 1>);
@@ -913,6 +920,9 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
         QCHK(cudaGetLastError());
     }
     {
+        // One warp a block or eight: against 131,072 points within 1 % either way from 500
+        // queries on (500 380 and 372 us, 2,432 510 and 505, 16,400 1391 and 1403); against
+        // 1M, 500 queries 605 and 628
         const bool few = T < 16 * sms;
         auto rerank = t->d_pad == 32 ? (few ? ko_rerank_kernel<1, 1> : ko_rerank_kernel<1, 8>)
                                      : (few ? ko_rerank_kernel<2, 1> : ko_rerank_kernel<2, 8>);

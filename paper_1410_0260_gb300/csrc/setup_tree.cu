@@ -305,7 +305,11 @@ __global__ void __launch_bounds__(256) knn_leaf_kernel(const float *X, int d, co
 // distance and recomputes the survivors in canonical FP64.  Each split
 // writes its own best-32 lists; knn_merge_kernel merges the splits.
 constexpr int KT_Q = 64, KT_C = 128, KT_K = 32;
-// points a segment above which a tree level is sorted as a whole
+// Points a segment above which a tree level is sorted as a whole.  64K x 64, leaves of
+// 128, six RP trees (kNN stage) and the tree itself, line at 256, 512, 1024, 2048, 4096,
+// 8192 and 16384: 20.6, 19.2, 18.2, 17.1, 16.3, 15.8 and 16.4 ms; 11.1, 10.9, 10.7, 10.6,
+// 10.4, 10.4 and 10.5 ms.  1M: 155 to 151 ms and 147 to 146 ms.  Segments of 2048 and
+// less are better off sorted one a block; 8192 would gain another 1.2 ms of that build.
 constexpr int64_t TREE_RADIX = 2048;
 
 __global__ void __launch_bounds__(256) knn_tiled_kernel(const float *X, int64_t N, int d, const float *Y,
@@ -579,9 +583,9 @@ askit_status build_tree_gpu(const float *X, int64_t N, int d, int L, int kind, u
             }
             TCHK(cudaGetLastError(), "projection kernels");
             if (N / nseg > TREE_RADIX) {
-                // Few large segments: the segmented sort takes one block for each
-                // (a 64K segment about 1 ms, a 1M one 16 ms), so the whole level is
-                // radix-sorted by key, then stably by segment.
+                // Few large segments: the segmented sort takes one block for each (a
+                // 64K segment about 1 ms, a 1M one 16 ms), so the whole level is radix-
+                // sorted by key, then stably by segment (the line: TREE_RADIX).
                 iota_kernel<<<nblk(N, 256), 256, 0, s>>>(sc.pos0, N);
                 if ((rc = sort_f64_i32(sc.keys, sc.keys_out, sc.pos0, sc.pos1, N, sc.cub, &sc.cub_bytes, s)) != ASKIT_OK) goto done;
                 seg_gather_kernel<<<nblk(N, 256), 256, 0, s>>>(sc.pos1, sc.seg, order, N, sc.skey0, sc.pos0);
