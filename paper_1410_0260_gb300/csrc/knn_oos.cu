@@ -195,7 +195,10 @@ __global__ void ko_key_kernel(const float *hd, const int32_t *hi_, int nsplit, i
 // halves of eight lines, twice the cycles in the load unit, which bound the seed at
 // 91 %: 1.74 ms for 100,000 queries, 1.17 with this and the gathered offers below); the lanes' sums meet in a transposing butterfly.  Lane l ends with the
 // distance of pos(4 (l & 7) + (l >> 3)).
-template <int NJ, class F>
+// PACK: two coordinates an instruction, which the leaf scan gains from (50,000 queries
+// in a cluster of 65,536 points, 16 dimensions 32.5 -> 29.9 ms, 64 dimensions 86 -> 69)
+// and the seed and the re-rank lose by (100,000 queries 8.1 -> 8.6 ms).
+template <int NJ, bool PACK, class F>
 __device__ __forceinline__ float rows32(const float *Xt, const float4 (&y)[NJ], int lane, F pos) {
     const int sub = lane & 7, r4 = lane >> 3;
     float4 x[8][NJ];
@@ -209,14 +212,24 @@ __device__ __forceinline__ float rows32(const float *Xt, const float4 (&y)[NJ], 
 #pragma unroll
     for (int g = 0; g < 8; ++g) {
         a[g] = 0.f;
+        float2 s = make_float2(0.f, 0.f);
+        const float2 m1 = make_float2(-1.f, -1.f);
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
-            const float t0 = y[j].x - x[g][j].x, t1 = y[j].y - x[g][j].y, t2 = y[j].z - x[g][j].z, t3 = y[j].w - x[g][j].w;
-            a[g] = fmaf(t0, t0, a[g]);
-            a[g] = fmaf(t1, t1, a[g]);
-            a[g] = fmaf(t2, t2, a[g]);
-            a[g] = fmaf(t3, t3, a[g]);
+            if (!PACK) {
+                const float t0 = y[j].x - x[g][j].x, t1 = y[j].y - x[g][j].y, t2 = y[j].z - x[g][j].z, t3 = y[j].w - x[g][j].w;
+                a[g] = fmaf(t0, t0, a[g]);
+                a[g] = fmaf(t1, t1, a[g]);
+                a[g] = fmaf(t2, t2, a[g]);
+                a[g] = fmaf(t3, t3, a[g]);
+                continue;
+            }
+            const float2 t0 = __ffma2_rn(make_float2(x[g][j].x, x[g][j].y), m1, make_float2(y[j].x, y[j].y));
+            const float2 t1 = __ffma2_rn(make_float2(x[g][j].z, x[g][j].w), m1, make_float2(y[j].z, y[j].w));
+            s = __ffma2_rn(t0, t0, s);
+            s = __ffma2_rn(t1, t1, s);
         }
+        if (PACK) a[g] = s.x + s.y;
     }
     // lanes with bit m of sub set keep the upper half of the values left
 #pragma unroll
@@ -306,7 +319,7 @@ __global__ void __launch_bounds__(256) ko_seed_kernel(const float *Xt, const flo
         const int p0 = nstart[M + leaf[h]], np = nsize[M + leaf[h]];
         for (int b = 32 * (warp % W); b < np; b += 32 * W) {
             // rows past the leaf are other points or the zero rows past N
-            const float v = rows32<NJ>(Xt, y, lane, [&](int i) { return p0 + b + i; });
+            const float v = rows32<NJ, false>(Xt, y, lane, [&](int i) { return p0 + b + i; });
             const int i = b + 4 * (lane & 7) + (lane >> 3);
             gather_f32(l, i < np ? v : 3.4e38f, lists[warp], have, kappa, lane);
         }
@@ -333,7 +346,7 @@ __global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, cons
                                                            const int32_t *order, int64_t T, const int32_t *perm,
                                                            const int *cnt, const int32_t *cand, int kappa,
                                                            int32_t *ids, double *dist, int *n_ovf, int32_t *ovf,
-                                                           int32_t *wide) {
+                                                           int32_t *wide, const float *U, bool many) {
     __shared__ float sd[W][KO_CAP];
     __shared__ float sy[W][TC_K];
     __shared__ float sl[W][64];
@@ -343,7 +356,10 @@ __global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, cons
     if (q >= T) return;                                    // warp-uniform
     const int64_t src = order ? order[q] : q;
     const int n = cnt[q];
-    if (n >= KO_BAD || n < kappa) {                        // (fewer cannot be: U bounds kappa points)
+    // (fewer than kappa cannot be: U bounds kappa points.)  Where the home leaves hold
+    // fewer than kappa points U bounds nothing, no leaf can be left out, and many such
+    // queries are better off in the exhaustive search's tiles
+    if (n >= KO_BAD || n < kappa || (n > KO_CAP && many && !(U[q] < 3.0e38f))) {
         if (lane == 0) ovf[atomicAdd(n_ovf, 1)] = (int32_t)src;
         return;
     }
@@ -358,7 +374,7 @@ __global__ void __launch_bounds__(32 * W) ko_rerank_kernel(const float *Xt, cons
     float l = 3.4e38f;
     for (int b = 0; b < n; b += 32) {
         const int32_t mine = c[min(b + lane, n - 1)];
-        const float v = rows32<NJ>(Xt, y, lane, [&](int i) { return __shfl_sync(FULL, mine, i); });
+        const float v = rows32<NJ, false>(Xt, y, lane, [&](int i) { return __shfl_sync(FULL, mine, i); });
         const int i = b + 4 * (lane & 7) + (lane >> 3);
         if (i < n) sd[warp][i] = v;
         gather_f32(l, i < n ? v : 3.4e38f, sl[warp], have_l, kappa, lane);
@@ -425,12 +441,14 @@ __global__ void ko_radius_kernel(const float *nrmc, const int32_t *nstart, const
 
 // A query with too many candidates, a block per query: its warps take the leaves in
 // turn, 32 centers at a time (a lane each), and scan those that |y - c| - radius leaves
-// within sqrt(U).  FP32 distances within U, and within the warp's kappa-th FP64 one so
-// far, get their FP64 distance, 32 to a batch; the warps' lists are merged at the end.
+// within sqrt(U), or the root of the warp's kappa-th FP64 distance so far.  FP32
+// distances within the same limit get their FP64 distance, 32 to a batch; the warps'
+// lists are merged at the end.
 // Overflow comes with tight clusters or few intrinsic dimensions, where the balls rule
 // out nearly all leaves: 3,001 queries against 1M points of a curve in 3 dimensions
-// took 38.4 ms with the exhaustive search here, 1.7 so; 50,000 against 64 clusters of
-// 2,048 points 88.3 ms and 8.2.
+// took 38.4 ms with the exhaustive search here, 1.6 so; 50,000 against 64 clusters of
+// 2,048 points 88.3 ms and 7.6.  Where they rule out little -- two clusters of 65,536
+// points in 16 and in 64 dimensions -- 50,000 queries take 29.9 and 69 ms (92 and 231).
 constexpr int BA_WARPS = 8;
 template <int NJ>
 __global__ void __launch_bounds__(32 * BA_WARPS) ko_ball_kernel(const float *Xt, const float *Y, int d,
@@ -448,8 +466,8 @@ __global__ void __launch_bounds__(32 * BA_WARPS) ko_ball_kernel(const float *Xt,
     float4 y[NJ];
     load_query<NJ>(Y + src * d, d, lane, y);
     __syncthreads();
-    const float gam = sum_gam(d), su = sqrtf(U[q]) * (1.f + 2e-6f);
-    const float u = U[q] * (1.f + gam) + 1e-37f;           // FP32 distances of the kappa nearest are within this
+    const float gam = sum_gam(d);
+    float lim = U[q] * (1.f + gam) + 1e-37f;               // FP32 distances of the kappa nearest are within this
     double ld = DBL_MAX;
     int li = INT_MAX, have = 0;
     int32_t held = 0;                                      // lane < have: a candidate's tree position
@@ -462,6 +480,10 @@ __global__ void __launch_bounds__(32 * BA_WARPS) ko_ball_kernel(const float *Xt,
         }
         warp_offer(ld, li, cd, ci, kappa, false, lane);
         have = 0;
+        // the limit follows the list here alone: its two FP64 instructions would hold the
+        // warp's quarter of the SM in every step of the scan
+        const double kth = __shfl_sync(FULL, ld, kappa - 1);
+        if (kth < 1e38) lim = fminf(lim, __double2float_ru(kth) * (1.f + 2.f * gam) + 1e-37f);
     };
     for (int64_t l0 = 32 * (int64_t)warp; l0 < M; l0 += 32 * BA_WARPS) {
         const int64_t l = l0 + lane;
@@ -478,7 +500,7 @@ __global__ void __launch_bounds__(32 * BA_WARPS) ko_ball_kernel(const float *Xt,
                 acc = fmaf(t2, t2, acc);
                 acc = fmaf(t3, t3, acc);
             }
-            in = !(sqrtf(acc) * (1.f - gam - 4e-6f) - rad[l] > su);
+            in = !(sqrtf(acc) * (1.f - gam - 4e-6f) - rad[l] > sqrtf(lim) * (1.f + 2e-6f));
         }
         unsigned m = __ballot_sync(FULL, in);
         while (m) {
@@ -487,10 +509,8 @@ __global__ void __launch_bounds__(32 * BA_WARPS) ko_ball_kernel(const float *Xt,
             const int p0 = nstart[M + leaf], np = nsize[M + leaf];
             for (int b = 0; b < np; b += 32) {
                 // rows past the leaf are other points or the zero rows past N
-                const float v = rows32<NJ>(Xt, y, lane, [&](int i) { return p0 + b + i; });
+                const float v = rows32<NJ, true>(Xt, y, lane, [&](int i) { return p0 + b + i; });
                 const int i = b + 4 * (lane & 7) + (lane >> 3);
-                const double kth = __shfl_sync(FULL, ld, kappa - 1);
-                const float lim = kth < 1e38 ? fminf(u, __double2float_ru(kth) * (1.f + 2.f * gam) + 1e-37f) : u;
                 const unsigned hit = __ballot_sync(FULL, i < np && v <= lim);
                 // the lanes' rows are not in lane order: positions travel with the hits
                 if (hit) warp_collect(hit, p0 + i, have, held, lane, offer);
@@ -617,7 +637,7 @@ ko_shortlist_kernel(const __grid_constant__ CUtensorMap map_qh, const __grid_con
         auto flush = [&]() {
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                uint32_t m = ph[c];
+                uint32_t m = pk < KO_CAP ? ph[c] : 0u;     // a full list takes no more
                 while (m) {
                     const int j = __ffs(m) - 1;
                     m &= m - 1;
@@ -920,6 +940,9 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
         QCHK(cudaGetLastError());
     }
     {
+        // (Queries without a bound, 131,072 x 64, leaves of 12: 100 / 3,001 / 50,000 take 2.6 /
+        // 23 / 370 ms leaf by leaf, 8.0 / 64 / 239 in the exhaustive search's tiles, whose
+        // lines cross at about 14,400: 96 an SM.)
         // One warp a block or eight: against 131,072 points within 1 % either way from 500
         // queries on (500 380 and 372 us, 2,432 510 and 505, 16,400 1391 and 1403); against
         // 1M, 500 queries 605 and 628
@@ -927,7 +950,7 @@ askit_status knn_oos(askit_tree t, const float *Y, int64_t T, int kappa, int32_t
         auto rerank = t->d_pad == 32 ? (few ? ko_rerank_kernel<1, 1> : ko_rerank_kernel<1, 8>)
                                      : (few ? ko_rerank_kernel<2, 1> : ko_rerank_kernel<2, 8>);
         rerank<<<nblk(T, few ? 1 : 8), few ? 32 : 256, 0, s>>>(t->Xt, Y, d, order, T, t->perm, cnt, cand, kappa, ids, dist,
-                                                              n_ovf, ovf, wide);
+                                                              n_ovf, ovf, wide, U, T >= 96 * sms);
     }
     QCHK(cudaGetLastError());
     QCHK(cudaMemcpyAsync(h_n, n_ovf, sizeof h_n, cudaMemcpyDeviceToHost, s));

@@ -81,3 +81,22 @@ def test_overflowing_queries_do_not_cost_the_exhaustive_search():
         a, b = best(lambda: t.knn_targets(Y)), best(lambda: t.knn_points(rows))
         t.close()
         assert a < 0.5 * b, (a, b)
+
+
+@pytest.mark.parametrize("T", [300, 15001])
+def test_queries_without_a_bound_match_the_oracle(T):
+    """Home leaves of fewer than kappa points bound nothing: few such queries scan the
+    leaves, many take the exhaustive search."""
+    import oracle
+    from paper_1410_0260_gb300 import askit
+    rng = np.random.default_rng(T)
+    X = rng.standard_normal((3000, 5)).astype(np.float32)
+    X[1:50:2] = X[0:49:2]
+    Y = rng.standard_normal((T, 5)).astype(np.float32)
+    t = askit.Tree(torch.from_numpy(X).cuda(), askit.Config(leaf_size=8, kappa=32, s_max=8, h=1.0))
+    ids, dist = t.knn_targets(torch.from_numpy(Y).cuda())
+    t.sync()
+    t.close()
+    oi, od = oracle.knn_exact(X, 32, Y=Y)
+    assert np.array_equal(ids.cpu().numpy(), oi)
+    assert np.array_equal(dist.cpu().numpy(), od)
